@@ -129,6 +129,7 @@ struct Lane {
   std::vector<cudaEvent_t> ev_chain[NSLOT];
   float2* stw = nullptr;                    // stage twiddle tables of R1, R2, Q1, Q2
   const float2 *stwR1 = nullptr, *stwR2 = nullptr, *stwQ1 = nullptr, *stwQ2 = nullptr, *stwJ = nullptr;
+  const float2* wtwR2 = nullptr;            // stage-2 twiddles of the 64-values-per-thread FFT of R2 (null: none)
   float2* tw2buf = nullptr;
   Tw2 tw2L;                                 // exp(-2 pi i e/(2L))
   float2* tw3L = nullptr;                   // three-level exp(-2 pi i e/L)
@@ -408,13 +409,14 @@ int build_lane(pond_t h, Lane* ln) {
   }
   const int n1 = stage_tw_entries(1 << g.logR1), n2 = stage_tw_entries(1 << g.logR2);
   const int n3 = stage_tw_entries(1 << g.logQ1), n4 = stage_tw_entries(1 << g.logQ2);
-  const int n5 = stage_tw_entries(FUSED_J);
-  CK(cudaMalloc(&ln->stw, (size_t)std::max(1, n1 + n2 + n3 + n4 + n5) * sizeof(float2)));
+  const int n5 = stage_tw_entries(FUSED_J), n6 = wide_tw_entries(1 << g.logR2);
+  CK(cudaMalloc(&ln->stw, (size_t)std::max(1, n1 + n2 + n3 + n4 + n5 + n6) * sizeof(float2)));
   ln->stwR1 = ln->stw;
   ln->stwR2 = ln->stwR1 + n1;
   ln->stwQ1 = ln->stwR2 + n2;
   ln->stwQ2 = ln->stwQ1 + n3;
   ln->stwJ = ln->stwQ2 + n4;
+  ln->wtwR2 = n6 > 0 ? ln->stwJ + n5 : nullptr;
   auto nhi = [](int logn) { return logn > TW2_LOG ? (1ll << (logn - TW2_LOG)) : 1ll; };
   const long long total = TW2_LO + nhi(g.logL + 1) + 2 * 768;
   CK(cudaMalloc(&ln->tw2buf, total * sizeof(float2)));
@@ -430,6 +432,7 @@ int build_lane(pond_t h, Lane* ln) {
   CK(launch_stage_tw(const_cast<float2*>(ln->stwQ1), 1 << g.logQ1, h->st));
   CK(launch_stage_tw(const_cast<float2*>(ln->stwQ2), 1 << g.logQ2, h->st));
   CK(launch_stage_tw(const_cast<float2*>(ln->stwJ), FUSED_J, h->st));
+  CK(launch_wide_tw(const_cast<float2*>(ln->wtwR2), 1 << g.logR2, h->st));
   CK(launch_tw3(ln->tw3L, g.logL, -1, h->st));
   CK(launch_tw2(const_cast<float2*>(ln->tw2L.lo), const_cast<float2*>(ln->tw2L.hi), g.logL + 1, -1, h->st));
   CK(launch_tw3(ln->tw3M, g.logM, +1, h->st));
@@ -621,7 +624,7 @@ cudaError_t launch_ic(pond_t h, const Lane& ln, const float2* in, float* P, floa
   if (ln.ic_tc)
     return launch_inv_cols_det_tc(ln.g, in, P, part, cnt, vout, vstride, vofs, m_lo, m_hi, h->ic_ops, h->tc_err, st,
                                   ntr);
-  return launch_inv_cols_det(ln.g, in, P, part, cnt, vout, vstride, vofs, m_lo, m_hi, ln.stwR2, st, ntr);
+  return launch_inv_cols_det(ln.g, in, P, part, cnt, vout, vstride, vofs, m_lo, m_hi, ln.stwR2, ln.wtwR2, st, ntr);
 }
 
 int run_segment(pond_t h, int li, SegIn in, long long s, long long g_end) {

@@ -24,6 +24,7 @@
 #include <stdint.h>
 
 #include "passes.cuh"
+#include "passes_wide.cuh"
 
 namespace pond {
 
@@ -49,6 +50,19 @@ __global__ void k_make_stage_tw(float2* out, int R) {
     }
     off += n;
   }
+}
+
+// Stage 2's twiddles of the (ra, rb) line FFT (fft_wide.cuh), rb = na nb: row
+// b - 1 (b = 1 .. nb-1) holds w^{b t}, row nb - 2 + a (a = 1 .. na-1) w^{nb a t},
+// t < ra, w = exp(-2 pi i / (ra rb)).
+__global__ void k_make_wide_tw(float2* out, int ra, int rb, int na, int nb) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (na + nb - 2) * ra) return;
+  const int row = i / ra, t = i % ra;
+  const int e = row < nb - 1 ? (row + 1) * t : nb * (row - nb + 2) * t;
+  double s, c;
+  sincospi(-2.0 * (double)e / (double)(ra * rb), &s, &c);
+  out[i] = make_float2((float)c, (float)s);
 }
 
 // Anchor a covers the 2^clog bins k = 2^clog a + d (d < 2^clog); it holds the
@@ -610,6 +624,29 @@ cudaError_t launch_stage_tw(float2* out, int R, cudaStream_t st) {
 
 int stage_tw_entries(int R) { return stage_table_size(R); }
 
+#define POND_WIDE_RB(X) X(8) X(16) X(32) X(64)
+
+int wide_tw_entries(int R) {
+  switch (R / 64) {
+#define CASE(RB) case RB: return WideTw<64, RB>::SIZE;
+    POND_WIDE_RB(CASE)
+#undef CASE
+    default: return 0;
+  }
+}
+
+cudaError_t launch_wide_tw(float2* out, int R, cudaStream_t st) {
+  const int n = wide_tw_entries(R);
+  switch (R / 64) {
+#define CASE(RB) \
+  case RB: k_make_wide_tw<<<(n + 255) / 256, 256, 0, st>>>(out, 64, RB, WideSplit<RB>::NA, WideSplit<RB>::NB); break;
+    POND_WIDE_RB(CASE)
+#undef CASE
+    default: return cudaSuccess;
+  }
+  return cudaGetLastError();
+}
+
 cudaError_t launch_tw2(float2* lo, float2* hi, int logn, int sign, cudaStream_t st) {
   const long long nhi = logn > TW2_LOG ? (1ll << (logn - TW2_LOG)) : 1;
   const long long n = std::max<long long>(TW2_LO, nhi);
@@ -628,9 +665,10 @@ cudaError_t launch_tables(ChirpAnchor* anc, long long nanc, int clog, double du,
   return cudaGetLastError();
 }
 
-// Fused schedule: F2f for R1 = 512..4096 with J = 64, Ic for R2 = 16..2048.
+// Fused schedule: F2f for R1 = 512..4096 with J = 64, Ic for R2 = 16..2048
+// (the radix-16 form to 512, the 64-values-per-thread form from 512).
 #define POND_FUSED_R1(X) X(512) X(1024) X(2048) X(4096)
-#define POND_FUSED_R2(X) X(16) X(32) X(64) X(128) X(256) X(512) X(1024) X(2048)
+#define POND_FUSED_R2(X) X(16) X(32) X(64) X(128) X(256) X(512)
 
 bool fused_geometry(const Geom& g) {
   return g.logM - g.logR2 == 6 && g.logR1 >= 9 && g.logR1 <= 12 && g.logR2 >= 4 && g.logR2 <= 11;
@@ -728,7 +766,7 @@ int fused_groups(const Geom& g) {
 
 cudaError_t launch_inv_cols_det(const Geom& g, const float2* in, float* P, float* part, int* cnt, float2* vout,
                                 long long vstride, long long vofs, int m_lo, int m_hi, const float2* tw,
-                                cudaStream_t st, int ntr) {
+                                const float2* wtw, cudaStream_t st, int ntr) {
   const int R2 = 1 << g.logR2, R1 = 1 << g.logR1;
   const int nl = std::min(TILE / R2, g.nchan);
   const dim3 grid((unsigned)(R1 / nl), (unsigned)ntr);
@@ -737,6 +775,28 @@ cudaError_t launch_inv_cols_det(const Geom& g, const float2* in, float* P, float
   // several trials: each has its own L-element input, M-element P, partials and tickets
   const TrialStride ts = ntr > 1 ? TrialStride{g.L, g.M, (long long)fused_groups(g) * g.M, FUSED_J}
                                  : TrialStride{0, 0, 0, 0};
+  // 512-, 1024- and 2048-point columns that fill a tile (at least TILE / R2
+  // sub-channels; always so from 1024 on) take the form with 64 values per
+  // thread: per launch of 32 trials of the 2048-point column pass 755 -> 548 us,
+  // of up to 21 trials of the 512-point one 30.7 -> 21.3 us.  Shorter columns
+  // have no 64-point first stage to fill, and half tiles leave half the threads idle.
+  if (R2 >= 512 && nl * R2 == TILE) {
+    const int logG = lognch - (13 - g.logR2);
+    switch (R2) {
+#define CASE(R)                                                                                                  \
+  case R:                                                                                                        \
+    if (vout)                                                                                                    \
+      k_inv_cols_det_w<R, true><<<grid, WIDE_NT, wide_smem_bytes<64, R / 64>(), st>>>(                          \
+          in, P, part, cnt, vout, vstride, vofs, logG, g.logM - g.logR2, m_lo, m_hi, scale, wtw, ts);            \
+    else                                                                                                         \
+      k_inv_cols_det_w<R, false><<<grid, WIDE_NT, wide_smem_bytes<64, R / 64>(), st>>>(                         \
+          in, P, part, cnt, vout, vstride, vofs, logG, g.logM - g.logR2, m_lo, m_hi, scale, wtw, ts);            \
+    return cudaGetLastError();
+      CASE(512) CASE(1024) CASE(2048)
+#undef CASE
+      default: break;
+    }
+  }
   switch (R2) {
 #define CASE(R) case R: k_inv_cols_det<R><<<grid, NT, smem_inv_cols_det<R>(nl), st>>>(in, P, part, cnt, vout, vstride, vofs, g.logR1, lognch, g.logM - g.logR2, m_lo, m_hi, scale, tw, ts); break;
     POND_FUSED_R2(CASE)
@@ -770,6 +830,15 @@ cudaError_t set_kernel_attributes() {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_inv_cols_det<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_inv_cols_det<R>(TILE / R));
   POND_FUSED_R2(SET_C)
 #undef SET_C
+#define SET_W(R)                                                                                                     \
+  if (e == cudaSuccess)                                                                                              \
+    e = cudaFuncSetAttribute(k_inv_cols_det_w<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,                \
+                             wide_smem_bytes<64, R / 64>());                                                         \
+  if (e == cudaSuccess)                                                                                              \
+    e = cudaFuncSetAttribute(k_inv_cols_det_w<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,                 \
+                             wide_smem_bytes<64, R / 64>());
+  SET_W(512) SET_W(1024) SET_W(2048)
+#undef SET_W
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_fold_partial, cudaFuncAttributeMaxDynamicSharedMemorySize, fold_smem_bytes(MAX_NBINS));
   if (e == cudaSuccess)

@@ -107,6 +107,9 @@ cudaError_t launch_tw2(float2* lo, float2* hi, int logn, int sign, cudaStream_t 
 cudaError_t launch_tw3(float2* out, int logn, int sign, cudaStream_t st);
 cudaError_t launch_stage_tw(float2* out, int R, cudaStream_t st);
 int stage_tw_entries(int R);
+// Stage-2 twiddles of the 64-values-per-thread FFT of length R (512 .. 4096; none otherwise).
+cudaError_t launch_wide_tw(float2* out, int R, cudaStream_t st);
+int wide_tw_entries(int R);
 cudaError_t launch_fwd_cols(const Geom& g, SegIn in, float2* out, const float2* tw, cudaStream_t st);
 cudaError_t launch_fwd_rows(const Geom& g, const float2* in, float2* out, const float2* tw3L, Tw2 tw2L, const float2* tw,
                             cudaStream_t st);
@@ -129,10 +132,11 @@ cudaError_t launch_chirp_c64(float2* tab, const Geom& g, double du, double half,
 cudaError_t launch_inv_rows_chirp(const Geom& g, const float2* in, float2* out, const float2* tw3L, const float2* twJ,
                                   const ChirpAnchor* anc, int clog, cudaStream_t st);
 // ntr > 1: one launch over ntr trials, trial t reading in + t L and writing
-// P + t M, part + t G M, cnt + t FUSED_J (G = fused_groups)
+// P + t M, part + t G M, cnt + t FUSED_J (G = fused_groups); wtw: launch_wide_tw of R2
+// (null: the radix-16 stages with their tables tw)
 cudaError_t launch_inv_cols_det(const Geom& g, const float2* in, float* P, float* part, int* cnt, float2* vout,
                                 long long vstride, long long vofs, int m_lo, int m_hi, const float2* tw,
-                                cudaStream_t st, int ntr = 1);
+                                const float2* wtw, cudaStream_t st, int ntr = 1);
 // Batched lanes: Ir over ntr trials in one launch (trial t writes out + t L),
 // the chirp from the lane's Q0.32 table (table = true) or each trial's anchors
 cudaError_t launch_inv_rows_chirp_multi(const Geom& g, const float2* in, float2* out, int ntr, const float2* tw3L,
