@@ -713,11 +713,6 @@ size_t smem_inv_rows_chirp(int R1, int nl) {
   return ((size_t)TW3_SN + stage_table_size(FUSED_J) + (size_t)nl * FUSED_J + (size_t)nl * (R1 + R1 / 16)) *
          sizeof(float2);
 }
-// k_inv_rows_chirp_res: the row pass's tables and tile plus the resident rows
-// (8 bytes per bin) and their table words (4 bytes per bin), in the tile's layout
-size_t smem_inv_rows_res(int R1, int nl) {
-  return smem_inv_rows_chirp(R1, nl) + (size_t)nl * (R1 + R1 / 16) * (sizeof(float2) + sizeof(unsigned));
-}
 }  // namespace
 
 cudaError_t launch_inv_rows_chirp(const Geom& g, const float2* in, float2* out, const float2* tw3L, const float2* twJ,
@@ -741,13 +736,14 @@ cudaError_t launch_inv_rows_chirp_multi(const Geom& g, const float2* in, float2*
   if (ntr < 1) return cudaErrorInvalidValue;
   // table form: one CTA per row tile runs every trial; anchor form: one CTA
   // per (trial, row tile)
+  const RowTile rt = row_tile(g.logR1, g.logR2);
   const unsigned tiles = (unsigned)(R2 / nl);
   switch (R1) {
 #define CASE(R)                                                                                             \
   case R:                                                                                                   \
     if (table)                                                                                              \
-      k_inv_rows_chirp_res<R, FUSED_J><<<tiles, NT, smem_inv_rows_res(R, nl), st>>>(in, out, g.L, g.logR2,  \
-                                                                                    tw3L, twJ, mc, ntr);    \
+      k_inv_rows_table<R><<<tiles, TAB_GROUPS * WIDE_NT, table_smem_bytes<R>(rt), st>>>(in, out, g.L, rt,    \
+                                                                                        tw3L, mc, ntr);     \
     else                                                                                                    \
       k_inv_rows_chirp_multi<R, FUSED_J><<<dim3((unsigned)ntr, tiles), NT, smem_inv_rows_chirp(R, nl), st>>>( \
           in, out, g.L, g.logR2, tw3L, twJ, mc);                                                            \
@@ -819,8 +815,8 @@ cudaError_t set_kernel_attributes() {
 #undef SET_I
 #define SET_M(R)                                                                                       \
   if (e == cudaSuccess)                                                                                \
-    e = cudaFuncSetAttribute(k_inv_rows_chirp_res<R, FUSED_J>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                             (int)smem_inv_rows_res(R, TILE / R));                                        \
+    e = cudaFuncSetAttribute(k_inv_rows_table<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,          \
+                             (int)table_smem_bytes<R>(RowTile{0, 0, 0, row_stride_max(R), row_stride_max(R)}));             \
   if (e == cudaSuccess)                                                                                \
     e = cudaFuncSetAttribute(k_inv_rows_chirp_multi<R, FUSED_J>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                              (int)smem_inv_rows_chirp(R, TILE / R));

@@ -736,69 +736,9 @@ __global__ void __launch_bounds__(NT, 2) k_inv_rows_chirp(const float2* __restri
 // exp(-2 pi i r) for the phase r = u 2^-32 (mod 1) held as a Q0.32 word u: the
 // same final sine and cosine as chirp_from.
 __device__ __forceinline__ float2 chirp_q32(unsigned u) {
-  const float r = (float)(int)u * 2.3283064365386963e-10f;   // 2^-32
   float s, c;
-  __sincosf(6.2831853071795865f * r, &s, &c);
+  __sincosf((float)(int)u * 1.4629180792671596e-9f, &s, &c);   // 2 pi 2^-32
   return make_float2(c, -s);
-}
-
-// IrK, table form: Ir for the ntr trials of one batched launch with the rows
-// resident.  CTA b (one per SM, R2 / nl of them) copies its nl rows of the
-// shared spectrum and their table words (stored in the spectrum's row layout)
-// into shared memory once, in the tile's padded layout, then runs every trial
-// of the launch on them: each length-64 run applies the trial's chirp as it
-// first reads its bins from those copies, and its F2f steps and blocked store
-// for the column pass go to out + t out_tstride.  A run is read and written
-// by the same four lanes, so the trials need no block barrier.  The rows are
-// read from L2 or HBM once per launch instead of once per trial (per trial and
-// segment, passes and decimation: 51.3 us one trial per CTA at two CTAs per
-// SM, 48.2 with the rows resident and a chirped tile per trial).
-template <int R1, int J>
-__global__ void __launch_bounds__(NT, 1) k_inv_rows_chirp_res(const float2* __restrict__ in,
-                                                              float2* __restrict__ out, long long out_tstride,
-                                                              int logR2, const float2* __restrict__ tw3L,
-                                                              const float2* __restrict__ twJ, MultiChirp mc,
-                                                              int ntr) {
-  static_assert(J == 64 && R1 % (4 * J) == 0 && R1 >= NT, "row layout of the fused pass");
-  constexpr int NCH = R1 / J;
-  constexpr int LSTR = R1 + R1 / 16;
-  constexpr int LOGJ = ilog2c(J), LOGNCH = ilog2c(NCH), LOGR1 = ilog2c(R1);
-  extern __shared__ float2 smem[];
-  float2* st3 = smem;                              // [TW3_SN], w = exp(-2 pi i / L)
-  float2* stwj = st3 + TW3_SN;
-  float2* twk = stwj + stage_table_size(J);        // [nl][J]: e^{2 pi i k2 m1 / M}
-  const int R2 = 1 << logR2;
-  const int nl = min(TILE / R1, R2);
-  const int tot = nl * R1;
-  float2* rows = twk + nl * J;                     // [nl * LSTR], the tile's layout
-  float2* sm = rows + nl * LSTR;                   // [nl * LSTR], the runs' exchange
-  unsigned* tabw = reinterpret_cast<unsigned*>(sm + nl * LSTR);   // [nl * LSTR], the rows' table words
-  const int r0 = blockIdx.x * nl;
-  load_tw3(st3, tw3L);
-  load_twiddles<J>(stwj, twJ);
-  const float4* in4 = reinterpret_cast<const float4*>(in) + ((size_t)r0 << (LOGR1 - 1));
-  const uint2* a2 = reinterpret_cast<const uint2*>(mc.atab) + ((size_t)r0 << (LOGR1 - 1));
-  for (int i = threadIdx.x; i < tot / 2; i += NT) {
-    const int idx = 2 * i, o = pidx(idx >> LOGR1, idx & (R1 - 1), LSTR);   // k1 even: o + 1 is k1 + 1
-    const float4 rv = __ldg(in4 + i);
-    const uint2 w = __ldg(a2 + i);
-    rows[o] = make_float2(rv.x, rv.y);
-    rows[o + 1] = make_float2(rv.z, rv.w);
-    tabw[o] = w.x;
-    tabw[o + 1] = w.y;
-  }
-  __syncthreads();   // st3
-  for (int i = threadIdx.x; i < nl * J; i += NT) {
-    const unsigned k2 = (unsigned)(r0 + (i >> LOGJ)), m1 = (unsigned)(i & (J - 1));
-    twk[i] = cconj(tw3(st3, (k2 * m1) << LOGNCH));
-  }
-  __syncthreads();   // twk, the rows and their table words
-  for (int t = 0; t < ntr; ++t) {
-    const unsigned nm = __ldg(mc.nmul + t);
-    j_runs_load<R1, J>(sm, stwj, twk, out + (size_t)t * out_tstride, nl, logR2, [&](int slot) { return r0 + slot; },
-                       [&](int o) { return cmul(rows[o], chirp_q32(nm * tabw[o])); });
-    __syncwarp();    // the run's last reads of sm come before the next trial's writes
-  }
 }
 
 // IrK, anchor form: Ir for the ntr trials of one batched launch, one trial per

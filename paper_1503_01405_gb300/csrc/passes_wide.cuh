@@ -5,6 +5,11 @@
 
 namespace pond {
 
+// L2 prefetch distance (CTAs) of these passes, three CTAs per SM.  Batched
+// chunk of 128 trials / full-rate stream, ms: 38: 104.3 / 15.98, 114: 103.3 /
+// 15.97, 228: 103.5 / 16.09, 456: 105.4 / 16.34, none: 116.6 / 16.40.
+constexpr int WIDE_PF = 114;
+
 // ---------------------------------------------------------------------------
 // Ic: column pass after F2f: inverse length-R2 FFTs, discard, detect, sum
 // ---------------------------------------------------------------------------
@@ -42,9 +47,9 @@ __global__ void __launch_bounds__(WIDE_NT, 3) k_inv_cols_det_w(const float2* __r
   const int m1 = blockIdx.x >> logG, gi = blockIdx.x & ((1 << logG) - 1);
   const float2* blk = in + (size_t)blockIdx.x * TILE;   // block m1 G + g
   if (tid < 4) {
-    // the block of CTA blockIdx.x + PF_DIST (in launch order, the next trial's
+    // the block of CTA blockIdx.x + WIDE_PF (in launch order, the next trial's
     // blocks after this trial's last), in four quarters
-    const unsigned nx = gridDim.x, lin = blockIdx.y * nx + blockIdx.x + PF_DIST;
+    const unsigned nx = gridDim.x, lin = blockIdx.y * nx + blockIdx.x + WIDE_PF;
     if (lin < nx * gridDim.y) {
       const float2* nb = in - blockIdx.y * ts.in + (size_t)(lin / nx) * ts.in + (size_t)(lin % nx) * TILE;
       constexpr unsigned qb = TILE * (unsigned)sizeof(float2) / 4;
@@ -70,6 +75,8 @@ __global__ void __launch_bounds__(WIDE_NT, 3) k_inv_cols_det_w(const float2* __r
   __syncthreads();
   float p[RB];
 #pragma unroll
+  for (int k = 0; k < RB; ++k) p[k] = 0.f;
+#pragma unroll 1   // one copy of the DFT in the instruction cache
   for (int u = 0; u < BPT; ++u) {
     const int line = h * BPT + u;
     const float2* src = smem + line * WSTR + t2;
@@ -79,8 +86,7 @@ __global__ void __launch_bounds__(WIDE_NT, 3) k_inv_cols_det_w(const float2* __r
     w2.template dft<true>(v);
 #pragma unroll
     for (int k = 0; k < RB; ++k) {
-      const float q = u == 0 ? v[k].x * v[k].x : fmaf(v[k].x, v[k].x, p[k]);
-      p[k] = fmaf(v[k].y, v[k].y, q);
+      p[k] = fmaf(v[k].y, v[k].y, fmaf(v[k].x, v[k].x, p[k]));
       if constexpr (VOUT) {
         const int m = m1 + ((t2 + RA * k) << logJ);
         if (m >= m_lo && m < m_hi)
@@ -146,6 +152,138 @@ __global__ void __launch_bounds__(WIDE_NT, 3) k_inv_cols_det_w(const float2* __r
       if (m >= m_lo && m < m_hi) P[m - m_lo] = o[i] * s2;
     }
   }
+}
+
+// ---------------------------------------------------------------------------
+// Ir: per-trial row pass of batched plans with M = 64 R2
+// ---------------------------------------------------------------------------
+
+// A batched plan shares F2's spectrum X[k2 + R2 k1] (row k2, column k1) among
+// its trials.  For each trial a row tile (nl = TILE/R1 consecutive rows) takes the
+// trial's chirp (Eq. 4) and the length-64 inverse DFT of every (row, sub-channel)
+// run of J = 64 consecutive columns, scales output m1 by e^{2 pi i k2 m1 / M} and
+// stores it at ((m1 G + g) R2 + k2) nlc + ci, c = g nlc + ci, nlc = min(TILE/R2,
+// NCH), the blocks that the column pass reads.
+//
+// A thread transforms a whole run in registers.  Rows sit in shared memory with
+// one value of padding per run and a row stride of RowTile::rstr values, so that a warp's
+// lanes, which take the nlc sub-channels of a block first, then the tile's rows,
+// read distinct banks and store runs of nl nlc consecutive values.
+struct RowTile {
+  int logR2, lognl, lognlc;   // rows of the segment, rows per tile, sub-channels per block
+  int rstr;                   // row stride in shared memory, values
+  int tstr;                   // row stride of the table words (32 lanes on 4-byte banks)
+};
+
+template <int R1>
+__host__ __device__ constexpr int run_slots() { return TILE / R1; }
+
+// Row stride: NCH runs of 65 values, padded to (16 / nl or nlc, the larger) mod 16
+// while a half-warp covers several rows.
+inline RowTile row_tile(int logR1, int logR2) {
+  RowTile r;
+  const int lognch = logR1 - 6;
+  r.logR2 = logR2;
+  r.lognl = 13 - logR1;
+  r.lognlc = 13 - logR2 < lognch ? 13 - logR2 : lognch;
+  const int base = 65 << lognch, nlc = 1 << r.lognlc, s = 16 >> r.lognl;
+  const int want = nlc >= 16 ? 0 : (nlc > s ? nlc : s);
+  r.rstr = base + ((want - base) & 15);
+  // lanes of a warp: nlc sub-channels, then min(nl, 32 / nlc) rows, then blocks of nlc
+  const int rows = nlc >= 32 ? 1 : (32 / nlc < (1 << r.lognl) ? 32 / nlc : 1 << r.lognl);
+  r.tstr = base + (((rows > 1 ? 32 / rows : 0) - base) & 31);
+  return r;
+}
+// largest row stride of a line length (any R2): for shared-memory limits
+constexpr int row_stride_max(int R1) { return 65 * (R1 / 64) + 31; }
+
+constexpr int TWK_STR = 65;   // stride of a row's 64 factors e^{2 pi i k2 m1 / M}
+
+// Thread -> run: sub-channels of a block fastest, then rows, then blocks.
+struct Run {
+  int slot, c;
+};
+__device__ __forceinline__ Run run_of(const RowTile& rt, int id) {
+  Run r;
+  r.slot = (id >> rt.lognlc) & ((1 << rt.lognl) - 1);
+  r.c = (id & ((1 << rt.lognlc) - 1)) | ((id >> (rt.lognlc + rt.lognl)) << rt.lognlc);
+  return r;
+}
+
+// The run's 64-point inverse DFT, the factors twk[m1] and the blocked store.
+template <int R1>
+__device__ __forceinline__ void run_finish(float2* v, const RowTile& rt, const Run& r, unsigned k2, const float2* twk,
+                                           float2* __restrict__ out) {
+  constexpr int LOGNCH = ilog2c(R1 / 64);
+  wide_dft<64, true>(v);
+  const unsigned g = (unsigned)r.c >> rt.lognlc, ci = (unsigned)r.c & ((1u << rt.lognlc) - 1);
+  float2* dst = out + ((((g << rt.logR2) + k2) << rt.lognlc) + ci);
+  const float2* w = twk + r.slot * TWK_STR;
+#pragma unroll
+  for (int m1 = 0; m1 < 64; ++m1) dst[(unsigned)m1 << (LOGNCH + rt.logR2)] = cmul(v[m1], w[m1]);
+}
+
+// e^{2 pi i k2 m1 / M} = conj(w^{k2 m1 NCH}), k2 m1 NCH < L, of rows row_of(0 .. nl-1).
+template <int R1, class RowOf>
+__device__ __forceinline__ void make_twk(float2* twk, const float2* st3, int nl, RowOf row_of) {
+  for (int i = threadIdx.x; i < nl * 64; i += blockDim.x) {
+    const unsigned k2 = (unsigned)row_of(i >> 6), m1 = (unsigned)(i & 63);
+    twk[(i >> 6) * TWK_STR + m1] = cconj(tw3(st3, (k2 * m1) << ilog2c(R1 / 64)));
+  }
+}
+
+// Table form: the rows and their Q0.32 table words resident for every trial of the launch.
+// Four warps run a trial of the tile, GROUPS trials at a time; a run is read from the
+// resident copies and stored from registers, so there is no exchange and no
+// barrier after the tile's load.  Bound by the issue slots (chirp and DFT, 34
+// instructions per value) next to the 64 MiB that each trial writes (4.8 TB/s).
+// Full-rate batched plan: 19.9 us per trial with the runs split over four lanes
+// and exchanged through shared memory (78 % of that pipe), 13.5 here; the 8 s
+// chunk of 128 trials 126 -> 103 ms.
+constexpr int TAB_GROUPS = 3;   // 384 threads of 168 registers: one CTA per SM
+
+template <int R1>
+__global__ void __launch_bounds__(TAB_GROUPS * WIDE_NT, 1)
+    k_inv_rows_table(const float2* __restrict__ in, float2* __restrict__ out, long long out_tstride, RowTile rt,
+                     const float2* __restrict__ tw3L, MultiChirp mc, int ntr) {
+  constexpr int NLR = run_slots<R1>(), LOGR1 = ilog2c(R1);
+  extern __shared__ float2 smem[];
+  float2* st3 = smem;                                       // [TW3_SN], w = exp(-2 pi i / L)
+  float2* twk = st3 + TW3_SN;                               // [NLR][TWK_STR]
+  float2* rows = twk + NLR * TWK_STR + (NLR * TWK_STR & 1); // [NLR * rstr]
+  unsigned* tabw = reinterpret_cast<unsigned*>(rows + NLR * rt.rstr);
+  const int r0 = blockIdx.x * NLR;
+  load_tw3(st3, tw3L);
+  const float2* src = in + ((size_t)r0 << LOGR1);
+  const unsigned* tsrc = mc.atab + ((size_t)r0 << LOGR1);
+#pragma unroll 8
+  for (int i = threadIdx.x; i < TILE; i += TAB_GROUPS * WIDE_NT) {
+    const int slot = i >> LOGR1, k1 = i & (R1 - 1), o = k1 + (k1 >> 6);
+    rows[slot * rt.rstr + o] = __ldg(src + i);
+    tabw[slot * rt.tstr + o] = __ldg(tsrc + i);
+  }
+  __syncthreads();   // st3
+  make_twk<R1>(twk, st3, NLR, [&](int slot) { return r0 + slot; });
+  __syncthreads();   // twk, the rows and their table words
+  const Run r = run_of(rt, (int)threadIdx.x & (WIDE_NT - 1));
+  const int o = r.slot * rt.rstr + 65 * r.c, ot = r.slot * rt.tstr + 65 * r.c;
+  int t = (int)threadIdx.x / WIDE_NT;
+  unsigned next = t < ntr ? __ldg(mc.nmul + t) : 0u;
+  for (; t < ntr; t += TAB_GROUPS) {
+    const unsigned nm = next;
+    if (t + TAB_GROUPS < ntr) next = __ldg(mc.nmul + t + TAB_GROUPS);   // ahead of its use
+    float2 v[64];
+#pragma unroll
+    for (int j = 0; j < 64; ++j) v[j] = cmul(rows[o + j], chirp_q32(nm * tabw[ot + j]));
+    run_finish<R1>(v, rt, r, (unsigned)(r0 + r.slot), twk, out + (size_t)t * out_tstride);
+  }
+}
+
+template <int R1>
+size_t table_smem_bytes(const RowTile& rt) {
+  constexpr int NLR = run_slots<R1>();
+  return (size_t)(TW3_SN + NLR * TWK_STR + (NLR * TWK_STR & 1) + NLR * rt.rstr) * sizeof(float2) +
+         (size_t)NLR * rt.tstr * sizeof(unsigned);
 }
 
 // Shared memory of a tile of nl lines of RA x RB.
