@@ -115,7 +115,8 @@ struct Lane {
   Geom g;
   double dm_max = 0;                        // largest DM of the lane (sets the overlap)
   std::vector<int> trials;
-  // two buffer slots: consecutive segments alternate slots and streams
+  int group = 1;                            // segments per launch (single-DM plans; buffers below hold that many)
+  // two buffer slots: consecutive groups of segments alternate slots and streams
   float2* bufA[NSLOT] = {};
   float2* bufB[NSLOT] = {};
   float* P[NSLOT] = {};
@@ -137,6 +138,7 @@ struct Lane {
   int8_t* carry[2] = {nullptr, nullptr};
   int carry_cur = 0;
   long long seg_start = 0, carry_pos = 0, segments = 0;
+  long long groups = 0;                     // launched so far (buffer slot = groups mod NSLOT)
   // batched lanes with several trials per launch (POND_TRIALS_MULTI_*)
   int mode = POND_TRIALS_PER_TRIAL;
   int kt = 1;                               // trials per launch
@@ -213,6 +215,7 @@ struct pond_s {
   long long v_cap = 0;
   // stream state
   long long total_in = 0;
+  int fold_rows = 0;                        // partial rows of the fold
   bool flushed = false;
   long long outputs = 0;
   // time series: [ts_drained, ts_complete) complete on the device; ts_hi = one past the last touched
@@ -397,14 +400,20 @@ int build_lane(pond_t h, Lane* ln) {
   ln->fused = !h->multi && three;
   ln->fused_multi = h->multi && three;
   ln->ic_tc = three && h->tc_terms == 3;
+  // Several segments per launch: one segment of a 2^24-point plan is 2.2 waves of
+  // CTAs and a short one a fraction of a wave, so a launch of each pass over a group
+  // of segments fills the chip where one per segment drains it.  Kept voltages
+  // and per-stage timing take one segment at a time, as do the tensor-core forms.
+  ln->group = h->multi || h->timing || h->want_voltages || h->tc_terms ? 1 : fold_slots(g);
+  const size_t K = (size_t)ln->group;
   for (int k = 0; k < NSLOT; ++k) {
-    CK(cudaMalloc(&ln->bufA[k], g.L * sizeof(float2)));
-    CK(cudaMalloc(&ln->bufB[k], g.L * sizeof(float2)));
-    CK(cudaMalloc(&ln->P[k], g.M * sizeof(float)));
+    CK(cudaMalloc(&ln->bufA[k], K * g.L * sizeof(float2)));
+    CK(cudaMalloc(&ln->bufB[k], K * g.L * sizeof(float2)));
+    CK(cudaMalloc(&ln->P[k], K * g.M * sizeof(float)));
     if ((ln->fused || ln->fused_multi) && fused_groups(g) > 1) {
-      CK(cudaMalloc(&ln->part[k], (size_t)fused_groups(g) * g.M * sizeof(float)));
-      CK(cudaMalloc(&ln->cnt[k], FUSED_J * sizeof(int)));
-      CK(cudaMemsetAsync(ln->cnt[k], 0, FUSED_J * sizeof(int), h->st));
+      CK(cudaMalloc(&ln->part[k], K * fused_groups(g) * g.M * sizeof(float)));
+      CK(cudaMalloc(&ln->cnt[k], K * FUSED_J * sizeof(int)));
+      CK(cudaMemsetAsync(ln->cnt[k], 0, K * FUSED_J * sizeof(int), h->st));
     }
   }
   const int n1 = stage_tw_entries(1 << g.logR1), n2 = stage_tw_entries(1 << g.logR2);
@@ -617,25 +626,27 @@ void update_complete(pond_t h) {
   h->ts_complete = std::max(h->ts_complete, (gn * h->dec_den) / h->dec_num);
 }
 
-// Process segment s of lane li; g_end bounds the emitted channel samples.
 // The column pass of a three-pass lane: FP32 or tensor-core form.
 cudaError_t launch_ic(pond_t h, const Lane& ln, const float2* in, float* P, float* part, int* cnt, float2* vout,
-                      long long vstride, long long vofs, int m_lo, int m_hi, cudaStream_t st, int ntr = 1) {
+                      long long vstride, long long vofs, const MSpan& span, cudaStream_t st, int nu = 1) {
   if (ln.ic_tc)
-    return launch_inv_cols_det_tc(ln.g, in, P, part, cnt, vout, vstride, vofs, m_lo, m_hi, h->ic_ops, h->tc_err, st,
-                                  ntr);
-  return launch_inv_cols_det(ln.g, in, P, part, cnt, vout, vstride, vofs, m_lo, m_hi, ln.stwR2, ln.wtwR2, st, ntr);
+    return launch_inv_cols_det_tc(ln.g, in, P, part, cnt, vout, vstride, vofs, span.m_lo,
+                                  (int)std::min<long long>(span.m_hi, span.m_end), h->ic_ops, h->tc_err, st, nu);
+  return launch_inv_cols_det(ln.g, in, P, part, cnt, vout, vstride, vofs, span, ln.stwR2, ln.wtwR2, st, nu);
 }
 
-int run_segment(pond_t h, int li, SegIn in, long long s, long long g_end) {
+// Process segments s .. s + nseg - 1 of lane li (nseg <= ln.group), whose input is
+// src; g_end bounds the emitted channel samples.
+int run_segments(pond_t h, int li, const SegSrc& src, long long s, int nseg, long long g_end) {
   Lane& ln = h->lanes[li];
   const Geom& g = ln.g;
   const long long m_lo = std::max(g.n_past, h->g_first - s * g.S_c);
-  const long long m_hi = std::min(g.M - g.n_fut, g_end - s * g.S_c);
-  ln.segments = s + 1;
+  const long long m_hi = std::min(g.M - g.n_fut, g_end - (s + nseg - 1) * g.S_c);   // of the last segment
+  ln.segments = s + nseg;
   if (m_hi <= m_lo) return POND_OK;
-  const long long g0 = s * g.S_c + m_lo;         // first output of this segment
-  const long long nv = m_hi - m_lo;
+  const long long g0 = s * g.S_c + m_lo;         // first output of the first segment
+  const long long nv = m_hi - m_lo + (nseg - 1) * g.S_c;
+  const MSpan span{(int)m_lo, (int)(g.M - g.n_fut), g_end - s * g.S_c, g.S_c};
   const long long j_lo = (g0 * h->dec_den) / h->dec_num;
   const long long j_hi = ((g0 + nv - 1) * h->dec_den) / h->dec_num;
   if (h->ts_first < 0) {
@@ -650,47 +661,54 @@ int run_segment(pond_t h, int li, SegIn in, long long s, long long g_end) {
     if (h->v_len + nv > h->v_cap) RC(spill_voltages(h));
     vout = h->vbuf;
   }
-  {  // F1 may load 8 bytes (4 columns of a row), or one sample's N / S pairs, at a time when both runs allow it
-    const int nl1 = std::min(TILE >> g.logR2, 1 << g.logR1);
-    in.vec8 = in.ch == 1 && (nl1 % 4 == 0) && ((uintptr_t)in.a % 8 == 0) && (in.a_len % 8 == 0) &&
-              (in.b_len == 0 || (uintptr_t)in.b % 8 == 0);
-    in.pair4 = in.ch == 2 && ((uintptr_t)in.a % 4 == 0) && (in.a_len % 4 == 0) && (in.b_len % 4 == 0) &&
-               (in.b_len == 0 || (uintptr_t)in.b % 4 == 0);
-  }
-  // consecutive segments alternate buffer slots and streams, so one segment's
+  // consecutive groups alternate buffer slots and streams, so one group's
   // passes fill the other's tail waves; fold / decimation stay in segment order.
   // With per-stage timing everything runs on st, so each stage's events
   // bracket that stage alone.
-  const int slot = (int)(s % NSLOT);
+  const int slot = (int)(ln.groups++ % NSLOT);
   cudaStream_t cs = (slot && !h->timing) ? h->sx[slot] : h->st;
   float2 *bufA = ln.bufA[slot], *bufB = ln.bufB[slot];
   float* P = ln.P[slot];
   h->ev_cur = SegEvents{};
   RC(record(h, 0, cs));
-  CK(launch_fwd_cols(g, in, bufA, ln.stwR2, cs));
+  CK(launch_fwd_cols(g, src, bufA, ln.stwR2, cs, nseg));
   RC(record(h, 1 + ST_F1, cs));
-  if (ln.fused) {
-    // three passes: F2f takes the chirp and the first inverse factor, Ic the rest
+  if (!h->multi) {
     const Trial& t = h->trials[ln.trials[0]];
-    CK(launch_fwd_rows_inv(g, bufA, bufB, ln.tw3L, ln.tw2L, ln.stwR1, ln.stwJ, t.anc, t.clog, t.ctab, cs));
-    RC(record(h, 1 + ST_F2F, cs));
-    // P of this slot is free once the fold of segment s - NSLOT has read it
+    if (ln.fused) {
+      // three passes: F2f takes the chirp and the first inverse factor, Ic the rest
+      CK(launch_fwd_rows_inv(g, bufA, bufB, ln.tw3L, ln.tw2L, ln.stwR1, ln.stwJ, t.anc, t.clog, t.ctab, cs, nseg));
+      RC(record(h, 1 + ST_F2F, cs));
+      h->launches += 4;
+    } else {
+      CK(launch_fwd_rows(g, bufA, bufB, ln.tw3L, ln.tw2L, ln.stwR1, cs, nseg));
+      RC(record(h, 1 + ST_F2, cs));
+      // the chirp is applied as I1 loads the spectrum
+      CK(launch_inv_cols(g, bufB, bufA, t.anc, t.clog, ln.stwQ2, cs, nseg));
+      RC(record(h, 1 + ST_I1, cs));
+      h->launches += 5;
+    }
+    // P of this slot is free once the fold of the group before the last has read it
     if (!h->timing) CK(cudaStreamWaitEvent(cs, h->ev_pfree[slot], 0));
-    CK(launch_ic(h, ln, bufB, P, ln.part[slot], ln.cnt[slot], vout, h->v_cap, h->v_len, (int)m_lo, (int)m_hi, cs));
-    RC(record(h, 1 + ST_IC, cs));
+    if (ln.fused) {
+      CK(launch_ic(h, ln, bufB, P, ln.part[slot], ln.cnt[slot], vout, h->v_cap, h->v_len, span, cs, nseg));
+      RC(record(h, 1 + ST_IC, cs));
+    } else {
+      CK(launch_inv_rows(g, bufA, P, vout, h->v_cap, h->v_len, span, ln.tw3M, ln.stwQ1, cs, nseg));
+      RC(record(h, 1 + ST_I2, cs));
+    }
     // folds run in segment order on their own stream (on st with per-stage timing)
     cudaStream_t fs = h->timing ? cs : h->sf;
     if (!h->timing) {
       CK(cudaEventRecord(h->ev_pready[slot], cs));
       CK(cudaStreamWaitEvent(fs, h->ev_pready[slot], 0));
     }
-    CK(launch_fold_dec(P, nv, g0, h->fold_rule, h->nbins, h->dec_num, h->dec_den, j_lo, j_hi - j_lo + 1,
-                       h->ts + (size_t)ln.trials[0] * h->ring, h->ts_cnt + (size_t)ln.trials[0] * h->ring, h->ring,
-                       h->psum, h->phits, fs));
+    const FoldSegs f{s, g0, g.S_c, g.M, nv, nseg};
+    CK(launch_fold_dec(g, P, f, h->fold_rule, h->nbins, h->dec_num, h->dec_den, h->ts, h->ts_cnt, h->ring, h->psum,
+                       h->phits, fs));
     RC(record(h, 1 + ST_FOLD, fs));
     RC(record(h, 1 + ST_DEC, fs, true));
     if (!h->timing) CK(cudaEventRecord(h->ev_pfree[slot], fs));
-    h->launches += 4;
   } else {
     CK(launch_fwd_rows(g, bufA, bufB, ln.tw3L, ln.tw2L, ln.stwR1, cs));
     RC(record(h, 1 + ST_F2, cs));
@@ -698,6 +716,7 @@ int run_segment(pond_t h, int li, SegIn in, long long s, long long g_end) {
     if (ln.mode == POND_TRIALS_MULTI_ANCHOR || ln.mode == POND_TRIALS_MULTI_TABLE) {
       // kt trials per launch: the row pass with each trial's chirp, the column
       // pass with detection, then the decimation of every trial's series row
+      const MSpan trials{span.m_lo, (int)m_hi, m_hi, 0};
       const int ntr = (int)ln.trials.size();
       for (int b = 0, q0 = 0; q0 < ntr; ++b, q0 += ln.kt) {
         const int nq = std::min(ln.kt, ntr - q0);
@@ -705,8 +724,7 @@ int run_segment(pond_t h, int li, SegIn in, long long s, long long g_end) {
         CK(launch_inv_rows_chirp_multi(g, bufB, ln.bufT[slot], nq, ln.tw3L, ln.stwJ, mc,
                                        ln.mode == POND_TRIALS_MULTI_TABLE, cs));
         if (b == 0) RC(record(h, 1 + ST_IR, cs));
-        CK(launch_ic(h, ln, ln.bufT[slot], ln.Pm[slot], ln.partm[slot], ln.cntm[slot], nullptr, 0, 0, (int)m_lo,
-                     (int)m_hi, cs, nq));
+        CK(launch_ic(h, ln, ln.bufT[slot], ln.Pm[slot], ln.partm[slot], ln.cntm[slot], nullptr, 0, 0, trials, cs, nq));
         if (b == 0) RC(record(h, 1 + ST_IC, cs));
         // the block's series rows are updated in segment order
         CK(cudaStreamWaitEvent(cs, ln.ev_chain[(slot + NSLOT - 1) % NSLOT][b], 0));
@@ -735,30 +753,20 @@ int run_segment(pond_t h, int li, SegIn in, long long s, long long g_end) {
           // the trial's chirp and the first inverse factor as Ir loads the shared spectrum's rows
           CK(launch_inv_rows_chirp(g, bufB, bufA, ln.tw3L, ln.stwJ, t.anc, t.clog, cs));
           if (q == 0) RC(record(h, 1 + ST_IR, cs));
-          CK(launch_ic(h, ln, bufA, P, ln.part[slot], ln.cnt[slot], vout, h->v_cap, h->v_len, (int)m_lo,
-                       (int)m_hi, cs));
+          CK(launch_ic(h, ln, bufA, P, ln.part[slot], ln.cnt[slot], nullptr, 0, 0, span, cs));
           if (q == 0) RC(record(h, 1 + ST_IC, cs));
         } else {
           // four passes: every trial's chirp is applied as I1 loads the shared forward spectrum
           CK(launch_inv_cols(g, bufB, bufA, t.anc, t.clog, ln.stwQ2, cs));
           if (q == 0) RC(record(h, 1 + ST_I1, cs));
-          CK(launch_inv_rows(g, bufA, P, vout, h->v_cap, h->v_len, (int)m_lo, (int)m_hi, ln.tw3M, ln.stwQ1, cs));
+          CK(launch_inv_rows(g, bufA, P, nullptr, 0, 0, span, ln.tw3M, ln.stwQ1, cs));
           if (q == 0) RC(record(h, 1 + ST_I2, cs));
         }
-        // each trial's series row (and the fold partials) is updated in segment order
+        // each trial's series row is updated in segment order
         CK(cudaStreamWaitEvent(cs, ln.ev_chain[(slot + NSLOT - 1) % NSLOT][q], 0));
-        if (!h->multi) {
-          // fold and decimation in one launch; the profile is merged when read
-          CK(launch_fold_dec(P, nv, g0, h->fold_rule, h->nbins, h->dec_num, h->dec_den, j_lo, j_hi - j_lo + 1,
-                             h->ts + (size_t)d * h->ring, h->ts_cnt + (size_t)d * h->ring, h->ring, h->psum,
-                             h->phits, cs));
-          RC(record(h, 1 + ST_FOLD, cs));
-          RC(record(h, 1 + ST_DEC, cs, true));
-        } else {
-          CK(launch_decimate(P, nv, g0, h->dec_num, h->dec_den, j_lo, j_hi - j_lo + 1, h->ts + (size_t)d * h->ring,
-                             h->ts_cnt + (size_t)d * h->ring, h->ring, cs));
-          if (q == 0) RC(record(h, 1 + ST_DEC, cs, true));
-        }
+        CK(launch_decimate(P, nv, g0, h->dec_num, h->dec_den, j_lo, j_hi - j_lo + 1, h->ts + (size_t)d * h->ring,
+                           h->ts_cnt + (size_t)d * h->ring, h->ring, cs));
+        if (q == 0) RC(record(h, 1 + ST_DEC, cs, true));
         CK(cudaEventRecord(ln.ev_chain[slot][q], cs));
         h->launches += 3;
       }
@@ -767,6 +775,30 @@ int run_segment(pond_t h, int li, SegIn in, long long s, long long g_end) {
   if (h->want_voltages) h->v_len += nv;
   h->ts_hi = std::max(h->ts_hi, j_hi + 1);
   if (li == 0) h->outputs += nv;
+  return POND_OK;
+}
+
+// Run the lane's next n segments (their input in the carry and the avail bytes at d) in
+// groups of at most ln.group; a group's series samples stay well inside the device ring.
+int run_lane(pond_t h, int li, const int8_t* d, long long avail, long long n, long long g_end) {
+  Lane& ln = h->lanes[li];
+  const Geom& g = ln.g;
+  const long long per = (g.S_c * h->dec_den) / h->dec_num + 2;   // series samples per segment
+  const long long most = std::max(1ll, std::min<long long>(ln.group, h->ring / (4 * per)));
+  while (n > 0) {
+    const int k = (int)std::min(n, most);
+    SegSrc src;
+    src.carry_end = ln.carry[ln.carry_cur] + (h->total_in - ln.carry_pos) * h->ch;
+    src.d = d;
+    src.avail = avail;
+    src.r0 = (ln.seg_start - h->total_in) * h->ch;
+    src.step = g.S * h->ch;
+    src.bytes = g.N * h->ch;
+    src.ch = h->ch;
+    RC(run_segments(h, li, src, ln.seg_start / g.S, k, g_end));
+    ln.seg_start += k * g.S;
+    n -= k;
+  }
   return POND_OK;
 }
 
@@ -779,23 +811,7 @@ int ingest_device(pond_t h, const int8_t* d, long long n) {
   for (size_t li = 0; li < h->lanes.size(); ++li) {
     Lane& ln = h->lanes[li];
     const Geom& g = ln.g;
-    while (ln.seg_start + g.N <= end) {
-      SegIn in;
-      in.ch = ch;
-      if (ln.seg_start < h->total_in) {
-        in.a = ln.carry[ln.carry_cur] + (ln.seg_start - ln.carry_pos) * ch;
-        in.a_len = (h->total_in - ln.seg_start) * ch;
-        in.b = d;
-        in.b_len = g.N * ch - in.a_len;
-      } else {
-        in.a = d + (ln.seg_start - h->total_in) * ch;
-        in.a_len = g.N * ch;
-        in.b = nullptr;
-        in.b_len = 0;
-      }
-      RC(run_segment(h, (int)li, in, ln.seg_start / g.S, 1ll << 62));
-      ln.seg_start += g.S;
-    }
+    if (ln.seg_start + g.N <= end) RC(run_lane(h, (int)li, d, n * ch, (end - g.N - ln.seg_start) / g.S + 1, 1ll << 62));
   }
   // Each lane's carry is double-buffered: the buffer rewritten below was last
   // read by the previous ingest's segments, so st waits for that ingest's
@@ -947,7 +963,8 @@ int measure_lane(pond_t h, const pond_opts* o, long long nfft, double* t_fwd, do
     ce = launch_tables(anc, nanc, clog, o->fs_hz / (double)nfft * 1e-6, std::fabs(o->bw_mhz) / 2, o->f0_mhz, 0.0,
                        h->sgn, h->st);
   const int reps = 3;
-  SegIn in{ln.carry[0], g.N * h->ch, nullptr, 0, 0, h->ch};
+  const SegSrc in{ln.carry[0] + g.N * h->ch, nullptr, 0, -g.N * h->ch, 0, g.N * h->ch, h->ch};
+  const MSpan span{(int)g.n_past, (int)(g.n_past + nv), g.M, 0};
   for (int it = 0; it <= reps && ce == cudaSuccess; ++it) {      // first pass warms up
     if (it == 1) ce = cudaEventRecord(e[0], h->st);
     if (ce == cudaSuccess) ce = launch_fwd_cols(g, in, ln.bufA[0], ln.stwR2, h->st);
@@ -959,13 +976,11 @@ int measure_lane(pond_t h, const pond_opts* o, long long nfft, double* t_fwd, do
     if (ln.fused_multi) {   // the per-trial passes the plan will run
       if (ce == cudaSuccess) ce = launch_inv_rows_chirp(g, ln.bufB[0], ln.bufA[0], ln.tw3L, ln.stwJ, anc, clog, h->st);
       if (ce == cudaSuccess)
-        ce = launch_ic(h, ln, ln.bufA[0], ln.P[0], ln.part[0], ln.cnt[0], nullptr, 0, 0, (int)g.n_past,
-                       (int)(g.n_past + nv), h->st);
+        ce = launch_ic(h, ln, ln.bufA[0], ln.P[0], ln.part[0], ln.cnt[0], nullptr, 0, 0, span, h->st);
     } else {
       if (ce == cudaSuccess) ce = launch_inv_cols(g, ln.bufB[0], ln.bufA[0], anc, clog, ln.stwQ2, h->st);
       if (ce == cudaSuccess)
-        ce = launch_inv_rows(g, ln.bufA[0], ln.P[0], nullptr, 0, 0, (int)g.n_past, (int)(g.n_past + nv), ln.tw3M,
-                             ln.stwQ1, h->st);
+        ce = launch_inv_rows(g, ln.bufA[0], ln.P[0], nullptr, 0, 0, span, ln.tw3M, ln.stwQ1, h->st);
     }
     if (ce == cudaSuccess) ce = launch_decimate(ln.P[0], nv, 0, 8, 1, 0, nv / 8, T, C, nv / 8 + 1, h->st);
   }
@@ -1101,6 +1116,7 @@ int time_trials(pond_t h, Lane* ln, int mode, int kt, int split, double* us) {
   const int nq = std::min(kt, (int)ln->trials.size());
   const long long m_lo = g.n_past, m_hi = g.M - g.n_fut, g0 = m_lo, nv = m_hi - m_lo;
   const long long j_lo = (g0 * h->dec_den) / h->dec_num, j_hi = ((g0 + nv - 1) * h->dec_den) / h->dec_num;
+  const MSpan span{(int)m_lo, (int)m_hi, m_hi, 0};
   // the four-pass form at this split: its own Q1 / Q2 tables
   Geom gq = g;
   float2* tq = nullptr;
@@ -1127,7 +1143,7 @@ int time_trials(pond_t h, Lane* ln, int mode, int kt, int split, double* us) {
         const Trial& t = h->trials[ln->trials[q]];
         ce = launch_inv_cols(gq, ln->bufB[0], ln->bufA[0], t.anc, t.clog, tq2, h->st);
         if (ce == cudaSuccess)
-          ce = launch_inv_rows(gq, ln->bufA[0], ln->P[0], nullptr, 0, 0, (int)m_lo, (int)m_hi, ln->tw3M, tq1, h->st);
+          ce = launch_inv_rows(gq, ln->bufA[0], ln->P[0], nullptr, 0, 0, span, ln->tw3M, tq1, h->st);
         if (ce == cudaSuccess)
           ce = launch_decimate(ln->P[0], nv, g0, h->dec_num, h->dec_den, j_lo, j_hi - j_lo + 1,
                                h->ts + (size_t)ln->trials[q] * h->ring, h->ts_cnt + (size_t)ln->trials[q] * h->ring,
@@ -1138,8 +1154,7 @@ int time_trials(pond_t h, Lane* ln, int mode, int kt, int split, double* us) {
         const Trial& t = h->trials[ln->trials[q]];
         ce = launch_inv_rows_chirp(g, ln->bufB[0], ln->bufA[0], ln->tw3L, ln->stwJ, t.anc, t.clog, h->st);
         if (ce == cudaSuccess)
-          ce = launch_ic(h, *ln, ln->bufA[0], ln->P[0], ln->part[0], ln->cnt[0], nullptr, 0, 0, (int)m_lo, (int)m_hi,
-                         h->st);
+          ce = launch_ic(h, *ln, ln->bufA[0], ln->P[0], ln->part[0], ln->cnt[0], nullptr, 0, 0, span, h->st);
         if (ce == cudaSuccess)
           ce = launch_decimate(ln->P[0], nv, g0, h->dec_num, h->dec_den, j_lo, j_hi - j_lo + 1,
                                h->ts + (size_t)ln->trials[q] * h->ring, h->ts_cnt + (size_t)ln->trials[q] * h->ring,
@@ -1150,8 +1165,7 @@ int time_trials(pond_t h, Lane* ln, int mode, int kt, int split, double* us) {
       ce = launch_inv_rows_chirp_multi(g, ln->bufB[0], ln->bufT[0], nq, ln->tw3L, ln->stwJ, mc,
                                        mode == POND_TRIALS_MULTI_TABLE, h->st);
       if (ce == cudaSuccess)
-        ce = launch_ic(h, *ln, ln->bufT[0], ln->Pm[0], ln->partm[0], ln->cntm[0], nullptr, 0, 0, (int)m_lo, (int)m_hi,
-                       h->st, nq);
+        ce = launch_ic(h, *ln, ln->bufT[0], ln->Pm[0], ln->partm[0], ln->cntm[0], nullptr, 0, 0, span, h->st, nq);
       if (ce == cudaSuccess && h->dec_num < 64 * h->dec_den)
         ce = launch_decimate_multi(ln->Pm[0], g.M, nv, g0, h->dec_num, h->dec_den, j_lo, j_hi - j_lo + 1, h->ts,
                                    h->ts_cnt, h->ring, ln->d_rows, nq, h->st);
@@ -1509,14 +1523,15 @@ int plan_impl(pond_t* out, const pond_opts* o) {
     CKD(cudaMemsetAsync(h->ts_cnt, 0, (size_t)ntr * h->ring * sizeof(int), h->st));
   }
   if (!multi) {
+    h->fold_rows = fold_slots(h->lanes[0].g) * fold_parts_seg(h->lanes[0].g);
     CKD(cudaMalloc(&h->prof_sum, h->nbins * sizeof(double)));
     CKD(cudaMalloc(&h->prof_hits, h->nbins * sizeof(long long)));
-    CKD(cudaMalloc(&h->psum, (size_t)MAX_FOLD_PARTS * h->nbins * sizeof(double)));
-    CKD(cudaMalloc(&h->phits, (size_t)MAX_FOLD_PARTS * h->nbins * sizeof(long long)));
+    CKD(cudaMalloc(&h->psum, (size_t)h->fold_rows * h->nbins * sizeof(double)));
+    CKD(cudaMalloc(&h->phits, (size_t)h->fold_rows * h->nbins * sizeof(long long)));
     CKD(cudaMemsetAsync(h->prof_sum, 0, h->nbins * sizeof(double), h->st));
     CKD(cudaMemsetAsync(h->prof_hits, 0, h->nbins * sizeof(long long), h->st));
-    CKD(cudaMemsetAsync(h->psum, 0, (size_t)MAX_FOLD_PARTS * h->nbins * sizeof(double), h->st));
-    CKD(cudaMemsetAsync(h->phits, 0, (size_t)MAX_FOLD_PARTS * h->nbins * sizeof(long long), h->st));
+    CKD(cudaMemsetAsync(h->psum, 0, (size_t)h->fold_rows * h->nbins * sizeof(double), h->st));
+    CKD(cudaMemsetAsync(h->phits, 0, (size_t)h->fold_rows * h->nbins * sizeof(long long), h->st));
   }
   if (h->want_voltages) {
     h->v_cap = std::max<long long>(4 * h->lanes[0].g.S_c, 1 << 16);
@@ -1653,16 +1668,9 @@ int pond_flush(pond_t h) {
   for (size_t li = 0; li < h->lanes.size(); ++li) {
     Lane& ln = h->lanes[li];
     const Geom& g = ln.g;
-    while ((ln.seg_start / g.S) * g.S_c + g.n_past < g_end) {
-      SegIn in;
-      in.ch = h->ch;
-      in.a = ln.carry[ln.carry_cur] + (ln.seg_start - ln.carry_pos) * h->ch;
-      in.a_len = std::max(0ll, h->total_in - ln.seg_start) * h->ch;
-      in.b = nullptr;
-      in.b_len = 0;
-      RC(run_segment(h, (int)li, in, ln.seg_start / g.S, g_end));
-      ln.seg_start += g.S;
-    }
+    // segments whose first output lies before g_end
+    const long long s = ln.seg_start / g.S, first = s * g.S_c + g.n_past;
+    if (first < g_end) RC(run_lane(h, (int)li, nullptr, 0, (g_end - 1 - first) / g.S_c + 1, g_end));
   }
   RC(join_streams(h));
   h->flushed = true;
@@ -1689,8 +1697,8 @@ int pond_reset(pond_t h) {
   if (!h->multi) {
     CK(cudaMemsetAsync(h->prof_sum, 0, h->nbins * sizeof(double), h->st));
     CK(cudaMemsetAsync(h->prof_hits, 0, h->nbins * sizeof(long long), h->st));
-    CK(cudaMemsetAsync(h->psum, 0, (size_t)MAX_FOLD_PARTS * h->nbins * sizeof(double), h->st));
-    CK(cudaMemsetAsync(h->phits, 0, (size_t)MAX_FOLD_PARTS * h->nbins * sizeof(long long), h->st));
+    CK(cudaMemsetAsync(h->psum, 0, (size_t)h->fold_rows * h->nbins * sizeof(double), h->st));
+    CK(cudaMemsetAsync(h->phits, 0, (size_t)h->fold_rows * h->nbins * sizeof(long long), h->st));
   }
   CK(cudaMemsetAsync(h->ts, 0, (size_t)ntr * h->ring * sizeof(float), h->st));
   CK(cudaMemsetAsync(h->ts_cnt, 0, (size_t)ntr * h->ring * sizeof(int), h->st));
@@ -1720,7 +1728,7 @@ int pond_profile(pond_t h, double* sum, int64_t* hits, pond_meta* meta) {
   if (h->multi) return fail(POND_E_STATE, "a batched plan does not fold");
   CK(cudaSetDevice(h->device));
   RC(join_streams(h));
-  CK(launch_fold_snapshot(h->psum, h->phits, h->nbins, h->prof_sum, h->prof_hits, h->st));
+  CK(launch_fold_snapshot(h->psum, h->phits, h->fold_rows, h->nbins, h->prof_sum, h->prof_hits, h->st));
   if (sum) CK(cudaMemcpyAsync(sum, h->prof_sum, h->nbins * sizeof(double), cudaMemcpyDeviceToHost, h->st));
   if (hits) CK(cudaMemcpyAsync(hits, h->prof_hits, h->nbins * sizeof(long long), cudaMemcpyDeviceToHost, h->st));
   CK(cudaStreamSynchronize(h->st));

@@ -145,91 +145,237 @@ __global__ void k_make_tw2(float2* lo, float2* hi, int logn, int sign) {
 constexpr int FOLD_WARPS = 4;
 constexpr int FOLD_U = 4;        // 32-sample groups in flight per warp
 
-// bin(g) = min(floor(frac(g * inc) * nbins), nbins - 1), FP64, correctly rounded.
-__device__ __forceinline__ int fold_bin(long long g, double inc, int nbins) {
-  const double x = __dmul_rn((double)g, inc);
-  const double ph = __dsub_rn(x, floor(x));
-  const int b = (int)__dmul_rn(ph, (double)nbins);
-  return b < nbins - 1 ? b : nbins - 1;
+// The fold's phase rules: phase(g) in cycles and whether it is known to run
+// forwards over samples [ga, gb] in its FP64 evaluation.  Each FP64 operation
+// is rounded on its own, so bins are those of a plain evaluation.
+struct ConstPeriod {
+  double inc;
+  __device__ __forceinline__ double operator()(long long g) const { return __dmul_rn((double)g, inc); }
+  __device__ __forceinline__ bool forwards(long long, long long) const { return true; }   // one rounded product: monotone
+};
+
+// Polynomial phase model, Horner's rule.
+struct PhaseRule {
+  FoldPhase r;
+  __device__ __forceinline__ double operator()(long long g) const {
+    const double tau = __dsub_rn(__dmul_rn((double)g, r.dt), r.t_ref);
+    double x = r.c[r.nc - 1];
+    for (int k = r.nc - 2; k >= 0; --k) x = __dadd_rn(__dmul_rn(x, tau), r.c[k]);
+    return x;
+  }
+  // phi' at the middle less its largest change over the span, times dt, against the
+  // evaluation's rounding (sum |c_i| |tau|^i eps, with room to spare)
+  __device__ bool forwards(long long ga, long long gb) const {
+    const double t0 = (double)ga * r.dt - r.t_ref, t1 = (double)gb * r.dt - r.t_ref;
+    const double tm = 0.5 * (t0 + t1), half = 0.5 * (t1 - t0), ta = fmax(fabs(t0), fabs(t1));
+    double d = 0.0, dd = 0.0, mag = 0.0, pm = 1.0, pa1 = 1.0, pa2 = 0.0;
+    for (int i = 0; i < r.nc; ++i) {
+      const double c = fabs(r.c[i]);
+      if (i >= 1) {
+        d += i * r.c[i] * pm;
+        pm *= tm;
+      }
+      if (i >= 2) {
+        pa2 = i == 2 ? 1.0 : pa2 * ta;
+        dd += i * (i - 1) * c * pa2;
+      }
+      mag += c * pa1;
+      pa1 *= ta;
+    }
+    // tau itself is rounded: to |g dt| + |t_ref| ulps, times the slope
+    const double slope = d + dd * half;
+    const double err = 1e-14 * (mag + slope * (fabs((double)gb * r.dt) + fabs(r.t_ref)));
+    return (d - dd * half) * r.dt > err;   // false for NaN
+  }
+};
+
+// bin = min(floor((phi - floor(phi)) nbins), nbins - 1); key = floor(phi) nbins + bin.
+__device__ __forceinline__ int phase_bin(double x, int nbins, double* key = nullptr) {
+  const double q = floor(x);
+  const int t = (int)__dmul_rn(__dsub_rn(x, q), (double)nbins), b = t < nbins - 1 ? t : nbins - 1;
+  if (key) *key = q * (double)nbins + (double)b;   // an integer below 2^53: exact
+  return b;
 }
 
-// The bin of g under the fold's phase rule: the constant period, or the
-// polynomial phase model (Horner's rule, each FP64 multiply and add rounded
-// on its own; bin = min(floor((phi - floor(phi)) nbins), nbins - 1)).
-__device__ __forceinline__ int fold_bin(long long g, const FoldPhase& r, int nbins) {
-  if (r.nc == 0) return fold_bin(g, r.inc, nbins);
-  const double tau = __dsub_rn(__dmul_rn((double)g, r.dt), r.t_ref);
-  double x = r.c[r.nc - 1];
-  for (int k = r.nc - 2; k >= 0; --k) x = __dadd_rn(__dmul_rn(x, tau), r.c[k]);
-  const int b = (int)__dmul_rn(__dsub_rn(x, floor(x)), (double)nbins);
-  return b < nbins - 1 ? b : nbins - 1;
+// Fold a window of 32 FOLD_RUN channel samples [c, ..) of P (global index g + i) whose
+// phase runs forwards: lane l takes FOLD_RUN consecutive samples, evaluates the phase at
+// the first and last of them and, where the bin changes in between, finds the
+// change by bisection, so a window costs two to seven phase evaluations per lane
+// instead of FOLD_RUN (an SM retires two FP64 operations per clock, which bounded the
+// per-sample form: a 2^20-sample segment 34.7 -> 7 us, nine segments of 113k samples with a
+// phase model 579 -> 83 us).  Each lane's one or two FP32 sums are joined with its neighbours' of the
+// same bin in FP64, in lane order.  False (nothing added) when a lane's samples span more
+// than two bins or the window comes back to a bin.
+constexpr int FOLD_RUN = 32, FOLD_WIN = 32 * FOLD_RUN;
+template <class Rule>
+__device__ __forceinline__ bool fold_window(const float* __restrict__ P, long long c, long long g, const Rule& rule,
+                                            int nbins, int b0, double* myh, int* myc) {
+  const int lane = threadIdx.x & 31;
+  float v[FOLD_RUN];
+  const float4* src = reinterpret_cast<const float4*>(P + c) + lane * (FOLD_RUN / 4);
+#pragma unroll
+  for (int i = 0; i < FOLD_RUN / 4; ++i) {
+    const float4 q = __ldg(src + i);
+    v[4 * i] = q.x;
+    v[4 * i + 1] = q.y;
+    v[4 * i + 2] = q.z;
+    v[4 * i + 3] = q.w;
+  }
+  const long long ga = g + lane * FOLD_RUN;
+  double kf, kt;
+  const int bf = phase_bin(rule(ga), nbins, &kf), bt = phase_bin(rule(ga + FOLD_RUN - 1), nbins, &kt);
+  int split = FOLD_RUN;   // samples before the change of bin
+  bool ok = true;
+  if (__any_sync(0xffffffffu, kf != kt)) {
+    int lo = 0, hi = FOLD_RUN - 1;   // key(lo) = kf, key(hi) > kf
+    double kh = kt;
+#pragma unroll 1
+    for (int s = 0; s < 5; ++s) {
+      const int mid = (lo + hi) >> 1;
+      double km;
+      phase_bin(rule(ga + mid), nbins, &km);
+      if (km > kf) {
+        hi = mid;
+        kh = km;
+      } else {
+        lo = mid;
+      }
+    }
+    if (kf != kt) {
+      split = hi;
+      ok = kh == kt;
+    }
+  }
+  const double k0 = __shfl_sync(0xffffffffu, kf, 0), k1 = __shfl_sync(0xffffffffu, kt, 31);
+  if (!__all_sync(0xffffffffu, ok) || !(k1 - k0 < (double)nbins)) return false;
+  float sl = 0.f, sr = 0.f;
+  {
+    float l[4] = {0.f, 0.f, 0.f, 0.f}, r[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < FOLD_RUN; ++i) {
+      l[i & 3] += i < split ? v[i] : 0.f;
+      r[i & 3] += i < split ? 0.f : v[i];
+    }
+    sl = (l[0] + l[1]) + (l[2] + l[3]);
+    sr = (r[0] + r[1]) + (r[2] + r[3]);
+  }
+  // chain of the lanes' last bins: lane l continues lane l-1's sum when all its
+  // samples lie in that bin
+  const bool two = split < FOLD_RUN;
+  const double kp = __shfl_up_sync(0xffffffffu, kt, 1), kn = __shfl_down_sync(0xffffffffu, kf, 1);
+  const bool joins = lane > 0 && kp == kf;   // the first part belongs to the previous lane's bin
+  double s = two ? (double)sr : (double)sl;
+  int n = two ? FOLD_RUN - split : FOLD_RUN;
+  bool open = joins && !two;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const double ps = __shfl_up_sync(0xffffffffu, s, d);
+    const int pn = __shfl_up_sync(0xffffffffu, n, d);
+    const bool po = __shfl_up_sync(0xffffffffu, open, d);
+    if (lane >= d && open) {
+      s += ps;
+      n += pn;
+      open = po;
+    }
+  }
+  const double ps = __shfl_up_sync(0xffffffffu, s, 1);
+  const int pn = __shfl_up_sync(0xffffffffu, n, 1);
+  if (two) {
+    const int e = bf >= b0 ? bf - b0 : bf - b0 + nbins;
+    myh[e] += joins ? ps + (double)sl : (double)sl;
+    myc[e] += joins ? pn + split : split;
+  }
+  __syncwarp();
+  if (lane == 31 || kn != kt) {
+    const int e = bt >= b0 ? bt - b0 : bt - b0 + nbins;
+    myh[e] += s;
+    myc[e] += n;
+  }
+  __syncwarp();
+  return true;
+}
+
+// Fold 32 channel samples, one per lane, into the warp's histogram (b < 0: none).
+__device__ __forceinline__ void fold_group(int b, float p, int nbins, int b0, double* myh, int* myc, float* mybuf) {
+  const int lane = threadIdx.x & 31;
+  const bool ok = b >= 0;
+  const unsigned peers = __match_any_sync(0xffffffffu, b);
+  const int first = __ffs(peers) - 1;
+  const int last = 31 - __clz(peers);
+  const unsigned span = (last == 31 ? 0xffffffffu : ((1u << (last + 1)) - 1u)) & ~((1u << first) - 1u);
+  if (__all_sync(0xffffffffu, peers == span)) {
+    // every bin's lanes are contiguous: segmented scan in a fixed tree order
+    float x = p;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const float y = __shfl_up_sync(0xffffffffu, x, d);
+      if (lane - d >= first) x += y;
+    }
+    if (ok && lane == last) {
+      const int e = b >= b0 ? b - b0 : b - b0 + nbins;
+      myh[e] += (double)x;
+      myc[e] += last - first + 1;
+    }
+  } else {
+    // a period shorter than a warp: the group leader sums its lanes in order
+    mybuf[lane] = p;
+    __syncwarp();
+    if (ok && lane == first) {
+      float sum = 0.f;
+      unsigned m = peers;
+      while (m) {
+        sum += mybuf[__ffs(m) - 1];
+        m &= m - 1;
+      }
+      const int e = b >= b0 ? b - b0 : b - b0 + nbins;
+      myh[e] += (double)sum;
+      myc[e] += __popc(peers);
+    }
+  }
+  __syncwarp();
 }
 
 // Fold channel samples [c0, c1) of P (global index g0 + c) into this warp's
-// histogram (FOLD_WARPS warps share the chunk: warp w takes groups of
-// 32 * FOLD_U samples w, w + FOLD_WARPS, ...).  Bin b is kept at entry
-// (b - b0) mod nbins, so a chunk that spans a short cyclic run of bins starting
-// at b0 needs only that run's entries.
+// histogram; FOLD_WARPS warps share the chunk.  Where there is a window for every warp, whole
+// windows whose phase runs forwards go through fold_window (with fewer, one warp would
+// work through what four share sample by sample: 15,600 samples 5 against 20 us); the
+// rest goes sample by sample, FOLD_U groups of 32 per warp and
+// step (their loads and phases in flight before the groups are added in order).
+// Bin b is kept at entry (b - b0) mod nbins, so a chunk that spans a short cyclic
+// run of bins starting at b0 needs only that run's entries.
 template <class Rule>
 __device__ __forceinline__ void fold_chunk(const float* __restrict__ P, long long c0, long long c1, long long g0,
                                            const Rule& rule, int nbins, int b0, double* myh, int* myc, float* mybuf) {
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // FOLD_U groups of 32 samples per warp and iteration: their loads and FP64
-  // bin computations are all in flight before the groups are scanned in order
-  for (long long base = c0 + (long long)w * 32 * FOLD_U; base < c1; base += FOLD_WARPS * 32 * FOLD_U) {
-    float pv[FOLD_U];
-    int bv[FOLD_U];
+  auto by_sample = [&](long long a, long long e, int step) {
+    for (long long base = a; base < e; base += step) {
+      float pv[FOLD_U];
+      int bv[FOLD_U];
 #pragma unroll
-    for (int u = 0; u < FOLD_U; ++u) {
-      const long long i = base + u * 32 + lane;
-      pv[u] = 0.f;
-      bv[u] = -1;
-      if (i < c1) {
-        pv[u] = __ldg(P + i);
-        bv[u] = fold_bin(g0 + i, rule, nbins);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < FOLD_U; ++u) {
-      const int b = bv[u];
-      const bool ok = b >= 0;
-      const float p = pv[u];
-      const unsigned peers = __match_any_sync(0xffffffffu, b);
-      const int first = __ffs(peers) - 1;
-      const int last = 31 - __clz(peers);
-      const unsigned span = (last == 31 ? 0xffffffffu : ((1u << (last + 1)) - 1u)) & ~((1u << first) - 1u);
-      if (__all_sync(0xffffffffu, peers == span)) {
-        // every bin's lanes are contiguous: segmented scan in a fixed tree order
-        float x = p;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-          const float y = __shfl_up_sync(0xffffffffu, x, d);
-          if (lane - d >= first) x += y;
-        }
-        if (ok && lane == last) {
-          const int e = b >= b0 ? b - b0 : b - b0 + nbins;
-          myh[e] += (double)x;
-          myc[e] += last - first + 1;
-        }
-      } else {
-        // a period shorter than a warp: the group leader sums its lanes in order
-        mybuf[lane] = p;
-        __syncwarp();
-        if (ok && lane == first) {
-          float sum = 0.f;
-          unsigned m = peers;
-          while (m) {
-            sum += mybuf[__ffs(m) - 1];
-            m &= m - 1;
-          }
-          const int e = b >= b0 ? b - b0 : b - b0 + nbins;
-          myh[e] += (double)sum;
-          myc[e] += __popc(peers);
+      for (int u = 0; u < FOLD_U; ++u) {
+        const long long i = base + u * 32 + lane;
+        pv[u] = 0.f;
+        bv[u] = -1;
+        if (i < e) {
+          pv[u] = __ldg(P + i);
+          bv[u] = phase_bin(rule(g0 + i), nbins);
         }
       }
-      __syncwarp();
+#pragma unroll
+      for (int u = 0; u < FOLD_U; ++u) fold_group(bv[u], pv[u], nbins, b0, myh, myc, mybuf);
     }
+  };
+  long long tail = c0;
+  if ((reinterpret_cast<uintptr_t>(P + c0) & 15) == 0 && c1 - c0 >= FOLD_WARPS * FOLD_WIN &&
+      rule.forwards(g0 + c0, g0 + c1)) {
+    const int nwin = (int)((c1 - c0) / FOLD_WIN);
+    for (int i = w; i < nwin; i += FOLD_WARPS) {
+      const long long c = c0 + (long long)i * FOLD_WIN;
+      if (!fold_window(P, c, g0 + c, rule, nbins, b0, myh, myc)) by_sample(c, c + FOLD_WIN, 32 * FOLD_U);
+    }
+    tail = c0 + (long long)nwin * FOLD_WIN;
   }
+  by_sample(tail + (long long)w * 32 * FOLD_U, c1, FOLD_WARPS * 32 * FOLD_U);
 }
 
 // Shared-memory layout of the fold kernels: [FOLD_WARPS][nbins] FP64 sums,
@@ -264,7 +410,7 @@ __global__ void __launch_bounds__(FOLD_WARPS * 32) k_fold_partial(const float* _
   const FoldSmem f = fold_smem_init(fsm, nbins, nbins);
   const int w = threadIdx.x >> 5;
   const long long c0 = (long long)blockIdx.x * chunk;
-  fold_chunk(P, c0, min(n, c0 + chunk), g0, inc, nbins, 0, f.hsum + w * nbins, f.hcnt + w * nbins,
+  fold_chunk(P, c0, min(n, c0 + chunk), g0, ConstPeriod{inc}, nbins, 0, f.hsum + w * nbins, f.hcnt + w * nbins,
              f.pbuf + w * 32);
   __syncthreads();
   for (int b = threadIdx.x; b < nbins; b += blockDim.x) {
@@ -285,120 +431,140 @@ __device__ __forceinline__ long long ceil_div_ll(long long a, long long b) { ret
 // Series samples spanning at most DEC_SPAN channel samples load them together.
 constexpr int DEC_SPAN = 16;
 
-// Fold + decimation of one segment's valid span [g0, g0 + n) in one launch.
-// CTA b owns the series samples j in [j_lo + b jpc, j_lo + (b+1) jpc) and the
-// channel samples they cover: it folds them (its histogram is added to
-// partial row b, which accumulates over the segments of the stream and is
-// merged when the profile is read) and then sums each of its series samples
-// (one thread per j for spans under 64 channel samples, else one warp per j
-// with four partial sums).  Every j belongs to one CTA, so no atomics.
+// The sum of P[g0 .. g0 + n) over g in [a, e) by one thread (spans under 64 samples).
+__device__ __forceinline__ float dec_span(const float* __restrict__ P, long long a, long long e) {
+  float s = 0.f;
+  if (e - a <= DEC_SPAN) {
+    // loads issued together, added in sample order
+    float v[DEC_SPAN];
+#pragma unroll
+    for (int i = 0; i < DEC_SPAN; ++i) v[i] = a + i < e ? __ldg(P + a + i) : 0.f;
+#pragma unroll
+    for (int i = 0; i < DEC_SPAN; ++i)
+      if (a + i < e) s += v[i];
+  } else {
+    for (long long g = a; g < e; ++g) s += __ldg(P + g);
+  }
+  return s;
+}
+
+// The same by one warp: four partial sums per lane, then a fixed tree.
+__device__ __forceinline__ float dec_span_warp(const float* __restrict__ P, long long a, long long e, int lane) {
+  float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+  long long g = a + lane;
+  for (; g + 96 < e; g += 128) {
+    s0 += __ldg(P + g);
+    s1 += __ldg(P + g + 32);
+    s2 += __ldg(P + g + 64);
+    s3 += __ldg(P + g + 96);
+  }
+  if (g < e) s0 += __ldg(P + g);
+  if (g + 32 < e) s1 += __ldg(P + g + 32);
+  if (g + 64 < e) s2 += __ldg(P + g + 64);
+  float s = (s0 + s1) + (s2 + s3);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  return s;
+}
+
+// Fold + decimation of the valid spans of nseg consecutive segments in one launch.
+// The first parts nseg CTAs fold: CTA (y, x) adds chunk x of segment y to partial
+// row (s mod slots) parts + x, which accumulates over the stream and is merged
+// when the profile is read; a launch holds at most `slots` segments, so no two of
+// its CTAs share a row and every row takes its segments in order however they
+// are grouped.  The other CTAs own the series samples j: one thread per j for spans under
+// 64 channel samples, else one warp.  A sample that straddles segments adds one
+// sum per segment, in order, as separate launches would.  No atomics.
 template <bool MODEL>
-__global__ void __launch_bounds__(FOLD_WARPS * 32) k_fold_dec(const float* __restrict__ P, long long n,
-                                                              long long g0, FoldPhase rule, int nbins,
+__global__ void __launch_bounds__(FOLD_WARPS * 32) k_fold_dec(const float* __restrict__ P, FoldSegs f, FoldPhase rule,
+                                                              int nbins, int slots, int parts, long long chunk,
                                                               long long num, long long den, long long j_lo,
-                                                              long long nj, long long jpc,
-                                                              float* __restrict__ T, int* __restrict__ C,
-                                                              long long ring, double* __restrict__ psum,
+                                                              long long nj, float* __restrict__ T,
+                                                              int* __restrict__ C, long long ring,
+                                                              double* __restrict__ psum,
                                                               long long* __restrict__ phits) {
   extern __shared__ unsigned char fsm[];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long ja = j_lo + (long long)blockIdx.x * jpc;
-  const long long jb = min(j_lo + nj, ja + jpc);
-  const long long ga = max(ceil_div_ll(ja * num, den), g0);
-  const long long gb = min(ceil_div_ll(jb * num, den), g0 + n);
-  // at the constant period the phase grows with g, so a chunk shorter than one
-  // period (with a margin of two bins) covers the cyclic run of bins
-  // fold_bin(ga) .. fold_bin(gb - 1); a phase model keeps every bin
-  int b0 = 0, used = nbins;
-  if (!MODEL && gb > ga && (double)(gb - 1 - ga) * rule.inc < 1.0 - 2.0 / nbins) {
-    b0 = fold_bin(ga, rule.inc, nbins);
-    const int b1 = fold_bin(gb - 1, rule.inc, nbins);
-    used = (b1 >= b0 ? b1 - b0 : b1 - b0 + nbins) + 1;
+  const int nfold = parts * f.nseg;
+  if ((int)blockIdx.x < nfold) {
+    const int y = blockIdx.x / parts, x = blockIdx.x - y * parts;
+    const long long n = min(f.S_c, f.n_left - y * f.S_c), c0 = x * chunk, c1 = min(n, c0 + chunk);
+    if (c1 <= c0) return;
+    const long long gy = f.g0 + y * f.S_c;
+    // at the constant period the phase grows with g, so a chunk shorter than one
+    // period (with a margin of two bins) covers the cyclic run of bins
+    // of its first and last sample; a phase model keeps every bin
+    int b0 = 0, used = nbins;
+    if (!MODEL && (double)(c1 - 1 - c0) * rule.inc < 1.0 - 2.0 / nbins) {
+      const ConstPeriod cp{rule.inc};
+      b0 = phase_bin(cp(gy + c0), nbins);
+      const int b1 = phase_bin(cp(gy + c1 - 1), nbins);
+      used = (b1 >= b0 ? b1 - b0 : b1 - b0 + nbins) + 1;
+    }
+    const FoldSmem fs = fold_smem_init(fsm, nbins, used);
+    const float* Py = P + y * f.M;
+    if constexpr (MODEL)
+      fold_chunk(Py, c0, c1, gy, PhaseRule{rule}, nbins, b0, fs.hsum + w * nbins, fs.hcnt + w * nbins, fs.pbuf + w * 32);
+    else
+      fold_chunk(Py, c0, c1, gy, ConstPeriod{rule.inc}, nbins, b0, fs.hsum + w * nbins, fs.hcnt + w * nbins, fs.pbuf + w * 32);
+    __syncthreads();
+    const size_t row = (size_t)((f.s0 + y) % slots) * parts + x;
+    for (int e = threadIdx.x; e < used; e += blockDim.x) {
+      double s = 0.0;
+      int h = 0;
+#pragma unroll
+      for (int q = 0; q < FOLD_WARPS; ++q) {
+        s += fs.hsum[q * nbins + e];
+        h += fs.hcnt[q * nbins + e];
+      }
+      const int b = b0 + e < nbins ? b0 + e : b0 + e - nbins;
+      psum[row * nbins + b] += s;
+      phits[row * nbins + b] += h;
+    }
+    return;
   }
-  const FoldSmem f = fold_smem_init(fsm, nbins, used);
-  if constexpr (MODEL)
-    fold_chunk(P, ga - g0, gb - g0, g0, rule, nbins, b0, f.hsum + w * nbins, f.hcnt + w * nbins, f.pbuf + w * 32);
-  else
-    fold_chunk(P, ga - g0, gb - g0, g0, rule.inc, nbins, b0, f.hsum + w * nbins, f.hcnt + w * nbins,
-               f.pbuf + w * 32);
-  __syncthreads();
-  for (int e = threadIdx.x; e < used; e += blockDim.x) {
-    double s = 0.0;
-    int h = 0;
-#pragma unroll
-    for (int k = 0; k < FOLD_WARPS; ++k) {
-      s += f.hsum[k * nbins + e];
-      h += f.hcnt[k * nbins + e];
-    }
-    const int b = b0 + e < nbins ? b0 + e : b0 + e - nbins;
-    psum[(size_t)blockIdx.x * nbins + b] += s;
-    phits[(size_t)blockIdx.x * nbins + b] += h;
+  const long long g_end = f.g0 + f.n_left;
+  const bool by_warp = num >= 64 * den;
+  const long long jj = by_warp ? (long long)(blockIdx.x - nfold) * FOLD_WARPS + w
+                               : (long long)(blockIdx.x - nfold) * (FOLD_WARPS * 32) + threadIdx.x;
+  if (jj >= nj) return;
+  const long long j = j_lo + jj, slot = j % ring;
+  long long a = max(ceil_div_ll(j * num, den), f.g0);
+  const long long e = min(ceil_div_ll((j + 1) * num, den), g_end);
+  const int c = (int)max(e - a, 0ll);
+  const bool owner = !by_warp || lane == 0;
+  float t = owner ? T[slot] : 0.f;
+  while (a < e) {   // uniform over a warp in the by_warp form
+    const long long y = (a - f.g0) / f.S_c, base = f.g0 + y * f.S_c, ey = min(e, base + f.S_c);
+    t += by_warp ? dec_span_warp(P + y * f.M, a - base, ey - base, lane) : dec_span(P + y * f.M, a - base, ey - base);
+    a = ey;
   }
-  if (num < 64 * den) {
-    for (long long j = ja + threadIdx.x; j < jb; j += blockDim.x) {
-      const long long a = max(ceil_div_ll(j * num, den), g0), e = min(ceil_div_ll((j + 1) * num, den), g0 + n);
-      float s = 0.f;
-      if (e - a <= DEC_SPAN) {
-        // loads issued together, added in sample order
-        float v[DEC_SPAN];
-#pragma unroll
-        for (int i = 0; i < DEC_SPAN; ++i) v[i] = a + i < e ? __ldg(P + (a + i - g0)) : 0.f;
-#pragma unroll
-        for (int i = 0; i < DEC_SPAN; ++i)
-          if (a + i < e) s += v[i];
-      } else {
-        for (long long g = a; g < e; ++g) s += __ldg(P + (g - g0));
-      }
-      const long long slot = j % ring;
-      T[slot] += s;
-      C[slot] += (int)max(e - a, 0ll);
-    }
-  } else {
-    for (long long j = ja + w; j < jb; j += FOLD_WARPS) {
-      const long long a = max(ceil_div_ll(j * num, den), g0), e = min(ceil_div_ll((j + 1) * num, den), g0 + n);
-      float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-      long long g = a + lane;
-      for (; g + 96 < e; g += 128) {
-        s0 += __ldg(P + (g - g0));
-        s1 += __ldg(P + (g + 32 - g0));
-        s2 += __ldg(P + (g + 64 - g0));
-        s3 += __ldg(P + (g + 96 - g0));
-      }
-      if (g < e) s0 += __ldg(P + (g - g0));
-      if (g + 32 < e) s1 += __ldg(P + (g + 32 - g0));
-      if (g + 64 < e) s2 += __ldg(P + (g + 64 - g0));
-      float s = (s0 + s1) + (s2 + s3);
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-      if (lane == 0) {
-        const long long slot = j % ring;
-        T[slot] += s;
-        C[slot] += (int)max(e - a, 0ll);
-      }
-    }
+  if (owner) {
+    T[slot] = t;
+    C[slot] += c;
   }
 }
 
-// A CTA merges 32 consecutive bins: warp y sums parts y, y + 8, y + 16, ... in
+// A CTA merges 32 consecutive bins: warp y of W sums parts y, y + W, y + 2 W, ... in
 // order (lanes read 32 consecutive bins of a part: coalesced), then lane x of
-// warp 0 adds the eight warp sums of bin x in a fixed order.  ACC adds the
+// warp 0 adds the warp sums of bin x in a fixed order.  ACC adds the
 // result to the profile, otherwise it replaces it.
-constexpr int MERGE_WARPS = 8;
+constexpr int MERGE_WARPS = 8, SNAP_WARPS = 32;
 
-template <typename H, bool ACC>
-__global__ void __launch_bounds__(MERGE_WARPS * 32) k_fold_merge(const double* __restrict__ psum,
+template <typename H, bool ACC, int W>
+__global__ void __launch_bounds__(W * 32) k_fold_merge(const double* __restrict__ psum,
                                                                  const H* __restrict__ phits, int nparts,
                                                                  int nbins, double* __restrict__ prof_sum,
                                                                  long long* __restrict__ prof_hits) {
-  __shared__ double ss[MERGE_WARPS][32];
-  __shared__ long long sh[MERGE_WARPS][32];
+  __shared__ double ss[W][32];
+  __shared__ long long sh[W][32];
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
   const int b = blockIdx.x * 32 + x;
   double s = 0.0;
   long long h = 0;
   if (b < nbins) {
 #pragma unroll 4
-    for (int k = y; k < nparts; k += MERGE_WARPS) {
+    for (int k = y; k < nparts; k += W) {
       s += __ldg(psum + (size_t)k * nbins + b);
       h += (long long)__ldg(phits + (size_t)k * nbins + b);
     }
@@ -410,7 +576,7 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32) k_fold_merge(const double* _
     double t = 0.0;
     long long c = 0;
 #pragma unroll
-    for (int k = 0; k < MERGE_WARPS; ++k) {
+    for (int k = 0; k < W; ++k) {
       t += ss[k][x];
       c += sh[k][x];
     }
@@ -687,10 +853,10 @@ size_t smem_inv_cols_det(int nl) {
 
 cudaError_t launch_fwd_rows_inv(const Geom& g, const float2* in, float2* out, const float2* tw3L, Tw2 tw2L,
                                 const float2* tw, const float2* twJ, const ChirpAnchor* anc, int clog,
-                                const float2* ctab, cudaStream_t st) {
+                                const float2* ctab, cudaStream_t st, int nseg) {
   const int R2 = 1 << g.logR2, R1 = 1 << g.logR1;
   const int nl = std::min(TILE / R1, R2);
-  const unsigned grid = (unsigned)(R2 / nl);
+  const dim3 grid((unsigned)(R2 / nl), (unsigned)nseg);
   switch (R1) {
 #define CASE(R)                                                                                             \
   case R:                                                                                                   \
@@ -761,15 +927,15 @@ int fused_groups(const Geom& g) {
 }
 
 cudaError_t launch_inv_cols_det(const Geom& g, const float2* in, float* P, float* part, int* cnt, float2* vout,
-                                long long vstride, long long vofs, int m_lo, int m_hi, const float2* tw,
-                                const float2* wtw, cudaStream_t st, int ntr) {
+                                long long vstride, long long vofs, const MSpan& span, const float2* tw,
+                                const float2* wtw, cudaStream_t st, int nu) {
   const int R2 = 1 << g.logR2, R1 = 1 << g.logR1;
   const int nl = std::min(TILE / R2, g.nchan);
-  const dim3 grid((unsigned)(R1 / nl), (unsigned)ntr);
+  const dim3 grid((unsigned)(R1 / nl), (unsigned)nu);
   const float scale = 1.0f / (float)(1u << g.logM);
   const int lognch = g.logR1 - (g.logM - g.logR2);
-  // several trials: each has its own L-element input, M-element P, partials and tickets
-  const TrialStride ts = ntr > 1 ? TrialStride{g.L, g.M, (long long)fused_groups(g) * g.M, FUSED_J}
+  // several trials or segments: each has its own L-element input, M-element P, partials and tickets
+  const TrialStride ts = nu > 1 ? TrialStride{g.L, g.M, (long long)fused_groups(g) * g.M, FUSED_J}
                                  : TrialStride{0, 0, 0, 0};
   // 512-, 1024- and 2048-point columns that fill a tile (at least TILE / R2
   // sub-channels; always so from 1024 on) take the form with 64 values per
@@ -783,10 +949,10 @@ cudaError_t launch_inv_cols_det(const Geom& g, const float2* in, float* P, float
   case R:                                                                                                        \
     if (vout)                                                                                                    \
       k_inv_cols_det_w<R, true><<<grid, WIDE_NT, wide_smem_bytes<64, R / 64>(), st>>>(                          \
-          in, P, part, cnt, vout, vstride, vofs, logG, g.logM - g.logR2, m_lo, m_hi, scale, wtw, ts);            \
+          in, P, part, cnt, vout, vstride, vofs, logG, g.logM - g.logR2, span, scale, wtw, ts);            \
     else                                                                                                         \
       k_inv_cols_det_w<R, false><<<grid, WIDE_NT, wide_smem_bytes<64, R / 64>(), st>>>(                         \
-          in, P, part, cnt, vout, vstride, vofs, logG, g.logM - g.logR2, m_lo, m_hi, scale, wtw, ts);            \
+          in, P, part, cnt, vout, vstride, vofs, logG, g.logM - g.logR2, span, scale, wtw, ts);            \
     return cudaGetLastError();
       CASE(512) CASE(1024) CASE(2048)
 #undef CASE
@@ -794,7 +960,7 @@ cudaError_t launch_inv_cols_det(const Geom& g, const float2* in, float* P, float
     }
   }
   switch (R2) {
-#define CASE(R) case R: k_inv_cols_det<R><<<grid, NT, smem_inv_cols_det<R>(nl), st>>>(in, P, part, cnt, vout, vstride, vofs, g.logR1, lognch, g.logM - g.logR2, m_lo, m_hi, scale, tw, ts); break;
+#define CASE(R) case R: k_inv_cols_det<R><<<grid, NT, smem_inv_cols_det<R>(nl), st>>>(in, P, part, cnt, vout, vstride, vofs, g.logR1, lognch, g.logM - g.logR2, span, scale, tw, ts); break;
     POND_FUSED_R2(CASE)
 #undef CASE
     default: return cudaErrorInvalidValue;
@@ -845,27 +1011,27 @@ cudaError_t set_kernel_attributes() {
 }
 
 // The pass launchers pick the FP32 or the tensor-core instantiation.
-cudaError_t launch_fwd_cols(const Geom& g, SegIn in, float2* out, const float2* tw, cudaStream_t st) {
-  return g.tc_terms ? launch_fwd_cols_tc(g, in, out, tw, st) : launch_fwd_cols_t<false>(g, in, out, tw, st);
+cudaError_t launch_fwd_cols(const Geom& g, const SegSrc& in, float2* out, const float2* tw, cudaStream_t st, int nseg) {
+  return g.tc_terms ? launch_fwd_cols_tc(g, in, out, tw, st, nseg) : launch_fwd_cols_t<false>(g, in, out, tw, st, nseg);
 }
 
 cudaError_t launch_fwd_rows(const Geom& g, const float2* in, float2* out, const float2* tw3L, Tw2 tw2L, const float2* tw,
-                            cudaStream_t st) {
-  return g.tc_terms ? launch_fwd_rows_tc(g, in, out, tw3L, tw2L, tw, st)
-                    : launch_fwd_rows_t<false>(g, in, out, tw3L, tw2L, tw, st);
+                            cudaStream_t st, int nseg) {
+  return g.tc_terms ? launch_fwd_rows_tc(g, in, out, tw3L, tw2L, tw, st, nseg)
+                    : launch_fwd_rows_t<false>(g, in, out, tw3L, tw2L, tw, st, nseg);
 }
 
 cudaError_t launch_inv_cols(const Geom& g, const float2* in, float2* out, const ChirpAnchor* anc,
-                            int clog, const float2* tw, cudaStream_t st) {
-  return g.tc_terms ? launch_inv_cols_tc(g, in, out, anc, clog, tw, st)
-                    : launch_inv_cols_t<false>(g, in, out, anc, clog, tw, st);
+                            int clog, const float2* tw, cudaStream_t st, int nseg) {
+  return g.tc_terms ? launch_inv_cols_tc(g, in, out, anc, clog, tw, st, nseg)
+                    : launch_inv_cols_t<false>(g, in, out, anc, clog, tw, st, nseg);
 }
 
 cudaError_t launch_inv_rows(const Geom& g, const float2* buf, float* P, float2* vout, long long vstride,
-                            long long vofs, int m_lo, int m_hi, const float2* tw3M, const float2* tw,
-                               cudaStream_t st) {
-  return g.tc_terms ? launch_inv_rows_tc(g, buf, P, vout, vstride, vofs, m_lo, m_hi, tw3M, tw, st)
-                    : launch_inv_rows_t<false>(g, buf, P, vout, vstride, vofs, m_lo, m_hi, tw3M, tw, st);
+                            long long vofs, const MSpan& span, const float2* tw3M, const float2* tw,
+                            cudaStream_t st, int nseg) {
+  return g.tc_terms ? launch_inv_rows_tc(g, buf, P, vout, vstride, vofs, span, tw3M, tw, st, nseg)
+                    : launch_inv_rows_t<false>(g, buf, P, vout, vstride, vofs, span, tw3M, tw, st, nseg);
 }
 
 size_t fold_smem_bytes(int nbins) {
@@ -885,40 +1051,47 @@ cudaError_t launch_fold(const float* P, long long n, long long g0, double inc, i
   long long chunk;
   const int parts = fold_parts(n, &chunk);
   k_fold_partial<<<parts, FOLD_WARPS * 32, fold_smem_bytes(nbins), st>>>(P, n, g0, inc, nbins, chunk, psum, phits);
-  k_fold_merge<int, true><<<(nbins + 31) / 32, MERGE_WARPS * 32, 0, st>>>(psum, phits, parts, nbins, prof_sum,
+  k_fold_merge<int, true, MERGE_WARPS><<<(nbins + 31) / 32, MERGE_WARPS * 32, 0, st>>>(psum, phits, parts, nbins, prof_sum,
                                                                           prof_hits);
   return cudaGetLastError();
 }
 
-cudaError_t launch_fold_dec(const float* P, long long n, long long g0, const FoldPhase& ph, int nbins, long long num,
-                            long long den, long long j_lo, long long nj, float* T, int* C, long long ring,
-                            double* psum, long long* phits, cudaStream_t st) {
-  if (n <= 0 || nj <= 0) return cudaSuccess;
-  // whole series samples per CTA: at least FOLD_MIN_SAMPLES channel samples
-  // each, at most MAX_FOLD_PARTS CTAs.  The fold runs beside the passes of the
-  // next segments, and each resident fold CTA holds registers a pass CTA would
-  // use: a few long-lived CTAs displace less than many short ones (full rate,
-  // 105k samples per segment, CTAs: 304: 112.5k, 152: 113.9k, 76: 114.8k,
-  // 38: 114.8k, 19: 114.0k Msamples/s), while segments of a million samples
-  // (one sub-channel) still spread over every SM.
-  constexpr long long FOLD_MIN_SAMPLES = 1400;
-  const long long per_j = std::max(1ll, num / den);
-  long long jpc = std::max((nj + MAX_FOLD_PARTS - 1) / MAX_FOLD_PARTS, (FOLD_MIN_SAMPLES + per_j - 1) / per_j);
-  jpc = std::min(jpc, nj);
-  const unsigned parts = (unsigned)((nj + jpc - 1) / jpc);
+// Segments per launch: 2^25 bins' worth (four segments of a 2^24-point plan, so
+// that a pass runs many waves of CTAs), at most 16.
+int fold_slots(const Geom& g) { return (int)std::max<long long>(1, std::min<long long>(16, (1ll << 25) / g.L)); }
+
+// Fold CTAs per segment: whole windows, one per warp and more where 1024 partial rows
+// would not hold them.
+static long long fold_chunk_len(const Geom& g) {
+  const long long most = std::max(1, std::min(64, 1024 / fold_slots(g)));
+  const long long step = (long long)FOLD_WARPS * FOLD_WIN;
+  return ((g.S_c + most - 1) / most + step - 1) / step * step;
+}
+int fold_parts_seg(const Geom& g) { return (int)((g.S_c + fold_chunk_len(g) - 1) / fold_chunk_len(g)); }
+
+cudaError_t launch_fold_dec(const Geom& g, const float* P, const FoldSegs& f, const FoldPhase& ph, int nbins, long long num,
+                            long long den, float* T, int* C, long long ring, double* psum, long long* phits,
+                            cudaStream_t st) {
+  if (f.n_left <= 0) return cudaSuccess;
+  const int slots = fold_slots(g), parts = fold_parts_seg(g);
+  if (f.nseg > slots) return cudaErrorInvalidValue;
+  const long long chunk = fold_chunk_len(g);
+  const long long j_lo = (f.g0 * den) / num, nj = ((f.g0 + f.n_left - 1) * den) / num - j_lo + 1;
+  const long long per = num >= 64 * den ? FOLD_WARPS : FOLD_WARPS * 32;
+  const unsigned blocks = (unsigned)(parts * f.nseg + (nj + per - 1) / per);
   if (ph.nc > 0)
-    k_fold_dec<true><<<parts, FOLD_WARPS * 32, fold_smem_bytes(nbins), st>>>(P, n, g0, ph, nbins, num, den, j_lo, nj,
-                                                                           jpc, T, C, ring, psum, phits);
+    k_fold_dec<true><<<blocks, FOLD_WARPS * 32, fold_smem_bytes(nbins), st>>>(P, f, ph, nbins, slots, parts, chunk, num, den,
+                                                                            j_lo, nj, T, C, ring, psum, phits);
   else
-    k_fold_dec<false><<<parts, FOLD_WARPS * 32, fold_smem_bytes(nbins), st>>>(P, n, g0, ph, nbins, num, den, j_lo, nj,
-                                                                            jpc, T, C, ring, psum, phits);
+    k_fold_dec<false><<<blocks, FOLD_WARPS * 32, fold_smem_bytes(nbins), st>>>(P, f, ph, nbins, slots, parts, chunk, num,
+                                                                             den, j_lo, nj, T, C, ring, psum, phits);
   return cudaGetLastError();
 }
 
-cudaError_t launch_fold_snapshot(const double* psum, const long long* phits, int nbins, double* prof_sum,
+cudaError_t launch_fold_snapshot(const double* psum, const long long* phits, int rows, int nbins, double* prof_sum,
                                  long long* prof_hits, cudaStream_t st) {
-  k_fold_merge<long long, false><<<(nbins + 31) / 32, MERGE_WARPS * 32, 0, st>>>(psum, phits, MAX_FOLD_PARTS, nbins,
-                                                                                prof_sum, prof_hits);
+  k_fold_merge<long long, false, SNAP_WARPS><<<(nbins + 31) / 32, SNAP_WARPS * 32, 0, st>>>(psum, phits, rows, nbins,
+                                                                                          prof_sum, prof_hits);
   return cudaGetLastError();
 }
 

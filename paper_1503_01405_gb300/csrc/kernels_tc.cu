@@ -32,24 +32,25 @@ cudaError_t launch_inv_cols_det_tc(const Geom& g, const float2* in, float* P, fl
   return cudaGetLastError();
 }
 
-cudaError_t launch_fwd_cols_tc(const Geom& g, SegIn in, float2* out, const float2* tw, cudaStream_t st) {
-  return launch_fwd_cols_t<true>(g, in, out, tw, st);
+cudaError_t launch_fwd_cols_tc(const Geom& g, const SegSrc& in, float2* out, const float2* tw, cudaStream_t st,
+                               int nseg) {
+  return launch_fwd_cols_t<true>(g, in, out, tw, st, nseg);
 }
 
 cudaError_t launch_fwd_rows_tc(const Geom& g, const float2* in, float2* out, const float2* tw3L, Tw2 tw2L, const float2* tw,
-                               cudaStream_t st) {
-  return launch_fwd_rows_t<true>(g, in, out, tw3L, tw2L, tw, st);
+                               cudaStream_t st, int nseg) {
+  return launch_fwd_rows_t<true>(g, in, out, tw3L, tw2L, tw, st, nseg);
 }
 
 cudaError_t launch_inv_cols_tc(const Geom& g, const float2* in, float2* out, const ChirpAnchor* anc,
-                               int clog, const float2* tw, cudaStream_t st) {
-  return launch_inv_cols_t<true>(g, in, out, anc, clog, tw, st);
+                               int clog, const float2* tw, cudaStream_t st, int nseg) {
+  return launch_inv_cols_t<true>(g, in, out, anc, clog, tw, st, nseg);
 }
 
 cudaError_t launch_inv_rows_tc(const Geom& g, const float2* buf, float* P, float2* vout, long long vstride,
-                               long long vofs, int m_lo, int m_hi, const float2* tw3M, const float2* tw,
-                               cudaStream_t st) {
-  return launch_inv_rows_t<true>(g, buf, P, vout, vstride, vofs, m_lo, m_hi, tw3M, tw, st);
+                               long long vofs, const MSpan& span, const float2* tw3M, const float2* tw,
+                               cudaStream_t st, int nseg) {
+  return launch_inv_rows_t<true>(g, buf, P, vout, vstride, vofs, span, tw3M, tw, st, nseg);
 }
 
 // One CTA waits, with the tensor-core stages' bounded wait, on a barrier that

@@ -102,8 +102,8 @@ struct Lin {
   }
 };
 
-// Per-trial strides (elements) of a column pass launched over several trials
-// (blockIdx.y = trial); all zero for a single trial.
+// Strides (elements) of a column pass launched over several trials or segments
+// (blockIdx.y); all zero for a single one.
 struct TrialStride {
   long long in, P, part;
   int cnt;
@@ -196,11 +196,34 @@ __device__ __forceinline__ float2 f1_pair(const SegIn& in, long long q) {
   }
 }
 
+// Segment y's two runs and how they may be loaded (nl: columns per CTA).
+__device__ __forceinline__ SegIn seg_runs(const SegSrc& s, unsigned y, int nl) {
+  SegIn in;
+  const long long r = s.r0 + (long long)y * s.step;
+  in.ch = s.ch;
+  if (r < 0) {
+    in.a = s.carry_end + r;
+    in.a_len = min(-r, s.bytes);
+    in.b = s.d;
+    in.b_len = min(s.bytes - in.a_len, s.avail);
+  } else {
+    in.a = s.d + r;
+    in.a_len = max(0ll, min(s.bytes, s.avail - r));
+    in.b = nullptr;
+    in.b_len = 0;
+  }
+  in.vec8 = in.ch == 1 && (nl & 3) == 0 && ((uintptr_t)in.a & 7) == 0 && (in.a_len & 7) == 0 &&
+            (in.b_len == 0 || ((uintptr_t)in.b & 7) == 0);
+  in.pair4 = in.ch == 2 && ((uintptr_t)in.a & 3) == 0 && (in.a_len & 3) == 0 && (in.b_len & 3) == 0 &&
+             (in.b_len == 0 || ((uintptr_t)in.b & 3) == 0);
+  return in;
+}
+
 // z viewed as [R2][R1] (z[n1 + R1 n2]); a CTA transforms nl adjacent columns n1
 // and stores them in place (the twiddle exp(-2 pi i n1 k2 / L) is F2's).
 template <int R2, bool TC>
-__global__ void __launch_bounds__(NT, 2) k_fwd_cols(SegIn in, float2* __restrict__ out, int logR1,
-                                                    const float2* __restrict__ tw, TcArgs tca) {
+__global__ void __launch_bounds__(NT, 2) k_fwd_cols(SegSrc src, float2* __restrict__ out, int logR1,
+                                                    long long ostride, const float2* __restrict__ tw, TcArgs tca) {
   extern __shared__ float2 smem[];
   float2* stw = smem;
   float2* sm = smem + stage_table_size(R2);
@@ -209,6 +232,8 @@ __global__ void __launch_bounds__(NT, 2) k_fwd_cols(SegIn in, float2* __restrict
   const int nl = min(TILE / R2, R1);
   const int lognl = __ffs(nl) - 1;
   const int tot = nl * R2;
+  const SegIn in = seg_runs(src, blockIdx.y, nl);
+  out += blockIdx.y * ostride;
   load_twiddles<R2>(stw, tw);
   tc::Ctx tcc;
   if constexpr (TC) tc::setup(tcc, sm, tile_f2<R2, TC, LSTR>(nl), tca);
@@ -518,6 +543,8 @@ __global__ void __launch_bounds__(NT, 2) k_fwd_rows(const float2* __restrict__ i
   constexpr int LSTR = line_stride(R1);
   constexpr int LOGR1 = ilog2c(R1);
   load_tw3(st3, tw3L);
+  in += (size_t)blockIdx.y << logL;
+  out += (size_t)blockIdx.y << logL;
   const int R2 = 1 << logR2;
   const int nl = min(TILE / R1, R2);   // 2 * pairs
   const int np = nl >> 1;
@@ -636,6 +663,8 @@ __global__ void __launch_bounds__(NT, 2) k_fwd_rows_inv(const float2* __restrict
   float2* stw = st3 + TW3_SN;
   float2* stwj = stw + stage_table_size(R1);
   float2* twk = stwj + stage_table_size(J);        // [nl][J]: e^{2 pi i k2 m1 / M}
+  in += (size_t)blockIdx.y << logL;
+  out += (size_t)blockIdx.y << logL;
   const int R2 = 1 << logR2;
   const int nl = min(TILE / R1, R2);
   const int np = nl >> 1;
@@ -823,6 +852,8 @@ __global__ void __launch_bounds__(NT, 2) k_inv_cols(const float2* __restrict__ i
                                                     int logQ1, int logM, int logR1, int logR2, int nchan,
                                                     const ChirpAnchor* __restrict__ anc, int clog,
                                                     const float2* __restrict__ tw, TcArgs tca) {
+  in += (size_t)blockIdx.y << (logR1 + logR2);
+  out += (size_t)blockIdx.y << (logR1 + logR2);
   extern __shared__ float2 smem[];
   ChirpAnchor* sanc = reinterpret_cast<ChirpAnchor*>(smem);   // [ANC_STAGE]
   float2* stw = smem + ANC_BYTES / sizeof(float2);
@@ -909,10 +940,13 @@ template <int Q1, bool TC>
 __global__ void __launch_bounds__(NT, 2) k_inv_rows(const float2* __restrict__ buf, float* __restrict__ P,
                                                     float2* __restrict__ vout, long long vstride,
                                                     long long vofs, int logQ2, int logM, int nchan,
-                                                    int m_lo, int m_hi, float scale,
+                                                    MSpan span, float scale,
                                                     const float2* __restrict__ tw3M,
                                                     const float2* __restrict__ tw, TcArgs tca) {
   extern __shared__ float2 smem[];
+  buf += ((size_t)blockIdx.y << logM) * nchan;
+  P += (size_t)blockIdx.y << logM;
+  const int m_lo = span.m_lo, m_hi = span.hi(blockIdx.y);
   float2* st3 = smem;                              // [TW3_SN], w = exp(+2 pi i / M)
   float2* stw = smem + TW3_SN;
   float2* sm = stw + stage_table_size(Q1);
@@ -1026,11 +1060,12 @@ __global__ void __launch_bounds__(NT, 2) k_inv_cols_det(const float2* __restrict
                                                         float* __restrict__ part, int* __restrict__ cnt,
                                                         float2* __restrict__ vout, long long vstride,
                                                         long long vofs, int logR1, int lognch, int logJ,
-                                                        int m_lo, int m_hi, float scale,
+                                                        MSpan span, float scale,
                                                         const float2* __restrict__ tw, TrialStride ts) {
   extern __shared__ float2 smem[];
   __shared__ int s_last;
-  // batched launches: blockIdx.y is the trial, with its own input, P, partials and tickets
+  const int m_lo = span.m_lo, m_hi = span.hi(blockIdx.y);
+  // blockIdx.y is the trial or segment, with its own input, P, partials and tickets
   in += blockIdx.y * ts.in;
   P += blockIdx.y * ts.P;
   part += blockIdx.y * ts.part;
@@ -1187,12 +1222,12 @@ cudaError_t set_attributes_t() {
 }
 
 template <bool TC>
-cudaError_t launch_fwd_cols_t(const Geom& g, SegIn in, float2* out, const float2* tw, cudaStream_t st) {
+cudaError_t launch_fwd_cols_t(const Geom& g, const SegSrc& in, float2* out, const float2* tw, cudaStream_t st, int nseg) {
   const int R2 = 1 << g.logR2, R1 = 1 << g.logR1;
   const int nl = std::min(TILE / R2, R1);
-  const unsigned grid = (unsigned)(R1 / nl);
+  const dim3 grid((unsigned)(R1 / nl), (unsigned)nseg);
   switch (R2) {
-#define CASE(R) case R: k_fwd_cols<R, TC><<<grid, NT, smem_bytes<R, TC, col_stride<R>()>(nl), st>>>(in, out, g.logR1, tw, g.tc_fwd); break;
+#define CASE(R) case R: k_fwd_cols<R, TC><<<grid, NT, smem_bytes<R, TC, col_stride<R>()>(nl), st>>>(in, out, g.logR1, g.L, tw, g.tc_fwd); break;
     POND_FOR_R(CASE)
 #undef CASE
     default: return cudaErrorInvalidValue;
@@ -1202,10 +1237,10 @@ cudaError_t launch_fwd_cols_t(const Geom& g, SegIn in, float2* out, const float2
 
 template <bool TC>
 cudaError_t launch_fwd_rows_t(const Geom& g, const float2* in, float2* out, const float2* tw3L, Tw2 tw2L, const float2* tw,
-                              cudaStream_t st) {
+                              cudaStream_t st, int nseg) {
   const int R2 = 1 << g.logR2, R1 = 1 << g.logR1;
   const int nl = std::min(TILE / R1, R2);
-  const unsigned grid = (unsigned)(R2 / nl);
+  const dim3 grid((unsigned)(R2 / nl), (unsigned)nseg);
   switch (R1) {
 #define CASE(R) case R: k_fwd_rows<R, TC><<<grid, NT, smem_bytes<R, TC>(nl) + TW3_BYTES, st>>>(in, out, g.logR2, g.logL, tw3L, tw2L, tw, g.tc_fwd); break;
     POND_FOR_R(CASE)
@@ -1217,11 +1252,11 @@ cudaError_t launch_fwd_rows_t(const Geom& g, const float2* in, float2* out, cons
 
 template <bool TC>
 cudaError_t launch_inv_cols_t(const Geom& g, const float2* in, float2* out, const ChirpAnchor* anc,
-                              int clog, const float2* tw, cudaStream_t st) {
+                              int clog, const float2* tw, cudaStream_t st, int nseg) {
   const int Q2 = 1 << g.logQ2, Q1 = 1 << g.logQ1;
   const int lines = g.nchan * Q1;
   const int nl = std::min(TILE / Q2, lines);
-  const unsigned grid = (unsigned)(lines / nl);
+  const dim3 grid((unsigned)(lines / nl), (unsigned)nseg);
   switch (Q2) {
 #define CASE(R) case R: k_inv_cols<R, TC><<<grid, NT, smem_bytes<R, TC, col_stride<R>()>(nl) + ANC_BYTES, st>>>(in, out, g.logQ1, g.logM, g.logR1, g.logR2, g.nchan, anc, clog, tw, g.tc_inv); break;
     POND_FOR_R(CASE)
@@ -1233,15 +1268,15 @@ cudaError_t launch_inv_cols_t(const Geom& g, const float2* in, float2* out, cons
 
 template <bool TC>
 cudaError_t launch_inv_rows_t(const Geom& g, const float2* buf, float* P, float2* vout, long long vstride,
-                              long long vofs, int m_lo, int m_hi, const float2* tw3M, const float2* tw,
-                               cudaStream_t st) {
+                              long long vofs, const MSpan& span, const float2* tw3M, const float2* tw,
+                              cudaStream_t st, int nseg) {
   const int Q2 = 1 << g.logQ2, Q1 = 1 << g.logQ1;
   const int b2 = std::min(TILE / (Q1 * g.nchan), Q2);
   const int nl = g.nchan * b2;
-  const unsigned grid = (unsigned)(Q2 / b2);
+  const dim3 grid((unsigned)(Q2 / b2), (unsigned)nseg);
   const float scale = 1.0f / (float)(1u << g.logM);
   switch (Q1) {
-#define CASE(R) case R: k_inv_rows<R, TC><<<grid, NT, smem_bytes<R, TC>(nl) + TW3_BYTES, st>>>(buf, P, vout, vstride, vofs, g.logQ2, g.logM, g.nchan, m_lo, m_hi, scale, tw3M, tw, g.tc_inv); break;
+#define CASE(R) case R: k_inv_rows<R, TC><<<grid, NT, smem_bytes<R, TC>(nl) + TW3_BYTES, st>>>(buf, P, vout, vstride, vofs, g.logQ2, g.logM, g.nchan, span, scale, tw3M, tw, g.tc_inv); break;
     POND_FOR_R(CASE)
 #undef CASE
     default: return cudaErrorInvalidValue;
@@ -1250,13 +1285,13 @@ cudaError_t launch_inv_rows_t(const Geom& g, const float2* buf, float* P, float2
 }
 
 // Tensor-core instantiations (kernels_tc.cu).
-cudaError_t launch_fwd_cols_tc(const Geom& g, SegIn in, float2* out, const float2* tw, cudaStream_t st);
+cudaError_t launch_fwd_cols_tc(const Geom& g, const SegSrc& in, float2* out, const float2* tw, cudaStream_t st, int nseg);
 cudaError_t launch_fwd_rows_tc(const Geom& g, const float2* in, float2* out, const float2* tw3L, Tw2 tw2L, const float2* tw,
-                               cudaStream_t st);
+                               cudaStream_t st, int nseg);
 cudaError_t launch_inv_cols_tc(const Geom& g, const float2* in, float2* out, const ChirpAnchor* anc,
-                               int clog, const float2* tw, cudaStream_t st);
+                               int clog, const float2* tw, cudaStream_t st, int nseg);
 cudaError_t launch_inv_rows_tc(const Geom& g, const float2* buf, float* P, float2* vout, long long vstride,
-                               long long vofs, int m_lo, int m_hi, const float2* tw3M, const float2* tw,
-                               cudaStream_t st);
+                               long long vofs, const MSpan& span, const float2* tw3M, const float2* tw,
+                               cudaStream_t st, int nseg);
 
 }  // namespace pond

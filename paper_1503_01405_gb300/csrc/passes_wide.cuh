@@ -31,14 +31,15 @@ template <int R2, bool VOUT>
 __global__ void __launch_bounds__(WIDE_NT, 3) k_inv_cols_det_w(const float2* __restrict__ in, float* __restrict__ P,
                                                                float* __restrict__ part, int* __restrict__ cnt,
                                                                float2* __restrict__ vout, long long vstride,
-                                                               long long vofs, int logG, int logJ, int m_lo, int m_hi,
+                                                               long long vofs, int logG, int logJ, MSpan span,
                                                                float scale, const float2* __restrict__ tw,
                                                                TrialStride ts) {
   constexpr int RA = 64, RB = R2 / RA, NL = TILE / R2, BPT = 64 / RB;
   constexpr int WSTR = wide_stride<RA, RB>();
   extern __shared__ float2 smem[];
   __shared__ int s_last;
-  // batched launches: blockIdx.y is the trial, with its own input, P, partials and tickets
+  const int m_lo = span.m_lo, m_hi = span.hi(blockIdx.y);
+  // blockIdx.y is the trial or segment, with its own input, P, partials and tickets
   in += blockIdx.y * ts.in;
   P += blockIdx.y * ts.P;
   part += blockIdx.y * ts.part;
@@ -47,7 +48,7 @@ __global__ void __launch_bounds__(WIDE_NT, 3) k_inv_cols_det_w(const float2* __r
   const int m1 = blockIdx.x >> logG, gi = blockIdx.x & ((1 << logG) - 1);
   const float2* blk = in + (size_t)blockIdx.x * TILE;   // block m1 G + g
   if (tid < 4) {
-    // the block of CTA blockIdx.x + WIDE_PF (in launch order, the next trial's
+    // the block of CTA blockIdx.x + WIDE_PF (in launch order, the next unit's
     // blocks after this trial's last), in four quarters
     const unsigned nx = gridDim.x, lin = blockIdx.y * nx + blockIdx.x + WIDE_PF;
     if (lin < nx * gridDim.y) {

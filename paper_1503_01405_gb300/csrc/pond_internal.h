@@ -11,7 +11,7 @@ namespace pond {
 
 constexpr int CHIRP_LOG_MAX = 15;            // at most 2^15 bins per chirp anchor
 constexpr int MAX_NBINS = 4096;              // fold bins (per-warp FP64 histograms in smem)
-constexpr int MAX_FOLD_PARTS = 304;          // fold CTAs per segment (2 per SM)
+constexpr int MAX_FOLD_PARTS = 304;          // CTAs of launch_fold (2 per SM)
 
 // Taylor coefficients of the dedispersion phase phi (cycles) about an anchor
 // bin: phi(k_a + d) = phi0 + phi1 d + phi2 d^2 + phi3 d^3.  The first three
@@ -63,6 +63,30 @@ struct SegIn {
                   // one complex sample's two N / S pairs (4 bytes) at a time
 };
 
+// The input of consecutive segments, one per blockIdx.y of a launch.  Byte r of
+// the stream, counted from the first new byte: carry_end[r] for r < 0, d[r] for
+// 0 <= r < avail, zero beyond.  Segment y starts at byte r0 + y step and spans
+// `bytes` bytes; F1 forms its two runs and alignment flags from these.
+struct SegSrc {
+  const int8_t* carry_end;
+  const int8_t* d;
+  long long avail, r0, step, bytes;
+  int ch;
+};
+
+// Emitted span of segment y of a launch: m_lo <= m < min(m_hi, m_end - y m_step).
+// Batched launches (blockIdx.y = trial) have m_step = 0.
+struct MSpan {
+  int m_lo, m_hi;
+  long long m_end, m_step;
+#ifdef __CUDACC__
+  __device__ __forceinline__ int hi(unsigned y) const {
+    const long long e = m_end - (long long)y * m_step;
+    return e < m_hi ? (int)e : m_hi;
+  }
+#endif
+};
+
 constexpr int TC_W_BYTES = 3 * 32 * 32 * 2;   // W16 hi, mid, lo parts of one direction
 
 // Tensor-core stage arguments: the W16 parts of one transform direction
@@ -110,14 +134,17 @@ int stage_tw_entries(int R);
 // Stage-2 twiddles of the 64-values-per-thread FFT of length R (512 .. 4096; none otherwise).
 cudaError_t launch_wide_tw(float2* out, int R, cudaStream_t st);
 int wide_tw_entries(int R);
-cudaError_t launch_fwd_cols(const Geom& g, SegIn in, float2* out, const float2* tw, cudaStream_t st);
+// Passes over nseg consecutive segments per launch (blockIdx.y): segment y reads
+// and writes its own L elements of the buffers (M of P).
+cudaError_t launch_fwd_cols(const Geom& g, const SegSrc& in, float2* out, const float2* tw, cudaStream_t st,
+                            int nseg = 1);
 cudaError_t launch_fwd_rows(const Geom& g, const float2* in, float2* out, const float2* tw3L, Tw2 tw2L, const float2* tw,
-                            cudaStream_t st);
+                            cudaStream_t st, int nseg = 1);
 cudaError_t launch_inv_cols(const Geom& g, const float2* in, float2* out, const ChirpAnchor* anc,
-                            int clog, const float2* tw, cudaStream_t st);
+                            int clog, const float2* tw, cudaStream_t st, int nseg = 1);
 cudaError_t launch_inv_rows(const Geom& g, const float2* buf, float* P, float2* vout, long long vstride,
-                            long long vofs, int m_lo, int m_hi, const float2* tw3M, const float2* tw,
-                               cudaStream_t st);
+                            long long vofs, const MSpan& span, const float2* tw3M, const float2* tw,
+                            cudaStream_t st, int nseg = 1);
 // Fused schedule (F1, F2f, Ic) for single-trial FP32 plans whose geometry has
 // J = M / R2 = FUSED_J; fused_groups = sub-channel groups per m1 in Ic.
 constexpr int FUSED_J = 64;
@@ -126,17 +153,17 @@ int fused_groups(const Geom& g);
 // ctab non-null: the chirp from that per-bin table (launch_chirp_c64), else from the anchors
 cudaError_t launch_fwd_rows_inv(const Geom& g, const float2* in, float2* out, const float2* tw3L, Tw2 tw2L,
                                 const float2* tw, const float2* twJ, const ChirpAnchor* anc, int clog,
-                                const float2* ctab, cudaStream_t st);
+                                const float2* ctab, cudaStream_t st, int nseg = 1);
 cudaError_t launch_chirp_c64(float2* tab, const Geom& g, double du, double half, double f0, double alpha, int sgn,
                              cudaStream_t st);
 cudaError_t launch_inv_rows_chirp(const Geom& g, const float2* in, float2* out, const float2* tw3L, const float2* twJ,
                                   const ChirpAnchor* anc, int clog, cudaStream_t st);
-// ntr > 1: one launch over ntr trials, trial t reading in + t L and writing
-// P + t M, part + t G M, cnt + t FUSED_J (G = fused_groups); wtw: launch_wide_tw of R2
+// nu > 1: one launch over nu trials or segments, the u-th reading in + u L and writing
+// P + u M, part + u G M, cnt + u FUSED_J (G = fused_groups); wtw: launch_wide_tw of R2
 // (null: the radix-16 stages with their tables tw)
 cudaError_t launch_inv_cols_det(const Geom& g, const float2* in, float* P, float* part, int* cnt, float2* vout,
-                                long long vstride, long long vofs, int m_lo, int m_hi, const float2* tw,
-                                const float2* wtw, cudaStream_t st, int ntr = 1);
+                                long long vstride, long long vofs, const MSpan& span, const float2* tw,
+                                const float2* wtw, cudaStream_t st, int nu = 1);
 // Batched lanes: Ir over ntr trials in one launch (trial t writes out + t L),
 // the chirp from the lane's Q0.32 table (table = true) or each trial's anchors
 cudaError_t launch_inv_rows_chirp_multi(const Geom& g, const float2* in, float2* out, int ntr, const float2* tw3L,
@@ -173,13 +200,22 @@ struct FoldPhase {
   double dt = 0, t_ref = 0;
   double c[8] = {};
 };
-// Fold + decimation of one segment (single-DM plans): the fold adds to
-// per-CTA partial rows [MAX_FOLD_PARTS][nbins] that accumulate over the
-// stream; launch_fold_snapshot merges them into the profile (replacing it).
-cudaError_t launch_fold_dec(const float* P, long long n, long long g0, const FoldPhase& ph, int nbins, long long num,
-                            long long den, long long j_lo, long long nj, float* T, int* C, long long ring,
-                            double* psum, long long* phits, cudaStream_t st);
-cudaError_t launch_fold_snapshot(const double* psum, const long long* phits, int nbins, double* prof_sum,
+// Fold + decimation of nseg consecutive segments s0 .. (single-DM plans).  Segment y's
+// power is P + y M, n_y = min(S_c, n_left - y S_c) samples from g0 + y S_c on.  The
+// fold of segment s adds to the fold_parts rows of its slot s mod fold_slots of the
+// partials [fold_rows][nbins], which accumulate over the stream, so the sums do not depend
+// on how the segments are grouped into launches (nseg <= fold_slots);
+// launch_fold_snapshot merges the rows into the profile (replacing it).
+struct FoldSegs {
+  long long s0, g0, S_c, M, n_left;
+  int nseg;
+};
+int fold_slots(const Geom& g);   // also the most segments per launch
+int fold_parts_seg(const Geom& g);
+cudaError_t launch_fold_dec(const Geom& g, const float* P, const FoldSegs& f, const FoldPhase& ph, int nbins, long long num,
+                            long long den, float* T, int* C, long long ring, double* psum, long long* phits,
+                            cudaStream_t st);
+cudaError_t launch_fold_snapshot(const double* psum, const long long* phits, int rows, int nbins, double* prof_sum,
                                  long long* prof_hits, cudaStream_t st);
 cudaError_t launch_decimate(const float* P, long long n, long long g0, long long num, long long den,
                             long long j_lo, long long nj, float* T, int* C, long long ring, cudaStream_t st);
