@@ -129,8 +129,8 @@ struct Lane {
   // per trial of the lane and slot: after that trial's fold / decimation of a segment
   std::vector<cudaEvent_t> ev_chain[NSLOT];
   float2* stw = nullptr;                    // stage twiddle tables of R1, R2, Q1, Q2
-  const float2 *stwR1 = nullptr, *stwR2 = nullptr, *stwQ1 = nullptr, *stwQ2 = nullptr, *stwJ = nullptr;
-  const float2* wtwR2 = nullptr;            // stage-2 twiddles of the 64-values-per-thread FFT of R2 (null: none)
+  const float2 *stwR1 = nullptr, *stwR2 = nullptr, *stwQ1 = nullptr, *stwQ2 = nullptr;
+  const float2 *wtwR1 = nullptr, *wtwR2 = nullptr;   // stage-2 twiddles of the 64-values-per-thread FFTs (512 and more)
   float2* tw2buf = nullptr;
   Tw2 tw2L;                                 // exp(-2 pi i e/(2L))
   float2* tw3L = nullptr;                   // three-level exp(-2 pi i e/L)
@@ -147,6 +147,7 @@ struct Lane {
   float* partm[NSLOT] = {};                 // [kt][G][M] column-pass group partials
   int* cntm[NSLOT] = {};                    // [kt][FUSED_J] column-pass tickets
   unsigned* atab = nullptr;                 // table form: Q0.32 phase of one DM step per bin (row layout)
+  unsigned* words = nullptr;                // anchor form: [trial][L] phase words, or null
   unsigned* d_nmul = nullptr;               // per lane trial: its DM in DM steps
   const ChirpAnchor** d_anc = nullptr;      // per lane trial: its anchor table
   int* d_clog = nullptr;
@@ -418,14 +419,14 @@ int build_lane(pond_t h, Lane* ln) {
   }
   const int n1 = stage_tw_entries(1 << g.logR1), n2 = stage_tw_entries(1 << g.logR2);
   const int n3 = stage_tw_entries(1 << g.logQ1), n4 = stage_tw_entries(1 << g.logQ2);
-  const int n5 = stage_tw_entries(FUSED_J), n6 = wide_tw_entries(1 << g.logR2);
+  const int n5 = wide_tw_entries(1 << g.logR1), n6 = wide_tw_entries(1 << g.logR2);
   CK(cudaMalloc(&ln->stw, (size_t)std::max(1, n1 + n2 + n3 + n4 + n5 + n6) * sizeof(float2)));
   ln->stwR1 = ln->stw;
   ln->stwR2 = ln->stwR1 + n1;
   ln->stwQ1 = ln->stwR2 + n2;
   ln->stwQ2 = ln->stwQ1 + n3;
-  ln->stwJ = ln->stwQ2 + n4;
-  ln->wtwR2 = n6 > 0 ? ln->stwJ + n5 : nullptr;
+  ln->wtwR1 = ln->stwQ2 + n4;
+  ln->wtwR2 = ln->wtwR1 + n5;
   auto nhi = [](int logn) { return logn > TW2_LOG ? (1ll << (logn - TW2_LOG)) : 1ll; };
   const long long total = TW2_LO + nhi(g.logL + 1) + 2 * 768;
   CK(cudaMalloc(&ln->tw2buf, total * sizeof(float2)));
@@ -440,7 +441,7 @@ int build_lane(pond_t h, Lane* ln) {
   CK(launch_stage_tw(const_cast<float2*>(ln->stwR2), 1 << g.logR2, h->st));
   CK(launch_stage_tw(const_cast<float2*>(ln->stwQ1), 1 << g.logQ1, h->st));
   CK(launch_stage_tw(const_cast<float2*>(ln->stwQ2), 1 << g.logQ2, h->st));
-  CK(launch_stage_tw(const_cast<float2*>(ln->stwJ), FUSED_J, h->st));
+  CK(launch_wide_tw(const_cast<float2*>(ln->wtwR1), 1 << g.logR1, h->st));
   CK(launch_wide_tw(const_cast<float2*>(ln->wtwR2), 1 << g.logR2, h->st));
   CK(launch_tw3(ln->tw3L, g.logL, -1, h->st));
   CK(launch_tw2(const_cast<float2*>(ln->tw2L.lo), const_cast<float2*>(ln->tw2L.hi), g.logL + 1, -1, h->st));
@@ -463,6 +464,7 @@ void free_lane(Lane* ln) {
     ln->ev_chain[k].clear();
   }
   cudaFree(ln->atab);
+  cudaFree(ln->words);
   cudaFree(ln->d_nmul);
   cudaFree(ln->d_anc);
   cudaFree(ln->d_clog);
@@ -677,11 +679,11 @@ int run_segments(pond_t h, int li, const SegSrc& src, long long s, int nseg, lon
     const Trial& t = h->trials[ln.trials[0]];
     if (ln.fused) {
       // three passes: F2f takes the chirp and the first inverse factor, Ic the rest
-      CK(launch_fwd_rows_inv(g, bufA, bufB, ln.tw3L, ln.tw2L, ln.stwR1, ln.stwJ, t.anc, t.clog, t.ctab, cs, nseg));
+      CK(launch_fwd_rows_inv(g, bufA, bufB, ln.tw3L, ln.tw2L, ln.wtwR1, t.anc, t.clog, t.ctab, cs, nseg));
       RC(record(h, 1 + ST_F2F, cs));
       h->launches += 4;
     } else {
-      CK(launch_fwd_rows(g, bufA, bufB, ln.tw3L, ln.tw2L, ln.stwR1, cs, nseg));
+      CK(launch_fwd_rows(g, bufA, bufB, ln.tw3L, ln.tw2L, ln.stwR1, ln.wtwR1, cs, nseg));
       RC(record(h, 1 + ST_F2, cs));
       // the chirp is applied as I1 loads the spectrum
       CK(launch_inv_cols(g, bufB, bufA, t.anc, t.clog, ln.stwQ2, cs, nseg));
@@ -710,7 +712,7 @@ int run_segments(pond_t h, int li, const SegSrc& src, long long s, int nseg, lon
     RC(record(h, 1 + ST_DEC, fs, true));
     if (!h->timing) CK(cudaEventRecord(h->ev_pfree[slot], fs));
   } else {
-    CK(launch_fwd_rows(g, bufA, bufB, ln.tw3L, ln.tw2L, ln.stwR1, cs));
+    CK(launch_fwd_rows(g, bufA, bufB, ln.tw3L, ln.tw2L, ln.stwR1, ln.wtwR1, cs));
     RC(record(h, 1 + ST_F2, cs));
     h->launches += 2;
     if (ln.mode == POND_TRIALS_MULTI_ANCHOR || ln.mode == POND_TRIALS_MULTI_TABLE) {
@@ -720,8 +722,9 @@ int run_segments(pond_t h, int li, const SegSrc& src, long long s, int nseg, lon
       const int ntr = (int)ln.trials.size();
       for (int b = 0, q0 = 0; q0 < ntr; ++b, q0 += ln.kt) {
         const int nq = std::min(ln.kt, ntr - q0);
-        const MultiChirp mc{ln.atab, ln.d_nmul + q0, ln.d_anc + q0, ln.d_clog + q0};
-        CK(launch_inv_rows_chirp_multi(g, bufB, ln.bufT[slot], nq, ln.tw3L, ln.stwJ, mc,
+        const MultiChirp mc{ln.atab, ln.d_nmul + q0, ln.words ? ln.words + (size_t)q0 * g.L : nullptr, ln.d_anc + q0,
+                            ln.d_clog + q0};
+        CK(launch_inv_rows_chirp_multi(g, bufB, ln.bufT[slot], nq, ln.tw3L, mc,
                                        ln.mode == POND_TRIALS_MULTI_TABLE, cs));
         if (b == 0) RC(record(h, 1 + ST_IR, cs));
         CK(launch_ic(h, ln, ln.bufT[slot], ln.Pm[slot], ln.partm[slot], ln.cntm[slot], nullptr, 0, 0, trials, cs, nq));
@@ -751,7 +754,7 @@ int run_segments(pond_t h, int li, const SegSrc& src, long long s, int nseg, lon
         const Trial& t = h->trials[d];
         if (ln.mode == POND_TRIALS_PER_TRIAL) {
           // the trial's chirp and the first inverse factor as Ir loads the shared spectrum's rows
-          CK(launch_inv_rows_chirp(g, bufB, bufA, ln.tw3L, ln.stwJ, t.anc, t.clog, cs));
+          CK(launch_inv_rows_chirp(g, bufB, bufA, ln.tw3L, t.anc, t.clog, cs));
           if (q == 0) RC(record(h, 1 + ST_IR, cs));
           CK(launch_ic(h, ln, bufA, P, ln.part[slot], ln.cnt[slot], nullptr, 0, 0, span, cs));
           if (q == 0) RC(record(h, 1 + ST_IC, cs));
@@ -968,13 +971,13 @@ int measure_lane(pond_t h, const pond_opts* o, long long nfft, double* t_fwd, do
   for (int it = 0; it <= reps && ce == cudaSuccess; ++it) {      // first pass warms up
     if (it == 1) ce = cudaEventRecord(e[0], h->st);
     if (ce == cudaSuccess) ce = launch_fwd_cols(g, in, ln.bufA[0], ln.stwR2, h->st);
-    if (ce == cudaSuccess) ce = launch_fwd_rows(g, ln.bufA[0], ln.bufB[0], ln.tw3L, ln.tw2L, ln.stwR1, h->st);
+    if (ce == cudaSuccess) ce = launch_fwd_rows(g, ln.bufA[0], ln.bufB[0], ln.tw3L, ln.tw2L, ln.stwR1, ln.wtwR1, h->st);
   }
   if (ce == cudaSuccess) ce = cudaEventRecord(e[1], h->st);
   for (int it = 0; it <= reps && ce == cudaSuccess; ++it) {
     if (it == 1) ce = cudaEventRecord(e[2], h->st);
     if (ln.fused_multi) {   // the per-trial passes the plan will run
-      if (ce == cudaSuccess) ce = launch_inv_rows_chirp(g, ln.bufB[0], ln.bufA[0], ln.tw3L, ln.stwJ, anc, clog, h->st);
+      if (ce == cudaSuccess) ce = launch_inv_rows_chirp(g, ln.bufB[0], ln.bufA[0], ln.tw3L, anc, clog, h->st);
       if (ce == cudaSuccess)
         ce = launch_ic(h, ln, ln.bufA[0], ln.P[0], ln.part[0], ln.cnt[0], nullptr, 0, 0, span, h->st);
     } else {
@@ -1107,6 +1110,20 @@ int alloc_multi(Lane* ln, int kt) {
   return POND_OK;
 }
 
+// The anchor form's phase words for every trial of the lane, while they stay below
+// WORDS_MAX bytes (otherwise the row pass evaluates the anchors per bin).
+constexpr size_t WORDS_MAX = 8ull << 30;
+int make_words(pond_t h, Lane* ln) {
+  const size_t n = (size_t)ln->g.L * ln->trials.size();
+  if (n * sizeof(unsigned) > WORDS_MAX) return POND_OK;
+  CK(cudaMalloc(&ln->words, n * sizeof(unsigned)));
+  for (size_t q = 0; q < ln->trials.size(); ++q) {
+    const Trial& t = h->trials[ln->trials[q]];
+    CK(launch_chirp_words(ln->words + q * ln->g.L, ln->g, t.anc, t.clog, h->st));
+  }
+  return POND_OK;
+}
+
 // Device time per trial (us) of one block of min(kt, ntrials) trials of the
 // lane in the given mode (row pass, column pass, decimation), on slot 0, by
 // CUDA events over three launches after a warm-up.  The series rows it adds to
@@ -1152,7 +1169,7 @@ int time_trials(pond_t h, Lane* ln, int mode, int kt, int split, double* us) {
     } else if (mode == POND_TRIALS_PER_TRIAL) {
       for (int q = 0; q < nq && ce == cudaSuccess; ++q) {
         const Trial& t = h->trials[ln->trials[q]];
-        ce = launch_inv_rows_chirp(g, ln->bufB[0], ln->bufA[0], ln->tw3L, ln->stwJ, t.anc, t.clog, h->st);
+        ce = launch_inv_rows_chirp(g, ln->bufB[0], ln->bufA[0], ln->tw3L, t.anc, t.clog, h->st);
         if (ce == cudaSuccess)
           ce = launch_ic(h, *ln, ln->bufA[0], ln->P[0], ln->part[0], ln->cnt[0], nullptr, 0, 0, span, h->st);
         if (ce == cudaSuccess)
@@ -1161,8 +1178,8 @@ int time_trials(pond_t h, Lane* ln, int mode, int kt, int split, double* us) {
                                h->ring, h->st);
       }
     } else {
-      const MultiChirp mc{ln->atab, ln->d_nmul, ln->d_anc, ln->d_clog};
-      ce = launch_inv_rows_chirp_multi(g, ln->bufB[0], ln->bufT[0], nq, ln->tw3L, ln->stwJ, mc,
+      const MultiChirp mc{ln->atab, ln->d_nmul, ln->words, ln->d_anc, ln->d_clog};
+      ce = launch_inv_rows_chirp_multi(g, ln->bufB[0], ln->bufT[0], nq, ln->tw3L, mc,
                                        mode == POND_TRIALS_MULTI_TABLE, h->st);
       if (ce == cudaSuccess)
         ce = launch_ic(h, *ln, ln->bufT[0], ln->Pm[0], ln->partm[0], ln->cntm[0], nullptr, 0, 0, span, h->st, nq);
@@ -1245,6 +1262,12 @@ int apply_tune(pond_t h, Lane* ln, const TrialTune& t) {
   ln->cand_split = t.csplit;
   ln->cand_us = t.cus;
   if (t.mode == POND_TRIALS_FOUR_PASS) RC(use_split(h, ln, t.split));
+  if (t.mode == POND_TRIALS_MULTI_ANCHOR) {
+    if (!ln->words) RC(make_words(h, ln));
+  } else {
+    cudaFree(ln->words);
+    ln->words = nullptr;
+  }
   if (t.mode == POND_TRIALS_PER_TRIAL || t.mode == POND_TRIALS_FOUR_PASS) {
     free_multi(ln);
     return POND_OK;
@@ -1304,6 +1327,7 @@ int setup_trials(pond_t h, const pond_opts* o, Lane* ln) {
     // the requested form (the table form only where the DMs allow it), else the table form where possible
     if (!multi_ok) return POND_OK;
     ln->mode = (req == POND_TRIALS_MULTI_ANCHOR) ? POND_TRIALS_MULTI_ANCHOR : best_multi;
+    if (ln->mode == POND_TRIALS_MULTI_ANCHOR) RC(make_words(h, ln));
     return alloc_multi(ln, kt_req ? kt_req : std::min(32, ntr));
   }
   // autotune: time every candidate on this lane, keep the fastest per trial
@@ -1330,7 +1354,10 @@ int setup_trials(pond_t h, const pond_opts* o, Lane* ln) {
     auto it = g_trial_tune.find(key);
     if (it != g_trial_tune.end()) return apply_tune(h, ln, it->second);
   }
-  if (!kts.empty()) RC(alloc_multi(ln, *std::max_element(kts.begin(), kts.end())));
+  if (!kts.empty()) {
+    RC(alloc_multi(ln, *std::max_element(kts.begin(), kts.end())));
+    RC(make_words(h, ln));
+  }
   CK(cudaMemsetAsync(ln->bufB[0], 0, (size_t)g.L * sizeof(float2), h->st));
   TrialTune t;
   size_t best = 0;

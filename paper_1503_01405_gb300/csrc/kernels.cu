@@ -685,13 +685,15 @@ __global__ void k_make_chirp_table(unsigned* tab, int logR1, int logR2, double d
 }
 
 // The inverse filter of Eq. 4 per bin as FP32 (cos, -sin) of 2 pi phi(k), in
-// the spectrum's row layout (bin k2 + R2 k1 at k2 R1 + k1): phi in FP64 with the
+// F2f's order: row k2, then the position j in a run of 64 columns, then the run c (bin
+// k2 + R2 (64 c + j) at k2 R1 + j NCH + c, NCH = R1 / 64).  phi in FP64 with the
 // anchors' formula, reduced mod 1, then FP64 sincospi, rounded once to FP32.
 __global__ void k_make_chirp_c64(float2* tab, int logR1, int logR2, double du, double half, double f0, double alpha,
                                  int sgn) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (1ll << (logR1 + logR2))) return;
-  const long long k2 = i >> logR1, k1 = i & ((1ll << logR1) - 1);
+  const long long k2 = i >> logR1, e = i & ((1ll << logR1) - 1), nch = 1ll << (logR1 - 6);
+  const long long k1 = ((e & (nch - 1)) << 6) + (e >> (logR1 - 6));
   const double k = (double)(k2 + (k1 << logR2));
   const double f = sgn > 0 ? __dsub_rn(__dmul_rn(k, du), half) : __dsub_rn(half, __dmul_rn(k, du));
   const double g = f0 + f;
@@ -701,6 +703,15 @@ __global__ void k_make_chirp_c64(float2* tab, int logR1, int logR2, double du, d
   double sn, cs;
   sincospi(2.0 * r, &sn, &cs);
   tab[i] = make_float2((float)cs, (float)-sn);
+}
+
+// A trial's phase words (anchor_word), in the same order as the table above.
+__global__ void k_make_chirp_words(unsigned* words, int logR1, int logR2, const ChirpAnchor* __restrict__ anc, int clog) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (1ll << (logR1 + logR2))) return;
+  const long long k2 = i >> logR1, e = i & ((1ll << logR1) - 1), nch = 1ll << (logR1 - 6);
+  const unsigned k = (unsigned)(k2 + ((((e & (nch - 1)) << 6) + (e >> (logR1 - 6))) << logR2));
+  words[i] = anchor_word(anc[k >> clog], clog, k);
 }
 
 // Byte copy between device buffers (any alignment): 16-byte words where both
@@ -762,6 +773,11 @@ cudaError_t launch_chirp_c64(float2* tab, const Geom& g, double du, double half,
                              cudaStream_t st) {
   const long long n = g.L;
   k_make_chirp_c64<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(tab, g.logR1, g.logR2, du, half, f0, alpha, sgn);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_chirp_words(unsigned* words, const Geom& g, const ChirpAnchor* anc, int clog, cudaStream_t st) {
+  k_make_chirp_words<<<(unsigned)((g.L + 255) / 256), 256, 0, st>>>(words, g.logR1, g.logR2, anc, clog);
   return cudaGetLastError();
 }
 
@@ -841,10 +857,6 @@ bool fused_geometry(const Geom& g) {
 }
 
 namespace {
-size_t smem_fwd_rows_inv(int R1, int nl) {
-  return ((size_t)TW3_SN + stage_table_size(R1) + stage_table_size(FUSED_J) + (size_t)nl * FUSED_J +
-          (size_t)nl * (R1 + R1 / 16)) * sizeof(float2);
-}
 template <int R2>
 size_t smem_inv_cols_det(int nl) {
   return ((size_t)stage_table_size(R2) + (size_t)nl * col_stride<R2>()) * sizeof(float2);
@@ -852,20 +864,19 @@ size_t smem_inv_cols_det(int nl) {
 }  // namespace
 
 cudaError_t launch_fwd_rows_inv(const Geom& g, const float2* in, float2* out, const float2* tw3L, Tw2 tw2L,
-                                const float2* tw, const float2* twJ, const ChirpAnchor* anc, int clog,
-                                const float2* ctab, cudaStream_t st, int nseg) {
-  const int R2 = 1 << g.logR2, R1 = 1 << g.logR1;
-  const int nl = std::min(TILE / R1, R2);
-  const dim3 grid((unsigned)(R2 / nl), (unsigned)nseg);
-  switch (R1) {
+                                const float2* wtw, const ChirpAnchor* anc, int clog, const float2* ctab,
+                                cudaStream_t st, int nseg) {
+  const RowTile rt = row_tile(g.logR1, g.logR2);
+  const dim3 tiles((unsigned)(g.L / TILE), (unsigned)nseg);
+  switch (1 << g.logR1) {
 #define CASE(R)                                                                                             \
   case R:                                                                                                   \
     if (ctab)                                                                                               \
-      k_fwd_rows_inv<R, FUSED_J, true><<<grid, NT, smem_fwd_rows_inv(R, nl), st>>>(                        \
-          in, out, g.logR2, g.logL, tw3L, tw2L, tw, twJ, anc, clog, ctab);                                  \
+      k_fwd_rows_w<R, ROW_TABLE><<<tiles, WIDE_NT, fwd_rows_smem_bytes<R>(rt), st>>>(in, out, rt, tw3L,     \
+                                                                                     tw2L, wtw, anc, clog, ctab); \
     else                                                                                                    \
-      k_fwd_rows_inv<R, FUSED_J, false><<<grid, NT, smem_fwd_rows_inv(R, nl), st>>>(                       \
-          in, out, g.logR2, g.logL, tw3L, tw2L, tw, twJ, anc, clog, ctab);                                  \
+      k_fwd_rows_w<R, ROW_ANCHORS><<<tiles, WIDE_NT, fwd_rows_smem_bytes<R>(rt), st>>>(in, out, rt, tw3L,   \
+                                                                                       tw2L, wtw, anc, clog, ctab); \
     break;
     POND_FUSED_R1(CASE)
 #undef CASE
@@ -874,20 +885,18 @@ cudaError_t launch_fwd_rows_inv(const Geom& g, const float2* in, float2* out, co
   return cudaGetLastError();
 }
 
-namespace {
-size_t smem_inv_rows_chirp(int R1, int nl) {
-  return ((size_t)TW3_SN + stage_table_size(FUSED_J) + (size_t)nl * FUSED_J + (size_t)nl * (R1 + R1 / 16)) *
-         sizeof(float2);
-}
-}  // namespace
-
-cudaError_t launch_inv_rows_chirp(const Geom& g, const float2* in, float2* out, const float2* tw3L, const float2* twJ,
-                                  const ChirpAnchor* anc, int clog, cudaStream_t st) {
-  const int R2 = 1 << g.logR2, R1 = 1 << g.logR1;
-  const int nl = std::min(TILE / R1, R2);
-  const unsigned grid = (unsigned)(R2 / nl);
-  switch (R1) {
-#define CASE(R) case R: k_inv_rows_chirp<R, FUSED_J><<<grid, NT, smem_inv_rows_chirp(R, nl), st>>>(in, out, g.logR2, tw3L, twJ, anc, clog); break;
+// Ir with the anchor chirp over ntr trials (mc), or over the one trial anc1 (mc.anc null).
+static cudaError_t launch_inv_rows_anchor(const Geom& g, const float2* in, float2* out, int ntr, const float2* tw3L,
+                                          MultiChirp mc, const ChirpAnchor* anc1, int clog1, cudaStream_t st) {
+  const RowTile rt = row_tile(g.logR1, g.logR2);
+  const unsigned tiles = (unsigned)(g.L / TILE);
+  const dim3 grid((unsigned)ntr, tiles);
+  switch (1 << g.logR1) {
+#define CASE(R)                                                                                             \
+  case R:                                                                                                   \
+    k_inv_rows_anchor<R><<<grid, WIDE_NT, anchor_smem_bytes<R>(rt), st>>>(in, out, g.L, rt, tw3L, mc, anc1, \
+                                                                          clog1);                           \
+    break;
     POND_FUSED_R1(CASE)
 #undef CASE
     default: return cudaErrorInvalidValue;
@@ -895,24 +904,39 @@ cudaError_t launch_inv_rows_chirp(const Geom& g, const float2* in, float2* out, 
   return cudaGetLastError();
 }
 
+cudaError_t launch_inv_rows_chirp(const Geom& g, const float2* in, float2* out, const float2* tw3L,
+                                  const ChirpAnchor* anc, int clog, cudaStream_t st) {
+  return launch_inv_rows_anchor(g, in, out, 1, tw3L, MultiChirp{}, anc, clog, st);
+}
+
 cudaError_t launch_inv_rows_chirp_multi(const Geom& g, const float2* in, float2* out, int ntr, const float2* tw3L,
-                                        const float2* twJ, MultiChirp mc, bool table, cudaStream_t st) {
-  const int R2 = 1 << g.logR2, R1 = 1 << g.logR1;
-  const int nl = std::min(TILE / R1, R2);
+                                        MultiChirp mc, bool table, cudaStream_t st) {
   if (ntr < 1) return cudaErrorInvalidValue;
-  // table form: one CTA per row tile runs every trial; anchor form: one CTA
-  // per (trial, row tile)
+  if (!table && !mc.words) return launch_inv_rows_anchor(g, in, out, ntr, tw3L, mc, nullptr, 0, st);
   const RowTile rt = row_tile(g.logR1, g.logR2);
-  const unsigned tiles = (unsigned)(R2 / nl);
-  switch (R1) {
+  const unsigned tiles = (unsigned)(g.L / TILE);
+  if (!table) {
+    // trials per CTA: four waves of three CTAs per SM, then as many trials as leave them
+    const int tpc = std::max(1, std::min(ntr, (int)((long long)tiles * ntr / (12ll * std::max(1, g.sms)))));
+    const dim3 grid((unsigned)((ntr + tpc - 1) / tpc), tiles);
+    switch (1 << g.logR1) {
 #define CASE(R)                                                                                             \
   case R:                                                                                                   \
-    if (table)                                                                                              \
-      k_inv_rows_table<R><<<tiles, TAB_GROUPS * WIDE_NT, table_smem_bytes<R>(rt), st>>>(in, out, g.L, rt,    \
-                                                                                        tw3L, mc, ntr);     \
-    else                                                                                                    \
-      k_inv_rows_chirp_multi<R, FUSED_J><<<dim3((unsigned)ntr, tiles), NT, smem_inv_rows_chirp(R, nl), st>>>( \
-          in, out, g.L, g.logR2, tw3L, twJ, mc);                                                            \
+    k_inv_rows_words<R><<<grid, WIDE_NT, anchor_smem_bytes<R>(rt), st>>>(in, out, g.L, rt, tw3L, mc.words,  \
+                                                                         ntr, tpc);                         \
+    break;
+      POND_FUSED_R1(CASE)
+#undef CASE
+      default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+  }
+  // table form: one CTA per row tile runs every trial
+  switch (1 << g.logR1) {
+#define CASE(R)                                                                                             \
+  case R:                                                                                                   \
+    k_inv_rows_table<R><<<tiles, TAB_GROUPS * WIDE_NT, table_smem_bytes<R>(rt), st>>>(in, out, g.L, rt,    \
+                                                                                      tw3L, mc, ntr);       \
     break;
     POND_FUSED_R1(CASE)
 #undef CASE
@@ -970,24 +994,21 @@ cudaError_t launch_inv_cols_det(const Geom& g, const float2* in, float* P, float
 
 cudaError_t set_kernel_attributes() {
   cudaError_t e = set_attributes_t<false>();
-#define SET_F(R) \
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fwd_rows_inv<R, FUSED_J, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_fwd_rows_inv(R, TILE / R)); \
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fwd_rows_inv<R, FUSED_J, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_fwd_rows_inv(R, TILE / R));
+#define SET_F(R)                                                                                               \
+  {                                                                                                            \
+    const RowTile rt{0, 0, 0, row_stride_max(R), row_stride_max(R)};                                           \
+    auto attr = [&](auto* f, size_t bytes) {                                                                   \
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); \
+    };                                                                                                         \
+    attr(k_fwd_rows_w<R, ROW_SPECTRUM>, fwd_rows_smem_bytes<R>(rt));                                           \
+    attr(k_fwd_rows_w<R, ROW_ANCHORS>, fwd_rows_smem_bytes<R>(rt));                                            \
+    attr(k_fwd_rows_w<R, ROW_TABLE>, fwd_rows_smem_bytes<R>(rt));                                              \
+    attr(k_inv_rows_words<R>, anchor_smem_bytes<R>(rt));                                                       \
+    attr(k_inv_rows_anchor<R>, anchor_smem_bytes<R>(rt));                                                      \
+    attr(k_inv_rows_table<R>, table_smem_bytes<R>(rt));                                                        \
+  }
   POND_FUSED_R1(SET_F)
 #undef SET_F
-#define SET_I(R) \
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_inv_rows_chirp<R, FUSED_J>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_inv_rows_chirp(R, TILE / R));
-  POND_FUSED_R1(SET_I)
-#undef SET_I
-#define SET_M(R)                                                                                       \
-  if (e == cudaSuccess)                                                                                \
-    e = cudaFuncSetAttribute(k_inv_rows_table<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,          \
-                             (int)table_smem_bytes<R>(RowTile{0, 0, 0, row_stride_max(R), row_stride_max(R)}));             \
-  if (e == cudaSuccess)                                                                                \
-    e = cudaFuncSetAttribute(k_inv_rows_chirp_multi<R, FUSED_J>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                             (int)smem_inv_rows_chirp(R, TILE / R));
-  POND_FUSED_R1(SET_M)
-#undef SET_M
 #define SET_C(R) \
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_inv_cols_det<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_inv_cols_det<R>(TILE / R));
   POND_FUSED_R2(SET_C)
@@ -1016,9 +1037,23 @@ cudaError_t launch_fwd_cols(const Geom& g, const SegSrc& in, float2* out, const 
 }
 
 cudaError_t launch_fwd_rows(const Geom& g, const float2* in, float2* out, const float2* tw3L, Tw2 tw2L, const float2* tw,
-                            cudaStream_t st, int nseg) {
-  return g.tc_terms ? launch_fwd_rows_tc(g, in, out, tw3L, tw2L, tw, st, nseg)
-                    : launch_fwd_rows_t<false>(g, in, out, tw3L, tw2L, tw, st, nseg);
+                            const float2* wtw, cudaStream_t st, int nseg) {
+  if (g.tc_terms) return launch_fwd_rows_tc(g, in, out, tw3L, tw2L, tw, st, nseg);
+  const RowTile rt = row_tile(g.logR1, g.logR2);
+  const dim3 tiles((unsigned)(g.L / TILE), (unsigned)nseg);
+  if (g.L >= TILE) {
+    switch (1 << g.logR1) {
+#define CASE(R)                                                                                             \
+  case R:                                                                                                   \
+    k_fwd_rows_w<R, ROW_SPECTRUM><<<tiles, WIDE_NT, fwd_rows_smem_bytes<R>(rt), st>>>(in, out, rt, tw3L,    \
+                                                                                      tw2L, wtw, nullptr, 0, nullptr); \
+    return cudaGetLastError();
+      POND_FUSED_R1(CASE)
+#undef CASE
+      default: break;
+    }
+  }
+  return launch_fwd_rows_t<false>(g, in, out, tw3L, tw2L, tw, st, nseg);
 }
 
 cudaError_t launch_inv_cols(const Geom& g, const float2* in, float2* out, const ChirpAnchor* anc,

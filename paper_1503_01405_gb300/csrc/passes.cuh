@@ -40,26 +40,31 @@
 
 namespace pond {
 
-// exp(-2 pi i phi(k)) from the anchor table: the phase mod 1 is exact to
-// < 1e-7 cycles (FP64-built fixed point, see k_make_chirp_anchors); the final
-// sine and cosine of 2 pi r, |r| <= 1/2 + 1e-3, use the hardware approximation
-// (absolute error about 4e-7 on [-pi, pi]).
-__device__ __forceinline__ float2 chirp_from(const ChirpAnchor& a, int clog, unsigned k) {
+// exp(-2 pi i r) for the phase r = u 2^-32 (mod 1) held as a Q0.32 word u; the
+// sine and cosine use the hardware approximation (absolute error about 4e-7 on [-pi, pi]).
+__device__ __forceinline__ float2 chirp_q32(unsigned u) {
+  float s, c;
+  __sincosf((float)(int)u * 1.4629180792671596e-9f, &s, &c);   // 2 pi 2^-32
+  return make_float2(c, -s);
+}
+
+// phi(k) mod 1 from the anchor table as a Q0.32 word: exact to < 1e-7 cycles
+// (FP64-built fixed point, see k_make_chirp_anchors).
+__device__ __forceinline__ unsigned anchor_word(const ChirpAnchor& a, int clog, unsigned k) {
   const int d = (int)(k & ((1u << clog) - 1)) - (int)((1u << clog) >> 1);   // |d| <= 2^14
   const unsigned dd = (unsigned)(d * d);
   // top 32 bits of phi0 + phi1 d + phi2 d^2 mod 1 in Q0.64: the high words
   // multiply mod 2^32, the low words contribute their products' high words
-  // (each truncation loses < 2^-32 cycles)
+  // (each truncation loses < 2^-32 cycles); the cubic term (below 1e-2 cycles) in FP32
   const unsigned p1h = (unsigned)(a.p1 >> 32), p1l = (unsigned)a.p1;
   const unsigned p2h = (unsigned)(a.p2 >> 32), p2l = (unsigned)a.p2;
-  const unsigned u = a.p0 + p1h * (unsigned)d + (unsigned)(((long long)p1l * d) >> 32) + p2h * dd +
-                     __umulhi(p2l, dd);
   const float df = (float)d;
-  float r = (float)(int)u * 2.3283064365386963e-10f;   // 2^-32
-  r = fmaf(a.p3 * df, df * df, r);
-  float s, c;
-  __sincosf(6.2831853071795865f * r, &s, &c);
-  return make_float2(c, -s);
+  return a.p0 + p1h * (unsigned)d + (unsigned)(((long long)p1l * d) >> 32) + p2h * dd + __umulhi(p2l, dd) +
+         (unsigned)__float2int_rn(a.p3 * df * (df * df) * 4294967296.f);
+}
+
+__device__ __forceinline__ float2 chirp_from(const ChirpAnchor& a, int clog, unsigned k) {
+  return chirp_q32(anchor_word(a, clog, k));
 }
 
 // Chirp anchors an I1 CTA stages in shared memory (16 KiB) before its lookups.
@@ -569,273 +574,6 @@ __global__ void __launch_bounds__(NT, 2) k_fwd_rows(const float2* __restrict__ i
   f2_split<R1, LSTR>(sm, q0, np, R2, logR2, logL, tw2L, [&](int, int row, int k1, float2 X) {
     out[((unsigned)row << LOGR1) + (unsigned)k1] = X;
   });
-}
-
-// Length-J (= 64 = 16 x 4) inverse DFT of every (slot, c) run of a row tile
-// (row stride R1 + R1/16, run c at c (J + J/16)), four lanes of one warp per
-// run (run = threadIdx.x / 4, lane t4): the Stockham radix-16 step (outputs of
-// butterfly t4 to 16 t4 + k) in registers, the exchange through the run's own
-// line with warp-level barriers, the radix-4 step (butterflies t4 + 4q, outputs
-// to t' + 16 j), then twk[slot][m1] = e^{2 pi i k2 m1 / M} and the store of
-// element (k2 = row_of(slot), m1, c) at ((m1 G + g) R2 + k2) nl_c + ci,
-// c = g nl_c + ci, nl_c = min(8192 / R2, NCH) (the column pass's blocks).
-// The run's first read takes element o of the tile (its offset in the padded
-// layout) from load(o); the runs' stores go to sm.
-template <int R1, int J, class RowOf, class Load>
-__device__ __forceinline__ void j_runs_load(float2* sm, const float2* stwj, const float2* twk,
-                                            float2* __restrict__ out, int nl, int logR2, RowOf row_of, Load load) {
-  static_assert(J == 64, "radix-16 x radix-4 runs");
-  constexpr int NCH = R1 / J;
-  constexpr int LSTR = R1 + R1 / 16;
-  constexpr int LOGNCH = ilog2c(NCH);
-  const int lognl = min(13 - logR2, LOGNCH);
-  const int run = (int)threadIdx.x >> 2, t4 = (int)threadIdx.x & 3;
-  if (run < nl * NCH) {                            // whole warps (8 runs each) in or out
-    const int slot = run >> LOGNCH, c = run & (NCH - 1);
-    const int lo = slot * LSTR + c * (J + J / 16);
-    float2* line = sm + lo;
-    float2 v[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = load(lo + pidx(0, t4 + 4 * i, 0));
-    Dft<16, true>::run(v);
-    __syncwarp();                                  // the run is read before it is overwritten
-#pragma unroll
-    for (int k = 0; k < 16; ++k) line[pidx(0, 16 * t4 + k, 0)] = v[k];
-    __syncwarp();
-    const unsigned k2 = (unsigned)row_of(slot);
-    const unsigned g = (unsigned)c >> lognl, ci = (unsigned)c & ((1u << lognl) - 1);
-    const unsigned ofs0 = (((g << logR2) + k2) << lognl) + ci;
-    const int mstep = LOGNCH + logR2;              // log2 of the m1 stride (G R2 nl_c)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int t = t4 + 4 * q;
-      float2 w[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) w[j] = line[t + 17 * j];   // element t + 16 j (t < 16)
-#pragma unroll
-      for (int j = 1; j < 4; ++j) w[j] = cmul(w[j], cconj(stwj[(j - 1) * 16 + t]));
-      Dft<4, true>::run(w);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int m1 = t + 16 * j;
-        out[ofs0 + ((unsigned)m1 << mstep)] = cmul(w[j], twk[slot * J + m1]);
-      }
-    }
-  }
-}
-
-// The runs of the tile held in sm.
-template <int R1, int J, class RowOf>
-__device__ __forceinline__ void j_runs(float2* sm, const float2* stwj, const float2* twk, float2* __restrict__ out,
-                                       int nl, int logR2, RowOf row_of) {
-  j_runs_load<R1, J>(sm, stwj, twk, out, nl, logR2, row_of, [&](int o) { return sm[o]; });
-}
-
-// ---------------------------------------------------------------------------
-// F2f: F2 with the chirp and the first factor of every sub-channel's inverse
-// ---------------------------------------------------------------------------
-
-// When R2 divides M, row k2 holds for sub-channel c the J = M/R2 bins
-// c M + k2 + R2 j (j < J) at columns c J + j, and with m = m1 + J m2
-//   v_c[m] = sum_k2 e^{2 pi i k2 m2 / R2} e^{2 pi i k2 m1 / M}
-//            sum_j Y_c[k2 + R2 j] e^{2 pi i j m1 / J}
-// (times 1/M, applied on detection).  The inner sum is a length-J inverse DFT
-// within the row, so F2f applies the chirp (Eq. 4) to the split spectrum in
-// shared memory, transforms every (row, sub-channel) run of J bins, scales by
-// e^{2 pi i k2 m1 / M} and stores element (k2, m1, c) blocked for the column
-// pass (Ic): with nl = min(TILE/R2, NCH) sub-channels per Ic CTA and
-// c = g nl + ci, at ((m1 G + g) R2 + k2) nl + ci, so that each Ic CTA reads one
-// contiguous block (its stores here are runs of 4 sub-channels, 32 bytes).
-// The row stride R1 + R1/16 makes each run a line of stride J + J/16.
-template <int R1, int J, bool CTAB>
-__global__ void __launch_bounds__(NT, 2) k_fwd_rows_inv(const float2* __restrict__ in, float2* __restrict__ out,
-                                                        int logR2, int logL, const float2* __restrict__ tw3L,
-                                                        Tw2 tw2L, const float2* __restrict__ tw,
-                                                        const float2* __restrict__ twJ,
-                                                        const ChirpAnchor* __restrict__ anc, int clog,
-                                                        const float2* __restrict__ ctab) {
-  static_assert(J >= 16 && J % 16 == 0 && R1 % (4 * J) == 0 && R1 >= NT, "row layout of the fused pass");
-  constexpr int NCH = R1 / J;                 // sub-channels
-  constexpr int LSTR = R1 + R1 / 16;
-  constexpr int LOGJ = ilog2c(J), LOGNCH = ilog2c(NCH), LOGR1 = ilog2c(R1);
-  extern __shared__ float2 smem[];
-  float2* st3 = smem;                              // [TW3_SN], w = exp(-2 pi i / L)
-  float2* stw = st3 + TW3_SN;
-  float2* stwj = stw + stage_table_size(R1);
-  float2* twk = stwj + stage_table_size(J);        // [nl][J]: e^{2 pi i k2 m1 / M}
-  in += (size_t)blockIdx.y << logL;
-  out += (size_t)blockIdx.y << logL;
-  const int R2 = 1 << logR2;
-  const int nl = min(TILE / R1, R2);
-  const int np = nl >> 1;
-  float2* sm = twk + nl * J;
-  load_tw3(st3, tw3L);
-  load_twiddles<R1>(stw, tw);
-  load_twiddles<J>(stwj, twJ);
-  const int q0 = blockIdx.x * np;
-  if (threadIdx.x < 4 && np == 1 && blockIdx.x + PF_DIST < gridDim.x) {
-    // the two rows of CTA blockIdx.x + PF_DIST (q and its mirror R2 - q), and
-    // with the per-bin chirp table the same rows of the table
-    const int q = q0 + PF_DIST, row = (threadIdx.x & 1) == 0 ? q : R2 - q;
-    if (threadIdx.x < 2) prefetch_l2(in + ((size_t)row << LOGR1), R1 * (unsigned)sizeof(float2));
-    else if (CTAB) prefetch_l2(ctab + ((size_t)row << LOGR1), R1 * (unsigned)sizeof(float2));
-  }
-  f2_stage1<R1, LSTR>(in, sm, st3, q0, np, R2, nl);
-  // e^{2 pi i k2 m1 / M} = conj(w^{k2 m1 NCH}), k2 m1 NCH < L
-  for (int i = threadIdx.x; i < nl * J; i += NT) {
-    const unsigned k2 = (unsigned)f2_line(i >> LOGJ, q0, np, R2), m1 = (unsigned)(i & (J - 1));
-    twk[i] = cconj(tw3(st3, (k2 * m1) << LOGNCH));
-  }
-  __syncthreads();
-  Stages<R1, 16, false, LSTR>::run(sm, nl, stw);          // the stages after the first
-  f2_split<R1, LSTR>(sm, q0, np, R2, logR2, logL, tw2L, [&](int slot, int row, int k1, float2 X) {
-    if constexpr (CTAB) {
-      // the chirp of bin row + R2 k1 from the plan's table (row layout: consecutive lanes, consecutive words)
-      sm[pidx(slot, k1, LSTR)] = cmul(X, __ldg(ctab + ((size_t)row << LOGR1) + k1));
-    } else {
-      const unsigned k = (unsigned)row + ((unsigned)k1 << logR2);
-      const ChirpAnchor a = anc[k >> clog];   // every row spans the band: L1/L2-resident table
-      sm[pidx(slot, k1, LSTR)] = cmul(X, chirp_from(a, clog, k));
-    }
-  });
-  __syncthreads();
-  j_runs<R1, J>(sm, stwj, twk, out, nl, logR2, [&](int slot) { return f2_line(slot, q0, np, R2); });
-}
-
-// ---------------------------------------------------------------------------
-// Ir: per-trial row pass of batched plans with M = 64 R2
-// ---------------------------------------------------------------------------
-
-// A batched plan shares F2's spectrum X[k2 + R2 k1] (row k2, column k1) among
-// its trials, so the chirp cannot move into F2.  For each trial a CTA takes
-// nl = min(TILE/R1, R2) consecutive rows, applies the trial's chirp (Eq. 4) as
-// it loads them and runs F2f's length-64 runs and blocked store; the column
-// pass (Ic) then completes the trial's sub-channel inverses.
-template <int R1, int J>
-__global__ void __launch_bounds__(NT, 2) k_inv_rows_chirp(const float2* __restrict__ in, float2* __restrict__ out,
-                                                          int logR2, const float2* __restrict__ tw3L,
-                                                          const float2* __restrict__ twJ,
-                                                          const ChirpAnchor* __restrict__ anc, int clog) {
-  static_assert(J == 64 && R1 % (4 * J) == 0 && R1 >= NT, "row layout of the fused pass");
-  constexpr int NCH = R1 / J;
-  constexpr int LSTR = R1 + R1 / 16;
-  constexpr int LOGJ = ilog2c(J), LOGNCH = ilog2c(NCH), LOGR1 = ilog2c(R1);
-  extern __shared__ float2 smem[];
-  float2* st3 = smem;                              // [TW3_SN], w = exp(-2 pi i / L)
-  float2* stwj = st3 + TW3_SN;
-  float2* twk = stwj + stage_table_size(J);        // [nl][J]: e^{2 pi i k2 m1 / M}
-  const int R2 = 1 << logR2;
-  const int nl = min(TILE / R1, R2);
-  float2* sm = twk + nl * J;
-  load_tw3(st3, tw3L);
-  load_twiddles<J>(stwj, twJ);
-  const int r0 = blockIdx.x * nl;
-  const int tot = nl * R1;
-  // rows r0 .. r0 + nl - 1 are contiguous: 16-byte loads of columns k1, k1 + 1
-  const float4* in4 = reinterpret_cast<const float4*>(in) + ((size_t)r0 << (LOGR1 - 1));
-  constexpr int H = EPT / 2;
-  float4 r[H];
-#pragma unroll
-  for (int u = 0; u < H; ++u) {
-    const int idx = 2 * ((int)threadIdx.x + u * NT);
-    if (idx < tot) r[u] = __ldg(in4 + (idx >> 1));
-  }
-#pragma unroll
-  for (int u = 0; u < H; ++u) {
-    const int idx = 2 * ((int)threadIdx.x + u * NT);
-    if (idx < tot) {
-      const int slot = idx >> LOGR1, k1 = idx & (R1 - 1);
-      const unsigned ka = (unsigned)(r0 + slot) + ((unsigned)k1 << logR2), kb = ka + (1u << logR2);
-      const ChirpAnchor a = anc[ka >> clog], b = anc[kb >> clog];
-      float2* p = sm + pidx(slot, k1, LSTR);        // k1 even: no pad between the two
-      p[0] = cmul(make_float2(r[u].x, r[u].y), chirp_from(a, clog, ka));
-      p[1] = cmul(make_float2(r[u].z, r[u].w), chirp_from(b, clog, kb));
-    }
-  }
-  __syncthreads();   // st3 and the tile
-  // e^{2 pi i k2 m1 / M} = conj(w^{k2 m1 NCH}), k2 m1 NCH < L
-  for (int i = threadIdx.x; i < nl * J; i += NT) {
-    const unsigned k2 = (unsigned)(r0 + (i >> LOGJ)), m1 = (unsigned)(i & (J - 1));
-    twk[i] = cconj(tw3(st3, (k2 * m1) << LOGNCH));
-  }
-  __syncthreads();
-  j_runs<R1, J>(sm, stwj, twk, out, nl, logR2, [&](int slot) { return r0 + slot; });
-}
-
-// exp(-2 pi i r) for the phase r = u 2^-32 (mod 1) held as a Q0.32 word u: the
-// same final sine and cosine as chirp_from.
-__device__ __forceinline__ float2 chirp_q32(unsigned u) {
-  float s, c;
-  __sincosf((float)(int)u * 1.4629180792671596e-9f, &s, &c);   // 2 pi 2^-32
-  return make_float2(c, -s);
-}
-
-// IrK, anchor form: Ir for the ntr trials of one batched launch, one trial per
-// CTA.  blockIdx.y is the row tile (nl rows of the shared spectrum) and
-// blockIdx.x the trial, so the CTAs that read the same rows are adjacent in
-// launch order and find them in L2 after the first.  Trial t's output (the
-// blocked layout of F2f) goes to out + t out_tstride.  The anchor chirp costs
-// about 20 more instructions per bin than the table's, and two CTAs per SM
-// hide them better than the rows-resident form's one (per trial and segment,
-// 32 trials per launch: 55.1 us here, 57.8 with the rows and each trial's
-// anchors resident).
-template <int R1, int J>
-__global__ void __launch_bounds__(NT, 2) k_inv_rows_chirp_multi(const float2* __restrict__ in,
-                                                                float2* __restrict__ out, long long out_tstride,
-                                                                int logR2, const float2* __restrict__ tw3L,
-                                                                const float2* __restrict__ twJ, MultiChirp mc) {
-  static_assert(J == 64 && R1 % (4 * J) == 0 && R1 >= NT, "row layout of the fused pass");
-  constexpr int NCH = R1 / J;
-  constexpr int LSTR = R1 + R1 / 16;
-  constexpr int LOGJ = ilog2c(J), LOGNCH = ilog2c(NCH), LOGR1 = ilog2c(R1);
-  extern __shared__ float2 smem[];
-  float2* st3 = smem;                              // [TW3_SN], w = exp(-2 pi i / L)
-  float2* stwj = st3 + TW3_SN;
-  float2* twk = stwj + stage_table_size(J);        // [nl][J]: e^{2 pi i k2 m1 / M}
-  const int R2 = 1 << logR2;
-  const int nl = min(TILE / R1, R2);
-  float2* sm = twk + nl * J;
-  const int t = blockIdx.x;
-  const int r0 = blockIdx.y * nl;
-  const int tot = nl * R1;
-  if (t == 0 && threadIdx.x == 0) {
-    // trials run fastest in launch order: the first trial's CTA of a row tile
-    // warms L2 with the rows of a later tile
-    const unsigned rn = blockIdx.y + max(1u, (unsigned)PF_DIST / gridDim.x);
-    if (rn < gridDim.y) prefetch_l2(in + (((size_t)rn * nl) << LOGR1), (unsigned)tot * (unsigned)sizeof(float2));
-  }
-  load_tw3(st3, tw3L);
-  load_twiddles<J>(stwj, twJ);
-  // rows r0 .. r0 + nl - 1 are contiguous: 16-byte loads of columns k1, k1 + 1
-  const float4* in4 = reinterpret_cast<const float4*>(in) + ((size_t)r0 << (LOGR1 - 1));
-  constexpr int H = EPT / 2;
-  float4 r[H];
-#pragma unroll
-  for (int u = 0; u < H; ++u) {
-    const int idx = 2 * ((int)threadIdx.x + u * NT);
-    if (idx < tot) r[u] = __ldg(in4 + (idx >> 1));
-  }
-  const ChirpAnchor* anc = mc.anc[t];
-  const int clog = __ldg(mc.clog + t);
-#pragma unroll
-  for (int u = 0; u < H; ++u) {
-    const int idx = 2 * ((int)threadIdx.x + u * NT);
-    if (idx < tot) {
-      const int slot = idx >> LOGR1, k1 = idx & (R1 - 1);
-      const unsigned ka = (unsigned)(r0 + slot) + ((unsigned)k1 << logR2), kb = ka + (1u << logR2);
-      const ChirpAnchor a = anc[ka >> clog], b = anc[kb >> clog];
-      float2* p = sm + pidx(slot, k1, LSTR);
-      p[0] = cmul(make_float2(r[u].x, r[u].y), chirp_from(a, clog, ka));
-      p[1] = cmul(make_float2(r[u].z, r[u].w), chirp_from(b, clog, kb));
-    }
-  }
-  __syncthreads();   // st3 and the tile
-  for (int i = threadIdx.x; i < nl * J; i += NT) {
-    const unsigned k2 = (unsigned)(r0 + (i >> LOGJ)), m1 = (unsigned)(i & (J - 1));
-    twk[i] = cconj(tw3(st3, (k2 * m1) << LOGNCH));
-  }
-  __syncthreads();
-  j_runs<R1, J>(sm, stwj, twk, out + (size_t)t * out_tstride, nl, logR2, [&](int slot) { return r0 + slot; });
 }
 
 // ---------------------------------------------------------------------------

@@ -200,6 +200,20 @@ constexpr int row_stride_max(int R1) { return 65 * (R1 / 64) + 31; }
 
 constexpr int TWK_STR = 65;   // stride of a row's 64 factors e^{2 pi i k2 m1 / M}
 
+// The three-level table (load_tw3) by NTHR threads, all loads in flight together.
+template <int NTHR>
+__device__ __forceinline__ void load_tw3_all(float2* st, const float2* __restrict__ g) {
+  float2 w[(TW3_N + NTHR - 1) / NTHR];
+#pragma unroll
+  for (int u = 0; u < (TW3_N + NTHR - 1) / NTHR; ++u)
+    if ((int)threadIdx.x + u * NTHR < TW3_N) w[u] = __ldg(g + threadIdx.x + u * NTHR);
+#pragma unroll
+  for (int u = 0; u < (TW3_N + NTHR - 1) / NTHR; ++u) {
+    const int i = (int)threadIdx.x + u * NTHR;
+    if (i < TW3_N) st[i < 256 ? i + (i >> 4) : i + 16] = w[u];
+  }
+}
+
 // Thread -> run: sub-channels of a block fastest, then rows, then blocks.
 struct Run {
   int slot, c;
@@ -209,6 +223,21 @@ __device__ __forceinline__ Run run_of(const RowTile& rt, int id) {
   r.slot = (id >> rt.lognlc) & ((1 << rt.lognl) - 1);
   r.c = (id & ((1 << rt.lognlc) - 1)) | ((id >> (rt.lognlc + rt.lognl)) << rt.lognlc);
   return r;
+}
+
+// A run's bins k0 + R2 j times the chirp from a trial's anchors (chirp_from).
+template <class Bin>
+__device__ __forceinline__ void run_chirp_anchors(float2* v, const ChirpAnchor* __restrict__ anc, int clog, unsigned k0,
+                                                  int logR2, Bin bin) {
+  // bins that share an anchor: the run starts at a multiple of min(2^clog, M) plus k2 < R2
+  const int amask = clog > logR2 ? (1 << (clog - logR2)) - 1 : 0;
+  ChirpAnchor a;
+#pragma unroll
+  for (int j = 0; j < 64; ++j) {
+    const unsigned k = k0 + ((unsigned)j << logR2);
+    if ((j & amask) == 0) a = anc[k >> clog];
+    v[j] = cmul(bin(j), chirp_from(a, clog, k));
+  }
 }
 
 // The run's 64-point inverse DFT, the factors twk[m1] and the blocked store.
@@ -251,10 +280,10 @@ __global__ void __launch_bounds__(TAB_GROUPS * WIDE_NT, 1)
   extern __shared__ float2 smem[];
   float2* st3 = smem;                                       // [TW3_SN], w = exp(-2 pi i / L)
   float2* twk = st3 + TW3_SN;                               // [NLR][TWK_STR]
-  float2* rows = twk + NLR * TWK_STR + (NLR * TWK_STR & 1); // [NLR * rstr]
+  float2* rows = twk + NLR * TWK_STR; // [NLR * rstr]
   unsigned* tabw = reinterpret_cast<unsigned*>(rows + NLR * rt.rstr);
   const int r0 = blockIdx.x * NLR;
-  load_tw3(st3, tw3L);
+  load_tw3_all<TAB_GROUPS * WIDE_NT>(st3, tw3L);
   const float2* src = in + ((size_t)r0 << LOGR1);
   const unsigned* tsrc = mc.atab + ((size_t)r0 << LOGR1);
 #pragma unroll 8
@@ -283,8 +312,271 @@ __global__ void __launch_bounds__(TAB_GROUPS * WIDE_NT, 1)
 template <int R1>
 size_t table_smem_bytes(const RowTile& rt) {
   constexpr int NLR = run_slots<R1>();
-  return (size_t)(TW3_SN + NLR * TWK_STR + (NLR * TWK_STR & 1) + NLR * rt.rstr) * sizeof(float2) +
+  return (size_t)(TW3_SN + NLR * TWK_STR + NLR * rt.rstr) * sizeof(float2) +
          (size_t)NLR * rt.tstr * sizeof(unsigned);
+}
+
+// Word form: the anchor chirp with its phases read from per-trial tables of Q0.32 words
+// ([row][j][c]: consecutive lanes, consecutive words) made from the anchors once
+// per plan.  A CTA keeps its rows resident and runs tpc trials of the launch on
+// them (blockIdx.x: trials x tpc ..), so a trial reads 4 bytes per bin and
+// writes 8.  21 trials of 2^19 bins: 53 us per launch with
+// the anchors evaluated per bin and trial, 36 here.
+template <int R1>
+__global__ void __launch_bounds__(WIDE_NT, 3)
+    k_inv_rows_words(const float2* __restrict__ in, float2* __restrict__ out, long long out_tstride, RowTile rt,
+                     const float2* __restrict__ tw3L, const unsigned* __restrict__ words, int ntr, int tpc) {
+  constexpr int NLR = run_slots<R1>(), LOGR1 = ilog2c(R1), NCH = R1 / 64;
+  extern __shared__ float2 smem[];
+  float2* st3 = smem;                       // [TW3_SN], w = exp(-2 pi i / L)
+  float2* twk = st3 + TW3_SN;               // [NLR][TWK_STR]
+  float2* rows = twk + NLR * TWK_STR;       // [NLR * rstr]
+  const int r0 = blockIdx.y * NLR;
+  {
+    const float2* src = in + ((size_t)r0 << LOGR1);
+    float2 v[64];   // the tile: 64 loads in flight per thread
+#pragma unroll
+    for (int u = 0; u < 64; ++u) v[u] = __ldg(src + threadIdx.x + u * WIDE_NT);
+    load_tw3_all<WIDE_NT>(st3, tw3L);
+#pragma unroll
+    for (int u = 0; u < 64; ++u) {
+      const int i = (int)threadIdx.x + u * WIDE_NT, k1 = i & (R1 - 1);
+      rows[(i >> LOGR1) * rt.rstr + k1 + (k1 >> 6)] = v[u];
+    }
+  }
+  __syncthreads();   // st3 and the rows
+  make_twk<R1>(twk, st3, NLR, [&](int slot) { return r0 + slot; });
+  __syncthreads();
+  const Run r = run_of(rt, (int)threadIdx.x);
+  const float2* row = rows + r.slot * rt.rstr + 65 * r.c;
+  const unsigned* wr = words + ((size_t)(r0 + r.slot) << LOGR1) + r.c;
+  const int t1 = min(ntr, ((int)blockIdx.x + 1) * tpc);
+  for (int t = (int)blockIdx.x * tpc; t < t1; ++t) {
+    // nothing of the run (its values, its outputs' offsets) is held across trials: 64
+    // of each would not fit the registers
+    RowTile ro = rt;
+    asm volatile("" : "+r"(ro.logR2)::"memory");
+    const unsigned* wt = wr + (size_t)t * out_tstride;
+    float2 v[64];
+#pragma unroll
+    for (int j = 0; j < 64; ++j) v[j].x = __uint_as_float(__ldg(wt + j * NCH));
+#pragma unroll
+    for (int j = 0; j < 64; ++j) v[j] = cmul(row[j], chirp_q32(__float_as_uint(v[j].x)));
+    run_finish<R1>(v, ro, r, (unsigned)(r0 + r.slot), twk, out + (size_t)t * out_tstride);
+  }
+}
+
+// Anchor form: one CTA per (trial, row tile), the chirp evaluated from the trial's anchors
+// as the tile is loaded (lanes over consecutive columns: their anchors lie side by side).
+// For lanes whose word tables would be too large, and for one trial per launch.
+// blockIdx.x is the trial and runs fastest, so the CTAs that share rows are
+// adjacent in launch order and all but the first find them in L2.  With mc.anc null
+// the launch's one trial takes its anchors from anc1, clog1.
+template <int R1>
+__global__ void __launch_bounds__(WIDE_NT, 3)
+    k_inv_rows_anchor(const float2* __restrict__ in, float2* __restrict__ out, long long out_tstride, RowTile rt,
+                      const float2* __restrict__ tw3L, MultiChirp mc, const ChirpAnchor* __restrict__ anc1, int clog1) {
+  constexpr int NLR = run_slots<R1>(), LOGR1 = ilog2c(R1);
+  extern __shared__ float2 smem[];
+  float2* st3 = smem;                       // [TW3_SN], w = exp(-2 pi i / L)
+  float2* twk = st3 + TW3_SN;               // [NLR][TWK_STR]
+  float2* rows = twk + NLR * TWK_STR;       // [NLR * rstr]
+  const int r0 = blockIdx.y * NLR, t = blockIdx.x;
+  const float2* src = in + ((size_t)r0 << LOGR1);
+  {
+    float2 v[64];   // the tile: 64 loads in flight per thread
+#pragma unroll
+    for (int u = 0; u < 64; ++u) v[u] = __ldg(src + threadIdx.x + u * WIDE_NT);
+    load_tw3_all<WIDE_NT>(st3, tw3L);
+    if (t == 0 && threadIdx.x == 0) {
+      // the first trial's CTA of a row tile warms L2 with the rows of a later tile
+      const unsigned rn = blockIdx.y + max(1u, (unsigned)WIDE_PF / gridDim.x);
+      if (rn < gridDim.y) prefetch_l2(in + (((size_t)rn * NLR) << LOGR1), TILE * (unsigned)sizeof(float2));
+    }
+    const ChirpAnchor* anc = mc.anc ? mc.anc[t] : anc1;
+    const int clog = mc.anc ? __ldg(mc.clog + t) : clog1;
+#pragma unroll
+    for (int u = 0; u < 64; ++u) {
+      const int i = (int)threadIdx.x + u * WIDE_NT, slot = i >> LOGR1, k1 = i & (R1 - 1);
+      const unsigned k = (unsigned)(r0 + slot) + ((unsigned)k1 << rt.logR2);
+      const ChirpAnchor a = anc[k >> clog];
+      rows[slot * rt.rstr + k1 + (k1 >> 6)] = cmul(v[u], chirp_from(a, clog, k));
+    }
+  }
+  __syncthreads();   // st3 and the rows
+  make_twk<R1>(twk, st3, NLR, [&](int slot) { return r0 + slot; });
+  __syncthreads();
+  const Run r = run_of(rt, (int)threadIdx.x);
+  const float2* row = rows + r.slot * rt.rstr + 65 * r.c;
+  float2 v[64];
+#pragma unroll
+  for (int j = 0; j < 64; ++j) v[j] = row[j];
+  run_finish<R1>(v, rt, r, (unsigned)(r0 + r.slot), twk, out + (size_t)t * out_tstride);
+}
+
+template <int R1>
+size_t anchor_smem_bytes(const RowTile& rt) {
+  constexpr int NLR = run_slots<R1>();
+  return (size_t)(TW3_SN + NLR * TWK_STR + NLR * rt.rstr) * sizeof(float2);
+}
+
+// ---------------------------------------------------------------------------
+// F2, F2f: row FFTs of the forward transform, real-input split, and (F2f) the
+// chirp with the first factor of every sub-channel's inverse
+// ---------------------------------------------------------------------------
+
+// L2 prefetch distance of F2 and F2f, at most three CTAs per SM (full-rate stream, ms:
+// 20: 14.46, 38: 14.59, 114: 15.0, none: 15.4).
+constexpr int ROW_PF = 20;
+
+enum RowMode { ROW_SPECTRUM = 0, ROW_ANCHORS = 1, ROW_TABLE = 2 };
+
+// Rows k2 and R2 - k2 share a CTA (f2_line), each a (64, RB) line, RB = R1 / 64 =
+// NCH.  Stage 1 takes the rows straight from global memory with the inter-pass
+// twiddle w^{n1 k2}, n1 = t + RB (8 a + b), factored as w^{8 RB k2 a} (inside the
+// first DFT) and w^{k2 (t + RB b)}; stage 2 works in place (a thread reads and writes the
+// same column), after which run c of a row is row c of its line.  Then, with
+// A = Z[k], B = conj(Z[L-k]), W = exp(-i pi k / L):
+//   X[k] = (A + B) / 2 - i W (A - B) / 2,
+// evaluated for every bin on its own (both bins of a pair load the same two
+// values, so this costs one more shared-memory read per bin and saves the write, the read and
+// the barrier of a split spectrum).  W = Wb s[j], Wb per run, s[j] = exp(-i pi j / R1).
+//   ROW_SPECTRUM: X[k2 + R2 k1] to row k2, column k1 (the batched trials read it);
+//   ROW_TABLE / ROW_ANCHORS (F2f): times the chirp, from the per-bin table (laid out
+//   [row][j][c]: consecutive lanes, consecutive words) or the anchors, then the run's
+//   length-64 inverse DFT and blocked store (run_finish).
+// F2f runs two CTAs per SM: at the 168 registers of three, the run's 64 chirp loads are
+// split into batches whose latency shows (101 us per launch at three, 71 at two).
+// Bound by instruction issue (43 %) and memory latency in turn.  Full rate, launches of
+// four 2^24-point segments: 56.0 -> 45 us per segment; 24.8 M warp
+// instructions per segment against 31.0 M with radix-16 stages.  blockIdx.y is
+// the segment.
+template <int R1, int MODE>
+__global__ void __launch_bounds__(WIDE_NT, MODE == ROW_SPECTRUM ? 3 : 2)
+    k_fwd_rows_w(const float2* __restrict__ in, float2* __restrict__ out, RowTile rt,
+                 const float2* __restrict__ tw3L, Tw2 tw2L, const float2* __restrict__ tw,
+                 const ChirpAnchor* __restrict__ anc, int clog, const float2* __restrict__ ctab) {
+  constexpr int RB = R1 / 64, NLR = run_slots<R1>(), BPT = 64 / RB, LOGR1 = ilog2c(R1), LOGRB = ilog2c(RB);
+  extern __shared__ float2 smem[];
+  float2* st3 = smem;                          // [TW3_SN], w = exp(-2 pi i / L)
+  float2* uni = st3 + TW3_SN;                  // [NLR][16]: w^{RB k2 b} (b < 8), w^{8 RB k2 a} at 8 + a
+  float2* sj = uni + NLR * 16;                 // [64]: exp(-i pi j / R1)
+  float2* wbt = sj + 64;                       // [NLR][RB]: exp(-i pi (k2 + 64 R2 c) / L) / 2
+  float2* twk = wbt + NLR * RB;                // [NLR][TWK_STR]
+  float2* sm = twk + NLR * TWK_STR;   // [NLR * rstr]
+  const int tid = (int)threadIdx.x, R2 = 1 << rt.logR2, np = NLR / 2, q0 = blockIdx.x * np;
+  in += (size_t)blockIdx.y << (LOGR1 + rt.logR2);    // segment blockIdx.y
+  out += (size_t)blockIdx.y << (LOGR1 + rt.logR2);
+  auto row_of = [&](int slot) { return f2_line(slot, q0, np, R2); };
+  if (tid < 4 && np == 1 && blockIdx.x + ROW_PF < gridDim.x) {
+    // the two rows of CTA blockIdx.x + ROW_PF (q and its mirror R2 - q), and
+    // with the per-bin chirp table the same rows of the table
+    const int q = q0 + ROW_PF, row = (tid & 1) == 0 ? q : R2 - q;
+    if (tid < 2) prefetch_l2(in + ((size_t)row << LOGR1), R1 * (unsigned)sizeof(float2));
+    else if (MODE == ROW_TABLE) prefetch_l2(ctab + ((size_t)row << LOGR1), R1 * (unsigned)sizeof(float2));
+  }
+  {
+    // stage 1: butterfly t of the line, inputs n1 = t + RB j
+    const int slot = tid >> LOGRB, t = tid & (RB - 1);
+    const unsigned k2 = (unsigned)row_of(slot);
+    const float2* src = in + ((size_t)k2 << LOGR1) + t;
+    float2 v[64];
+#pragma unroll
+    for (int j = 0; j < 64; ++j) v[j] = __ldg(src + j * RB);
+    load_tw3_all<WIDE_NT>(st3, tw3L);
+    if (tid < 64) sj[tid] = tw2(tw2L, (unsigned)tid << rt.logR2);
+    if (tid < NLR * RB) {   // always: NLR RB = 128 threads
+      const unsigned kr = (unsigned)row_of(slot) + ((unsigned)(64 * t) << rt.logR2);
+      wbt[tid] = cscale(tw2(tw2L, kr), 0.5f);
+    }
+    __syncthreads();   // st3
+    for (int i = tid; i < NLR * 16; i += WIDE_NT) {
+      const unsigned e = (unsigned)(i & 7) * (unsigned)((i & 8) ? 8 * RB : RB);
+      uni[i] = tw3(st3, (unsigned)row_of(i >> 4) * e);
+    }
+    if (MODE != ROW_SPECTRUM) make_twk<R1>(twk, st3, NLR, row_of);
+    const float2 wt = tw3(st3, k2 * (unsigned)t);
+    __syncthreads();   // uni
+    const float2* un = uni + slot * 16;
+    wide_dft<64, false>(
+        v, [&](float2 x, int a) { return a == 0 ? x : cmul(x, un[8 + a]); },
+        [&](float2 x, int b) { return cmul(x, b == 0 ? wt : cmul(wt, un[b])); });
+    float2* dst = sm + slot * rt.rstr + 65 * t;
+#pragma unroll
+    for (int j = 0; j < 64; ++j) dst[j] = v[j];
+  }
+  {
+    const int t2 = tid & 63;
+    WideTw<64, RB> w2;
+    w2.load(tw, t2);
+    __syncthreads();
+#pragma unroll 1
+    for (int u = 0; u < BPT; ++u) {
+      float2* p = sm + ((tid >> 6) + 2 * u) * rt.rstr + t2;
+      float2 v[RB];
+#pragma unroll
+      for (int j = 0; j < RB; ++j) v[j] = p[65 * j];
+      w2.template dft<false>(v);
+#pragma unroll
+      for (int j = 0; j < RB; ++j) p[65 * j] = v[j];
+    }
+  }
+  __syncthreads();
+  // X of (slot, c, j): partner Z[L - k] at column R1 - 1 - k1 of the mirrored row;
+  // rows 0 and R2/2 (tile 0) pair with themselves, row 0 at column R1 - k1 (mod R1)
+  struct Pair {
+    int oa, ob, ob0;   // own value j at oa + j; the partner's at ob - j, for j = 0 at ob0
+  };
+  auto pair_of = [&](int slot, int c) {
+    Pair q;
+    const bool self = q0 == 0 && (slot == 0 || slot == np);
+    const int ps = self ? slot : (slot < np ? slot + np : slot - np);
+    q.oa = slot * rt.rstr + 65 * c;
+    q.ob = ps * rt.rstr + 65 * (RB - 1 - c) + 63;
+    q.ob0 = q.ob;
+    if (self && slot == 0) {
+      q.ob += 1;
+      q.ob0 = c == 0 ? 0 : 65 * (RB - c);
+    }
+    return q;
+  };
+  auto split = [&](float2 A, float2 Z, float2 W) {   // W holds the factor 1/2
+    const float2 B = cconj(Z), E = cadd(A, B), WO = cmul(W, csub(A, B));
+    return make_float2(fmaf(0.5f, E.x, WO.y), fmaf(0.5f, E.y, -WO.x));
+  };
+  if constexpr (MODE == ROW_SPECTRUM) {
+#pragma unroll 8
+    for (int u = 0; u < 64; ++u) {
+      const int i = tid + u * WIDE_NT, slot = i >> LOGR1, k1 = i & (R1 - 1), c = k1 >> 6, j = k1 & 63;
+      const Pair q = pair_of(slot, c);
+      const float2 W = cmul(wbt[slot * RB + c], sj[j]);
+      out[((size_t)row_of(slot) << LOGR1) + k1] = split(sm[q.oa + j], sm[j == 0 ? q.ob0 : q.ob - j], W);
+    }
+  } else {
+    const Run r = run_of(rt, tid);
+    const unsigned k2 = (unsigned)row_of(r.slot);
+    const Pair q = pair_of(r.slot, r.c);
+    const float2 wb = wbt[r.slot * RB + r.c];
+    auto bin = [&](int j) { return split(sm[q.oa + j], sm[j == 0 ? q.ob0 : q.ob - j], cmul(wb, sj[j])); };
+    float2 v[64];
+    if constexpr (MODE == ROW_TABLE) {
+      const float2* ct = ctab + ((size_t)k2 << LOGR1) + r.c;
+#pragma unroll
+      for (int j = 0; j < 64; ++j) v[j] = __ldg(ct + j * RB);
+#pragma unroll
+      for (int j = 0; j < 64; ++j) v[j] = cmul(bin(j), v[j]);
+    } else {
+      run_chirp_anchors(v, anc, clog, k2 + ((unsigned)(64 * r.c) << rt.logR2), rt.logR2, bin);
+    }
+    run_finish<R1>(v, rt, r, k2, twk, out);
+  }
+}
+
+template <int R1>
+size_t fwd_rows_smem_bytes(const RowTile& rt) {
+  constexpr int NLR = run_slots<R1>();
+  return (size_t)(TW3_SN + NLR * 16 + 64 + WIDE_NT + NLR * TWK_STR + NLR * rt.rstr) *
+         sizeof(float2);
 }
 
 // Shared memory of a tile of nl lines of RA x RB.

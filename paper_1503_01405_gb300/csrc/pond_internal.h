@@ -34,6 +34,7 @@ struct __align__(16) ChirpAnchor {
 struct MultiChirp {
   const unsigned* atab;            // table form: [L], bin k2 + R2 k1 at k2 R1 + k1
   const unsigned* nmul;            // table form: per trial of the launch, n_d
+  const unsigned* words;           // anchor form: [trial][L] phase words (launch_chirp_words), or null
   const ChirpAnchor* const* anc;   // anchor form: per trial of the launch
   const int* clog;                 // anchor form: per trial of the launch
 };
@@ -138,8 +139,9 @@ int wide_tw_entries(int R);
 // and writes its own L elements of the buffers (M of P).
 cudaError_t launch_fwd_cols(const Geom& g, const SegSrc& in, float2* out, const float2* tw, cudaStream_t st,
                             int nseg = 1);
+// wtw: launch_wide_tw of R1 (rows of 512 and more; tw: the radix-16 tables of the others)
 cudaError_t launch_fwd_rows(const Geom& g, const float2* in, float2* out, const float2* tw3L, Tw2 tw2L, const float2* tw,
-                            cudaStream_t st, int nseg = 1);
+                            const float2* wtw, cudaStream_t st, int nseg = 1);
 cudaError_t launch_inv_cols(const Geom& g, const float2* in, float2* out, const ChirpAnchor* anc,
                             int clog, const float2* tw, cudaStream_t st, int nseg = 1);
 cudaError_t launch_inv_rows(const Geom& g, const float2* buf, float* P, float2* vout, long long vstride,
@@ -152,11 +154,11 @@ bool fused_geometry(const Geom& g);
 int fused_groups(const Geom& g);
 // ctab non-null: the chirp from that per-bin table (launch_chirp_c64), else from the anchors
 cudaError_t launch_fwd_rows_inv(const Geom& g, const float2* in, float2* out, const float2* tw3L, Tw2 tw2L,
-                                const float2* tw, const float2* twJ, const ChirpAnchor* anc, int clog,
-                                const float2* ctab, cudaStream_t st, int nseg = 1);
+                                const float2* wtw, const ChirpAnchor* anc, int clog, const float2* ctab,
+                                cudaStream_t st, int nseg = 1);
 cudaError_t launch_chirp_c64(float2* tab, const Geom& g, double du, double half, double f0, double alpha, int sgn,
                              cudaStream_t st);
-cudaError_t launch_inv_rows_chirp(const Geom& g, const float2* in, float2* out, const float2* tw3L, const float2* twJ,
+cudaError_t launch_inv_rows_chirp(const Geom& g, const float2* in, float2* out, const float2* tw3L,
                                   const ChirpAnchor* anc, int clog, cudaStream_t st);
 // nu > 1: one launch over nu trials or segments, the u-th reading in + u L and writing
 // P + u M, part + u G M, cnt + u FUSED_J (G = fused_groups); wtw: launch_wide_tw of R2
@@ -167,7 +169,7 @@ cudaError_t launch_inv_cols_det(const Geom& g, const float2* in, float* P, float
 // Batched lanes: Ir over ntr trials in one launch (trial t writes out + t L),
 // the chirp from the lane's Q0.32 table (table = true) or each trial's anchors
 cudaError_t launch_inv_rows_chirp_multi(const Geom& g, const float2* in, float2* out, int ntr, const float2* tw3L,
-                                        const float2* twJ, MultiChirp mc, bool table, cudaStream_t st);
+                                        MultiChirp mc, bool table, cudaStream_t st);
 // Tensor-core column pass (split-BF16, three terms) for R2 = 2048 and at least
 // four sub-channels: same outputs and arguments as launch_inv_cols_det, plus
 // its operand block (build_ic_tc_ops, ic_tc_ops_bytes() bytes on the device)
@@ -182,6 +184,8 @@ int ic_tc_ops_bytes();
 cudaError_t launch_copy_bytes(int8_t* dst, const int8_t* src, long long n, cudaStream_t st);
 // Host-to-device copy from mapped pinned memory by `blocks` CTAs (the copy engines are not used).
 cudaError_t launch_copy_host(int8_t* dst, const int8_t* src, long long n, int blocks, cudaStream_t st);
+// Phase words of one trial from its anchors, in F2f's order (row, position in a run, run).
+cudaError_t launch_chirp_words(unsigned* words, const Geom& g, const ChirpAnchor* anc, int clog, cudaStream_t st);
 cudaError_t launch_chirp_table(unsigned* tab, const Geom& g, double du, double half, double f0, double alpha, int sgn,
                                cudaStream_t st);
 cudaError_t launch_decimate_multi(const float* P, long long pstride, long long n, long long g0, long long num,
