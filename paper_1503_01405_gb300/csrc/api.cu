@@ -130,7 +130,8 @@ struct Lane {
   std::vector<cudaEvent_t> ev_chain[NSLOT];
   float2* stw = nullptr;                    // stage twiddle tables of R1, R2, Q1, Q2
   const float2 *stwR1 = nullptr, *stwR2 = nullptr, *stwQ1 = nullptr, *stwQ2 = nullptr;
-  const float2 *wtwR1 = nullptr, *wtwR2 = nullptr;   // stage-2 twiddles of the 64-values-per-thread FFTs (512 and more)
+  // stage-2 twiddles of the 64-values-per-thread FFTs (lengths 512 and more): F2 (R1), Ic (R2)
+  const float2 *wtwR1 = nullptr, *wtwR2 = nullptr;
   float2* tw2buf = nullptr;
   Tw2 tw2L;                                 // exp(-2 pi i e/(2L))
   float2* tw3L = nullptr;                   // three-level exp(-2 pi i e/L)
@@ -419,7 +420,7 @@ int build_lane(pond_t h, Lane* ln) {
   }
   const int n1 = stage_tw_entries(1 << g.logR1), n2 = stage_tw_entries(1 << g.logR2);
   const int n3 = stage_tw_entries(1 << g.logQ1), n4 = stage_tw_entries(1 << g.logQ2);
-  const int n5 = wide_tw_entries(1 << g.logR1), n6 = wide_tw_entries(1 << g.logR2);
+  const int n5 = wide_tw_entries(1 << g.logR1, false), n6 = wide_tw_entries(1 << g.logR2, false);
   CK(cudaMalloc(&ln->stw, (size_t)std::max(1, n1 + n2 + n3 + n4 + n5 + n6) * sizeof(float2)));
   ln->stwR1 = ln->stw;
   ln->stwR2 = ln->stwR1 + n1;
@@ -441,8 +442,8 @@ int build_lane(pond_t h, Lane* ln) {
   CK(launch_stage_tw(const_cast<float2*>(ln->stwR2), 1 << g.logR2, h->st));
   CK(launch_stage_tw(const_cast<float2*>(ln->stwQ1), 1 << g.logQ1, h->st));
   CK(launch_stage_tw(const_cast<float2*>(ln->stwQ2), 1 << g.logQ2, h->st));
-  CK(launch_wide_tw(const_cast<float2*>(ln->wtwR1), 1 << g.logR1, h->st));
-  CK(launch_wide_tw(const_cast<float2*>(ln->wtwR2), 1 << g.logR2, h->st));
+  CK(launch_wide_tw(const_cast<float2*>(ln->wtwR1), 1 << g.logR1, false, h->st));
+  CK(launch_wide_tw(const_cast<float2*>(ln->wtwR2), 1 << g.logR2, false, h->st));
   CK(launch_tw3(ln->tw3L, g.logL, -1, h->st));
   CK(launch_tw2(const_cast<float2*>(ln->tw2L.lo), const_cast<float2*>(ln->tw2L.hi), g.logL + 1, -1, h->st));
   CK(launch_tw3(ln->tw3M, g.logM, +1, h->st));
@@ -679,7 +680,7 @@ int run_segments(pond_t h, int li, const SegSrc& src, long long s, int nseg, lon
     const Trial& t = h->trials[ln.trials[0]];
     if (ln.fused) {
       // three passes: F2f takes the chirp and the first inverse factor, Ic the rest
-      CK(launch_fwd_rows_inv(g, bufA, bufB, ln.tw3L, ln.tw2L, ln.wtwR1, t.anc, t.clog, t.ctab, cs, nseg));
+      CK(launch_fwd_rows_inv(g, bufA, bufB, ln.tw2L, ln.wtwR1, t.anc, t.clog, t.ctab, cs, nseg));
       RC(record(h, 1 + ST_F2F, cs));
       h->launches += 4;
     } else {
@@ -724,7 +725,7 @@ int run_segments(pond_t h, int li, const SegSrc& src, long long s, int nseg, lon
         const int nq = std::min(ln.kt, ntr - q0);
         const MultiChirp mc{ln.atab, ln.d_nmul + q0, ln.words ? ln.words + (size_t)q0 * g.L : nullptr, ln.d_anc + q0,
                             ln.d_clog + q0};
-        CK(launch_inv_rows_chirp_multi(g, bufB, ln.bufT[slot], nq, ln.tw3L, mc,
+        CK(launch_inv_rows_chirp_multi(g, bufB, ln.bufT[slot], nq, ln.tw2L, mc,
                                        ln.mode == POND_TRIALS_MULTI_TABLE, cs));
         if (b == 0) RC(record(h, 1 + ST_IR, cs));
         CK(launch_ic(h, ln, ln.bufT[slot], ln.Pm[slot], ln.partm[slot], ln.cntm[slot], nullptr, 0, 0, trials, cs, nq));
@@ -754,7 +755,7 @@ int run_segments(pond_t h, int li, const SegSrc& src, long long s, int nseg, lon
         const Trial& t = h->trials[d];
         if (ln.mode == POND_TRIALS_PER_TRIAL) {
           // the trial's chirp and the first inverse factor as Ir loads the shared spectrum's rows
-          CK(launch_inv_rows_chirp(g, bufB, bufA, ln.tw3L, t.anc, t.clog, cs));
+          CK(launch_inv_rows_chirp(g, bufB, bufA, ln.tw2L, t.anc, t.clog, cs));
           if (q == 0) RC(record(h, 1 + ST_IR, cs));
           CK(launch_ic(h, ln, bufA, P, ln.part[slot], ln.cnt[slot], nullptr, 0, 0, span, cs));
           if (q == 0) RC(record(h, 1 + ST_IC, cs));
@@ -977,7 +978,7 @@ int measure_lane(pond_t h, const pond_opts* o, long long nfft, double* t_fwd, do
   for (int it = 0; it <= reps && ce == cudaSuccess; ++it) {
     if (it == 1) ce = cudaEventRecord(e[2], h->st);
     if (ln.fused_multi) {   // the per-trial passes the plan will run
-      if (ce == cudaSuccess) ce = launch_inv_rows_chirp(g, ln.bufB[0], ln.bufA[0], ln.tw3L, anc, clog, h->st);
+      if (ce == cudaSuccess) ce = launch_inv_rows_chirp(g, ln.bufB[0], ln.bufA[0], ln.tw2L, anc, clog, h->st);
       if (ce == cudaSuccess)
         ce = launch_ic(h, ln, ln.bufA[0], ln.P[0], ln.part[0], ln.cnt[0], nullptr, 0, 0, span, h->st);
     } else {
@@ -1169,7 +1170,7 @@ int time_trials(pond_t h, Lane* ln, int mode, int kt, int split, double* us) {
     } else if (mode == POND_TRIALS_PER_TRIAL) {
       for (int q = 0; q < nq && ce == cudaSuccess; ++q) {
         const Trial& t = h->trials[ln->trials[q]];
-        ce = launch_inv_rows_chirp(g, ln->bufB[0], ln->bufA[0], ln->tw3L, t.anc, t.clog, h->st);
+        ce = launch_inv_rows_chirp(g, ln->bufB[0], ln->bufA[0], ln->tw2L, t.anc, t.clog, h->st);
         if (ce == cudaSuccess)
           ce = launch_ic(h, *ln, ln->bufA[0], ln->P[0], ln->part[0], ln->cnt[0], nullptr, 0, 0, span, h->st);
         if (ce == cudaSuccess)
@@ -1179,7 +1180,7 @@ int time_trials(pond_t h, Lane* ln, int mode, int kt, int split, double* us) {
       }
     } else {
       const MultiChirp mc{ln->atab, ln->d_nmul, ln->words, ln->d_anc, ln->d_clog};
-      ce = launch_inv_rows_chirp_multi(g, ln->bufB[0], ln->bufT[0], nq, ln->tw3L, mc,
+      ce = launch_inv_rows_chirp_multi(g, ln->bufB[0], ln->bufT[0], nq, ln->tw2L, mc,
                                        mode == POND_TRIALS_MULTI_TABLE, h->st);
       if (ce == cudaSuccess)
         ce = launch_ic(h, *ln, ln->bufT[0], ln->Pm[0], ln->partm[0], ln->cntm[0], nullptr, 0, 0, span, h->st, nq);

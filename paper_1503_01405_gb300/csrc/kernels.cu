@@ -808,24 +808,26 @@ int stage_tw_entries(int R) { return stage_table_size(R); }
 
 #define POND_WIDE_RB(X) X(8) X(16) X(32) X(64)
 
-int wide_tw_entries(int R) {
+int wide_tw_entries(int R, bool last64) {
   switch (R / 64) {
-#define CASE(RB) case RB: return WideTw<64, RB>::SIZE;
+#define CASE(RB) case RB: return last64 ? WideTw<RB, 64>::SIZE : WideTw<64, RB>::SIZE;
     POND_WIDE_RB(CASE)
 #undef CASE
     default: return 0;
   }
 }
 
-cudaError_t launch_wide_tw(float2* out, int R, cudaStream_t st) {
-  const int n = wide_tw_entries(R);
-  switch (R / 64) {
-#define CASE(RB) \
-  case RB: k_make_wide_tw<<<(n + 255) / 256, 256, 0, st>>>(out, 64, RB, WideSplit<RB>::NA, WideSplit<RB>::NB); break;
+cudaError_t launch_wide_tw(float2* out, int R, bool last64, cudaStream_t st) {
+  const int n = wide_tw_entries(R, last64);
+  if (n == 0) return cudaSuccess;
+  int na = 8, nb = 8;   // split of the last radix
+  switch (last64 ? 64 : R / 64) {
+#define CASE(RB) case RB: na = WideSplit<RB>::NA; nb = WideSplit<RB>::NB; break;
     POND_WIDE_RB(CASE)
 #undef CASE
-    default: return cudaSuccess;
+    default: return cudaErrorInvalidValue;
   }
+  k_make_wide_tw<<<(n + 255) / 256, 256, 0, st>>>(out, last64 ? R / 64 : 64, last64 ? 64 : R / 64, na, nb);
   return cudaGetLastError();
 }
 
@@ -863,7 +865,7 @@ size_t smem_inv_cols_det(int nl) {
 }
 }  // namespace
 
-cudaError_t launch_fwd_rows_inv(const Geom& g, const float2* in, float2* out, const float2* tw3L, Tw2 tw2L,
+cudaError_t launch_fwd_rows_inv(const Geom& g, const float2* in, float2* out, Tw2 tw2L,
                                 const float2* wtw, const ChirpAnchor* anc, int clog, const float2* ctab,
                                 cudaStream_t st, int nseg) {
   const RowTile rt = row_tile(g.logR1, g.logR2);
@@ -872,11 +874,9 @@ cudaError_t launch_fwd_rows_inv(const Geom& g, const float2* in, float2* out, co
 #define CASE(R)                                                                                             \
   case R:                                                                                                   \
     if (ctab)                                                                                               \
-      k_fwd_rows_w<R, ROW_TABLE><<<tiles, WIDE_NT, fwd_rows_smem_bytes<R>(rt), st>>>(in, out, rt, tw3L,     \
-                                                                                     tw2L, wtw, anc, clog, ctab); \
+      k_fwd_rows_w<R, ROW_TABLE><<<tiles, WIDE_NT, fwd_rows_smem_bytes<R>(rt), st>>>(in, out, rt, tw2L, wtw, anc, clog, ctab); \
     else                                                                                                    \
-      k_fwd_rows_w<R, ROW_ANCHORS><<<tiles, WIDE_NT, fwd_rows_smem_bytes<R>(rt), st>>>(in, out, rt, tw3L,   \
-                                                                                       tw2L, wtw, anc, clog, ctab); \
+      k_fwd_rows_w<R, ROW_ANCHORS><<<tiles, WIDE_NT, fwd_rows_smem_bytes<R>(rt), st>>>(in, out, rt, tw2L, wtw, anc, clog, ctab); \
     break;
     POND_FUSED_R1(CASE)
 #undef CASE
@@ -886,7 +886,7 @@ cudaError_t launch_fwd_rows_inv(const Geom& g, const float2* in, float2* out, co
 }
 
 // Ir with the anchor chirp over ntr trials (mc), or over the one trial anc1 (mc.anc null).
-static cudaError_t launch_inv_rows_anchor(const Geom& g, const float2* in, float2* out, int ntr, const float2* tw3L,
+static cudaError_t launch_inv_rows_anchor(const Geom& g, const float2* in, float2* out, int ntr, Tw2 tw2L,
                                           MultiChirp mc, const ChirpAnchor* anc1, int clog1, cudaStream_t st) {
   const RowTile rt = row_tile(g.logR1, g.logR2);
   const unsigned tiles = (unsigned)(g.L / TILE);
@@ -894,7 +894,7 @@ static cudaError_t launch_inv_rows_anchor(const Geom& g, const float2* in, float
   switch (1 << g.logR1) {
 #define CASE(R)                                                                                             \
   case R:                                                                                                   \
-    k_inv_rows_anchor<R><<<grid, WIDE_NT, anchor_smem_bytes<R>(rt), st>>>(in, out, g.L, rt, tw3L, mc, anc1, \
+    k_inv_rows_anchor<R><<<grid, WIDE_NT, anchor_smem_bytes<R>(rt), st>>>(in, out, g.L, rt, tw2L, mc, anc1, \
                                                                           clog1);                           \
     break;
     POND_FUSED_R1(CASE)
@@ -904,15 +904,15 @@ static cudaError_t launch_inv_rows_anchor(const Geom& g, const float2* in, float
   return cudaGetLastError();
 }
 
-cudaError_t launch_inv_rows_chirp(const Geom& g, const float2* in, float2* out, const float2* tw3L,
+cudaError_t launch_inv_rows_chirp(const Geom& g, const float2* in, float2* out, Tw2 tw2L,
                                   const ChirpAnchor* anc, int clog, cudaStream_t st) {
-  return launch_inv_rows_anchor(g, in, out, 1, tw3L, MultiChirp{}, anc, clog, st);
+  return launch_inv_rows_anchor(g, in, out, 1, tw2L, MultiChirp{}, anc, clog, st);
 }
 
-cudaError_t launch_inv_rows_chirp_multi(const Geom& g, const float2* in, float2* out, int ntr, const float2* tw3L,
+cudaError_t launch_inv_rows_chirp_multi(const Geom& g, const float2* in, float2* out, int ntr, Tw2 tw2L,
                                         MultiChirp mc, bool table, cudaStream_t st) {
   if (ntr < 1) return cudaErrorInvalidValue;
-  if (!table && !mc.words) return launch_inv_rows_anchor(g, in, out, ntr, tw3L, mc, nullptr, 0, st);
+  if (!table && !mc.words) return launch_inv_rows_anchor(g, in, out, ntr, tw2L, mc, nullptr, 0, st);
   const RowTile rt = row_tile(g.logR1, g.logR2);
   const unsigned tiles = (unsigned)(g.L / TILE);
   if (!table) {
@@ -922,7 +922,7 @@ cudaError_t launch_inv_rows_chirp_multi(const Geom& g, const float2* in, float2*
     switch (1 << g.logR1) {
 #define CASE(R)                                                                                             \
   case R:                                                                                                   \
-    k_inv_rows_words<R><<<grid, WIDE_NT, anchor_smem_bytes<R>(rt), st>>>(in, out, g.L, rt, tw3L, mc.words,  \
+    k_inv_rows_words<R><<<grid, WIDE_NT, anchor_smem_bytes<R>(rt), st>>>(in, out, g.L, rt, tw2L, mc.words,  \
                                                                          ntr, tpc);                         \
     break;
       POND_FUSED_R1(CASE)
@@ -936,7 +936,7 @@ cudaError_t launch_inv_rows_chirp_multi(const Geom& g, const float2* in, float2*
 #define CASE(R)                                                                                             \
   case R:                                                                                                   \
     k_inv_rows_table<R><<<tiles, TAB_GROUPS * WIDE_NT, table_smem_bytes<R>(rt), st>>>(in, out, g.L, rt,    \
-                                                                                      tw3L, mc, ntr);       \
+                                                                                      tw2L, mc, ntr);       \
     break;
     POND_FUSED_R1(CASE)
 #undef CASE
@@ -1045,8 +1045,7 @@ cudaError_t launch_fwd_rows(const Geom& g, const float2* in, float2* out, const 
     switch (1 << g.logR1) {
 #define CASE(R)                                                                                             \
   case R:                                                                                                   \
-    k_fwd_rows_w<R, ROW_SPECTRUM><<<tiles, WIDE_NT, fwd_rows_smem_bytes<R>(rt), st>>>(in, out, rt, tw3L,    \
-                                                                                      tw2L, wtw, nullptr, 0, nullptr); \
+    k_fwd_rows_w<R, ROW_SPECTRUM><<<tiles, WIDE_NT, fwd_rows_smem_bytes<R>(rt), st>>>(in, out, rt, tw2L, wtw, nullptr, 0, nullptr); \
     return cudaGetLastError();
       POND_FUSED_R1(CASE)
 #undef CASE

@@ -221,6 +221,8 @@ __device__ __forceinline__ SegIn seg_runs(const SegSrc& s, unsigned y, int nl) {
             (in.b_len == 0 || ((uintptr_t)in.b & 7) == 0);
   in.pair4 = in.ch == 2 && ((uintptr_t)in.a & 3) == 0 && (in.a_len & 3) == 0 && (in.b_len & 3) == 0 &&
              (in.b_len == 0 || ((uintptr_t)in.b & 3) == 0);
+  in.pair2 = in.ch == 1 && ((uintptr_t)in.a & 1) == 0 && (in.a_len & 1) == 0 && (in.b_len & 1) == 0 &&
+             (in.b_len == 0 || ((uintptr_t)in.b & 1) == 0);
   return in;
 }
 
@@ -254,11 +256,13 @@ __global__ void __launch_bounds__(NT, 2) k_fwd_cols(SegSrc src, float2* __restri
     if (in.a_len > 0) prefetch_range(in.a, min(in.a_len, tile * pa), min(in.a_len, (tile + 1) * pa));
     if (in.b_len > 0) prefetch_range(in.b, min(in.b_len, tile * pb), min(in.b_len, (tile + 1) * pb));
   }
-  // FP32 form, R2 >= 512, aligned runs: the first radix-16 stage takes its inputs
+  // FP32 form, R2 >= 512, runs aligned to one complex sample (segments of a one-channel
+  // plan start at any even byte: sample by sample they took 8.7 us of a 2^21-point
+  // segment's 25): the first radix-16 stage takes its inputs
   // straight from global memory (butterfly t of column b, columns fastest: a warp
   // reads the nl columns of 8 rows per load) and the stages after it start from
   // LS = 16; the unpack's shared-memory round trip and a barrier go away
-  const bool direct1 = !TC && R2 >= 512 && (in.vec8 || in.pair4);
+  const bool direct1 = !TC && R2 >= 512 && (in.pair2 || in.pair4);
   if (direct1) {
     constexpr int NB = R2 / 16;
     const int b = (int)threadIdx.x & (nl - 1), t = (int)threadIdx.x >> lognl;

@@ -200,20 +200,6 @@ constexpr int row_stride_max(int R1) { return 65 * (R1 / 64) + 31; }
 
 constexpr int TWK_STR = 65;   // stride of a row's 64 factors e^{2 pi i k2 m1 / M}
 
-// The three-level table (load_tw3) by NTHR threads, all loads in flight together.
-template <int NTHR>
-__device__ __forceinline__ void load_tw3_all(float2* st, const float2* __restrict__ g) {
-  float2 w[(TW3_N + NTHR - 1) / NTHR];
-#pragma unroll
-  for (int u = 0; u < (TW3_N + NTHR - 1) / NTHR; ++u)
-    if ((int)threadIdx.x + u * NTHR < TW3_N) w[u] = __ldg(g + threadIdx.x + u * NTHR);
-#pragma unroll
-  for (int u = 0; u < (TW3_N + NTHR - 1) / NTHR; ++u) {
-    const int i = (int)threadIdx.x + u * NTHR;
-    if (i < TW3_N) st[i < 256 ? i + (i >> 4) : i + 16] = w[u];
-  }
-}
-
 // Thread -> run: sub-channels of a block fastest, then rows, then blocks.
 struct Run {
   int slot, c;
@@ -253,12 +239,13 @@ __device__ __forceinline__ void run_finish(float2* v, const RowTile& rt, const R
   for (int m1 = 0; m1 < 64; ++m1) dst[(unsigned)m1 << (LOGNCH + rt.logR2)] = cmul(v[m1], w[m1]);
 }
 
-// e^{2 pi i k2 m1 / M} = conj(w^{k2 m1 NCH}), k2 m1 NCH < L, of rows row_of(0 .. nl-1).
+// e^{2 pi i k2 m1 / M} = conj(w^{k2 m1 NCH}), w = exp(-2 pi i / L), k2 m1 NCH < L, of
+// rows row_of(0 .. nl-1): one product of two table entries (tw2L steps by half a bin).
 template <int R1, class RowOf>
-__device__ __forceinline__ void make_twk(float2* twk, const float2* st3, int nl, RowOf row_of) {
+__device__ __forceinline__ void make_twk(float2* twk, const Tw2& tw2L, int nl, RowOf row_of) {
   for (int i = threadIdx.x; i < nl * 64; i += blockDim.x) {
     const unsigned k2 = (unsigned)row_of(i >> 6), m1 = (unsigned)(i & 63);
-    twk[(i >> 6) * TWK_STR + m1] = cconj(tw3(st3, (k2 * m1) << ilog2c(R1 / 64)));
+    twk[(i >> 6) * TWK_STR + m1] = cconj(tw2(tw2L, (k2 * m1) << (ilog2c(R1 / 64) + 1)));
   }
 }
 
@@ -275,15 +262,13 @@ constexpr int TAB_GROUPS = 3;   // 384 threads of 168 registers: one CTA per SM
 template <int R1>
 __global__ void __launch_bounds__(TAB_GROUPS * WIDE_NT, 1)
     k_inv_rows_table(const float2* __restrict__ in, float2* __restrict__ out, long long out_tstride, RowTile rt,
-                     const float2* __restrict__ tw3L, MultiChirp mc, int ntr) {
+                     Tw2 tw2L, MultiChirp mc, int ntr) {
   constexpr int NLR = run_slots<R1>(), LOGR1 = ilog2c(R1);
   extern __shared__ float2 smem[];
-  float2* st3 = smem;                                       // [TW3_SN], w = exp(-2 pi i / L)
-  float2* twk = st3 + TW3_SN;                               // [NLR][TWK_STR]
+  float2* twk = smem;                              // [NLR][TWK_STR]
   float2* rows = twk + NLR * TWK_STR; // [NLR * rstr]
   unsigned* tabw = reinterpret_cast<unsigned*>(rows + NLR * rt.rstr);
   const int r0 = blockIdx.x * NLR;
-  load_tw3_all<TAB_GROUPS * WIDE_NT>(st3, tw3L);
   const float2* src = in + ((size_t)r0 << LOGR1);
   const unsigned* tsrc = mc.atab + ((size_t)r0 << LOGR1);
 #pragma unroll 8
@@ -292,8 +277,7 @@ __global__ void __launch_bounds__(TAB_GROUPS * WIDE_NT, 1)
     rows[slot * rt.rstr + o] = __ldg(src + i);
     tabw[slot * rt.tstr + o] = __ldg(tsrc + i);
   }
-  __syncthreads();   // st3
-  make_twk<R1>(twk, st3, NLR, [&](int slot) { return r0 + slot; });
+  make_twk<R1>(twk, tw2L, NLR, [&](int slot) { return r0 + slot; });
   __syncthreads();   // twk, the rows and their table words
   const Run r = run_of(rt, (int)threadIdx.x & (WIDE_NT - 1));
   const int o = r.slot * rt.rstr + 65 * r.c, ot = r.slot * rt.tstr + 65 * r.c;
@@ -312,7 +296,7 @@ __global__ void __launch_bounds__(TAB_GROUPS * WIDE_NT, 1)
 template <int R1>
 size_t table_smem_bytes(const RowTile& rt) {
   constexpr int NLR = run_slots<R1>();
-  return (size_t)(TW3_SN + NLR * TWK_STR + NLR * rt.rstr) * sizeof(float2) +
+  return (size_t)(NLR * TWK_STR + NLR * rt.rstr) * sizeof(float2) +
          (size_t)NLR * rt.tstr * sizeof(unsigned);
 }
 
@@ -325,11 +309,10 @@ size_t table_smem_bytes(const RowTile& rt) {
 template <int R1>
 __global__ void __launch_bounds__(WIDE_NT, 3)
     k_inv_rows_words(const float2* __restrict__ in, float2* __restrict__ out, long long out_tstride, RowTile rt,
-                     const float2* __restrict__ tw3L, const unsigned* __restrict__ words, int ntr, int tpc) {
+                     Tw2 tw2L, const unsigned* __restrict__ words, int ntr, int tpc) {
   constexpr int NLR = run_slots<R1>(), LOGR1 = ilog2c(R1), NCH = R1 / 64;
   extern __shared__ float2 smem[];
-  float2* st3 = smem;                       // [TW3_SN], w = exp(-2 pi i / L)
-  float2* twk = st3 + TW3_SN;               // [NLR][TWK_STR]
+  float2* twk = smem;              // [NLR][TWK_STR]
   float2* rows = twk + NLR * TWK_STR;       // [NLR * rstr]
   const int r0 = blockIdx.y * NLR;
   {
@@ -337,15 +320,13 @@ __global__ void __launch_bounds__(WIDE_NT, 3)
     float2 v[64];   // the tile: 64 loads in flight per thread
 #pragma unroll
     for (int u = 0; u < 64; ++u) v[u] = __ldg(src + threadIdx.x + u * WIDE_NT);
-    load_tw3_all<WIDE_NT>(st3, tw3L);
 #pragma unroll
     for (int u = 0; u < 64; ++u) {
       const int i = (int)threadIdx.x + u * WIDE_NT, k1 = i & (R1 - 1);
       rows[(i >> LOGR1) * rt.rstr + k1 + (k1 >> 6)] = v[u];
     }
   }
-  __syncthreads();   // st3 and the rows
-  make_twk<R1>(twk, st3, NLR, [&](int slot) { return r0 + slot; });
+  make_twk<R1>(twk, tw2L, NLR, [&](int slot) { return r0 + slot; });
   __syncthreads();
   const Run r = run_of(rt, (int)threadIdx.x);
   const float2* row = rows + r.slot * rt.rstr + 65 * r.c;
@@ -375,11 +356,10 @@ __global__ void __launch_bounds__(WIDE_NT, 3)
 template <int R1>
 __global__ void __launch_bounds__(WIDE_NT, 3)
     k_inv_rows_anchor(const float2* __restrict__ in, float2* __restrict__ out, long long out_tstride, RowTile rt,
-                      const float2* __restrict__ tw3L, MultiChirp mc, const ChirpAnchor* __restrict__ anc1, int clog1) {
+                      Tw2 tw2L, MultiChirp mc, const ChirpAnchor* __restrict__ anc1, int clog1) {
   constexpr int NLR = run_slots<R1>(), LOGR1 = ilog2c(R1);
   extern __shared__ float2 smem[];
-  float2* st3 = smem;                       // [TW3_SN], w = exp(-2 pi i / L)
-  float2* twk = st3 + TW3_SN;               // [NLR][TWK_STR]
+  float2* twk = smem;              // [NLR][TWK_STR]
   float2* rows = twk + NLR * TWK_STR;       // [NLR * rstr]
   const int r0 = blockIdx.y * NLR, t = blockIdx.x;
   const float2* src = in + ((size_t)r0 << LOGR1);
@@ -387,7 +367,6 @@ __global__ void __launch_bounds__(WIDE_NT, 3)
     float2 v[64];   // the tile: 64 loads in flight per thread
 #pragma unroll
     for (int u = 0; u < 64; ++u) v[u] = __ldg(src + threadIdx.x + u * WIDE_NT);
-    load_tw3_all<WIDE_NT>(st3, tw3L);
     if (t == 0 && threadIdx.x == 0) {
       // the first trial's CTA of a row tile warms L2 with the rows of a later tile
       const unsigned rn = blockIdx.y + max(1u, (unsigned)WIDE_PF / gridDim.x);
@@ -403,8 +382,7 @@ __global__ void __launch_bounds__(WIDE_NT, 3)
       rows[slot * rt.rstr + k1 + (k1 >> 6)] = cmul(v[u], chirp_from(a, clog, k));
     }
   }
-  __syncthreads();   // st3 and the rows
-  make_twk<R1>(twk, st3, NLR, [&](int slot) { return r0 + slot; });
+  make_twk<R1>(twk, tw2L, NLR, [&](int slot) { return r0 + slot; });
   __syncthreads();
   const Run r = run_of(rt, (int)threadIdx.x);
   const float2* row = rows + r.slot * rt.rstr + 65 * r.c;
@@ -417,7 +395,7 @@ __global__ void __launch_bounds__(WIDE_NT, 3)
 template <int R1>
 size_t anchor_smem_bytes(const RowTile& rt) {
   constexpr int NLR = run_slots<R1>();
-  return (size_t)(TW3_SN + NLR * TWK_STR + NLR * rt.rstr) * sizeof(float2);
+  return (size_t)(NLR * TWK_STR + NLR * rt.rstr) * sizeof(float2);
 }
 
 // ---------------------------------------------------------------------------
@@ -428,6 +406,15 @@ size_t anchor_smem_bytes(const RowTile& rt) {
 // L2 prefetch distance of F2 and F2f, at most three CTAs per SM (full-rate stream, ms:
 // 20: 14.46, 38: 14.59, 114: 15.0, none: 15.4).
 constexpr int ROW_PF = 20;
+
+// The two entries of a tw2 lookup, loaded now and multiplied later.
+struct Tw2Pair {
+  float2 hi, lo;
+  Tw2Pair() = default;
+  __device__ __forceinline__ Tw2Pair(const Tw2& t, unsigned e)
+      : hi(__ldg(t.hi + (e >> TW2_LOG))), lo(__ldg(t.lo + (e & (TW2_LO - 1)))) {}
+  __device__ __forceinline__ float2 value() const { return cmul(hi, lo); }
+};
 
 enum RowMode { ROW_SPECTRUM = 0, ROW_ANCHORS = 1, ROW_TABLE = 2 };
 
@@ -454,12 +441,11 @@ enum RowMode { ROW_SPECTRUM = 0, ROW_ANCHORS = 1, ROW_TABLE = 2 };
 template <int R1, int MODE>
 __global__ void __launch_bounds__(WIDE_NT, MODE == ROW_SPECTRUM ? 3 : 2)
     k_fwd_rows_w(const float2* __restrict__ in, float2* __restrict__ out, RowTile rt,
-                 const float2* __restrict__ tw3L, Tw2 tw2L, const float2* __restrict__ tw,
+                 Tw2 tw2L, const float2* __restrict__ tw,
                  const ChirpAnchor* __restrict__ anc, int clog, const float2* __restrict__ ctab) {
   constexpr int RB = R1 / 64, NLR = run_slots<R1>(), BPT = 64 / RB, LOGR1 = ilog2c(R1), LOGRB = ilog2c(RB);
   extern __shared__ float2 smem[];
-  float2* st3 = smem;                          // [TW3_SN], w = exp(-2 pi i / L)
-  float2* uni = st3 + TW3_SN;                  // [NLR][16]: w^{RB k2 b} (b < 8), w^{8 RB k2 a} at 8 + a
+  float2* uni = smem;                          // [NLR][16]: w^{RB k2 b} (b < 8), w^{8 RB k2 a} at 8 + a
   float2* sj = uni + NLR * 16;                 // [64]: exp(-i pi j / R1)
   float2* wbt = sj + 64;                       // [NLR][RB]: exp(-i pi (k2 + 64 R2 c) / L) / 2
   float2* twk = wbt + NLR * RB;                // [NLR][TWK_STR]
@@ -476,26 +462,39 @@ __global__ void __launch_bounds__(WIDE_NT, MODE == ROW_SPECTRUM ? 3 : 2)
     else if (MODE == ROW_TABLE) prefetch_l2(ctab + ((size_t)row << LOGR1), R1 * (unsigned)sizeof(float2));
   }
   {
-    // stage 1: butterfly t of the line, inputs n1 = t + RB j
+    // stage 1: butterfly t of the line, inputs n1 = t + RB j.  The table entries of
+    // the twiddles are asked for ahead of the rows, their products formed behind them.
+    constexpr int NU = (NLR * 16 + WIDE_NT - 1) / WIDE_NT, NK = MODE != ROW_SPECTRUM ? NLR / 2 : 0;
     const int slot = tid >> LOGRB, t = tid & (RB - 1);
     const unsigned k2 = (unsigned)row_of(slot);
+    Tw2Pair pt(tw2L, 2 * k2 * (unsigned)t), pb(tw2L, k2 + ((unsigned)(64 * t) << rt.logR2)), ps, pu[NU], pk[NK + 1];
+    if (tid < 64) ps = Tw2Pair(tw2L, (unsigned)tid << rt.logR2);
+#pragma unroll
+    for (int i = 0; i < NU; ++i) {
+      const int q = tid + i * WIDE_NT;
+      if (q < NLR * 16)
+        pu[i] = Tw2Pair(tw2L, 2 * (unsigned)row_of(q >> 4) * ((unsigned)(q & 7) * (unsigned)((q & 8) ? 8 * RB : RB)));
+    }
+#pragma unroll
+    for (int i = 0; i < NK; ++i) {
+      const int q = tid + i * WIDE_NT;
+      pk[i] = Tw2Pair(tw2L, ((unsigned)row_of(q >> 6) * (unsigned)(q & 63)) << (LOGRB + 1));
+    }
     const float2* src = in + ((size_t)k2 << LOGR1) + t;
     float2 v[64];
 #pragma unroll
     for (int j = 0; j < 64; ++j) v[j] = __ldg(src + j * RB);
-    load_tw3_all<WIDE_NT>(st3, tw3L);
-    if (tid < 64) sj[tid] = tw2(tw2L, (unsigned)tid << rt.logR2);
-    if (tid < NLR * RB) {   // always: NLR RB = 128 threads
-      const unsigned kr = (unsigned)row_of(slot) + ((unsigned)(64 * t) << rt.logR2);
-      wbt[tid] = cscale(tw2(tw2L, kr), 0.5f);
+    const float2 wt = pt.value();
+    wbt[tid] = cscale(pb.value(), 0.5f);   // NLR RB = 128 entries
+    if (tid < 64) sj[tid] = ps.value();
+#pragma unroll
+    for (int i = 0; i < NU; ++i)
+      if (tid + i * WIDE_NT < NLR * 16) uni[tid + i * WIDE_NT] = pu[i].value();
+#pragma unroll
+    for (int i = 0; i < NK; ++i) {   // e^{2 pi i k2 m1 / M}, as make_twk
+      const int q = tid + i * WIDE_NT;
+      twk[(q >> 6) * TWK_STR + (q & 63)] = cconj(pk[i].value());
     }
-    __syncthreads();   // st3
-    for (int i = tid; i < NLR * 16; i += WIDE_NT) {
-      const unsigned e = (unsigned)(i & 7) * (unsigned)((i & 8) ? 8 * RB : RB);
-      uni[i] = tw3(st3, (unsigned)row_of(i >> 4) * e);
-    }
-    if (MODE != ROW_SPECTRUM) make_twk<R1>(twk, st3, NLR, row_of);
-    const float2 wt = tw3(st3, k2 * (unsigned)t);
     __syncthreads();   // uni
     const float2* un = uni + slot * 16;
     wide_dft<64, false>(
@@ -575,7 +574,7 @@ __global__ void __launch_bounds__(WIDE_NT, MODE == ROW_SPECTRUM ? 3 : 2)
 template <int R1>
 size_t fwd_rows_smem_bytes(const RowTile& rt) {
   constexpr int NLR = run_slots<R1>();
-  return (size_t)(TW3_SN + NLR * 16 + 64 + WIDE_NT + NLR * TWK_STR + NLR * rt.rstr) *
+  return (size_t)(NLR * 16 + 64 + WIDE_NT + NLR * TWK_STR + NLR * rt.rstr) *
          sizeof(float2);
 }
 

@@ -62,6 +62,7 @@ struct SegIn {
   int ch = 1;
   int pair4 = 0;  // ch 2, both runs 4-byte aligned with a_len, b_len % 4 == 0: F1 may load
                   // one complex sample's two N / S pairs (4 bytes) at a time
+  int pair2 = 0;  // ch 1, both runs 2-byte aligned with even lengths: one complex sample (2 bytes) at a time
 };
 
 // The input of consecutive segments, one per blockIdx.y of a launch.  Byte r of
@@ -132,9 +133,10 @@ cudaError_t launch_tw2(float2* lo, float2* hi, int logn, int sign, cudaStream_t 
 cudaError_t launch_tw3(float2* out, int logn, int sign, cudaStream_t st);
 cudaError_t launch_stage_tw(float2* out, int R, cudaStream_t st);
 int stage_tw_entries(int R);
-// Stage-2 twiddles of the 64-values-per-thread FFT of length R (512 .. 4096; none otherwise).
-cudaError_t launch_wide_tw(float2* out, int R, cudaStream_t st);
-int wide_tw_entries(int R);
+// Stage-2 twiddles of the 64-values-per-thread FFT of length R (512 .. 4096; none
+// otherwise), radices (64, R / 64) or, last64, (R / 64, 64).
+cudaError_t launch_wide_tw(float2* out, int R, bool last64, cudaStream_t st);
+int wide_tw_entries(int R, bool last64);
 // Passes over nseg consecutive segments per launch (blockIdx.y): segment y reads
 // and writes its own L elements of the buffers (M of P).
 cudaError_t launch_fwd_cols(const Geom& g, const SegSrc& in, float2* out, const float2* tw, cudaStream_t st,
@@ -153,12 +155,12 @@ constexpr int FUSED_J = 64;
 bool fused_geometry(const Geom& g);
 int fused_groups(const Geom& g);
 // ctab non-null: the chirp from that per-bin table (launch_chirp_c64), else from the anchors
-cudaError_t launch_fwd_rows_inv(const Geom& g, const float2* in, float2* out, const float2* tw3L, Tw2 tw2L,
+cudaError_t launch_fwd_rows_inv(const Geom& g, const float2* in, float2* out, Tw2 tw2L,
                                 const float2* wtw, const ChirpAnchor* anc, int clog, const float2* ctab,
                                 cudaStream_t st, int nseg = 1);
 cudaError_t launch_chirp_c64(float2* tab, const Geom& g, double du, double half, double f0, double alpha, int sgn,
                              cudaStream_t st);
-cudaError_t launch_inv_rows_chirp(const Geom& g, const float2* in, float2* out, const float2* tw3L,
+cudaError_t launch_inv_rows_chirp(const Geom& g, const float2* in, float2* out, Tw2 tw2L,
                                   const ChirpAnchor* anc, int clog, cudaStream_t st);
 // nu > 1: one launch over nu trials or segments, the u-th reading in + u L and writing
 // P + u M, part + u G M, cnt + u FUSED_J (G = fused_groups); wtw: launch_wide_tw of R2
@@ -168,7 +170,7 @@ cudaError_t launch_inv_cols_det(const Geom& g, const float2* in, float* P, float
                                 const float2* wtw, cudaStream_t st, int nu = 1);
 // Batched lanes: Ir over ntr trials in one launch (trial t writes out + t L),
 // the chirp from the lane's Q0.32 table (table = true) or each trial's anchors
-cudaError_t launch_inv_rows_chirp_multi(const Geom& g, const float2* in, float2* out, int ntr, const float2* tw3L,
+cudaError_t launch_inv_rows_chirp_multi(const Geom& g, const float2* in, float2* out, int ntr, Tw2 tw2L,
                                         MultiChirp mc, bool table, cudaStream_t st);
 // Tensor-core column pass (split-BF16, three terms) for R2 = 2048 and at least
 // four sub-channels: same outputs and arguments as launch_inv_cols_det, plus
