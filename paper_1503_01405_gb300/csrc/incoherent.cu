@@ -32,6 +32,7 @@
 
 #include "../../include/pond.h"
 #include "fft_block.cuh"
+#include "fft_wide.cuh"
 #include "pond_internal.h"
 
 namespace pond {
@@ -42,6 +43,8 @@ constexpr int FB_MIN_NCH = 64, FB_MAX_NCH = 2048;
 constexpr int FB_MAX_LOGNINT = 16;
 constexpr int DD_TD = 32;                  // outputs per shift-and-sum CTA
 constexpr int DD_WARPS = 8;
+constexpr int FBW_PF = 38;                 // L2 prefetch distance, CTAs (AID / scintillation us: 38: 674 / 338, 114: 676 /
+                                           // 338, 228: 677 / 339, 456: 679 / 341)
 
 enum FbForm { FB_AID1 = 0, FB_AID2 = 1, FB_CID = 2 };
 
@@ -172,6 +175,147 @@ __global__ void __launch_bounds__(NT, ONE ? 2 : 1) k_fb_power(FbArgs a, const fl
   }
 }
 
+// CPT consecutive real samples q .. of the (added) stream, or CPT N / S pairs, as bytes:
+// BPS bytes per sample, q CPT-aligned and the stream 16-byte aligned.
+template <int BYTES>
+__device__ __forceinline__ void load_bytes(const int8_t* p, unsigned (&w)[(BYTES + 3) / 4]) {
+  if constexpr (BYTES == 1) w[0] = (unsigned char)__ldg(p);
+  else if constexpr (BYTES == 2) w[0] = __ldg(reinterpret_cast<const unsigned short*>(p));
+  else if constexpr (BYTES == 4) w[0] = __ldg(reinterpret_cast<const unsigned*>(p));
+  else if constexpr (BYTES == 8) {
+    const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+    w[0] = v.x;
+    w[1] = v.y;
+  } else {
+    const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
+    w[0] = v.x;
+    w[1] = v.y;
+    w[2] = v.z;
+    w[3] = v.w;
+  }
+}
+template <int N>
+__device__ __forceinline__ float byte_of(const unsigned (&w)[N], int i) { return s8(w[i / 4], i & 3); }
+
+// Filterbank with 64 values per thread (fft_wide.cuh), R = 512 .. 4096: lines are (RA, 64),
+// RA = R / 64.  In stage 1 a thread takes the same RA rows of CPT = 64 / RA adjacent butterflies,
+// so a load brings CPT samples (a warp reads 128 bytes of one spectrum for AID with two
+// halves at R = 2048); stage 2 is one 64-point butterfly per thread, in place.  A line
+// has one value of padding per row of RA and, as stage 1's lanes are CPT rows
+// apart, one more per CPT rows: bin e sits at e + e / RA + e / 64.  Detection and integration as in
+// k_fb_power.  The radix-16 form kept the shared-memory pipe 62-72 % busy; against it
+// 2.56e8 N / S pairs in 1024 channels (AID) 468 -> 375 us, 1.28e8 pairs in 256
+// channels (CID, 16 spectra per sample) 347 -> 214 us.
+template <int R>
+__host__ __device__ constexpr int fbw_stride() {   // 8 mod 16: two 512-sample lines share a half-warp
+  constexpr int RA = R / 64, base = 64 * (RA + 1) + (RA < 64 ? RA : 0);
+  return base + ((8 - base) & 15);
+}
+template <int R, int FORM>
+__global__ void __launch_bounds__(WIDE_NT, 3) k_fb_power_w(FbArgs a, const float2* __restrict__ tw) {
+  constexpr int NCH = R / 2, NL = TILE / R, RA = R / 64, CPT = 64 / RA, WSTR = fbw_stride<R>();
+  constexpr int XP = CPT > 1 ? 1 : 0;                // the second padding
+  constexpr int SPL = FORM == FB_CID ? 1 : 2;        // spectra per line
+  constexpr int BPS = FORM == FB_AID1 ? 1 : 2;       // bytes per sample of a spectrum
+  constexpr int KPT = NCH / WIDE_NT;                 // channels per thread
+  extern __shared__ float2 smem[];
+  const int tid = (int)threadIdx.x;
+  const long long s0 = (long long)blockIdx.x * a.s_cta;
+  const int len = (int)min(a.s_cta, a.n_spec - s0);   // spectra of this CTA
+  const int nmask = (1 << a.lognint) - 1;
+  if (tid == 0 && blockIdx.x + FBW_PF < gridDim.x) {
+    // L2 prefetch of the input bytes of CTA blockIdx.x + FBW_PF (contiguous spectra)
+    const long long n0 = (long long)(blockIdx.x + FBW_PF) * a.s_cta;
+    const long long n1 = min(n0 + a.s_cta, a.n_spec);
+    prefetch_range(a.x, n0 * R * BPS, n1 * R * BPS);
+  }
+  float acc[KPT];
+#pragma unroll
+  for (int u = 0; u < KPT; ++u) acc[u] = 0.f;
+#pragma unroll 1
+  for (int p = 0; p < len; p += SPL * NL) {
+    {
+      const int l = tid / RA, t = (tid % RA) * CPT;   // RA threads of CPT butterflies per line
+      const int r = p + SPL * l;                      // spectrum within the CTA
+      const int8_t* xa = a.x + ((s0 + r) * R + t) * BPS;
+      float2 v[CPT][RA];
+#pragma unroll
+      for (int j = 0; j < RA; ++j) {
+        unsigned wa[(CPT * BPS + 3) / 4] = {}, wb[(CPT * BPS + 3) / 4] = {};
+        if (r < len) load_bytes<CPT * BPS>(xa + 64 * j * BPS, wa);
+        if (SPL == 2 && r + 1 < len) load_bytes<CPT * BPS>(xa + (R + 64 * j) * BPS, wb);
+#pragma unroll
+        for (int c = 0; c < CPT; ++c) {
+          if constexpr (FORM == FB_CID) v[c][j] = make_float2(byte_of(wa, 2 * c), byte_of(wa, 2 * c + 1));
+          else if constexpr (FORM == FB_AID2)
+            v[c][j] = make_float2(byte_of(wa, 2 * c) + byte_of(wa, 2 * c + 1), byte_of(wb, 2 * c) + byte_of(wb, 2 * c + 1));
+          else v[c][j] = make_float2(byte_of(wa, c), byte_of(wb, c));
+        }
+      }
+      float2* dst = smem + l * WSTR + (RA + 1) * t + XP * (tid % RA);
+#pragma unroll
+      for (int c = 0; c < CPT; ++c) {
+        wide_dft<RA, false>(v[c]);
+#pragma unroll
+        for (int j = 0; j < RA; ++j) dst[c * (RA + 1) + j] = v[c][j];
+      }
+    }
+    {
+      const int l = tid / RA, t = tid % RA;           // butterfly t < RA of line l
+      WideTw<RA, 64> w2;
+      w2.load(tw, t);
+      __syncthreads();
+      float2* q = smem + l * WSTR + t;
+      float2 v[64];
+#pragma unroll
+      for (int j = 0; j < 64; ++j) v[j] = q[j * (RA + 1) + XP * (j / CPT)];
+      w2.template dft<false>(v);
+#pragma unroll
+      for (int j = 0; j < 64; ++j) q[j * (RA + 1) + XP * (j / CPT)] = v[j];
+    }
+    __syncthreads();
+    // detect and integrate: thread-owned channels, spectra in order; a complete
+    // group (spectrum index = -1 mod nint; s0 is a multiple of nint) is written
+    // as row t of F by all threads together
+    auto at = [](int e) { return e + e / RA + XP * (e / 64); };
+#pragma unroll
+    for (int u = 0; u < KPT; ++u) {
+      const int k = tid + u * WIDE_NT;
+      const int ka = at(k), kc = at((R - k) & (R - 1));
+      float s = acc[u];
+#pragma unroll 4
+      for (int l = 0; l < NL; ++l) {
+        const int r = p + SPL * l;
+        if (r >= len) break;
+        const float2 A = smem[l * WSTR + ka], C = smem[l * WSTR + kc];
+        if constexpr (FORM == FB_CID) {
+          s += 0.5f * (A.x * C.y + A.y * C.x);
+          if ((r & nmask) == nmask) {
+            a.F[((s0 + r) >> a.lognint) * NCH + k] = s;
+            s = 0.f;
+          }
+        } else {
+          const float ar = A.x + C.x, ai = A.y - C.y, br = A.x - C.x, bi = A.y + C.y;
+          s += 0.25f * (ar * ar + ai * ai);
+          if ((r & nmask) == nmask) {
+            a.F[((s0 + r) >> a.lognint) * NCH + k] = s;
+            s = 0.f;
+          }
+          if (r + 1 < len) {
+            s += 0.25f * (br * br + bi * bi);
+            if (((r + 1) & nmask) == nmask) {
+              a.F[((s0 + r + 1) >> a.lognint) * NCH + k] = s;
+              s = 0.f;
+            }
+          }
+        }
+      }
+      acc[u] = s;
+    }
+    __syncthreads();   // the next pass's stage 1 overwrites the tile
+  }
+}
+
 // D[i] = sum_k F[t_first + i + d_k][k], i < n_out (nch a multiple of 32).
 __global__ void __launch_bounds__(DD_WARPS * 32) k_incoh_sum(const float* __restrict__ F, int nch,
                                                              const int* __restrict__ d, long long t_first,
@@ -275,6 +419,11 @@ size_t ips_smem_bytes() {
 }
 
 template <int R>
+constexpr int fbw_smem_bytes() {
+  return TILE / R * fbw_stride<R>() * (int)sizeof(float2);
+}
+
+template <int R>
 size_t fb_smem_bytes() {
   return ((size_t)stage_table_size(R) + (size_t)(TILE / R) * line_stride(R)) * sizeof(float2) +
          (size_t)(R / 2) * sizeof(float);
@@ -345,22 +494,37 @@ double rounded(double x) {
 
 template <int R>
 cudaError_t fb_attr() {
-  cudaError_t e = cudaFuncSetAttribute(pond::k_fb_power<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)pond::fb_smem_bytes<R>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(pond::k_fb_power<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)pond::fb_smem_bytes<R>());
+  cudaError_t e = cudaSuccess;
+  auto attr = [&](auto* f, int bytes) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  };
+  if constexpr (R >= 512) {
+    attr(pond::k_fb_power_w<R, pond::FB_AID1>, pond::fbw_smem_bytes<R>());
+    attr(pond::k_fb_power_w<R, pond::FB_AID2>, pond::fbw_smem_bytes<R>());
+    attr(pond::k_fb_power_w<R, pond::FB_CID>, pond::fbw_smem_bytes<R>());
+  } else {
+    attr(pond::k_fb_power<R, false>, (int)pond::fb_smem_bytes<R>());
+    attr(pond::k_fb_power<R, true>, (int)pond::fb_smem_bytes<R>());
+  }
   return e;
 }
 
+// Lines of 512 samples and more take 64 values per thread; shorter ones have no 64-point stage to fill.
 template <int R>
 cudaError_t fb_launch(const FbArgs& a, const float2* tw, cudaStream_t st) {
-  const long long blocks = (a.n_spec + a.s_cta - 1) / a.s_cta;
-  const long long per_pass = (long long)(a.form == pond::FB_CID ? 1 : 2) * (pond::TILE / R);
-  if (a.s_cta <= per_pass)
-    pond::k_fb_power<R, true><<<(unsigned)blocks, pond::NT, pond::fb_smem_bytes<R>(), st>>>(a, tw);
-  else
-    pond::k_fb_power<R, false><<<(unsigned)blocks, pond::NT, pond::fb_smem_bytes<R>(), st>>>(a, tw);
+  const unsigned blocks = (unsigned)((a.n_spec + a.s_cta - 1) / a.s_cta);
+  if constexpr (R >= 512) {
+    constexpr int bytes = pond::fbw_smem_bytes<R>();
+    if (a.form == pond::FB_AID1) pond::k_fb_power_w<R, pond::FB_AID1><<<blocks, pond::WIDE_NT, bytes, st>>>(a, tw);
+    else if (a.form == pond::FB_AID2) pond::k_fb_power_w<R, pond::FB_AID2><<<blocks, pond::WIDE_NT, bytes, st>>>(a, tw);
+    else pond::k_fb_power_w<R, pond::FB_CID><<<blocks, pond::WIDE_NT, bytes, st>>>(a, tw);
+  } else {
+    const long long per_pass = (long long)(a.form == pond::FB_CID ? 1 : 2) * (pond::TILE / R);
+    if (a.s_cta <= per_pass)
+      pond::k_fb_power<R, true><<<blocks, pond::NT, pond::fb_smem_bytes<R>(), st>>>(a, tw);
+    else
+      pond::k_fb_power<R, false><<<blocks, pond::NT, pond::fb_smem_bytes<R>(), st>>>(a, tw);
+  }
   return cudaGetLastError();
 }
 
@@ -491,7 +655,9 @@ extern "C" int pond_incoh_create(pond_incoh_t* out, const pond_incoh_opts* o) {
     if (e == cudaSuccess) e = cudaMemset(h->ips, 0, (o->ips_len / 2 + 1) * sizeof(double));
   }
   if (e == cudaSuccess) e = cudaMalloc(&h->d_delay, o->nchan * sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc(&h->stw, std::max(1, pond::stage_tw_entries(1 << h->logR)) * sizeof(float2));
+  const int wide = pond::wide_tw_entries(1 << h->logR, true);   // 0: radix-16 stages
+  if (e == cudaSuccess)
+    e = cudaMalloc(&h->stw, std::max(1, wide ? wide : pond::stage_tw_entries(1 << h->logR)) * sizeof(float2));
   if (e == cudaSuccess) e = cudaMalloc(&h->psum, (size_t)pond::MAX_FOLD_PARTS * o->nbins * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&h->phits, (size_t)pond::MAX_FOLD_PARTS * o->nbins * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&h->prof_sum, o->nbins * sizeof(double));
@@ -500,7 +666,9 @@ extern "C" int pond_incoh_create(pond_incoh_t* out, const pond_incoh_opts* o) {
     if (e == cudaSuccess) e = cudaEventCreate(&ev);
   if (e == cudaSuccess)
     e = cudaMemcpy(h->d_delay, h->delay.data(), o->nchan * sizeof(int), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = pond::launch_stage_tw(h->stw, 1 << h->logR, nullptr);
+  if (e == cudaSuccess)
+    e = wide ? pond::launch_wide_tw(h->stw, 1 << h->logR, true, nullptr)
+             : pond::launch_stage_tw(h->stw, 1 << h->logR, nullptr);
   if (e == cudaSuccess) e = cudaMemset(h->prof_sum, 0, o->nbins * sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(h->prof_hits, 0, o->nbins * sizeof(long long));
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
