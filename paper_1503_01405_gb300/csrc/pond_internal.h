@@ -122,6 +122,9 @@ cudaError_t launch_wait_probe(unsigned long long limit_ns, int* status, unsigned
 // W16 parts for the tensor-core stages, host-built: [fwd, inv][hi, mid, lo] in
 // the K-major operand layout (2 x 6 KiB).
 void build_w16_parts(uint16_t* out);
+// The library's own stream-ordered memory pool of the current device (scratch of the
+// entry points without a handle): it keeps a bounded amount between calls.
+cudaError_t scratch_pool(cudaMemPool_t* out);
 int run_boxcar(const float* d_series, int ndm, long long n, long long stride, double thr, pond_cand* host_out,
                size_t cap, size_t* n_found, cudaStream_t st);
 // Record msg as the calling thread's last error (pond_last_error) and return code.

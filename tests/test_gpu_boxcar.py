@@ -65,3 +65,56 @@ def test_candidates_from_a_batched_plan():
     best = max(cands, key=lambda c: c["snr"])
     assert best["trial"] == 2
     assert abs((best["index"] + best["width"] / 2) * 8e-6 - 0.03) < 1e-3
+
+
+def gpu_detect_strided(block, pad, thr):
+    """As gpu_detect with rows `pad` samples apart from their ends."""
+    import torch
+    t = torch.full((block.shape[0], block.shape[1] + pad), 7.0e9, device="cuda")
+    t[:, :block.shape[1]] = torch.from_numpy(np.ascontiguousarray(block, dtype=np.float32)).cuda()
+    c = pond.boxcar(t.data_ptr(), block.shape[0], block.shape[1], t.stride(0), thr,
+                    stream=torch.cuda.current_stream().cuda_stream)
+    return [(x["trial"], x["index"], x["width"], x["snr"]) for x in c]
+
+
+@pytest.mark.parametrize("pad", [0, 1], ids=["aligned", "odd_stride"])
+@pytest.mark.parametrize("n", [63, 64, 447, 448, 449, 512, 513, 897, 8191, 8193, 70001])
+def test_screened_points_at_the_edges(n, pad):
+    """Row lengths around a warp's 448 points, its 64-sample reach and the collection
+    chunk; pulses at both ends and across the seams; an outlier that widens the bound."""
+    rng = np.random.default_rng(n + pad)
+    block = (4e5 + 1.8e4 * rng.standard_normal((6, n))).astype(np.float32)
+    for t in (0, max(0, n - 1), max(0, n - 40), min(n - 1, 440), min(n - 1, 447), n // 2):
+        block[rng.integers(6), t:t + int(rng.integers(1, 64))] += np.float32(2e5)
+    block[2, n // 3] = 3e9
+    want = ob.detect(block)
+    assert gpu_detect_strided(block, pad, 6.0) == want
+
+
+@pytest.mark.parametrize("kind", ["ties", "two_values", "negative", "tiny_spread", "skewed", "sorted"])
+def test_order_statistics_of_awkward_rows(kind):
+    rng = np.random.default_rng(5)
+    n = 30000
+    x = {"ties": rng.integers(0, 12, (3, n)), "two_values": rng.integers(0, 2, (3, n)) * 5.0,
+         "negative": -1e3 + 5 * rng.standard_normal((3, n)), "tiny_spread": 1e6 + 0.25 * rng.integers(0, 9, (3, n)),
+         "skewed": rng.exponential(3.0, (3, n)) ** 2, "sorted": np.sort(rng.standard_normal((3, n)), axis=1)}[kind]
+    block = x.astype(np.float32)
+    block[1, 100:103] += np.float32(40 * (np.abs(block).max() + 1))
+    assert gpu_detect(block, thr=5.0) == ob.detect(block, threshold=5.0)
+
+
+def test_screened_and_dense_forms_agree():
+    """A threshold below 1 evaluates every point; its list cut at S/N 6 is the screened
+    list, also where rows hold infinities or NaN (and an overflowing list takes the dense form)."""
+    rng = np.random.default_rng(8)
+    block = (100 + 3 * rng.standard_normal((7, 20000))).astype(np.float32)
+    block[1, 5000:5008] += 30
+    block[2, 77] = np.inf
+    block[3, 900] = -np.inf
+    block[4, 901] = np.nan
+    block[5, 6000] = 1e30
+    every = gpu_detect(block, thr=0.5)
+    for thr in (1.0, 2.0, 6.0):
+        got = gpu_detect(block, thr=thr)
+        want = [c for c in every if c[3] >= thr]
+        assert got == want
