@@ -163,29 +163,8 @@ struct PhaseRule {
     for (int k = r.nc - 2; k >= 0; --k) x = __dadd_rn(__dmul_rn(x, tau), r.c[k]);
     return x;
   }
-  // phi' at the middle less its largest change over the span, times dt, against the
-  // evaluation's rounding (sum |c_i| |tau|^i eps, with room to spare)
   __device__ bool forwards(long long ga, long long gb) const {
-    const double t0 = (double)ga * r.dt - r.t_ref, t1 = (double)gb * r.dt - r.t_ref;
-    const double tm = 0.5 * (t0 + t1), half = 0.5 * (t1 - t0), ta = fmax(fabs(t0), fabs(t1));
-    double d = 0.0, dd = 0.0, mag = 0.0, pm = 1.0, pa1 = 1.0, pa2 = 0.0;
-    for (int i = 0; i < r.nc; ++i) {
-      const double c = fabs(r.c[i]);
-      if (i >= 1) {
-        d += i * r.c[i] * pm;
-        pm *= tm;
-      }
-      if (i >= 2) {
-        pa2 = i == 2 ? 1.0 : pa2 * ta;
-        dd += i * (i - 1) * c * pa2;
-      }
-      mag += c * pa1;
-      pa1 *= ta;
-    }
-    // tau itself is rounded: to |g dt| + |t_ref| ulps, times the slope
-    const double slope = d + dd * half;
-    const double err = 1e-14 * (mag + slope * (fabs((double)gb * r.dt) + fabs(r.t_ref)));
-    return (d - dd * half) * r.dt > err;   // false for NaN
+    return phase_forwards(r.c, r.nc, r.dt, r.t_ref, ga, gb);
   }
 };
 
@@ -714,19 +693,30 @@ __global__ void k_make_chirp_words(unsigned* words, int logR1, int logR2, const 
   words[i] = anchor_word(anc[k >> clog], clog, k);
 }
 
-// Byte copy between device buffers (any alignment): 16-byte words where both
-// sides allow, single bytes otherwise.
+// Byte copy between device buffers (any alignment): 16-byte words of dst, each from the
+// one to five aligned 4-byte words of src that hold its bytes; single bytes at the ends.
+// (A byte at a time where the sides disagree, the carry of an N / S stream pushed in odd
+// pieces took 141 us per push.)
 __global__ void k_copy_bytes(int8_t* __restrict__ dst, const int8_t* __restrict__ src, long long n) {
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if ((((uintptr_t)dst | (uintptr_t)src) & 15) == 0) {
-    const long long n16 = n >> 4;
-    for (long long i = i0; i < n16; i += stride)
-      reinterpret_cast<uint4*>(dst)[i] = __ldg(reinterpret_cast<const uint4*>(src) + i);
-    for (long long i = (n16 << 4) + i0; i < n; i += stride) dst[i] = src[i];
+  const long long head = min(n, (long long)(-(uintptr_t)dst & 15)), n16 = (n - head) >> 4;
+  const int8_t* s = src + head;
+  uint4* d = reinterpret_cast<uint4*>(dst + head);
+  const unsigned mis = (unsigned)((uintptr_t)s & 15), sh = (mis & 3) * 8;
+  if (mis == 0) {
+    for (long long i = i0; i < n16; i += stride) d[i] = __ldg(reinterpret_cast<const uint4*>(s) + i);
   } else {
-    for (long long i = i0; i < n; i += stride) dst[i] = src[i];
+    const unsigned* w = reinterpret_cast<const unsigned*>(s - (mis & 3));
+    for (long long i = i0; i < n16; i += stride) {
+      const unsigned* p = w + 4 * i;
+      const unsigned a = __ldg(p), b = __ldg(p + 1), c = __ldg(p + 2), e = __ldg(p + 3), f = sh ? __ldg(p + 4) : 0u;
+      d[i] = make_uint4(__funnelshift_r(a, b, sh), __funnelshift_r(b, c, sh), __funnelshift_r(c, e, sh),
+                        __funnelshift_r(e, f, sh));
+    }
   }
+  for (long long i = i0; i < head; i += stride) dst[i] = src[i];
+  for (long long i = head + (n16 << 4) + i0; i < n; i += stride) dst[i] = src[i];
 }
 
 // ---------------------------------------------------------------------------

@@ -209,6 +209,33 @@ struct FoldPhase {
   double dt = 0, t_ref = 0;
   double c[8] = {};
 };
+#ifdef __CUDACC__
+// True when the FP64 evaluation (Horner's rule) of the phase polynomial c[0 .. nc) in
+// tau = g dt - t_ref is known to grow from each sample of [ga, gb] to the next: phi' at the
+// middle less its largest change over the span, times dt, exceeds twice the
+// evaluation's rounding with room to spare.  False for NaN.
+__device__ inline bool phase_forwards(const double* c, int nc, double dt, double t_ref, long long ga, long long gb) {
+  const double t0 = (double)ga * dt - t_ref, t1 = (double)gb * dt - t_ref;
+  const double tm = 0.5 * (t0 + t1), half = 0.5 * (t1 - t0), ta = fmax(fabs(t0), fabs(t1));
+  double d = 0.0, dd = 0.0, mag = 0.0, pm = 1.0, pa1 = 1.0, pa2 = 0.0;
+  for (int i = 0; i < nc; ++i) {
+    const double a = fabs(c[i]);
+    if (i >= 1) {
+      d += i * c[i] * pm;
+      pm *= tm;
+    }
+    if (i >= 2) {
+      pa2 = i == 2 ? 1.0 : pa2 * ta;
+      dd += i * (i - 1) * a * pa2;
+    }
+    mag += a * pa1;
+    pa1 *= ta;
+  }
+  // tau itself is rounded: to |g dt| + |t_ref| ulps, times the slope
+  const double err = 1e-14 * (mag + (fabs(d) + dd * half) * (fabs((double)gb * dt) + fabs(t_ref)));
+  return (d - dd * half) * dt > err;
+}
+#endif
 // Fold + decimation of nseg consecutive segments s0 .. (single-DM plans).  Segment y's
 // power is P + y M, n_y = min(S_c, n_left - y S_c) samples from g0 + y S_c on.  The
 // fold of segment s adds to the fold_parts rows of its slot s mod fold_slots of the

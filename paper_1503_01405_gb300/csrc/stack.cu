@@ -9,11 +9,18 @@
 // are decided exactly as a plain FP64 evaluation decides them.
 //
 // The key K(g) = q nbins + b never decreases along the series for a phase
-// model that runs forwards (checked first, by k_stack_check), so the samples of
-// one (rotation, bin) pair form one contiguous run.  One thread per stack cell
-// (row, bin) finds the runs of its rotations by binary search on K and adds
-// their samples in sample order in FP64: no atomics, no partials to merge, and
-// the sums are those of a sequential loop over the series.
+// model that runs forwards (checked first), so the samples of
+// one (rotation, bin) pair form one contiguous run.  k_stack_starts evaluates K
+// where it changes, checks that it grows and writes the first sample of every key's run; one
+// thread per stack cell (row, bin) then adds the samples of its rotations' runs in
+// sample order in FP64: no atomics, no partials to merge, and
+// the sums are those of a sequential loop over the series.  The phase evaluations bound
+// it (an SM retires two FP64 operations per clock): with the check evaluating two keys per
+// sample and every cell finding its runs by binary search on K, a 60 s series (976,562
+// samples, 1024 bins) took 58 + 137 us, and 346 us with the host's
+// share, now 184.  Where the keys far outnumber
+// the samples (bins much finer than the sampling) the table of starts is not
+// worth its size and the cells search.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -68,6 +75,101 @@ __device__ long long first_at_or_after(const PhaseModel& m, long long lo, long l
 }
 
 __device__ int g_backwards;   // set when K decreases somewhere along the series
+
+__device__ __forceinline__ double phase_at(const PhaseModel& m, long long i) {
+  const double tau = __dsub_rn(__dmul_rn((double)(m.g0 + i), m.dt), m.t_ref);
+  double x = m.c[m.nc - 1];
+  for (int k = m.nc - 2; k >= 0; --k) x = __dadd_rn(__dmul_rn(x, tau), m.c[k]);
+  return x;
+}
+
+// start[K - K0] = first sample i with key >= K, for K0 <= K <= K0 + nk.  A warp takes
+// windows of 1024 samples.  Where the phase is known to run forwards over a window a
+// lane takes 32 consecutive samples: the keys at its first sample and at the next
+// lane's tell which keys begin in between, and each one's first sample is predicted from
+// the phases at the ends and corrected with exact keys (two evaluations per key).
+// Elsewhere every sample's key is evaluated and compared with the one before.
+constexpr int RUN = 32, WINDOW = 32 * RUN;
+__global__ void __launch_bounds__(128) k_stack_starts(PhaseModel m, long long n, long long K0, long long nk,
+                                                    unsigned* __restrict__ start) {
+  const int lane = threadIdx.x & 31;
+  const long long warps = gridDim.x * 4ll;
+  auto put = [&](long long lo, long long hi, long long i) {   // keys lo .. hi start at sample i
+    for (long long q = max(lo, K0); q <= min(hi, K0 + nk); ++q) start[q - K0] = (unsigned)i;
+  };
+  for (long long base = (blockIdx.x * 4ll + (threadIdx.x >> 5)) * WINDOW; base < n; base += warps * WINDOW) {
+    const long long end = min(n, base + WINDOW);   // the window and the step to the next one
+    if (base == 0 && lane == 0) put(K0, key_value(m, 0), 0);
+    if (end == n && lane == 0) put(key_value(m, n - 1) + 1, K0 + nk, n);
+    const long long last = min(end, n - 1);
+    if (pond::phase_forwards(m.c, m.nc, m.dt, m.t_ref, m.g0 + base, m.g0 + last)) {
+      const long long a = base + lane * RUN, e = min(last, a + RUN);
+      if (a >= e) continue;
+      const double xa = phase_at(m, a), xe = phase_at(m, e);
+      const long long ka = key_value(m, a), ke = key_value(m, e);
+      const float per = (float)(e - a) / (float)(xe - xa);
+      for (long long k = ka + 1; k <= ke;) {
+        // the first sample at or after the start of bin k
+        const double lead = (double)k / (double)m.nbins - xa;
+        long long i = a + max(1ll, min((long long)ceilf((float)lead * per), e - a));
+        long long ki = key_value(m, i);
+        while (ki < k) ki = key_value(m, ++i);            // ends: key(e) = ke >= k
+        for (long long kp; i - 1 > a && (kp = key_value(m, i - 1)) >= k;) {
+          ki = kp;
+          --i;
+        }
+        put(k, ki, i);
+        k = ki + 1;
+      }
+    } else {
+      // steps i -> i + 1 of samples base .. last, each key against the next
+      for (long long i0 = base; i0 < last; i0 += 31) {
+        const long long i = min(i0 + lane, last);
+        const long long k = key_value(m, i);
+        const long long prev = __shfl_up_sync(0xffffffffu, k, 1);
+        if (lane > 0 && i0 + lane <= last) {
+          if (k < prev) g_backwards = 1;
+          put(prev + 1, k, i);
+        }
+      }
+    }
+  }
+}
+
+// Cell (row, b) from the table of starts (rows as in k_stack_cells); nothing when the model
+// runs backwards.
+__global__ void __launch_bounds__(CELL_THREADS) k_stack_sums(const float* __restrict__ y, long long n, PhaseModel m,
+                                                             int mode, long long n_sub, long long q_first,
+                                                             long long rows, const unsigned* __restrict__ start,
+                                                             double* __restrict__ S, long long* __restrict__ H) {
+  if (g_backwards) return;
+  const long long cell = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (cell >= rows * m.nbins) return;
+  const long long row = cell / m.nbins;
+  const int b = (int)(cell - row * m.nbins);
+  long long lo = 0, hi = n, qa = row, qb = row;   // rotations from q_first
+  if (mode != POND_STACK_ROTATION) {
+    lo = row * n_sub;
+    hi = min(n, lo + n_sub);
+    qa = key_at(m, lo).q - q_first;
+    qb = key_at(m, hi - 1).q - q_first;
+  }
+  double s = 0.0;
+  long long h = 0;
+  for (long long q = qa; q <= qb; ++q) {
+    const unsigned* p = start + q * m.nbins + b;
+    const long long a = max(lo, (long long)p[0]), e = min(hi, (long long)p[1]);
+    long long i = a;
+    for (; i + 4 <= e; i += 4) {   // four loads in flight, added in order
+      const float v0 = __ldg(y + i), v1 = __ldg(y + i + 1), v2 = __ldg(y + i + 2), v3 = __ldg(y + i + 3);
+      s = __dadd_rn(__dadd_rn(__dadd_rn(__dadd_rn(s, (double)v0), (double)v1), (double)v2), (double)v3);
+    }
+    for (; i < e; ++i) s = __dadd_rn(s, (double)__ldg(y + i));
+    if (e > a) h += e - a;
+  }
+  S[cell] = s;
+  H[cell] = h;
+}
 
 __global__ void k_stack_check(PhaseModel m, long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i + 1 < n;
@@ -174,26 +276,51 @@ extern "C" int pond_fold_stack(const float* d_series, int64_t n, int64_t g0, dou
   if (n == 0) return POND_OK;
   if (!d_series || !d_sum || !d_hits) return pond::set_error(POND_E_ARG, "pond_fold_stack: null device pointer");
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  const int zero = 0;
+  auto failed = [](cudaError_t e) {
+    return pond::set_error(e == cudaErrorMemoryAllocation ? POND_E_OOM : POND_E_CUDA,
+                           (std::string("pond_fold_stack: ") + cudaGetErrorString(e)).c_str());
+  };
+  const char* backwards = "pond_fold_stack: the phase model runs backwards over the series";
+  const long long cells = *rows * (long long)nbins, q_last = host_rotation(m, n - 1);
+  const unsigned cell_blocks = (unsigned)((cells + CELL_THREADS - 1) / CELL_THREADS);
+  void* flag = nullptr;
   int back = 0;
-  cudaError_t e = cudaMemcpyToSymbolAsync(g_backwards, &zero, sizeof(int), 0, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) {
-    const long long blocks = std::min<long long>((n + 255) / 256, 4096);
-    k_stack_check<<<(unsigned)blocks, 256, 0, st>>>(m, n);
+  cudaError_t e = cudaGetSymbolAddress(&flag, g_backwards);
+  if (e == cudaSuccess) e = cudaMemsetAsync(flag, 0, sizeof(int), st);
+  if (e != cudaSuccess) return failed(e);
+  // the table holds a start per key: used while there are at most eight keys per sample
+  const double keys = ((double)q_last - (double)*first_rotation + 1.0) * nbins;
+  const unsigned blocks = (unsigned)std::min<long long>((n + 255) / 256, 4096);
+  if (q_last >= *first_rotation && keys <= 8.0 * (double)n + 65536.0 && n < (1ll << 32)) {
+    const long long nk = (q_last - *first_rotation + 1) * nbins, K0 = *first_rotation * (long long)nbins;
+    unsigned* start = nullptr;
+    cudaMemPool_t pool = nullptr;
+    e = pond::scratch_pool(&pool);
+    if (e == cudaSuccess)
+      e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&start), (size_t)(nk + 1) * sizeof(unsigned), pool, st);
+    if (e != cudaSuccess) return failed(e);
+    k_stack_starts<<<(unsigned)std::min<long long>((n + 4 * WINDOW - 1) / (4 * WINDOW), 4096), 128, 0, st>>>(m, n, K0, nk, start);
+    if (cells > 0)
+      k_stack_sums<<<cell_blocks, CELL_THREADS, 0, st>>>(d_series, n, m, mode, n_sub, *first_rotation, *rows, start,
+                                                         d_sum, reinterpret_cast<long long*>(d_hits));
     e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&back, flag, sizeof(int), cudaMemcpyDeviceToHost, st);
+    cudaFreeAsync(start, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return failed(e);
+    return back ? pond::set_error(POND_E_ARG, backwards) : POND_OK;
   }
-  if (e == cudaSuccess) e = cudaMemcpyFromSymbolAsync(&back, g_backwards, sizeof(int), 0, cudaMemcpyDeviceToHost, st);
+  k_stack_check<<<blocks, 256, 0, st>>>(m, n);
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&back, flag, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess)
-    return pond::set_error(POND_E_CUDA, (std::string("pond_fold_stack: ") + cudaGetErrorString(e)).c_str());
-  if (back) return pond::set_error(POND_E_ARG, "pond_fold_stack: the phase model runs backwards over the series");
-  const long long cells = *rows * (long long)nbins;
+  if (e != cudaSuccess) return failed(e);
+  if (back) return pond::set_error(POND_E_ARG, backwards);
   if (cells > 0) {
-    k_stack_cells<<<(unsigned)((cells + CELL_THREADS - 1) / CELL_THREADS), CELL_THREADS, 0, st>>>(
-        d_series, n, m, mode, n_sub, *first_rotation, *rows, d_sum, reinterpret_cast<long long*>(d_hits));
+    k_stack_cells<<<cell_blocks, CELL_THREADS, 0, st>>>(d_series, n, m, mode, n_sub, *first_rotation, *rows, d_sum,
+                                                        reinterpret_cast<long long*>(d_hits));
     e = cudaGetLastError();
-    if (e != cudaSuccess)
-      return pond::set_error(POND_E_CUDA, (std::string("pond_fold_stack: ") + cudaGetErrorString(e)).c_str());
+    if (e != cudaSuccess) return failed(e);
   }
   return POND_OK;
 }

@@ -46,3 +46,18 @@ def test_stack_errors_and_empty_series():
     rc = pond.lib().pond_fold_stack(y.data_ptr(), 1000, 0, 1e-3, c.ctypes.data, 2, 0.0, 16, 0, 0, None, None, 2,
                                     ctypes.byref(rows), ctypes.byref(q0), None)
     assert rc == pond.POND_E_OVERRUN and rows.value == 5
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 257, 5000])
+@pytest.mark.parametrize("period_samples", [0.37, 3.0, 700.3], ids=["undersampled", "coarse", "fine"])
+@pytest.mark.parametrize("mode,n_sub", [(st.ROTATION, 0), (st.SUBINT, 1), (st.SUBINT, 100)])
+def test_stack_key_tables_and_searches(n, period_samples, mode, n_sub):
+    """Short series and key counts from far below to far above the samples' (the
+    table of starts and the search), bit for bit."""
+    import torch
+    dt, nbins = 1e-3, 4096 if period_samples < 1 else 37
+    c = np.array([0.2, 1.0 / (period_samples * dt), 1e-3])
+    y = np.random.default_rng(n).normal(10.0, 3.0, n).astype(np.float32)
+    S_ref, H_ref, q0_ref = st.stack(y, 5, dt, c, 0.1, nbins, mode, n_sub)
+    S, H, q0 = pond.fold_stack(torch.from_numpy(y).cuda(), 5, dt, c, 0.1, nbins, mode, n_sub)
+    assert q0 == q0_ref and np.array_equal(H, H_ref) and np.array_equal(S, S_ref)
