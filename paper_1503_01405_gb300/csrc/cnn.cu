@@ -37,8 +37,9 @@ struct pond_cnn_s {
   __nv_bfloat16 *h1 = nullptr, *h2 = nullptr;
   uint8_t *a1 = nullptr, *a2 = nullptr;
   float *gap = nullptr, *prob = nullptr, *loss = nullptr, *dg = nullptr, *lmean = nullptr;
-  float *dz3 = nullptr, *dz2 = nullptr, *dz1 = nullptr, *part = nullptr;
+  float *dz2 = nullptr, *dz1 = nullptr, *part = nullptr;
   unsigned char* wtc = nullptr;   // the conv weights in the tensor-core operand layout
+  float* wf = nullptr;            // the conv weights in the training kernels' layouts
   int* tc_err = nullptr;          // set when a tensor-core MMA wait gave up
   int sms = 0;
 };
@@ -56,42 +57,36 @@ int cuda_fail(cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return cuda_fail(e_, #call); \
   } while (0)
 
-template <int T, int MODE>
-size_t fwd_smem() { return (size_t)(C * (T + 2 * PAD) + CONV) * sizeof(float); }
-template <int T>
-size_t wgt_smem() { return (size_t)(C * T + C * (T + 2 * PAD)) * sizeof(float); }
-
 cudaError_t set_attrs() {
-  cudaError_t e = cudaFuncSetAttribute(k_conv_fwd<256, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)fwd_smem<256, 0>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_conv_bwd_weight<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wgt_smem<256>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_conv_fwd<128, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)fwd_smem<128, 0>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_conv_fwd<64, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fwd_smem<64, 1>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_conv_bwd_data<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)fwd_smem<128, 0>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_conv_bwd_data<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fwd_smem<64, 0>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_cnn_infer_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+  cudaError_t e = cudaSuccess;
+  auto attr = [&](auto* f, int bytes) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  };
+  attr(k_conv_fwd<256, 0, false>, conv_smem_bytes<256>());
+  attr(k_conv_fwd<256, 0, true>, conv_smem_bytes<256>());
+  attr(k_conv_fwd<128, 0, false>, conv_smem_bytes<128>());
+  attr(k_conv_fwd<64, 1, false>, conv_smem_bytes<64>());
+  attr(k_conv_bwd_data<128, false>, conv_smem_bytes<128>());
+  attr(k_conv_bwd_data<64, true>, conv_smem_bytes<64>());
+  attr(k_conv_bwd_weight<256, false, false>, wgt_smem_bytes<256>());
+  attr(k_conv_bwd_weight<256, true, false>, wgt_smem_bytes<256>());
+  attr(k_conv_bwd_weight<128, false, false>, wgt_smem_bytes<128>());
+  attr(k_conv_bwd_weight<64, false, true>, wgt_smem_bytes<64>());
+  attr(k_cnn_infer_tc, TC_SMEM);
   return e;
 }
 
-// Refresh the tensor-core copy of the conv weights from the BF16 master copy.
+// Refresh the conv weights in the layouts of inference and training from the BF16 copy.
 cudaError_t refresh_wtc(pond_cnn_t n, cudaStream_t st) {
   k_cnn_tc_weights<<<(3 * CONV + 255) / 256, 256, 0, st>>>(n->wbf, n->wtc);
+  k_conv_weights<<<(3 * CONV + 255) / 256, 256, 0, st>>>(n->wbf, n->wf);
   return cudaGetLastError();
 }
 
 void free_net(pond_cnn_t n) {
   for (void* p : {(void*)n->theta, (void*)n->m, (void*)n->v, (void*)n->grad, (void*)n->wbf, (void*)n->z1,
                   (void*)n->z2, (void*)n->z3, (void*)n->h1, (void*)n->h2, (void*)n->a1, (void*)n->a2,
-                  (void*)n->gap, (void*)n->prob, (void*)n->loss, (void*)n->dg, (void*)n->lmean, (void*)n->dz3,
-                  (void*)n->dz2, (void*)n->dz1, (void*)n->part, (void*)n->wtc, (void*)n->tc_err})
+                  (void*)n->gap, (void*)n->prob, (void*)n->loss, (void*)n->dg, (void*)n->lmean, (void*)n->dz2, (void*)n->dz1, (void*)n->part, (void*)n->wtc, (void*)n->wf, (void*)n->tc_err})
     cudaFree(p);
   delete n;
 }
@@ -113,38 +108,42 @@ int load_params(pond_cnn_t n, const float* params) {
   return POND_OK;
 }
 
-__global__ void k_mean(const float* __restrict__ x, int n, float* __restrict__ out) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    float s = 0.f;
-    for (int i = 0; i < n; ++i) s += x[i];
-    *out = s / (float)n;
-  }
-}
+// The patches are the caller's: they need not be aligned for 8-byte loads.
+bool any_align(const __nv_bfloat16* x) { return ((uintptr_t)x & 7) != 0; }
+
+template <int T> dim3 conv_grid(int B) { return dim3((unsigned)((B + spb<T>() - 1) / spb<T>()), 2); }
 
 int forward(pond_cnn_t n, const __nv_bfloat16* x, int B, const int32_t* labels, cudaStream_t st) {
   const __nv_bfloat16* w = n->wbf;
-  k_conv_fwd<256, 0><<<B, THREADS, fwd_smem<256, 0>(), st>>>(x, w, n->theta + CONV, n->z1, n->h1, n->a1, nullptr);
-  k_conv_fwd<128, 0><<<B, THREADS, fwd_smem<128, 0>(), st>>>(n->h1, w + LAYER, n->theta + LAYER + CONV, n->z2,
-                                                             n->h2, n->a2, nullptr);
-  k_conv_fwd<64, 1><<<B, THREADS, fwd_smem<64, 1>(), st>>>(n->h2, w + 2 * LAYER, n->theta + 2 * LAYER + CONV,
-                                                           n->z3, nullptr, nullptr, n->gap);
-  k_head<<<(B + 127) / 128, 128, 0, st>>>(n->gap, w + FC_OFF, n->theta + FC_OFF + NCLS * C, labels, B, n->prob,
-                                          n->loss, n->dg, n->part);
+  const float* th = n->theta;
+  if (any_align(x))
+    k_conv_fwd<256, 0, true><<<conv_grid<256>(B), CT, conv_smem_bytes<256>(), st>>>(x, n->wf, th + CONV, B, n->z1, n->h1,
+                                                                                    n->a1, nullptr);
+  else
+    k_conv_fwd<256, 0, false><<<conv_grid<256>(B), CT, conv_smem_bytes<256>(), st>>>(x, n->wf, th + CONV, B, n->z1, n->h1,
+                                                                                     n->a1, nullptr);
+  k_conv_fwd<128, 0, false><<<conv_grid<128>(B), CT, conv_smem_bytes<128>(), st>>>(
+      n->h1, n->wf + 2 * WCONV, th + LAYER + CONV, B, n->z2, n->h2, n->a2, nullptr);
+  k_conv_fwd<64, 1, false><<<conv_grid<64>(B), CT, conv_smem_bytes<64>(), st>>>(
+      n->h2, n->wf + 4 * WCONV, th + 2 * LAYER + CONV, B, n->z3, nullptr, nullptr, n->gap);
+  k_head<<<(B + 3) / 4, 128, 0, st>>>(n->gap, w + FC_OFF, th + FC_OFF + NCLS * C, labels, B, n->prob, n->loss, n->dg,
+                                      n->part);
   CKC(cudaGetLastError());
   return POND_OK;
 }
 
 int backward(pond_cnn_t n, const __nv_bfloat16* x, int B, cudaStream_t st) {
-  const __nv_bfloat16* w = n->wbf;
-  const long long n3 = (long long)B * C * 64;
-  k_gap_bwd<<<(unsigned)((n3 + 255) / 256), 256, 0, st>>>(n->dg, n->z3, B, 64, n->dz3);
-  k_conv_bwd_weight<64><<<B, THREADS, wgt_smem<64>(), st>>>(n->dz3, n->h2, n->part, 2 * LAYER);
-  k_conv_bwd_data<64><<<B, THREADS, fwd_smem<64, 0>(), st>>>(n->dz3, w + 2 * LAYER, n->a2, n->z2, n->dz2);
-  k_conv_bwd_weight<128><<<B, THREADS, wgt_smem<128>(), st>>>(n->dz2, n->h1, n->part, LAYER);
-  k_conv_bwd_data<128><<<B, THREADS, fwd_smem<128, 0>(), st>>>(n->dz2, w + LAYER, n->a1, n->z1, n->dz1);
-  k_conv_bwd_weight<256><<<B, THREADS, wgt_smem<256>(), st>>>(n->dz1, x, n->part, 0);
-  k_reduce<<<(NPARAM + 255) / 256, 256, 0, st>>>(n->part, B, n->grad);
-  k_mean<<<1, 32, 0, st>>>(n->loss, B, n->lmean);
+  k_conv_bwd_weight<64, false, true><<<B, WT, wgt_smem_bytes<64>(), st>>>(n->z3, n->dg, n->h2, n->part, 2 * LAYER);
+  k_conv_bwd_data<64, true><<<conv_grid<64>(B), CT, conv_smem_bytes<64>(), st>>>(n->z3, n->dg, n->wf + 5 * WCONV, n->a2,
+                                                                                 n->z2, B, n->dz2);
+  k_conv_bwd_weight<128, false, false><<<B, WT, wgt_smem_bytes<128>(), st>>>(n->dz2, nullptr, n->h1, n->part, LAYER);
+  k_conv_bwd_data<128, false><<<conv_grid<128>(B), CT, conv_smem_bytes<128>(), st>>>(n->dz2, nullptr, n->wf + 3 * WCONV, n->a1,
+                                                                                     n->z1, B, n->dz1);
+  if (any_align(x))
+    k_conv_bwd_weight<256, true, false><<<B, WT, wgt_smem_bytes<256>(), st>>>(n->dz1, nullptr, x, n->part, 0);
+  else
+    k_conv_bwd_weight<256, false, false><<<B, WT, wgt_smem_bytes<256>(), st>>>(n->dz1, nullptr, x, n->part, 0);
+  k_reduce<<<REDUCE_BLOCKS + 1, RT, 0, st>>>(n->part, n->loss, B, n->grad, n->lmean);
   CKC(cudaGetLastError());
   return POND_OK;
 }
@@ -189,11 +188,11 @@ int pond_cnn_create(pond_cnn_t* out, const float* init_params, int32_t max_batch
   A(&n->loss, B * 4);
   A(&n->dg, B * C * 4);
   A(&n->lmean, 4);
-  A(&n->dz3, B * C * 64 * 4);
   A(&n->dz2, B * C * 128 * 4);
   A(&n->dz1, B * C * 256 * 4);
   A(&n->part, B * NPARAM * 4);
   A(&n->wtc, WTC_BYTES);
+  A(&n->wf, WF_FLOATS * 4);
   A(&n->tc_err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(n->tc_err, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n->sms, cudaDevAttrMultiProcessorCount, device);
