@@ -145,29 +145,63 @@ __global__ void __launch_bounds__(SORT_THREADS) k_bracket(const float* __restric
   __shared__ int s_lo, s_hi;
   const float* T = series + (size_t)blockIdx.x * stride;
   const int tid = threadIdx.x;
-  for (int i = tid; i < SAMPLE; i += SORT_THREADS) {
+  constexpr int V = SAMPLE / SORT_THREADS;   // element tid + SORT_THREADS u in register u
+  unsigned x[V];
+#pragma unroll
+  for (int u = 0; u < V; ++u) {
     // spread over the row, the place inside each stretch scattered
+    const int i = tid + u * SORT_THREADS;
     const long long a = (long long)i * n / SAMPLE, w = ((long long)(i + 1) * n) / SAMPLE - a;
-    key[i] = f32_key(T[min(n - 1, a + (w > 1 ? (long long)((unsigned)i * 2654435761u % (unsigned)w) : 0))]);
+    x[u] = f32_key(__ldg(T + min(n - 1, a + (w > 1 ? (long long)((unsigned)i * 2654435761u % (unsigned)w) : 0))));
   }
   if (tid == 0) {
     s_lo = -1;
     s_hi = SORT_THREADS;
   }
-  __syncthreads();
-  for (int k = 2; k <= SAMPLE; k <<= 1)
+  // bitonic sort: partners SORT_THREADS apart and more meet in registers, under 32 apart
+  // by shuffles, the 30 steps between through shared memory
+#pragma unroll 1
+  for (int k = 2; k <= SAMPLE; k <<= 1) {
+#pragma unroll 1
     for (int j = k >> 1; j > 0; j >>= 1) {
+      if (j >= SORT_THREADS) {
+        const int d = j / SORT_THREADS, kk = k / SORT_THREADS;
 #pragma unroll
-      for (int u = 0; u < SAMPLE / 2 / SORT_THREADS; ++u) {
-        const int p = tid + u * SORT_THREADS, i = 2 * p - (p & (j - 1)), q = i + j;
-        const unsigned x = key[i], y = key[q];
-        if ((x > y) == ((i & k) == 0)) {
-          key[i] = y;
-          key[q] = x;
+        for (int u = 0; u < V; ++u)
+#pragma unroll
+          for (int e = 1; e < V; e <<= 1)
+            if (e == d && (u & e) == 0) {
+              const unsigned lo = min(x[u], x[u | e]), hi = max(x[u], x[u | e]);
+              const bool up = (u & kk) == 0;
+              x[u] = up ? lo : hi;
+              x[u | e] = up ? hi : lo;
+            }
+      } else {
+        const bool low = (tid & j) == 0;
+        unsigned y[V];
+        if (j >= 32) {
+          __syncthreads();
+#pragma unroll
+          for (int u = 0; u < V; ++u) key[tid + u * SORT_THREADS] = x[u];
+          __syncthreads();
+#pragma unroll
+          for (int u = 0; u < V; ++u) y[u] = key[(tid ^ j) + u * SORT_THREADS];
+        } else {
+#pragma unroll
+          for (int u = 0; u < V; ++u) y[u] = __shfl_xor_sync(0xffffffffu, x[u], j);
+        }
+#pragma unroll
+        for (int u = 0; u < V; ++u) {
+          const bool up = ((tid + u * SORT_THREADS) & k) == 0;
+          x[u] = up == low ? min(x[u], y[u]) : max(x[u], y[u]);
         }
       }
-      __syncthreads();
     }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < V; ++u) key[tid + u * SORT_THREADS] = x[u];
+  __syncthreads();
   const float m = f32_unkey(key[SAMPLE / 2]);
   const float span = f32_unkey(key[SAMPLE / 4 * 3]) - f32_unkey(key[SAMPLE / 4]);   // about two MADs
   // radius of thread tid and the sample values within it
@@ -213,11 +247,24 @@ __global__ void __launch_bounds__(COLLECT_THREADS) k_collect(const float* __rest
   const float* T = series + (size_t)row * stride;
   const Bracket b = br[row];
   const long long i0 = (long long)blockIdx.x * COLLECT;
+  // value u of the thread: sample 4 (tid + COLLECT_THREADS (u / 4)) + u % 4 of the chunk
+  const int left = (int)min(n - i0, (long long)COLLECT);
   float v[COLLECT_V];
+  if (left == COLLECT && ((reinterpret_cast<uintptr_t>(T + i0)) & 15) == 0) {
 #pragma unroll
-  for (int u = 0; u < COLLECT_V; ++u) {
-    const long long i = i0 + tid + u * COLLECT_THREADS;
-    v[u] = i < n ? __ldg(T + i) : __int_as_float(0x7fc00000);
+    for (int u = 0; u < COLLECT_V; u += 4) {
+      const float4 q = __ldg(reinterpret_cast<const float4*>(T + i0) + tid + COLLECT_THREADS * (u / 4));
+      v[u] = q.x;
+      v[u + 1] = q.y;
+      v[u + 2] = q.z;
+      v[u + 3] = q.w;
+    }
+  } else {
+#pragma unroll
+    for (int u = 0; u < COLLECT_V; ++u) {
+      const int i = 4 * (tid + COLLECT_THREADS * (u / 4)) + u % 4;
+      v[u] = i < left ? __ldg(T + i0 + i) : 0.f;
+    }
   }
   // [0] values of C, [1] of D, [2] keys below, [3] values between
   unsigned cnt[4] = {0, 0, 0, 0};
@@ -227,7 +274,7 @@ __global__ void __launch_bounds__(COLLECT_THREADS) k_collect(const float* __rest
   for (int u = 0; u < COLLECT_V; ++u) {
     const float x = v[u];
     const unsigned k = f32_key(x);
-    const bool ok = i0 + tid + u * COLLECT_THREADS < n;
+    const bool ok = 4 * (tid + COLLECT_THREADS * (u / 4)) + u % 4 < left;
     nan |= ok && x != x;
     if (ok) {
       if (k >= b.klo && k <= b.khi) inc |= 1u << u;
@@ -501,29 +548,44 @@ __global__ void __launch_bounds__(SCREEN_WARPS * 32) k_screen(const float* __res
   for (int d = 16; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
   const bool any_odd = __any_sync(0xffffffffu, odd);
   // near the row's end a boxcar that does not fit is summed over what there is: that may
-  // set a bit for nothing, never clear one
-  unsigned mask = 0;
+  // set a bit for nothing, never clear one.  The points are marked one by one only in
+  // warps where some width's largest sum reaches its threshold.
+  float a1[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) a1[i] = a[i];
+  auto grow = [](float (&s)[16], int h) {   // s[i] += the sum that starts h samples on
+    if (h < 16) {
+      float nx[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i)
+        if (i < h) nx[i] = __shfl_down_sync(0xffffffffu, s[i], 1);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) s[i] += i + h < 16 ? s[i + h < 16 ? i + h : 0] : nx[(i + h) & 15];
+    } else {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) s[i] += __shfl_down_sync(0xffffffffu, s[i], h / 16);
+    }
+  };
+  float th[NW];
+  bool reach = any_odd || !(mx <= 1e36f);   // (sums that could overflow: mark by one)
 #pragma unroll
   for (int q = 0; q < NW; ++q) {
-    const int w = 1 << q;
-    if (q > 0) {
-      const int h = w / 2;   // a[i] += the sum that starts h samples on
-      if (h < 16) {
-        float nx[16];
+    if (q > 0) grow(a, 1 << (q - 1));
+    th[q] = z.th[q] - (float)(1 << q) * 9.5367432e-7f * mx;   // w maxabs 2^-20
+    float m = a[0];
 #pragma unroll
-        for (int i = 0; i < 16; ++i)
-          if (i < h) nx[i] = __shfl_down_sync(0xffffffffu, a[i], 1);
+    for (int i = 1; i < 16; ++i) m = fmaxf(m, a[i]);
+    reach |= !(m < th[q]);
+  }
+  unsigned mask = 0;
+  if (__any_sync(0xffffffffu, reach)) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) a[i] += i + h < 16 ? a[i + h < 16 ? i + h : 0] : nx[(i + h) & 15];
-      } else {
+    for (int q = 0; q < NW; ++q) {
+      if (q > 0) grow(a1, 1 << (q - 1));
 #pragma unroll
-        for (int i = 0; i < 16; ++i) a[i] += __shfl_down_sync(0xffffffffu, a[i], h / 16);
-      }
+      for (int i = 0; i < 16; ++i)
+        if (!(a1[i] < th[q])) mask |= 1u << i;
     }
-    const float th = z.th[q] - (float)w * 9.5367432e-7f * mx;   // w maxabs 2^-20
-#pragma unroll
-    for (int i = 0; i < 16; ++i)
-      if (!(a[i] < th)) mask |= 1u << i;
   }
   if (any_odd) mask = 0xffffu;
   const int t_lane = lane * 16;
@@ -591,35 +653,36 @@ __global__ void __launch_bounds__(128) k_suppress_hot(const uint2* __restrict__ 
   if (*nhot > hotcap) return;
   const unsigned m = (unsigned)*nhot;
   const long long words = (n + SCREEN_T - 1) / SCREEN_T * SCREEN_W;   // per row
-  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
+  // a warp per point: lanes over the (row, word) pairs of its neighbourhood
+  const int lane = threadIdx.x & 31;
+  for (unsigned i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < m; i += gridDim.x * blockDim.x >> 5) {
     const double s = S[i];
     if (!(s >= thr)) continue;
-    const int d = (int)hot[i].x, w = W[i];
-    const long long t = hot[i].y;
+    const uint2 p = hot[i];
+    const int d = (int)p.x, w = W[i];
+    const long long t = p.y;
     const int d0 = max(0, d - radius), d1 = min(ndm - 1, d + radius);
-    const long long a = max(0ll, t - w), b = min(n - 1, t + w);
-    bool keep = true;
-    for (int dd = d0; dd <= d1 && keep; ++dd)
-      for (long long q = a / 32; q <= b / 32 && keep; ++q) {
-        const unsigned word = bits[(size_t)dd * words + q];
-        unsigned in = word;
-        if (q == a / 32) in &= 0xffffffffu << (a & 31);
-        if (q == b / 32 && (b & 31) != 31) in &= (2u << (b & 31)) - 1u;
-        if (!in) continue;
-        const unsigned bs = base[(size_t)dd * words + q];
-        for (; in; in &= in - 1) {
-          const int bit = __ffs(in) - 1;
-          const long long tt = q * 32 + bit;
-          if (dd == d && tt == t) continue;
-          const double o = S[bs + __popc(word & ((1u << bit) - 1u))];
-          const bool earlier = dd < d || (dd == d && tt < t);
-          if (o > s || (o == s && earlier)) {
-            keep = false;
-            break;
-          }
-        }
+    const long long a = max(0ll, t - w), b = min(n - 1, t + w), q0 = a / 32;
+    const int per = (int)(b / 32 - q0) + 1, pairs = per * (d1 - d0 + 1);
+    bool lost = false;
+    for (int e = lane; e < pairs && !lost; e += 32) {
+      const int dd = d0 + e / per;
+      const long long q = q0 + e % per;
+      const unsigned word = bits[(size_t)dd * words + q];
+      unsigned in = word;
+      if (q == q0) in &= 0xffffffffu << (a & 31);
+      if (q == b / 32 && (b & 31) != 31) in &= (2u << (b & 31)) - 1u;
+      if (!in) continue;
+      const unsigned bs = base[(size_t)dd * words + q];
+      for (; in && !lost; in &= in - 1) {
+        const int bit = __ffs(in) - 1;
+        const long long tt = q * 32 + bit;
+        if (dd == d && tt == t) continue;
+        const double o = S[bs + __popc(word & ((1u << bit) - 1u))];
+        lost = o > s || (o == s && (dd < d || (dd == d && tt < t)));
       }
-    if (!keep) continue;
+    }
+    if (__any_sync(0xffffffffu, lost) || lane) continue;
     const unsigned long long k = atomicAdd(count, 1ull);
     if ((long long)k < cap) out[k] = make_cand(d, t, w, s);
   }
@@ -837,7 +900,7 @@ int run_boxcar(const float* d_series, int ndm, long long n, long long stride, do
                                                             hot, hotcap, nhot);
     k_exact<<<304, 128, 0, st>>>(d_series, n, stride, mu, sig, hot, hotcap, nhot, sc.at<double>(o_S),
                                  sc.at<unsigned char>(o_W));
-    k_suppress_hot<<<304, 128, 0, st>>>(hot, hotcap, nhot, sc.at<double>(o_S), sc.at<unsigned char>(o_W), bits, base,
+    k_suppress_hot<<<1216, 128, 0, st>>>(hot, hotcap, nhot, sc.at<double>(o_S), sc.at<unsigned char>(o_W), bits, base,
                                         ndm, n, thr, 2, dc, dcap, count);
     if (e == cudaSuccess) e = cudaGetLastError();
     Head h;
