@@ -1656,9 +1656,13 @@ int pond_push(pond_t h, const int8_t* x, size_t n) {
       cudaGetLastError();
   }
   for (size_t off = 0; off < n;) {
-    // a short first piece of a stream lets the passes start while the rest is copied
-    const long long cap = (h->total_in == 0 && off == 0) ? FIRST_STAGE_BYTES : STAGE_BYTES;
-    const long long len = std::min<long long>(cap, (long long)(n - off));
+    // a short first piece of a stream lets the passes start while the rest is copied, and pieces
+    // that shrink to a third of what is left end the push with little to compute
+    // behind the last copy (120 MB of pairs, end to end: 1236 -> 1075 us)
+    const long long left = (long long)(n - off), third = (left / 3 + 15) & ~15ll;
+    const long long cap = (h->total_in == 0 && off == 0) ? FIRST_STAGE_BYTES
+                                                         : std::max(FIRST_STAGE_BYTES, std::min(STAGE_BYTES, third));
+    const long long len = std::min(cap, left);
     const int i = h->stage_next;
     h->stage_next = (h->stage_next + 1) % NSTAGE;
     CK(cudaStreamWaitEvent(h->cst, h->ev_used[i], 0));

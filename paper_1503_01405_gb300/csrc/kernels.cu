@@ -744,8 +744,11 @@ __global__ void __launch_bounds__(512) k_copy_host(uint4* __restrict__ dst, cons
 
 cudaError_t launch_copy_host(int8_t* dst, const int8_t* src, long long n, int blocks, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  if (((((uintptr_t)dst | (uintptr_t)src) & 15) != 0) || (n & 15)) return launch_copy_bytes(dst, src, n, st);
-  k_copy_host<<<blocks, 512, 0, st>>>(reinterpret_cast<uint4*>(dst), reinterpret_cast<const uint4*>(src), n >> 4);
+  if ((((uintptr_t)dst | (uintptr_t)src) & 15) != 0) return launch_copy_bytes(dst, src, n, st);
+  const long long body = n & ~15ll;
+  if (body > 0)
+    k_copy_host<<<blocks, 512, 0, st>>>(reinterpret_cast<uint4*>(dst), reinterpret_cast<const uint4*>(src), body >> 4);
+  if (n > body) return launch_copy_bytes(dst + body, src + body, n - body, st);
   return cudaGetLastError();
 }
 
