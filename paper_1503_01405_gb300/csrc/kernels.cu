@@ -315,9 +315,9 @@ __device__ __forceinline__ void fold_group(int b, float p, int nbins, int b0, do
 }
 
 // Fold channel samples [c0, c1) of P (global index g0 + c) into this warp's
-// histogram; FOLD_WARPS warps share the chunk.  Where there is a window for every warp, whole
-// windows whose phase runs forwards go through fold_window (with fewer, one warp would
-// work through what four share sample by sample: 15,600 samples 5 against 20 us); the
+// histogram; FOLD_WARPS warps share the chunk.  From two windows on, whole windows whose
+// phase runs forwards go through fold_window (a single one would leave to one warp
+// what four share sample by sample: 15,600 samples 5 against 20 us); the
 // rest goes sample by sample, FOLD_U groups of 32 per warp and
 // step (their loads and phases in flight before the groups are added in order).
 // Bin b is kept at entry (b - b0) mod nbins, so a chunk that spans a short cyclic
@@ -345,7 +345,7 @@ __device__ __forceinline__ void fold_chunk(const float* __restrict__ P, long lon
     }
   };
   long long tail = c0;
-  if ((reinterpret_cast<uintptr_t>(P + c0) & 15) == 0 && c1 - c0 >= FOLD_WARPS * FOLD_WIN &&
+  if ((reinterpret_cast<uintptr_t>(P + c0) & 15) == 0 && c1 - c0 >= 2 * FOLD_WIN &&
       rule.forwards(g0 + c0, g0 + c1)) {
     const int nwin = (int)((c1 - c0) / FOLD_WIN);
     for (int i = w; i < nwin; i += FOLD_WARPS) {
@@ -987,6 +987,18 @@ cudaError_t launch_inv_cols_det(const Geom& g, const float2* in, float* P, float
 
 cudaError_t set_kernel_attributes() {
   cudaError_t e = set_attributes_t<false>();
+  // The small kernels that run between and beside the passes take the passes' division of
+  // L1 and shared memory: an SM changes it only when idle, and the CTAs of the next
+  // kernel crowd on the SMs that could (after a carry copy at the default division
+  // a segment's fold took 31.8 us instead of 8.1, four 64-bit-bound CTAs to an SM).  Not
+  // the copy from host memory: its loads in flight need the L1 (end to end 1057 -> 1230 us).
+  auto shared_first = [&](auto* f) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  };
+  shared_first(k_copy_bytes);
+  shared_first(k_decimate_short);
+  shared_first(k_decimate_short_multi);
 #define SET_F(R)                                                                                               \
   {                                                                                                            \
     const RowTile rt{0, 0, 0, row_stride_max(R), row_stride_max(R)};                                           \
@@ -1087,11 +1099,12 @@ cudaError_t launch_fold(const float* P, long long n, long long g0, double inc, i
 // that a pass runs many waves of CTAs), at most 16.
 int fold_slots(const Geom& g) { return (int)std::max<long long>(1, std::min<long long>(16, (1ll << 25) / g.L)); }
 
-// Fold CTAs per segment: whole windows, one per warp and more where 1024 partial rows
-// would not hold them.
+// Fold CTAs per segment: one window per warp, more where the partial rows of all slots
+// would exceed 1024.  Segments of 2^14 samples and less go by sample in CTAs of 1024:
+// a launch of one segment would otherwise be one to four CTAs.
 static long long fold_chunk_len(const Geom& g) {
-  const long long most = std::max(1, std::min(64, 1024 / fold_slots(g)));
-  const long long step = (long long)FOLD_WARPS * FOLD_WIN;
+  const long long most = std::max(1, std::min(MAX_FOLD_PARTS, 1024 / fold_slots(g)));
+  const long long step = g.S_c <= 1 << 14 ? 1024 : (long long)FOLD_WARPS * FOLD_WIN;
   return ((g.S_c + most - 1) / most + step - 1) / step * step;
 }
 int fold_parts_seg(const Geom& g) { return (int)((g.S_c + fold_chunk_len(g) - 1) / fold_chunk_len(g)); }
