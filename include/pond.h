@@ -261,8 +261,8 @@ int pond_plan_ex(pond_t* out, const pond_opts* opts);
  *   the input of the paper's GPU flow (Sec. 3.7, Fig. "gpuflow": the digitised
  *   voltages held on the host are sent to the device's global memory; Sec. 3.1:
  *   the ADC delivers 8-bit real samples of each half of the band).  The data
- *   move to the device in pieces of 128 MiB through two staging buffers while
- *   the passes run: page-locked (pinned, device-mapped) memory by a copy kernel
+ *   move to the device in pieces of 32 to 128 MiB (the first and the
+ *   last of a push are short) through two staging buffers while the passes run: page-locked (pinned, device-mapped) memory by a copy kernel
  *   on 8 CTAs that reads it over the host link, pageable memory by the copy
  *   engines.  The data are copied to the device before the call returns (pinned memory copies
  *   asynchronously, pageable memory through the driver's staging), so x may be
@@ -404,7 +404,9 @@ int pond_voltages(pond_t h, float* out_c, size_t cap, size_t* n_out, int64_t* fi
  *   point within 2 rows and w* samples has a larger s (equal s: the earlier
  *   point in (row, sample) order wins).  A row with sigma = 0 has none.
  *   Candidates go to HOST out[cap], sorted by (trial, index); *n_found gets
- *   their number.  Allocates device scratch (8 + 1 bytes per series sample).
+ *   their number.  Takes device scratch from a pool
+ *   (up to 256 MiB of it stay for the next call): about 3 bytes per series sample, and
+ *   8 + 1 more where more points than expected reach the threshold.
  *   Work runs on cuda_stream and the call waits for it.
  *   Errors: POND_E_ARG, POND_E_OVERRUN (more candidates than cap; *n_found is
  *   the number found), POND_E_OOM, POND_E_CUDA.

@@ -130,8 +130,8 @@ struct Lane {
   std::vector<cudaEvent_t> ev_chain[NSLOT];
   float2* stw = nullptr;                    // stage twiddle tables of R1, R2, Q1, Q2
   const float2 *stwR1 = nullptr, *stwR2 = nullptr, *stwQ1 = nullptr, *stwQ2 = nullptr;
-  // stage-2 twiddles of the 64-values-per-thread FFTs (lengths 512 and more): F2 (R1), Ic (R2)
-  const float2 *wtwR1 = nullptr, *wtwR2 = nullptr;
+  // stage-2 twiddles of the 64-values-per-thread FFTs (lengths 512 and more): F2 (R1), Ic (R2), I2 (Q1), I1 (Q2)
+  const float2 *wtwR1 = nullptr, *wtwR2 = nullptr, *wtwQ1 = nullptr, *wtwQ2 = nullptr;
   float2* tw2buf = nullptr;
   Tw2 tw2L;                                 // exp(-2 pi i e/(2L))
   float2* tw3L = nullptr;                   // three-level exp(-2 pi i e/L)
@@ -377,13 +377,14 @@ int build_trial(pond_t h, const pond_opts* o, Trial* t) {
   const double half = std::fabs(o->bw_mhz) / 2.0;
   const double alpha = K_DM * 1e6 * t->dm / (o->f0_mhz * o->f0_mhz);
   CK(launch_tables(t->anc, t->nanc, t->clog, du, half, o->f0_mhz, alpha, h->sgn, h->st));
-  // single-DM three-pass plans take the chirp from the per-bin table unless the
-  // anchors are asked for: with the table rows prefetched into L2 the fused row
-  // pass then overlaps the other segment stream better (full rate: 116.6k
-  // against 114.5k Msamples/s)
-  if ((o->chirp == POND_CHIRP_TABLE || o->chirp == POND_CHIRP_AUTO) && ln.fused) {
+  // single-DM plans take the chirp from the per-bin table unless the anchors are
+  // asked for: F2f of three-pass plans (with the table rows prefetched into L2 it
+  // overlaps the other segment stream better), and I1 of FP32 four-pass plans with columns
+  // of 512 points and more (the anchors cost it about 25 instructions per bin)
+  const bool four = !h->multi && !ln.fused && !h->tc_terms && inv_cols_table(ln.g);
+  if ((o->chirp == POND_CHIRP_TABLE || o->chirp == POND_CHIRP_AUTO) && (ln.fused || four)) {
     CK(cudaMalloc(&t->ctab, (size_t)ln.g.L * sizeof(float2)));
-    CK(launch_chirp_c64(t->ctab, ln.g, du, half, o->f0_mhz, alpha, h->sgn, h->st));
+    CK(launch_chirp_c64(t->ctab, ln.g, ln.fused, du, half, o->f0_mhz, alpha, h->sgn, h->st));
   }
   return POND_OK;
 }
@@ -421,13 +422,16 @@ int build_lane(pond_t h, Lane* ln) {
   const int n1 = stage_tw_entries(1 << g.logR1), n2 = stage_tw_entries(1 << g.logR2);
   const int n3 = stage_tw_entries(1 << g.logQ1), n4 = stage_tw_entries(1 << g.logQ2);
   const int n5 = wide_tw_entries(1 << g.logR1, false), n6 = wide_tw_entries(1 << g.logR2, false);
-  CK(cudaMalloc(&ln->stw, (size_t)std::max(1, n1 + n2 + n3 + n4 + n5 + n6) * sizeof(float2)));
+  const int n7 = wide_tw_entries(1 << g.logQ1, false), n8 = wide_tw_entries(1 << g.logQ2, false);
+  CK(cudaMalloc(&ln->stw, (size_t)std::max(1, n1 + n2 + n3 + n4 + n5 + n6 + n7 + n8) * sizeof(float2)));
   ln->stwR1 = ln->stw;
   ln->stwR2 = ln->stwR1 + n1;
   ln->stwQ1 = ln->stwR2 + n2;
   ln->stwQ2 = ln->stwQ1 + n3;
   ln->wtwR1 = ln->stwQ2 + n4;
   ln->wtwR2 = ln->wtwR1 + n5;
+  ln->wtwQ1 = ln->wtwR2 + n6;
+  ln->wtwQ2 = ln->wtwQ1 + n7;
   auto nhi = [](int logn) { return logn > TW2_LOG ? (1ll << (logn - TW2_LOG)) : 1ll; };
   const long long total = TW2_LO + nhi(g.logL + 1) + 2 * 768;
   CK(cudaMalloc(&ln->tw2buf, total * sizeof(float2)));
@@ -444,6 +448,8 @@ int build_lane(pond_t h, Lane* ln) {
   CK(launch_stage_tw(const_cast<float2*>(ln->stwQ2), 1 << g.logQ2, h->st));
   CK(launch_wide_tw(const_cast<float2*>(ln->wtwR1), 1 << g.logR1, false, h->st));
   CK(launch_wide_tw(const_cast<float2*>(ln->wtwR2), 1 << g.logR2, false, h->st));
+  CK(launch_wide_tw(const_cast<float2*>(ln->wtwQ1), 1 << g.logQ1, false, h->st));
+  CK(launch_wide_tw(const_cast<float2*>(ln->wtwQ2), 1 << g.logQ2, false, h->st));
   CK(launch_tw3(ln->tw3L, g.logL, -1, h->st));
   CK(launch_tw2(const_cast<float2*>(ln->tw2L.lo), const_cast<float2*>(ln->tw2L.hi), g.logL + 1, -1, h->st));
   CK(launch_tw3(ln->tw3M, g.logM, +1, h->st));
@@ -687,7 +693,7 @@ int run_segments(pond_t h, int li, const SegSrc& src, long long s, int nseg, lon
       CK(launch_fwd_rows(g, bufA, bufB, ln.tw3L, ln.tw2L, ln.stwR1, ln.wtwR1, cs, nseg));
       RC(record(h, 1 + ST_F2, cs));
       // the chirp is applied as I1 loads the spectrum
-      CK(launch_inv_cols(g, bufB, bufA, t.anc, t.clog, ln.stwQ2, cs, nseg));
+      CK(launch_inv_cols(g, bufB, bufA, t.anc, t.clog, t.ctab, ln.stwQ2, ln.wtwQ2, cs, nseg));
       RC(record(h, 1 + ST_I1, cs));
       h->launches += 5;
     }
@@ -697,7 +703,7 @@ int run_segments(pond_t h, int li, const SegSrc& src, long long s, int nseg, lon
       CK(launch_ic(h, ln, bufB, P, ln.part[slot], ln.cnt[slot], vout, h->v_cap, h->v_len, span, cs, nseg));
       RC(record(h, 1 + ST_IC, cs));
     } else {
-      CK(launch_inv_rows(g, bufA, P, vout, h->v_cap, h->v_len, span, ln.tw3M, ln.stwQ1, cs, nseg));
+      CK(launch_inv_rows(g, bufA, P, vout, h->v_cap, h->v_len, span, ln.tw3M, ln.stwQ1, ln.wtwQ1, cs, nseg));
       RC(record(h, 1 + ST_I2, cs));
     }
     // folds run in segment order on their own stream (on st with per-stage timing)
@@ -761,9 +767,9 @@ int run_segments(pond_t h, int li, const SegSrc& src, long long s, int nseg, lon
           if (q == 0) RC(record(h, 1 + ST_IC, cs));
         } else {
           // four passes: every trial's chirp is applied as I1 loads the shared forward spectrum
-          CK(launch_inv_cols(g, bufB, bufA, t.anc, t.clog, ln.stwQ2, cs));
+          CK(launch_inv_cols(g, bufB, bufA, t.anc, t.clog, nullptr, ln.stwQ2, nullptr, cs));
           if (q == 0) RC(record(h, 1 + ST_I1, cs));
-          CK(launch_inv_rows(g, bufA, P, nullptr, 0, 0, span, ln.tw3M, ln.stwQ1, cs));
+          CK(launch_inv_rows(g, bufA, P, nullptr, 0, 0, span, ln.tw3M, ln.stwQ1, ln.wtwQ1, cs));
           if (q == 0) RC(record(h, 1 + ST_I2, cs));
         }
         // each trial's series row is updated in segment order
@@ -982,9 +988,9 @@ int measure_lane(pond_t h, const pond_opts* o, long long nfft, double* t_fwd, do
       if (ce == cudaSuccess)
         ce = launch_ic(h, ln, ln.bufA[0], ln.P[0], ln.part[0], ln.cnt[0], nullptr, 0, 0, span, h->st);
     } else {
-      if (ce == cudaSuccess) ce = launch_inv_cols(g, ln.bufB[0], ln.bufA[0], anc, clog, ln.stwQ2, h->st);
+      if (ce == cudaSuccess) ce = launch_inv_cols(g, ln.bufB[0], ln.bufA[0], anc, clog, nullptr, ln.stwQ2, nullptr, h->st);
       if (ce == cudaSuccess)
-        ce = launch_inv_rows(g, ln.bufA[0], ln.P[0], nullptr, 0, 0, span, ln.tw3M, ln.stwQ1, h->st);
+        ce = launch_inv_rows(g, ln.bufA[0], ln.P[0], nullptr, 0, 0, span, ln.tw3M, ln.stwQ1, ln.wtwQ1, h->st);
     }
     if (ce == cudaSuccess) ce = launch_decimate(ln.P[0], nv, 0, 8, 1, 0, nv / 8, T, C, nv / 8 + 1, h->st);
   }
@@ -1138,16 +1144,19 @@ int time_trials(pond_t h, Lane* ln, int mode, int kt, int split, double* us) {
   // the four-pass form at this split: its own Q1 / Q2 tables
   Geom gq = g;
   float2* tq = nullptr;
-  const float2 *tq1 = nullptr, *tq2 = nullptr;
+  const float2 *tq1 = nullptr, *tq2 = nullptr, *tq1w = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   cudaError_t ce = cudaSuccess;
   if (mode == POND_TRIALS_FOUR_PASS) {
     gq.logQ1 = split;
     gq.logQ2 = g.logM - split;
     const int n1 = stage_tw_entries(1 << gq.logQ1), n2 = stage_tw_entries(1 << gq.logQ2);
-    ce = cudaMalloc(&tq, (size_t)std::max(1, n1 + n2) * sizeof(float2));
+    const int n3 = wide_tw_entries(1 << gq.logQ1, false);
+    ce = cudaMalloc(&tq, (size_t)std::max(1, n1 + n2 + n3) * sizeof(float2));
     tq1 = tq;
     tq2 = tq + n1;
+    tq1w = tq + n1 + n2;
+    if (ce == cudaSuccess) ce = launch_wide_tw(tq + n1 + n2, 1 << gq.logQ1, false, h->st);
     if (ce == cudaSuccess) ce = launch_stage_tw(tq, 1 << gq.logQ1, h->st);
     if (ce == cudaSuccess) ce = launch_stage_tw(tq + n1, 1 << gq.logQ2, h->st);
   }
@@ -1159,9 +1168,9 @@ int time_trials(pond_t h, Lane* ln, int mode, int kt, int split, double* us) {
     if (mode == POND_TRIALS_FOUR_PASS) {
       for (int q = 0; q < nq && ce == cudaSuccess; ++q) {
         const Trial& t = h->trials[ln->trials[q]];
-        ce = launch_inv_cols(gq, ln->bufB[0], ln->bufA[0], t.anc, t.clog, tq2, h->st);
+        ce = launch_inv_cols(gq, ln->bufB[0], ln->bufA[0], t.anc, t.clog, nullptr, tq2, nullptr, h->st);
         if (ce == cudaSuccess)
-          ce = launch_inv_rows(gq, ln->bufA[0], ln->P[0], nullptr, 0, 0, span, ln->tw3M, tq1, h->st);
+          ce = launch_inv_rows(gq, ln->bufA[0], ln->P[0], nullptr, 0, 0, span, ln->tw3M, tq1, tq1w, h->st);
         if (ce == cudaSuccess)
           ce = launch_decimate(ln->P[0], nv, g0, h->dec_num, h->dec_den, j_lo, j_hi - j_lo + 1,
                                h->ts + (size_t)ln->trials[q] * h->ring, h->ts_cnt + (size_t)ln->trials[q] * h->ring,
@@ -1212,9 +1221,12 @@ int use_split(pond_t h, Lane* ln, int q) {
   g.logQ1 = q;
   g.logQ2 = g.logM - q;
   const int n1 = stage_tw_entries(1 << g.logQ1), n2 = stage_tw_entries(1 << g.logQ2);
+  const int n3 = wide_tw_entries(1 << g.logQ1, false);
   cudaFree(ln->stwq);
   ln->stwq = nullptr;
-  CK(cudaMalloc(&ln->stwq, (size_t)std::max(1, n1 + n2) * sizeof(float2)));
+  CK(cudaMalloc(&ln->stwq, (size_t)std::max(1, n1 + n2 + n3) * sizeof(float2)));
+  ln->wtwQ1 = ln->stwq + n1 + n2;
+  CK(launch_wide_tw(ln->stwq + n1 + n2, 1 << g.logQ1, false, h->st));
   ln->stwQ1 = ln->stwq;
   ln->stwQ2 = ln->stwq + n1;
   CK(launch_stage_tw(ln->stwq, 1 << g.logQ1, h->st));

@@ -1,24 +1,11 @@
 // Segment kernels of the coherent-dedispersion path (PONDER Sec. 3.7).
 //
-// One overlap-save segment of N real int8 samples goes through four FFT passes
-// over a spectrum of L = N/2 complex bins (passes.cuh; FP32 instantiations
-// here), then fold and decimation:
+// Overlap-save segments of N real int8 samples go through three or four FFT passes
+// over a spectrum of L = N/2 complex bins (passes.cuh, passes_wide.cuh; FP32
+// instantiations here), several consecutive segments to a launch, then fold and decimation:
 //
-//  F1 k_fwd_cols   : unpack z[n] = x[2n] + i x[2n+1]; length-R2 FFTs down the
-//                    R1 columns n1 of z viewed as [R2][R1]; multiply by
-//                    exp(-2 pi i n1 k2 / L); store in place of the column.
-//  F2 k_fwd_rows   : length-R1 FFTs along the rows k2 (Z[k2 + R2 k1]); rows k2
-//                    and R2-k2 share a CTA so the real-input split
-//                    X[k] = (Z[k] + Z*[L-k])/2 - i e^{-i pi k/L} (Z[k] - Z*[L-k])/2
-//                    is local; multiply by the inverse ISM response (Eq. 4);
-//                    store Y[k] in natural order.
-//  I1 k_inv_cols   : per sub-channel c (bins cM..cM+M-1), inverse length-Q2
-//                    FFTs down the Q1 columns j1, multiply by exp(+2 pi i j1 m2 / M).
-//  I2 k_inv_rows   : inverse length-Q1 FFTs along rows m2 for all sub-channels
-//                    of the same m2 in one CTA: v_c[m2 + Q2 m1] / M, keep the
-//                    valid span n_past <= m < M - n_fut, detect |v|^2 and sum
-//                    over sub-channels into P (and optionally store v).
-//  k_fold_partial / k_fold_merge : deterministic fold of P (FP64 phase).
+//  k_fold_dec      : fold (FP64 phase) and decimation of a launch's segments.
+//  k_fold_partial / k_fold_merge : deterministic fold of a series (FP64 phase).
 //  k_decimate      : deterministic decimation of P into the time series.
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -664,15 +651,16 @@ __global__ void k_make_chirp_table(unsigned* tab, int logR1, int logR2, double d
 }
 
 // The inverse filter of Eq. 4 per bin as FP32 (cos, -sin) of 2 pi phi(k), in
-// F2f's order: row k2, then the position j in a run of 64 columns, then the run c (bin
-// k2 + R2 (64 c + j) at k2 R1 + j NCH + c, NCH = R1 / 64).  phi in FP64 with the
+// F2f's order (runs): row k2, then the position j in a run of 64 columns, then the run c (bin
+// k2 + R2 (64 c + j) at k2 R1 + j NCH + c, NCH = R1 / 64), or the spectrum's (bin k2 + R2 k1 at
+// k2 R1 + k1).  phi in FP64 with the
 // anchors' formula, reduced mod 1, then FP64 sincospi, rounded once to FP32.
-__global__ void k_make_chirp_c64(float2* tab, int logR1, int logR2, double du, double half, double f0, double alpha,
+__global__ void k_make_chirp_c64(float2* tab, int logR1, int logR2, bool runs, double du, double half, double f0, double alpha,
                                  int sgn) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (1ll << (logR1 + logR2))) return;
-  const long long k2 = i >> logR1, e = i & ((1ll << logR1) - 1), nch = 1ll << (logR1 - 6);
-  const long long k1 = ((e & (nch - 1)) << 6) + (e >> (logR1 - 6));
+  const long long k2 = i >> logR1, e = i & ((1ll << logR1) - 1);
+  const long long k1 = runs ? ((e & ((1ll << (logR1 - 6)) - 1)) << 6) + (e >> (logR1 - 6)) : e;
   const double k = (double)(k2 + (k1 << logR2));
   const double f = sgn > 0 ? __dsub_rn(__dmul_rn(k, du), half) : __dsub_rn(half, __dmul_rn(k, du));
   const double g = f0 + f;
@@ -762,10 +750,10 @@ cudaError_t launch_copy_bytes(int8_t* dst, const int8_t* src, long long n, cudaS
   return cudaGetLastError();
 }
 
-cudaError_t launch_chirp_c64(float2* tab, const Geom& g, double du, double half, double f0, double alpha, int sgn,
+cudaError_t launch_chirp_c64(float2* tab, const Geom& g, bool runs, double du, double half, double f0, double alpha, int sgn,
                              cudaStream_t st) {
   const long long n = g.L;
-  k_make_chirp_c64<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(tab, g.logR1, g.logR2, du, half, f0, alpha, sgn);
+  k_make_chirp_c64<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(tab, g.logR1, g.logR2, runs, du, half, f0, alpha, sgn);
   return cudaGetLastError();
 }
 
@@ -862,7 +850,7 @@ cudaError_t launch_fwd_rows_inv(const Geom& g, const float2* in, float2* out, Tw
                                 const float2* wtw, const ChirpAnchor* anc, int clog, const float2* ctab,
                                 cudaStream_t st, int nseg) {
   const RowTile rt = row_tile(g.logR1, g.logR2);
-  const dim3 tiles((unsigned)(g.L / TILE), (unsigned)nseg);
+  const dim3 tiles((unsigned)nseg, (unsigned)(g.L / TILE));   // segments fastest
   switch (1 << g.logR1) {
 #define CASE(R)                                                                                             \
   case R:                                                                                                   \
@@ -1027,6 +1015,15 @@ cudaError_t set_kernel_attributes() {
                              wide_smem_bytes<64, R / 64>());
   SET_W(512) SET_W(1024) SET_W(2048)
 #undef SET_W
+#define SET_I(R)                                                                                                     \
+  if (e == cudaSuccess)                                                                                              \
+    e = cudaFuncSetAttribute(k_inv_cols_w<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, wide_smem_bytes<64, R / 64>()); \
+  if (e == cudaSuccess)                                                                                              \
+    e = cudaFuncSetAttribute(k_inv_rows_w<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, inv_rows_w_smem<R>(0)); \
+  if (e == cudaSuccess)                                                                                              \
+    e = cudaFuncSetAttribute(k_inv_rows_w<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, inv_rows_w_smem<R>(0));
+  SET_I(512) SET_I(1024) SET_I(2048) SET_I(4096)
+#undef SET_I
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_fold_partial, cudaFuncAttributeMaxDynamicSharedMemorySize, fold_smem_bytes(MAX_NBINS));
   if (e == cudaSuccess)
@@ -1045,7 +1042,7 @@ cudaError_t launch_fwd_rows(const Geom& g, const float2* in, float2* out, const 
                             const float2* wtw, cudaStream_t st, int nseg) {
   if (g.tc_terms) return launch_fwd_rows_tc(g, in, out, tw3L, tw2L, tw, st, nseg);
   const RowTile rt = row_tile(g.logR1, g.logR2);
-  const dim3 tiles((unsigned)(g.L / TILE), (unsigned)nseg);
+  const dim3 tiles((unsigned)nseg, (unsigned)(g.L / TILE));   // segments fastest
   if (g.L >= TILE) {
     switch (1 << g.logR1) {
 #define CASE(R)                                                                                             \
@@ -1060,17 +1057,58 @@ cudaError_t launch_fwd_rows(const Geom& g, const float2* in, float2* out, const 
   return launch_fwd_rows_t<false>(g, in, out, tw3L, tw2L, tw, st, nseg);
 }
 
+// Lines of 512 and more points take 64 values per thread (I1 with the chirp from a table;
+// the anchors of batched trials stay with the radix-16 form, which stages them).
 cudaError_t launch_inv_cols(const Geom& g, const float2* in, float2* out, const ChirpAnchor* anc,
-                            int clog, const float2* tw, cudaStream_t st, int nseg) {
-  return g.tc_terms ? launch_inv_cols_tc(g, in, out, anc, clog, tw, st, nseg)
-                    : launch_inv_cols_t<false>(g, in, out, anc, clog, tw, st, nseg);
+                            int clog, const float2* ctab, const float2* tw, const float2* wtw, cudaStream_t st, int nseg) {
+  if (g.tc_terms) return launch_inv_cols_tc(g, in, out, anc, clog, tw, st, nseg);
+  if (ctab) {
+    const dim3 grid((unsigned)nseg, (unsigned)(g.L / TILE));   // segments fastest
+    switch (1 << g.logQ2) {
+#define CASE(R)                                                                                                     \
+  case R:                                                                                                           \
+    k_inv_cols_w<R><<<grid, WIDE_NT, wide_smem_bytes<64, R / 64>(), st>>>(in, out, g.logQ1, g.logM, g.logR1, g.logR2, \
+                                                                          ctab, wtw);                               \
+    return cudaGetLastError();
+      CASE(512) CASE(1024) CASE(2048) CASE(4096)
+#undef CASE
+      default: return cudaErrorInvalidValue;
+    }
+  }
+  return launch_inv_cols_t<false>(g, in, out, anc, clog, tw, st, nseg);
+}
+
+// The table form reads runs of 2^(logQ2 - 6 - s) consecutive bins, s = logR2 - logQ1: from four
+// on (a 32-byte sector) it wins (2^22 bins, runs of four: 44.0 us against 49.1 per segment),
+// at two it does not (2^23 bins: 61.8 us against 45.4).
+bool inv_cols_table(const Geom& g) {
+  return g.L >= TILE && g.logQ2 >= 9 && g.logQ2 <= 12 && g.logQ2 - 6 - (g.logR2 - g.logQ1) >= 2;
 }
 
 cudaError_t launch_inv_rows(const Geom& g, const float2* buf, float* P, float2* vout, long long vstride,
-                            long long vofs, const MSpan& span, const float2* tw3M, const float2* tw,
+                            long long vofs, const MSpan& span, const float2* tw3M, const float2* tw, const float2* wtw,
                             cudaStream_t st, int nseg) {
-  return g.tc_terms ? launch_inv_rows_tc(g, buf, P, vout, vstride, vofs, span, tw3M, tw, st, nseg)
-                    : launch_inv_rows_t<false>(g, buf, P, vout, vstride, vofs, span, tw3M, tw, st, nseg);
+  if (g.tc_terms) return launch_inv_rows_tc(g, buf, P, vout, vstride, vofs, span, tw3M, tw, st, nseg);
+  if (g.L >= TILE) {
+    const dim3 grid((unsigned)(g.L / TILE), (unsigned)nseg);
+    const int lognch = g.logL - g.logM;
+    const float scale = 1.0f / (float)(1u << g.logM);
+    switch (1 << g.logQ1) {
+#define CASE(R)                                                                                                     \
+  case R:                                                                                                           \
+    if (vout)                                                                                                       \
+      k_inv_rows_w<R, true><<<grid, WIDE_NT, inv_rows_w_smem<R>(lognch), st>>>(                                     \
+          buf, P, vout, vstride, vofs, g.logQ2, g.logM, lognch, span, scale, tw3M, wtw);                            \
+    else                                                                                                            \
+      k_inv_rows_w<R, false><<<grid, WIDE_NT, inv_rows_w_smem<R>(lognch), st>>>(                                    \
+          buf, P, vout, vstride, vofs, g.logQ2, g.logM, lognch, span, scale, tw3M, wtw);                            \
+    return cudaGetLastError();
+      CASE(512) CASE(1024) CASE(2048) CASE(4096)
+#undef CASE
+      default: break;
+    }
+  }
+  return launch_inv_rows_t<false>(g, buf, P, vout, vstride, vofs, span, tw3M, tw, st, nseg);
 }
 
 size_t fold_smem_bytes(int nbins) {

@@ -20,11 +20,13 @@
 //                    valid span n_past <= m < M - n_fut, detect |v|^2 and sum
 //                    over sub-channels into P (and optionally store v).
 //
-//  Single-trial FP32 plans with J = M / R2 = 64 run three passes instead
-//  (F1, F2f, Ic): F2f k_fwd_rows_inv is F2 followed, in the same tile, by the
-//  chirp and the length-J first factor of every sub-channel's inverse; Ic
-//  k_inv_cols_det takes the remaining length-R2 factor down the columns, then
-//  discards, detects and sums over sub-channels.  F1 is shared.
+//  FP32 plans with J = M / R2 = 64 run three passes instead (F1, F2f, Ic): F2f
+//  is F2 followed, in the same tile, by the chirp and the length-J first factor of
+//  every sub-channel's inverse (batched trials run that part as a pass of
+//  its own, Ir, on the shared spectrum); Ic takes the remaining length-R2 factor down the
+//  columns, then discards, detects and sums over sub-channels.  F1 is shared.
+//  In FP32, lines of 512 points and more of F2, I1 (with the chirp from a table) and I2,
+//  and F2f, Ir and Ic (R2 of 512 and more) keep 64 values per thread (passes_wide.cuh).
 //  Table lookups (twiddles, chirp anchors) sit in the load phases, where their
 //  latency overlaps the tile's own loads; I1 stages its CTA's chirp anchors in
 //  shared memory when they are few (one anchor covers up to 2^15 bins).
@@ -678,7 +680,9 @@ __global__ void __launch_bounds__(NT, 2) k_inv_cols(const float2* __restrict__ i
 // I2: inverse row FFTs, discard, detect, sum over sub-channels
 // ---------------------------------------------------------------------------
 
-template <int Q1, bool TC>
+// SEGS: several segments, blockIdx.y; one segment has its span in the launch's constants
+// (without the form for one, batched four-pass plans took 40.5 us instead of 36.7 per 2^23 bins).
+template <int Q1, bool TC, bool SEGS>
 __global__ void __launch_bounds__(NT, 2) k_inv_rows(const float2* __restrict__ buf, float* __restrict__ P,
                                                     float2* __restrict__ vout, long long vstride,
                                                     long long vofs, int logQ2, int logM, int nchan,
@@ -686,9 +690,7 @@ __global__ void __launch_bounds__(NT, 2) k_inv_rows(const float2* __restrict__ b
                                                     const float2* __restrict__ tw3M,
                                                     const float2* __restrict__ tw, TcArgs tca) {
   extern __shared__ float2 smem[];
-  buf += ((size_t)blockIdx.y << logM) * nchan;
-  P += (size_t)blockIdx.y << logM;
-  const int m_lo = span.m_lo, m_hi = span.hi(blockIdx.y);
+  if constexpr (SEGS) buf += ((size_t)blockIdx.y << logM) * nchan;
   float2* st3 = smem;                              // [TW3_SN], w = exp(+2 pi i / M)
   float2* stw = smem + TW3_SN;
   float2* sm = stw + stage_table_size(Q1);
@@ -743,6 +745,12 @@ __global__ void __launch_bounds__(NT, 2) k_inv_rows(const float2* __restrict__ b
   // (m = m2_0 + bb + Q2 m1) are shared by G = NT / no thread groups when no < NT;
   // group g sums sub-channels g, g + G, ..., and the G partial sums are added in
   // group order through shared memory.  P = scale^2 sum_c |v_c|^2.
+  int m_hi = span.m_hi;
+  if constexpr (SEGS) {
+    P += (size_t)blockIdx.y << logM;
+    m_hi = span.hi(blockIdx.y);
+  }
+  const int m_lo = span.m_lo;
   const int no = b2 * Q1;
   const float s2 = scale * scale;
   auto sample = [&](int o, int& m, int& bb, int& m1) {
@@ -948,16 +956,29 @@ size_t max_smem_t() {
   return m;
 }
 
+// FP32 rows of 2048 and more points are always k_fwd_rows_w's and k_inv_rows_w's (of 512
+// and 1024 points where the segment has a whole tile).
+template <bool TC>
+constexpr bool rows_here(int R) {
+  return TC || R <= 1024;
+}
+
 template <bool TC>
 cudaError_t set_attributes_t() {
   // I1 adds its staged anchors, F2 its twiddle table (the larger of the two)
   const int max_smem = (int)max_smem_t<TC>() + (ANC_BYTES > TW3_BYTES ? ANC_BYTES : TW3_BYTES);
   cudaError_t e = cudaSuccess;
-#define SET_ATTR(R)                                                                                   \
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fwd_cols<R, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem); \
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fwd_rows<R, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem); \
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_inv_cols<R, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem); \
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_inv_rows<R, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+  auto attr = [&](auto* f) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+  };
+#define SET_ATTR(R)                                                     \
+  attr(k_fwd_cols<R, TC>);                                              \
+  attr(k_inv_cols<R, TC>);                                              \
+  if constexpr (rows_here<TC>(R)) {                                     \
+    attr(k_fwd_rows<R, TC>);                                            \
+    attr(k_inv_rows<R, TC, false>);                                     \
+    if constexpr (!TC) attr(k_inv_rows<R, false, true>);                \
+  }
   POND_FOR_R(SET_ATTR)
 #undef SET_ATTR
   return e;
@@ -984,7 +1005,13 @@ cudaError_t launch_fwd_rows_t(const Geom& g, const float2* in, float2* out, cons
   const int nl = std::min(TILE / R1, R2);
   const dim3 grid((unsigned)(R2 / nl), (unsigned)nseg);
   switch (R1) {
-#define CASE(R) case R: k_fwd_rows<R, TC><<<grid, NT, smem_bytes<R, TC>(nl) + TW3_BYTES, st>>>(in, out, g.logR2, g.logL, tw3L, tw2L, tw, g.tc_fwd); break;
+#define CASE(R)                                                                                                          \
+  case R:                                                                                                                \
+    if constexpr (rows_here<TC>(R)) {                                                                                    \
+      k_fwd_rows<R, TC><<<grid, NT, smem_bytes<R, TC>(nl) + TW3_BYTES, st>>>(in, out, g.logR2, g.logL, tw3L, tw2L, tw, g.tc_fwd); \
+      break;                                                                                                             \
+    }                                                                                                                    \
+    return cudaErrorInvalidValue;
     POND_FOR_R(CASE)
 #undef CASE
     default: return cudaErrorInvalidValue;
@@ -1017,8 +1044,20 @@ cudaError_t launch_inv_rows_t(const Geom& g, const float2* buf, float* P, float2
   const int nl = g.nchan * b2;
   const dim3 grid((unsigned)(Q2 / b2), (unsigned)nseg);
   const float scale = 1.0f / (float)(1u << g.logM);
+  MSpan one = span;
+  one.m_hi = (int)std::min<long long>(span.m_hi, span.m_end);
   switch (Q1) {
-#define CASE(R) case R: k_inv_rows<R, TC><<<grid, NT, smem_bytes<R, TC>(nl) + TW3_BYTES, st>>>(buf, P, vout, vstride, vofs, g.logQ2, g.logM, g.nchan, span, scale, tw3M, tw, g.tc_inv); break;
+#define CASE(R)                                                                                                          \
+  case R:                                                                                                                \
+    if constexpr (rows_here<TC>(R)) {                                                                                    \
+      if (TC || nseg == 1) {                                                                                             \
+        k_inv_rows<R, TC, false><<<grid, NT, smem_bytes<R, TC>(nl) + TW3_BYTES, st>>>(buf, P, vout, vstride, vofs, g.logQ2, g.logM, g.nchan, one, scale, tw3M, tw, g.tc_inv); \
+      } else {                                                                                                           \
+        k_inv_rows<R, TC, !TC><<<grid, NT, smem_bytes<R, TC>(nl) + TW3_BYTES, st>>>(buf, P, vout, vstride, vofs, g.logQ2, g.logM, g.nchan, span, scale, tw3M, tw, g.tc_inv); \
+      }                                                                                                                  \
+      break;                                                                                                             \
+    }                                                                                                                    \
+    return cudaErrorInvalidValue;
     POND_FOR_R(CASE)
 #undef CASE
     default: return cudaErrorInvalidValue;

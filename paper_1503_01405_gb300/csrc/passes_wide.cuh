@@ -10,6 +10,12 @@ namespace pond {
 // 15.97, 228: 103.5 / 16.09, 456: 105.4 / 16.34, none: 116.6 / 16.40.
 constexpr int WIDE_PF = 114;
 
+// Shared memory of a tile of lines of RA x RB.
+template <int RA, int RB>
+constexpr int wide_smem_bytes() {
+  return TILE / (RA * RB) * wide_stride<RA, RB>() * (int)sizeof(float2);
+}
+
 // ---------------------------------------------------------------------------
 // Ic: column pass after F2f: inverse length-R2 FFTs, discard, detect, sum
 // ---------------------------------------------------------------------------
@@ -433,13 +439,17 @@ enum RowMode { ROW_SPECTRUM = 0, ROW_ANCHORS = 1, ROW_TABLE = 2 };
 //   [row][j][c]: consecutive lanes, consecutive words) or the anchors, then the run's
 //   length-64 inverse DFT and blocked store (run_finish).
 // F2f runs two CTAs per SM: at the 168 registers of three, the run's 64 chirp loads are
-// split into batches whose latency shows (101 us per launch at three, 71 at two).
+// split into batches whose latency shows (101 us per launch at three, 71 at two).  F2 runs
+// three for rows of 2048 and 4096 points (33.3 us against 36.9 per 2^23 bins); shorter rows
+// belong to segments of at most 128 tiles, which do not fill the SMs once, and take
+// the registers instead (2^20 bins beside another trial's passes: 8.0 us against 12.2).
 // Bound by instruction issue (43 %) and memory latency in turn.  Full rate, launches of
 // four 2^24-point segments: 56.0 -> 45 us per segment; 24.8 M warp
-// instructions per segment against 31.0 M with radix-16 stages.  blockIdx.y is
-// the segment.
+// instructions per segment against 31.0 M with radix-16 stages.  blockIdx.x is
+// the segment and runs fastest, so the segments of a launch share the chirp table's
+// rows in L2 (launches of four: 215 -> 188 us).
 template <int R1, int MODE>
-__global__ void __launch_bounds__(WIDE_NT, MODE == ROW_SPECTRUM ? 3 : 2)
+__global__ void __launch_bounds__(WIDE_NT, MODE == ROW_SPECTRUM && R1 > 1024 ? 3 : 2)
     k_fwd_rows_w(const float2* __restrict__ in, float2* __restrict__ out, RowTile rt,
                  Tw2 tw2L, const float2* __restrict__ tw,
                  const ChirpAnchor* __restrict__ anc, int clog, const float2* __restrict__ ctab) {
@@ -450,16 +460,18 @@ __global__ void __launch_bounds__(WIDE_NT, MODE == ROW_SPECTRUM ? 3 : 2)
   float2* wbt = sj + 64;                       // [NLR][RB]: exp(-i pi (k2 + 64 R2 c) / L) / 2
   float2* twk = wbt + NLR * RB;                // [NLR][TWK_STR]
   float2* sm = twk + NLR * TWK_STR;   // [NLR * rstr]
-  const int tid = (int)threadIdx.x, R2 = 1 << rt.logR2, np = NLR / 2, q0 = blockIdx.x * np;
-  in += (size_t)blockIdx.y << (LOGR1 + rt.logR2);    // segment blockIdx.y
-  out += (size_t)blockIdx.y << (LOGR1 + rt.logR2);
+  const int tid = (int)threadIdx.x, R2 = 1 << rt.logR2, np = NLR / 2, q0 = blockIdx.y * np;
+  in += (size_t)blockIdx.x << (LOGR1 + rt.logR2);
+  out += (size_t)blockIdx.x << (LOGR1 + rt.logR2);
   auto row_of = [&](int slot) { return f2_line(slot, q0, np, R2); };
-  if (tid < 4 && np == 1 && blockIdx.x + ROW_PF < gridDim.x) {
-    // the two rows of CTA blockIdx.x + ROW_PF (q and its mirror R2 - q), and
-    // with the per-bin chirp table the same rows of the table
-    const int q = q0 + ROW_PF, row = (tid & 1) == 0 ? q : R2 - q;
+  const unsigned ahead = max(1u, (unsigned)ROW_PF / gridDim.x);
+  if (tid < 4 && np == 1 && blockIdx.y + ahead < gridDim.y) {
+    // the two rows of a CTA ROW_PF later (q and its mirror R2 - q), and, once per
+    // launch of several segments, the same rows of the chirp table
+    const int q = q0 + (int)ahead, row = (tid & 1) == 0 ? q : R2 - q;
     if (tid < 2) prefetch_l2(in + ((size_t)row << LOGR1), R1 * (unsigned)sizeof(float2));
-    else if (MODE == ROW_TABLE) prefetch_l2(ctab + ((size_t)row << LOGR1), R1 * (unsigned)sizeof(float2));
+    else if (MODE == ROW_TABLE && blockIdx.x == 0)
+      prefetch_l2(ctab + ((size_t)row << LOGR1), R1 * (unsigned)sizeof(float2));
   }
   {
     // stage 1: butterfly t of the line, inputs n1 = t + RB j.  The table entries of
@@ -544,12 +556,19 @@ __global__ void __launch_bounds__(WIDE_NT, MODE == ROW_SPECTRUM ? 3 : 2)
     return make_float2(fmaf(0.5f, E.x, WO.y), fmaf(0.5f, E.y, -WO.x));
   };
   if constexpr (MODE == ROW_SPECTRUM) {
-#pragma unroll 8
-    for (int u = 0; u < 64; ++u) {
-      const int i = tid + u * WIDE_NT, slot = i >> LOGR1, k1 = i & (R1 - 1), c = k1 >> 6, j = k1 & 63;
-      const Pair q = pair_of(slot, c);
-      const float2 W = cmul(wbt[slot * RB + c], sj[j]);
-      out[((size_t)row_of(slot) << LOGR1) + k1] = split(sm[q.oa + j], sm[j == 0 ? q.ob0 : q.ob - j], W);
+    // lane: bin j of a run; two runs of a row at a time
+    const int j = tid & 63, c0 = tid >> 6;
+    const float2 s = sj[j];
+#pragma unroll 1
+    for (int slot = 0; slot < NLR; ++slot) {
+      const Pair q = pair_of(slot, c0);
+      const float2 *pa = sm + q.oa + j, *pb = sm + q.ob - j + (j == 0 && q.ob0 != q.ob), *wb = wbt + slot * RB + c0;
+      float2* o = out + ((size_t)row_of(slot) << LOGR1) + tid;
+#pragma unroll
+      for (int i = 0; i < RB / 2; ++i) {
+        const float2 Z = i == 0 && j == 0 ? sm[q.ob0] : pb[-130 * i];
+        o[128 * i] = split(pa[130 * i], Z, cmul(wb[2 * i], s));
+      }
     }
   } else {
     const Run r = run_of(rt, tid);
@@ -578,10 +597,167 @@ size_t fwd_rows_smem_bytes(const RowTile& rt) {
          sizeof(float2);
 }
 
-// Shared memory of a tile of nl lines of RA x RB.
-template <int RA, int RB>
-constexpr int wide_smem_bytes() {
-  return TILE / (RA * RB) * wide_stride<RA, RB>() * (int)sizeof(float2);
+// ---------------------------------------------------------------------------
+// I1: per-sub-channel inverse column FFTs (table chirp)
+// ---------------------------------------------------------------------------
+
+// Line (c, j1) holds Y[c M + j1 + Q1 j2], j2 < Q2, read from F2's rows (j2 = j2lo + 2^s
+// j2hi, s = logR2 - logQ1, at row j1 + Q1 j2lo, column c M/R2 + j2hi) and multiplied
+// by the chirp from the plan's per-bin table, which has the spectrum's layout.  The inverse
+// transform goes to natural order c M + j1 + Q1 m2.  Lines are (64, RB); lanes run over the
+// inputs of a line in stage 1 and over the lines in stage 2 (runs of nl values).
+// blockIdx.x is the segment and runs fastest: the segments of a launch share the table in
+// L2.  Bound by memory (three streams of 8 bytes a bin, one of them shared).  Launches of
+// four segments of 2^20 bins: 28.3 us with the chirp from anchors in the radix-16 form, 17.3 here.
+template <int Q2>
+__global__ void __launch_bounds__(WIDE_NT, 2)
+    k_inv_cols_w(const float2* __restrict__ in, float2* __restrict__ out, int logQ1, int logM, int logR1, int logR2,
+                 const float2* __restrict__ ctab, const float2* __restrict__ tw) {
+  constexpr int RA = 64, RB = Q2 / 64, NL = TILE / Q2, BPT = 64 / RB, LOGNL = ilog2c(NL);
+  constexpr int WSTR = wide_stride<RA, RB>();
+  extern __shared__ float2 smem[];
+  in += (size_t)blockIdx.x << (logR1 + logR2);
+  out += (size_t)blockIdx.x << (logR1 + logR2);
+  const int tid = (int)threadIdx.x, l0 = blockIdx.y * NL;
+  {
+    const int l = l0 + tid / RB, t = tid % RB, s = logR2 - logQ1;
+    const unsigned c = (unsigned)l >> logQ1, j1 = (unsigned)l & ((1u << logQ1) - 1), sm = (1u << s) - 1;
+    // offset of input j2: additive over the bits of t and of RB j
+    auto ofs = [&](unsigned j2) { return (j2 >> s) + ((j2 & sm) << (logQ1 + logR1)); };
+    const unsigned o = (c << (logM - logR2)) + (j1 << logR1) + ofs((unsigned)t);
+    const float2 *src = in + o, *ct = ctab + o;
+    float2 v[RA], h[RA];
+#pragma unroll
+    for (int j = 0; j < RA; ++j) v[j] = __ldg(src + ofs((unsigned)(RB * j)));
+#pragma unroll
+    for (int j = 0; j < RA; ++j) h[j] = __ldg(ct + ofs((unsigned)(RB * j)));
+#pragma unroll
+    for (int j = 0; j < RA; ++j) v[j] = cmul(v[j], h[j]);
+    wide_dft<RA, true>(v);
+    float2* dst = smem + (tid / RB) * WSTR + (RA + 1) * t;
+#pragma unroll
+    for (int j = 0; j < RA; ++j) dst[j] = v[j];
+  }
+  __syncthreads();
+  const int b = tid & (NL - 1);
+  const unsigned l = (unsigned)(l0 + b);
+  float2* o = out + ((l >> logQ1) << logM) + (l & ((1u << logQ1) - 1));
+#pragma unroll 1
+  for (int u = 0; u < BPT; ++u) {
+    const int t = (tid >> LOGNL) + u * (WIDE_NT / NL);
+    WideTw<RA, RB> w2;
+    w2.load(tw, t);
+    const float2* src = smem + b * WSTR + t;
+    float2 v[RB];
+#pragma unroll
+    for (int j = 0; j < RB; ++j) v[j] = src[j * (RA + 1)];
+    w2.template dft<true>(v);
+#pragma unroll
+    for (int k = 0; k < RB; ++k) o[(unsigned)(t + RA * k) << logQ1] = v[k];
+  }
 }
+
+// ---------------------------------------------------------------------------
+// I2: inverse row FFTs, discard, detect, sum over sub-channels
+// ---------------------------------------------------------------------------
+
+// Row m2 of sub-channel c: elements j1 < Q1 at c M + m2 Q1 + j1, scaled by
+// exp(+2 pi i j1 m2 / M) as they are loaded (factored as in F2f), inverse length-Q1
+// transform, sample m2 + Q2 m1.  A CTA takes b2 rows m2 of every sub-channel (lines c b2 +
+// bb).  In stage 2 a thread holds outputs m1 = t + 64 k of half of the lines: for
+// each bb it sums |v|^2 over its half of the sub-channels in registers, the halves meet
+// by shuffles, and the b2 Q1 powers go through shared memory so that neighbouring m
+// are stored together.  One sub-channel: the halves take different rows.
+// blockIdx.y is the segment.
+template <int Q1, bool VOUT>
+__global__ void __launch_bounds__(WIDE_NT, 2)
+    k_inv_rows_w(const float2* __restrict__ buf, float* __restrict__ P, float2* __restrict__ vout, long long vstride,
+                 long long vofs, int logQ2, int logM, int lognch, MSpan span, float scale,
+                 const float2* __restrict__ tw3M, const float2* __restrict__ tw) {
+  constexpr int RA = 64, RB = Q1 / 64, NL = TILE / Q1, LOGQ1 = ilog2c(Q1);
+  constexpr int WSTR = wide_stride<RA, RB>();
+  extern __shared__ float2 smem[];
+  float2* st3 = smem;                         // [TW3_SN], w = exp(+2 pi i / M)
+  float2* sm = st3 + TW3_SN;                  // [NL * WSTR]
+  float* pw = reinterpret_cast<float*>(sm + NL * WSTR);   // [b2 Q1]
+  buf += (size_t)blockIdx.y << (logM + lognch);
+  P += (size_t)blockIdx.y << logM;
+  const int m_lo = span.m_lo, m_hi = span.hi(blockIdx.y);
+  const int tid = (int)threadIdx.x, logb2 = ilog2c(NL) - lognch, b2 = 1 << logb2, m2_0 = blockIdx.x << logb2;
+  {
+    const int line = tid / RB, t = tid % RB;
+    const unsigned m2 = (unsigned)(m2_0 + (line & (b2 - 1)));
+    const float2* src = buf + ((size_t)(line >> logb2) << logM) + ((size_t)m2 << LOGQ1) + t;
+    float2 v[RA];
+#pragma unroll
+    for (int j = 0; j < RA; ++j) v[j] = __ldg(src + RB * j);
+    load_tw3(st3, tw3M);
+    __syncthreads();   // st3
+    // j1 = t + RB (8 a + b): w^{8 RB m2 a} inside the first DFT, w^{m2 (t + RB b)} after it
+    float2 wa[7], wb[8];
+#pragma unroll
+    for (int a = 1; a < 8; ++a) wa[a - 1] = tw3(st3, m2 * (unsigned)(8 * RB * a));
+#pragma unroll
+    for (int b = 0; b < 8; ++b) wb[b] = tw3(st3, m2 * (unsigned)(t + RB * b));
+    wide_dft<RA, true>(
+        v, [&](float2 x, int a) { return a == 0 ? x : cmul(x, wa[a - 1]); },
+        [&](float2 x, int b) { return cmul(x, wb[b]); });
+    float2* dst = sm + line * WSTR + (RA + 1) * t;
+#pragma unroll
+    for (int j = 0; j < RA; ++j) dst[j] = v[j];
+  }
+  const int t2 = (tid & 15) | ((tid >> 5) << 4), h = (tid >> 4) & 1;
+  WideTw<RA, RB> w2;
+  w2.load(tw, t2);
+  __syncthreads();
+  const float s2 = scale * scale;
+  // lines of this half: sub-channels c0 .. c0 + nc - 1 of rows bb0 .. bb0 + nb - 1
+  const int nc = lognch ? 1 << (lognch - 1) : 1, c0 = lognch ? h * nc : 0;
+  const int nb = lognch ? b2 : b2 / 2, bb0 = lognch ? 0 : h * nb;
+#pragma unroll 1
+  for (int bb = bb0; bb < bb0 + nb; ++bb) {
+    float p[RB];
+#pragma unroll
+    for (int k = 0; k < RB; ++k) p[k] = 0.f;
+#pragma unroll 1
+    for (int c = c0; c < c0 + nc; ++c) {
+      const float2* src = sm + ((c << logb2) + bb) * WSTR + t2;
+      float2 v[RB];
+#pragma unroll
+      for (int j = 0; j < RB; ++j) v[j] = src[j * (RA + 1)];
+      w2.template dft<true>(v);
+#pragma unroll
+      for (int k = 0; k < RB; ++k) {
+        p[k] = fmaf(v[k].y, v[k].y, fmaf(v[k].x, v[k].x, p[k]));
+        if constexpr (VOUT) {
+          const int m = m2_0 + bb + ((t2 + RA * k) << logQ2);
+          if (m >= m_lo && m < m_hi) vout[(size_t)c * vstride + vofs + (m - m_lo)] = cscale(v[k], scale);
+        }
+      }
+    }
+    if (lognch) {
+#pragma unroll
+      for (int k = 0; k < RB / 2; ++k) {
+        const float mine = h ? p[k + RB / 2] : p[k], other = h ? p[k] : p[k + RB / 2];
+        const float q = mine + __shfl_xor_sync(0xffffffffu, other, 16);
+        pw[((t2 + RA * (k + h * (RB / 2))) << logb2) + bb] = q * s2;
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < RB; ++k) pw[((t2 + RA * k) << logb2) + bb] = p[k] * s2;
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < Q1 << logb2; i += WIDE_NT) {
+    const int m = m2_0 + (i & (b2 - 1)) + ((i >> logb2) << logQ2);
+    if (m >= m_lo && m < m_hi) P[m - m_lo] = pw[i];
+  }
+}
+
+template <int Q1>
+constexpr int inv_rows_w_smem(int lognch) {   // the table, the tile and its powers
+  return TW3_BYTES + wide_smem_bytes<64, Q1 / 64>() + (TILE >> lognch) * (int)sizeof(float);
+}
+
 
 }  // namespace pond

@@ -65,7 +65,7 @@ struct SegIn {
   int pair2 = 0;  // ch 1, both runs 2-byte aligned with even lengths: one complex sample (2 bytes) at a time
 };
 
-// The input of consecutive segments, one per blockIdx.y of a launch.  Byte r of
+// The input of consecutive segments, one per blockIdx.x or .y of a launch.  Byte r of
 // the stream, counted from the first new byte: carry_end[r] for r < 0, d[r] for
 // 0 <= r < avail, zero beyond.  Segment y starts at byte r0 + y step and spans
 // `bytes` bytes; F1 forms its two runs and alignment flags from these.
@@ -140,18 +140,22 @@ int stage_tw_entries(int R);
 // otherwise), radices (64, R / 64) or, last64, (R / 64, 64).
 cudaError_t launch_wide_tw(float2* out, int R, bool last64, cudaStream_t st);
 int wide_tw_entries(int R, bool last64);
-// Passes over nseg consecutive segments per launch (blockIdx.y): segment y reads
-// and writes its own L elements of the buffers (M of P).
+// Passes over nseg consecutive segments per launch: segment y reads
+// and writes its own L elements of the buffers (M of P).  ctab (I1) non-null: the chirp from that
+// table in the spectrum's layout; wtw: launch_wide_tw of the line length.
 cudaError_t launch_fwd_cols(const Geom& g, const SegSrc& in, float2* out, const float2* tw, cudaStream_t st,
                             int nseg = 1);
 // wtw: launch_wide_tw of R1 (rows of 512 and more; tw: the radix-16 tables of the others)
 cudaError_t launch_fwd_rows(const Geom& g, const float2* in, float2* out, const float2* tw3L, Tw2 tw2L, const float2* tw,
                             const float2* wtw, cudaStream_t st, int nseg = 1);
 cudaError_t launch_inv_cols(const Geom& g, const float2* in, float2* out, const ChirpAnchor* anc,
-                            int clog, const float2* tw, cudaStream_t st, int nseg = 1);
+                            int clog, const float2* ctab, const float2* tw, const float2* wtw, cudaStream_t st,
+                            int nseg = 1);
 cudaError_t launch_inv_rows(const Geom& g, const float2* buf, float* P, float2* vout, long long vstride,
-                            long long vofs, const MSpan& span, const float2* tw3M, const float2* tw,
+                            long long vofs, const MSpan& span, const float2* tw3M, const float2* tw, const float2* wtw,
                             cudaStream_t st, int nseg = 1);
+// whether I1 of this geometry can take the chirp from a table (launch_chirp_c64, runs = false)
+bool inv_cols_table(const Geom& g);
 // Fused schedule (F1, F2f, Ic) for single-trial FP32 plans whose geometry has
 // J = M / R2 = FUSED_J; fused_groups = sub-channel groups per m1 in Ic.
 constexpr int FUSED_J = 64;
@@ -161,7 +165,7 @@ int fused_groups(const Geom& g);
 cudaError_t launch_fwd_rows_inv(const Geom& g, const float2* in, float2* out, Tw2 tw2L,
                                 const float2* wtw, const ChirpAnchor* anc, int clog, const float2* ctab,
                                 cudaStream_t st, int nseg = 1);
-cudaError_t launch_chirp_c64(float2* tab, const Geom& g, double du, double half, double f0, double alpha, int sgn,
+cudaError_t launch_chirp_c64(float2* tab, const Geom& g, bool runs, double du, double half, double f0, double alpha, int sgn,
                              cudaStream_t st);
 cudaError_t launch_inv_rows_chirp(const Geom& g, const float2* in, float2* out, Tw2 tw2L,
                                   const ChirpAnchor* anc, int clog, cudaStream_t st);

@@ -48,3 +48,43 @@ def test_three_pass_geometries(geo, bw, volt):
     assert rel(s, r.prof_sum) <= 1e-5 and rel(T, r.ts) <= 1e-5
     if volt:
         assert V.shape == r.voltages.shape and rel(V, r.voltages) <= 1e-5
+
+
+FOUR_PASS = [  # log2 nfft, sub-channels, inverse split Q1 x Q2 (rows of a tile: 8192 / (Q1 sub-channels))
+    (19, 1),    # 512 x 512, sixteen rows
+    (21, 1),    # 1024 x 1024, eight rows
+    (21, 8),    # 512 x 256 (short columns), two rows of every sub-channel
+    (22, 2),    # 1024 x 1024
+    (22, 16),   # 512 x 256, one row of every sub-channel
+    (23, 2),    # 2048 x 1024
+    (24, 1),    # 2048 x 4096
+]
+
+
+@pytest.mark.parametrize("chirp", [pond.POND_CHIRP_AUTO, pond.POND_CHIRP_ANCHORS], ids=["table", "anchors"])
+@pytest.mark.parametrize("geo", FOUR_PASS, ids=lambda g: f"nfft2^{g[0]}_nch{g[1]}")
+def test_four_pass_geometries(geo, chirp):
+    """The four-pass inverse at line lengths of 512 and more, its chirp from the
+    per-bin table or the anchors, powers and voltages."""
+    logn, nchan = geo
+    if chirp == pond.POND_CHIRP_ANCHORS and logn > 22:
+        pytest.skip("the anchor form is covered at the smaller lengths")
+    nfft, dm, period, nbins = 1 << logn, 0.02 * 2 ** (logn - 19), 0.0371, 128
+    p = pcd.make_plan(326.5, -16.0, 32e6, dm, nfft, nchan, nbins, period, 61.44e-6)
+    x = synth.make_stream(synth.StreamSpec(n=nfft + p.S + p.S // 3 + 77, seed=logn + nchan, dm=dm, period=period,
+                                           snr=40.0, duty=0.05, bw=-16.0))
+    out = {}
+    for volt in (False, True):
+        with pond.Engine(326.5, -16.0, 32e6, dm, nfft, nchan, nbins, period, want_voltages=volt, chirp=chirp,
+                         schedule=pond.POND_SCHEDULE_FOUR_PASS) as e:
+            e.push(x)
+            e.flush()
+            out[volt] = e.profile()[:2] + e.timeseries()
+            V = e.voltages()[0] if volt else None
+    for a, b in zip(out[False], out[True]):
+        assert np.array_equal(a, b)
+    s, h, T, C, j0 = out[True]
+    r = pcd.run(p, x, want_voltages=True)
+    assert np.array_equal(h, r.prof_hits) and np.array_equal(C, r.ts_counts) and j0 == r.ts_first
+    assert rel(s, r.prof_sum) <= 1e-5 and rel(T, r.ts) <= 1e-5
+    assert V.shape == r.voltages.shape and rel(V, r.voltages) <= 1e-5
