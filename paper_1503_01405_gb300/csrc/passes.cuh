@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(NT, 2) k_fwd_rows(const float2* __restrict__ i
   const int q0 = blockIdx.x * np;
   if constexpr (!TC && R1 >= 256) {
     if (threadIdx.x < 2 && np == 1 && blockIdx.x + PF_DIST < gridDim.x) {
-      const int q = q0 + PF_DIST, row = threadIdx.x == 0 ? q : R2 - q;   // as in k_fwd_rows_inv
+      const int q = q0 + PF_DIST, row = threadIdx.x == 0 ? q : R2 - q;   // as in k_fwd_rows_w
       prefetch_l2(in + ((size_t)row << LOGR1), R1 * (unsigned)sizeof(float2));
     }
     f2_stage1<R1, LSTR>(in, sm, st3, q0, np, R2, nl);
