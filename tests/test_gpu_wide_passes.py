@@ -58,6 +58,8 @@ FOUR_PASS = [  # log2 nfft, sub-channels, inverse split Q1 x Q2 (rows of a tile:
     (22, 16),   # 512 x 256, one row of every sub-channel
     (23, 2),    # 2048 x 1024
     (24, 1),    # 2048 x 4096
+    (23, 8),    # 1024 x 512, the chirp table read in runs of four bins
+    (23, 32),   # 256 x 512, runs of one bin: no table
 ]
 
 
