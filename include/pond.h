@@ -584,8 +584,8 @@ int pond_stack_rows(int64_t n, int64_t g0, double dt_s, const double* coef, int3
  * rows_cap); *rows and *first_rotation as from pond_stack_rows.  Work is
  * enqueued on cuda_stream (NULL = legacy default stream); the call waits for a
  * check that the phase model runs forwards over the whole series (a
- * non-decreasing (rotation, bin) key, which the stack relies on).  Calls that
- * overlap on the GPU share that check's flag and must be serialised.  Errors:
+ * non-decreasing (rotation, bin) key, which the stack relies on).  Calls from
+ * several threads and streams may overlap.  Errors:
  * as pond_stack_rows, POND_E_OVERRUN (rows > rows_cap; nothing written),
  * POND_E_ARG (the phase model runs backwards; null device pointer with n > 0),
  * POND_E_CUDA. */

@@ -26,7 +26,9 @@
 
 #include <algorithm>
 #include <cmath>
+#include <condition_variable>
 #include <cstdio>
+#include <mutex>
 #include <string>
 
 #include "../../include/pond.h"
@@ -74,7 +76,10 @@ __device__ long long first_at_or_after(const PhaseModel& m, long long lo, long l
   return lo;
 }
 
-__device__ int g_backwards;   // set when K decreases somewhere along the series
+// Flags of the calls in flight, one each: set when K decreases somewhere along that call's
+// series.  Device memory of the module, so a call needs no allocation for its flag.
+constexpr int FLAGS = 64;
+__device__ int g_backwards[FLAGS];
 
 __device__ __forceinline__ double phase_at(const PhaseModel& m, long long i) {
   const double tau = __dsub_rn(__dmul_rn((double)(m.g0 + i), m.dt), m.t_ref);
@@ -91,7 +96,7 @@ __device__ __forceinline__ double phase_at(const PhaseModel& m, long long i) {
 // Elsewhere every sample's key is evaluated and compared with the one before.
 constexpr int RUN = 32, WINDOW = 32 * RUN;
 __global__ void __launch_bounds__(128) k_stack_starts(PhaseModel m, long long n, long long K0, long long nk,
-                                                    unsigned* __restrict__ start) {
+                                                    unsigned* __restrict__ start, int* __restrict__ backwards) {
   const int lane = threadIdx.x & 31;
   const long long warps = gridDim.x * 4ll;
   auto put = [&](long long lo, long long hi, long long i) {   // keys lo .. hi start at sample i
@@ -128,7 +133,7 @@ __global__ void __launch_bounds__(128) k_stack_starts(PhaseModel m, long long n,
         const long long k = key_value(m, i);
         const long long prev = __shfl_up_sync(0xffffffffu, k, 1);
         if (lane > 0 && i0 + lane <= last) {
-          if (k < prev) g_backwards = 1;
+          if (k < prev) *backwards = 1;
           put(prev + 1, k, i);
         }
       }
@@ -137,12 +142,13 @@ __global__ void __launch_bounds__(128) k_stack_starts(PhaseModel m, long long n,
 }
 
 // Cell (row, b) from the table of starts (rows as in k_stack_cells); nothing when the model
-// runs backwards.
+// runs backwards (the table then has entries that no sample wrote).
 __global__ void __launch_bounds__(CELL_THREADS) k_stack_sums(const float* __restrict__ y, long long n, PhaseModel m,
                                                              int mode, long long n_sub, long long q_first,
                                                              long long rows, const unsigned* __restrict__ start,
+                                                             const int* __restrict__ backwards,
                                                              double* __restrict__ S, long long* __restrict__ H) {
-  if (g_backwards) return;
+  if (*backwards) return;
   const long long cell = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (cell >= rows * m.nbins) return;
   const long long row = cell / m.nbins;
@@ -171,10 +177,10 @@ __global__ void __launch_bounds__(CELL_THREADS) k_stack_sums(const float* __rest
   H[cell] = h;
 }
 
-__global__ void k_stack_check(PhaseModel m, long long n) {
+__global__ void k_stack_check(PhaseModel m, long long n, int* __restrict__ backwards) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i + 1 < n;
        i += (long long)gridDim.x * blockDim.x)
-    if (key_value(m, i + 1) < key_value(m, i)) g_backwards = 1;
+    if (key_value(m, i + 1) < key_value(m, i)) *backwards = 1;
 }
 
 // Cell (row, b): ROTATION rows are rotations q_first + row; SUBINT rows are the
@@ -252,6 +258,49 @@ int stack_args(int64_t n, int64_t g0, double dt_s, const double* coef, int32_t n
   return POND_OK;
 }
 
+// A call's own flag, from before its first launch to after it has waited for its stream;
+// waits for another call to end when all are taken.
+class Flag {
+ public:
+  Flag() {
+    std::unique_lock<std::mutex> lock(mu());
+    freed().wait(lock, [] { return taken() != ~0ull; });
+    while ((taken() >> i_) & 1) ++i_;
+    taken() |= 1ull << i_;
+  }
+  ~Flag() {
+    {
+      std::lock_guard<std::mutex> lock(mu());
+      taken() &= ~(1ull << i_);
+    }
+    freed().notify_one();
+  }
+  Flag(const Flag&) = delete;
+  Flag& operator=(const Flag&) = delete;
+  cudaError_t address(int** out) const {
+    void* p = nullptr;
+    const cudaError_t e = cudaGetSymbolAddress(&p, g_backwards);
+    *out = static_cast<int*>(p) + i_;
+    return e;
+  }
+
+ private:
+  static std::mutex& mu() {
+    static std::mutex m;
+    return m;
+  }
+  static std::condition_variable& freed() {
+    static std::condition_variable c;
+    return c;
+  }
+  static unsigned long long& taken() {
+    static unsigned long long t = 0;
+    return t;
+  }
+  static_assert(FLAGS == 64, "one bit per flag");
+  int i_ = 0;
+};
+
 }  // namespace
 
 extern "C" int pond_stack_rows(int64_t n, int64_t g0, double dt_s, const double* coef, int32_t ncoef, double t_ref_s,
@@ -283,9 +332,9 @@ extern "C" int pond_fold_stack(const float* d_series, int64_t n, int64_t g0, dou
   const char* backwards = "pond_fold_stack: the phase model runs backwards over the series";
   const long long cells = *rows * (long long)nbins, q_last = host_rotation(m, n - 1);
   const unsigned cell_blocks = (unsigned)((cells + CELL_THREADS - 1) / CELL_THREADS);
-  void* flag = nullptr;
-  int back = 0;
-  cudaError_t e = cudaGetSymbolAddress(&flag, g_backwards);
+  const Flag own;
+  int *flag = nullptr, back = 0;
+  cudaError_t e = own.address(&flag);
   if (e == cudaSuccess) e = cudaMemsetAsync(flag, 0, sizeof(int), st);
   if (e != cudaSuccess) return failed(e);
   // the table holds a start per key: used while there are at most eight keys per sample
@@ -299,10 +348,10 @@ extern "C" int pond_fold_stack(const float* d_series, int64_t n, int64_t g0, dou
     if (e == cudaSuccess)
       e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&start), (size_t)(nk + 1) * sizeof(unsigned), pool, st);
     if (e != cudaSuccess) return failed(e);
-    k_stack_starts<<<(unsigned)std::min<long long>((n + 4 * WINDOW - 1) / (4 * WINDOW), 4096), 128, 0, st>>>(m, n, K0, nk, start);
+    k_stack_starts<<<(unsigned)std::min<long long>((n + 4 * WINDOW - 1) / (4 * WINDOW), 4096), 128, 0, st>>>(m, n, K0, nk, start, flag);
     if (cells > 0)
       k_stack_sums<<<cell_blocks, CELL_THREADS, 0, st>>>(d_series, n, m, mode, n_sub, *first_rotation, *rows, start,
-                                                         d_sum, reinterpret_cast<long long*>(d_hits));
+                                                         flag, d_sum, reinterpret_cast<long long*>(d_hits));
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(&back, flag, sizeof(int), cudaMemcpyDeviceToHost, st);
     cudaFreeAsync(start, st);
@@ -310,7 +359,7 @@ extern "C" int pond_fold_stack(const float* d_series, int64_t n, int64_t g0, dou
     if (e != cudaSuccess) return failed(e);
     return back ? pond::set_error(POND_E_ARG, backwards) : POND_OK;
   }
-  k_stack_check<<<blocks, 256, 0, st>>>(m, n);
+  k_stack_check<<<blocks, 256, 0, st>>>(m, n, flag);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(&back, flag, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);

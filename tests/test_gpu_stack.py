@@ -61,3 +61,53 @@ def test_stack_key_tables_and_searches(n, period_samples, mode, n_sub):
     S_ref, H_ref, q0_ref = st.stack(y, 5, dt, c, 0.1, nbins, mode, n_sub)
     S, H, q0 = pond.fold_stack(torch.from_numpy(y).cuda(), 5, dt, c, 0.1, nbins, mode, n_sub)
     assert q0 == q0_ref and np.array_equal(H, H_ref) and np.array_equal(S, S_ref)
+
+
+@pytest.mark.parametrize("nbins", [64, 4096], ids=["table", "search"])
+def test_overlapping_calls_keep_their_own_verdict(nbins):
+    """Calls on two streams, one with a model that runs forwards and one whose model
+    turns round: each gets its own answer, the forward one the oracle's bit for bit."""
+    import threading
+
+    import torch
+    n, dt, rounds = 60_001, 1e-3, 100
+    y = np.random.default_rng(3).normal(10.0, 3.0, n).astype(np.float32)
+    per = 40.0 if nbins == 64 else 0.4      # samples per rotation: under and over eight keys per sample
+    good = np.array([0.2, 1.0 / (per * dt), 1e-3])
+    turns = np.array([0.2, 1.0 / (per * dt), -1.0 / (per * dt) / (n * dt)])    # the derivative is zero half-way
+    ref = st.stack(y, 5, dt, good, 0.0, nbins, st.SUBINT, 997)
+    d = torch.from_numpy(y).cuda()
+    torch.cuda.synchronize()
+    bad = []
+
+    def forwards():
+        s = torch.cuda.Stream()
+        for _ in range(rounds):
+            try:
+                S, H, q0 = pond.fold_stack(d, 5, dt, good, 0.0, nbins, st.SUBINT, 997, stream=s)
+            except pond.PondError as e:
+                bad.append(f"refused: {e}")
+                return
+            if q0 != ref[2] or not np.array_equal(H, ref[1]) or not np.array_equal(S, ref[0]):
+                bad.append("wrong stack")
+                return
+
+    def turned():
+        s = torch.cuda.Stream()
+        for _ in range(rounds):
+            try:
+                pond.fold_stack(d, 5, dt, turns, 0.0, nbins, st.SUBINT, 997, stream=s)
+            except pond.PondError as e:
+                if e.name != "ARG":
+                    bad.append(str(e))
+                    return
+            else:
+                bad.append("a model that turns round was accepted")
+                return
+
+    threads = [threading.Thread(target=f) for f in (forwards, turned, forwards, turned)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad, bad
