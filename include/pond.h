@@ -585,7 +585,9 @@ int pond_stack_rows(int64_t n, int64_t g0, double dt_s, const double* coef, int3
  * enqueued on cuda_stream (NULL = legacy default stream); the call waits for a
  * check that the phase model runs forwards over the whole series (a
  * non-decreasing (rotation, bin) key, which the stack relies on).  Calls from
- * several threads and streams may overlap.  Errors:
+ * several threads and streams may overlap.  Up to eight (rotation, bin) keys per
+ * sample a call is faster with 4 bytes of scratch per key, from the pool of
+ * pond_boxcar; it does without where they cannot be had.  Errors:
  * as pond_stack_rows, POND_E_OVERRUN (rows > rows_cap; nothing written),
  * POND_E_ARG (the phase model runs backwards; null device pointer with n > 0),
  * POND_E_CUDA. */

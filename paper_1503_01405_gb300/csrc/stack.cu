@@ -337,17 +337,27 @@ extern "C" int pond_fold_stack(const float* d_series, int64_t n, int64_t g0, dou
   cudaError_t e = own.address(&flag);
   if (e == cudaSuccess) e = cudaMemsetAsync(flag, 0, sizeof(int), st);
   if (e != cudaSuccess) return failed(e);
-  // the table holds a start per key: used while there are at most eight keys per sample
+  // the table holds a start per key (4 bytes of scratch): used while there are at most eight keys
+  // per sample and the scratch can be had; the cells search without one
   const double keys = ((double)q_last - (double)*first_rotation + 1.0) * nbins;
   const unsigned blocks = (unsigned)std::min<long long>((n + 255) / 256, 4096);
+  unsigned* start = nullptr;
+  long long nk = 0;
   if (q_last >= *first_rotation && keys <= 8.0 * (double)n + 65536.0 && n < (1ll << 32)) {
-    const long long nk = (q_last - *first_rotation + 1) * nbins, K0 = *first_rotation * (long long)nbins;
-    unsigned* start = nullptr;
+    nk = (q_last - *first_rotation + 1) * nbins;
     cudaMemPool_t pool = nullptr;
     e = pond::scratch_pool(&pool);
     if (e == cudaSuccess)
       e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&start), (size_t)(nk + 1) * sizeof(unsigned), pool, st);
-    if (e != cudaSuccess) return failed(e);
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      start = nullptr;
+    } else if (e != cudaSuccess) {
+      return failed(e);
+    }
+  }
+  if (start) {
+    const long long K0 = *first_rotation * (long long)nbins;
     k_stack_starts<<<(unsigned)std::min<long long>((n + 4 * WINDOW - 1) / (4 * WINDOW), 4096), 128, 0, st>>>(m, n, K0, nk, start, flag);
     if (cells > 0)
       k_stack_sums<<<cell_blocks, CELL_THREADS, 0, st>>>(d_series, n, m, mode, n_sub, *first_rotation, *rows, start,

@@ -1,0 +1,150 @@
+"""Calls at scratch limits: buffers that only make a call faster are done without when
+device memory is short, and results stay the same.
+
+The shortage is made on the host: a preloaded library stands in for the runtime's
+allocation calls of a child process and answers with an out-of-memory error once
+the bytes it has handed out would exceed a budget."""
+import ctypes
+import os
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+pytestmark = pytest.mark.gpu
+
+SHIM = r"""
+#define _GNU_SOURCE
+#include <dlfcn.h>
+#include <pthread.h>
+#include <stddef.h>
+static pthread_mutex_t mu = PTHREAD_MUTEX_INITIALIZER;
+static int armed;
+static size_t budget, live, peak;
+static struct { void *p; size_t n; } held[8192];
+static int nheld;
+static void *real(const char *name) {
+  static void *lib;
+  if (!lib) lib = dlopen("libcudart.so.13", RTLD_LAZY);
+  return dlsym(lib ? lib : RTLD_NEXT, name);
+}
+void shim_arm(size_t n) { pthread_mutex_lock(&mu); armed = 1; budget = n; live = peak = 0; nheld = 0; pthread_mutex_unlock(&mu); }
+size_t shim_disarm(void) { armed = 0; return peak; }
+static int fits(size_t n) { return !armed || (live + n <= budget && nheld < 8192); }
+static void took(void *p, size_t n) {
+  if (!armed) return;
+  held[nheld].p = p;
+  held[nheld++].n = n;
+  live += n;
+  if (live > peak) peak = live;
+}
+static void gave(void *p) {
+  pthread_mutex_lock(&mu);
+  if (armed && p)
+    for (int i = 0; i < nheld; ++i)
+      if (held[i].p == p) {
+        live -= held[i].n;
+        held[i] = held[--nheld];
+        break;
+      }
+  pthread_mutex_unlock(&mu);
+}
+int cudaMalloc(void **p, size_t n) {
+  int (*f)(void **, size_t) = real("cudaMalloc"), e;
+  pthread_mutex_lock(&mu);
+  if (!fits(n)) {
+    f(p, (size_t)1 << 60);   /* sets the runtime's last error */
+    *p = 0;
+    e = 2;
+  } else if (!(e = f(p, n))) took(*p, n);
+  pthread_mutex_unlock(&mu);
+  return e;
+}
+int cudaMallocFromPoolAsync(void **p, size_t n, void *pool, void *st) {
+  int (*f)(void **, size_t, void *, void *) = real("cudaMallocFromPoolAsync"), e;
+  pthread_mutex_lock(&mu);
+  if (!fits(n)) {
+    f(p, (size_t)1 << 60, pool, st);
+    *p = 0;
+    e = 2;
+  } else if (!(e = f(p, n, pool, st))) took(*p, n);
+  pthread_mutex_unlock(&mu);
+  return e;
+}
+int cudaFree(void *p) { gave(p); return ((int (*)(void *))real("cudaFree"))(p); }
+int cudaFreeAsync(void *p, void *st) { gave(p); return ((int (*)(void *, void *))real("cudaFreeAsync"))(p, st); }
+int cudaMemGetInfo(size_t *fr, size_t *tot) {
+  int e = ((int (*)(size_t *, size_t *))real("cudaMemGetInfo"))(fr, tot);
+  if (!e && armed && *fr > budget - live) *fr = budget - live;
+  return e;
+}
+"""
+NO_LIMIT = 1 << 50
+
+
+@pytest.fixture(scope="module")
+def shim(tmp_path_factory):
+    d = tmp_path_factory.mktemp("shim")
+    (d / "shim.c").write_text(SHIM)
+    so = d / "shim.so"
+    subprocess.run(["gcc", "-shared", "-fPIC", "-O1", "-w", "-o", str(so), str(d / "shim.c"), "-ldl", "-lpthread"],
+                   check=True)
+    from paper_1503_01405_gb300 import build
+    build.build()
+    return str(so)
+
+
+@pytest.mark.parametrize("case", ["stack_without_table"])
+def test_short_of_memory(shim, case):
+    r = subprocess.run([sys.executable, os.path.abspath(__file__), case], cwd=ROOT, text=True, capture_output=True,
+                       timeout=300, env=dict(os.environ, LD_PRELOAD=shim, SHIM=shim))
+    assert r.returncode == 0 and "ok" in r.stdout.split(), r.stdout[-2000:] + r.stderr[-2000:]
+
+
+class Budget:
+    """Allocations of the block may hold n bytes at most; .peak afterwards."""
+    lib = None
+
+    def __init__(self, n=NO_LIMIT):
+        if Budget.lib is None:
+            Budget.lib = ctypes.CDLL(os.environ["SHIM"])
+            Budget.lib.shim_disarm.restype = ctypes.c_size_t
+        self.n = n
+
+    def __enter__(self):
+        Budget.lib.shim_arm(ctypes.c_size_t(self.n))
+        return self
+
+    def __exit__(self, *a):
+        self.peak = Budget.lib.shim_disarm()
+
+
+def stack_without_table():
+    """pond_fold_stack needs no memory of its own: without the table of key starts the
+    cells search, in the same order."""
+    import torch
+
+    from paper_1503_01405_gb300 import pond
+    n, dt, nbins = 200_003, 1e-3, 64
+    c = np.array([0.2, 100.0, 1e-3])         # ten samples a rotation: 6.4 keys a sample
+    y = torch.from_numpy(np.random.default_rng(1).normal(10.0, 3.0, n).astype(np.float32)).cuda()
+    S_ref, H_ref, q_ref = pond.fold_stack(y, 3, dt, c, 0.0, nbins)
+    S = torch.zeros(S_ref.shape, dtype=torch.float64, device="cuda")
+    H = torch.zeros(H_ref.shape, dtype=torch.int64, device="cuda")
+    rows, q0 = ctypes.c_int64(), ctypes.c_int64()
+    torch.cuda.synchronize()
+    with Budget(0):
+        rc = pond.lib().pond_fold_stack(y.data_ptr(), n, 3, dt, c.ctypes.data, 3, 0.0, nbins, 0, 0, S.data_ptr(),
+                                        H.data_ptr(), S.shape[0], ctypes.byref(rows), ctypes.byref(q0), None)
+    torch.cuda.synchronize()
+    assert rc == pond.POND_OK, pond.lib().pond_last_error()
+    assert q0.value == q_ref and np.array_equal(S.cpu().numpy(), S_ref) and np.array_equal(H.cpu().numpy(), H_ref)
+
+
+if __name__ == "__main__":
+    sys.path.insert(0, ROOT)
+    globals()[sys.argv[1]]()
+    print("ok")
