@@ -1117,13 +1117,38 @@ int alloc_multi(Lane* ln, int kt) {
   return POND_OK;
 }
 
+// Room for a buffer that a plan can do without: a quarter of the free device memory beyond the
+// 1 GiB left for what the plan still has to allocate (rings, staging, voltages).
+size_t spare_bytes() {
+  constexpr size_t KEEP = 1ull << 30;
+  size_t free_b = 0, total = 0;
+  if (cudaMemGetInfo(&free_b, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return free_b > KEEP ? (free_b - KEEP) / 4 : 0;
+}
+
+// cudaMalloc of such a buffer; *p is null when there is no room.
+template <class T>
+cudaError_t malloc_spare(T** p, size_t bytes) {
+  *p = nullptr;
+  if (bytes > spare_bytes()) return cudaSuccess;
+  const cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaErrorMemoryAllocation) return e;
+  cudaGetLastError();
+  *p = nullptr;
+  return cudaSuccess;
+}
+
 // The anchor form's phase words for every trial of the lane, while they stay below
-// WORDS_MAX bytes (otherwise the row pass evaluates the anchors per bin).
+// WORDS_MAX bytes and there is room (otherwise the row pass evaluates the anchors per bin).
 constexpr size_t WORDS_MAX = 8ull << 30;
 int make_words(pond_t h, Lane* ln) {
   const size_t n = (size_t)ln->g.L * ln->trials.size();
   if (n * sizeof(unsigned) > WORDS_MAX) return POND_OK;
-  CK(cudaMalloc(&ln->words, n * sizeof(unsigned)));
+  CK(malloc_spare(&ln->words, n * sizeof(unsigned)));
+  if (!ln->words) return POND_OK;
   for (size_t q = 0; q < ln->trials.size(); ++q) {
     const Trial& t = h->trials[ln->trials[q]];
     CK(launch_chirp_words(ln->words + q * ln->g.L, ln->g, t.anc, t.clog, h->st));
@@ -1275,9 +1300,7 @@ int apply_tune(pond_t h, Lane* ln, const TrialTune& t) {
   ln->cand_split = t.csplit;
   ln->cand_us = t.cus;
   if (t.mode == POND_TRIALS_FOUR_PASS) RC(use_split(h, ln, t.split));
-  if (t.mode == POND_TRIALS_MULTI_ANCHOR) {
-    if (!ln->words) RC(make_words(h, ln));
-  } else {
+  if (t.mode != POND_TRIALS_MULTI_ANCHOR) {
     cudaFree(ln->words);
     ln->words = nullptr;
   }
@@ -1285,7 +1308,8 @@ int apply_tune(pond_t h, Lane* ln, const TrialTune& t) {
     free_multi(ln);
     return POND_OK;
   }
-  return t.kt != ln->kt || !ln->bufT[0] ? alloc_multi(ln, t.kt) : POND_OK;
+  if (t.kt != ln->kt || !ln->bufT[0]) RC(alloc_multi(ln, t.kt));
+  return t.mode == POND_TRIALS_MULTI_ANCHOR && !ln->words ? make_words(h, ln) : POND_OK;
 }
 
 // Choose how the lane runs its trials (after its trials' anchors exist and the
@@ -1340,8 +1364,8 @@ int setup_trials(pond_t h, const pond_opts* o, Lane* ln) {
     // the requested form (the table form only where the DMs allow it), else the table form where possible
     if (!multi_ok) return POND_OK;
     ln->mode = (req == POND_TRIALS_MULTI_ANCHOR) ? POND_TRIALS_MULTI_ANCHOR : best_multi;
-    if (ln->mode == POND_TRIALS_MULTI_ANCHOR) RC(make_words(h, ln));
-    return alloc_multi(ln, kt_req ? kt_req : std::min(32, ntr));
+    RC(alloc_multi(ln, kt_req ? kt_req : std::min(32, ntr)));
+    return ln->mode == POND_TRIALS_MULTI_ANCHOR ? make_words(h, ln) : POND_OK;
   }
   // autotune: time every candidate on this lane, keep the fastest per trial
   struct Cand {

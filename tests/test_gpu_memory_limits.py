@@ -97,7 +97,7 @@ def shim(tmp_path_factory):
     return str(so)
 
 
-@pytest.mark.parametrize("case", ["stack_without_table"])
+@pytest.mark.parametrize("case", ["stack_without_table", "trials_without_words"])
 def test_short_of_memory(shim, case):
     r = subprocess.run([sys.executable, os.path.abspath(__file__), case], cwd=ROOT, text=True, capture_output=True,
                        timeout=300, env=dict(os.environ, LD_PRELOAD=shim, SHIM=shim))
@@ -142,6 +142,47 @@ def stack_without_table():
     torch.cuda.synchronize()
     assert rc == pond.POND_OK, pond.lib().pond_last_error()
     assert q0.value == q_ref and np.array_equal(S.cpu().numpy(), S_ref) and np.array_equal(H.cpu().numpy(), H_ref)
+
+
+def samples(n):
+    import torch
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    x = torch.randn(n, generator=g, device="cuda").mul_(20.0).clamp_(-127, 127).to(torch.int8)
+    torch.cuda.synchronize()
+    return x
+
+
+def engine(x, budget, *args, **kw):
+    """Outputs of one stream through an engine made under the budget, and the peak of its allocations."""
+    from paper_1503_01405_gb300 import pond
+    with Budget(budget) as b:
+        with pond.Engine(326.5, 16.0, 32e6, *args, **kw) as e:
+            e.push_tensor(x)
+            e.flush()
+            out = list(e.timeseries())
+            if not kw.get("dms"):
+                out += e.profile()[:2]
+    return out, b.peak
+
+
+def same(a, b):
+    return len(a) == len(b) and all(np.array_equal(p, q) for p, q in zip(a, b))
+
+
+def trials_without_words():
+    """The anchor form over several trials per launch without its per-trial phase words
+    (blocks of three and of two trials): the same series."""
+    from paper_1503_01405_gb300 import pond
+    nfft, ndm = 1 << 20, 8
+    x = samples(5 * nfft + 1234)
+    args = (0.0, nfft, 16, 1, 1.0)
+    kw = dict(t_dec=32e-6, dms=[0.31 + 0.0137 * d ** 1.3 for d in range(ndm)],
+              trial_mode=pond.POND_TRIALS_MULTI_ANCHOR, trials_per_launch=3)
+    ref, peak = engine(x, NO_LIMIT, *args, **kw)
+    words = ndm * (nfft // 2) * 4
+    out, less = engine(x, peak - words // 2, *args, **kw)
+    assert less <= peak - words and same(out, ref)
 
 
 if __name__ == "__main__":
