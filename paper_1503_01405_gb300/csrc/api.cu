@@ -367,6 +367,30 @@ int anchor_log(const pond_opts* o, long long nfft, double dm) {
   return clog;
 }
 
+// Room for a buffer that a plan can do without: a quarter of the free device memory beyond the
+// 1 GiB left for what the plan still has to allocate (rings, staging, voltages).
+size_t spare_bytes() {
+  constexpr size_t KEEP = 1ull << 30;
+  size_t free_b = 0, total = 0;
+  if (cudaMemGetInfo(&free_b, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return free_b > KEEP ? (free_b - KEEP) / 4 : 0;
+}
+
+// cudaMalloc of such a buffer; *p is null when there is no room.
+template <class T>
+cudaError_t malloc_spare(T** p, size_t bytes) {
+  *p = nullptr;
+  if (bytes > spare_bytes()) return cudaSuccess;
+  const cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaErrorMemoryAllocation) return e;
+  cudaGetLastError();
+  *p = nullptr;
+  return cudaSuccess;
+}
+
 int build_trial(pond_t h, const pond_opts* o, Trial* t) {
   const Lane& ln = h->lanes[t->lane];
   const long long nfft = ln.g.N;
@@ -389,6 +413,40 @@ int build_trial(pond_t h, const pond_opts* o, Trial* t) {
   return POND_OK;
 }
 
+// The lane's per-slot buffers, of ln->group segments each (G: sub-channel groups of the
+// column pass that leave partials).
+cudaError_t alloc_slots(Lane* ln, int G) {
+  const Geom& g = ln->g;
+  const size_t K = (size_t)ln->group;
+  cudaError_t e = cudaSuccess;
+  auto take = [&](auto** p, size_t n) {
+    if (e == cudaSuccess) e = cudaMalloc(p, n * sizeof(**p));
+  };
+  for (int k = 0; k < NSLOT; ++k) {
+    take(&ln->bufA[k], K * g.L);
+    take(&ln->bufB[k], K * g.L);
+    take(&ln->P[k], K * g.M);
+    if (G) {
+      take(&ln->part[k], K * G * g.M);
+      take(&ln->cnt[k], K * FUSED_J);
+    }
+  }
+  return e;
+}
+
+void free_slots(Lane* ln) {
+  for (int k = 0; k < NSLOT; ++k) {
+    cudaFree(ln->bufA[k]);
+    cudaFree(ln->bufB[k]);
+    cudaFree(ln->P[k]);
+    cudaFree(ln->part[k]);
+    cudaFree(ln->cnt[k]);
+    ln->bufA[k] = ln->bufB[k] = nullptr;
+    ln->P[k] = ln->part[k] = nullptr;
+    ln->cnt[k] = nullptr;
+  }
+}
+
 int build_lane(pond_t h, Lane* ln) {
   if (h->tc_terms) {
     ln->g.tc_terms = h->tc_terms;
@@ -407,18 +465,23 @@ int build_lane(pond_t h, Lane* ln) {
   // CTAs and a short one a fraction of a wave, so a launch of each pass over a group
   // of segments fills the chip where one per segment drains it.  Kept voltages
   // and per-stage timing take one segment at a time, as do the tensor-core forms.
-  ln->group = h->multi || h->timing || h->want_voltages || h->tc_terms ? 1 : fold_slots(g);
-  const size_t K = (size_t)ln->group;
-  for (int k = 0; k < NSLOT; ++k) {
-    CK(cudaMalloc(&ln->bufA[k], K * g.L * sizeof(float2)));
-    CK(cudaMalloc(&ln->bufB[k], K * g.L * sizeof(float2)));
-    CK(cudaMalloc(&ln->P[k], K * g.M * sizeof(float)));
-    if ((ln->fused || ln->fused_multi) && fused_groups(g) > 1) {
-      CK(cudaMalloc(&ln->part[k], K * fused_groups(g) * g.M * sizeof(float)));
-      CK(cudaMalloc(&ln->cnt[k], K * FUSED_J * sizeof(int)));
-      CK(cudaMemsetAsync(ln->cnt[k], 0, K * FUSED_J * sizeof(int), h->st));
-    }
+  // Groups of up to fold_slots segments while their buffers fit the room to spare.
+  const int G = (ln->fused || ln->fused_multi) && fused_groups(g) > 1 ? fused_groups(g) : 0;
+  ln->group = 1;
+  if (!h->multi && !h->timing && !h->want_voltages && !h->tc_terms) {
+    const size_t per = NSLOT * (2 * g.L * sizeof(float2) + (1 + G) * g.M * sizeof(float));
+    ln->group = (int)std::max<size_t>(1, std::min<size_t>(fold_slots(g), spare_bytes() / per));
   }
+  for (;; ln->group /= 2) {
+    const cudaError_t e = alloc_slots(ln, G);
+    if (e == cudaSuccess) break;
+    free_slots(ln);
+    if (e != cudaErrorMemoryAllocation || ln->group == 1) CK(e);
+    cudaGetLastError();
+  }
+  if (G)
+    for (int k = 0; k < NSLOT; ++k)
+      CK(cudaMemsetAsync(ln->cnt[k], 0, (size_t)ln->group * FUSED_J * sizeof(int), h->st));
   const int n1 = stage_tw_entries(1 << g.logR1), n2 = stage_tw_entries(1 << g.logR2);
   const int n3 = stage_tw_entries(1 << g.logQ1), n4 = stage_tw_entries(1 << g.logQ2);
   const int n5 = wide_tw_entries(1 << g.logR1, false), n6 = wide_tw_entries(1 << g.logR2, false);
@@ -457,12 +520,8 @@ int build_lane(pond_t h, Lane* ln) {
 }
 
 void free_lane(Lane* ln) {
+  free_slots(ln);
   for (int k = 0; k < NSLOT; ++k) {
-    cudaFree(ln->bufA[k]);
-    cudaFree(ln->bufB[k]);
-    cudaFree(ln->P[k]);
-    cudaFree(ln->part[k]);
-    cudaFree(ln->cnt[k]);
     cudaFree(ln->bufT[k]);
     cudaFree(ln->Pm[k]);
     cudaFree(ln->partm[k]);
@@ -1115,30 +1174,6 @@ int alloc_multi(Lane* ln, int kt) {
   }
   ln->kt = kt;
   return POND_OK;
-}
-
-// Room for a buffer that a plan can do without: a quarter of the free device memory beyond the
-// 1 GiB left for what the plan still has to allocate (rings, staging, voltages).
-size_t spare_bytes() {
-  constexpr size_t KEEP = 1ull << 30;
-  size_t free_b = 0, total = 0;
-  if (cudaMemGetInfo(&free_b, &total) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  return free_b > KEEP ? (free_b - KEEP) / 4 : 0;
-}
-
-// cudaMalloc of such a buffer; *p is null when there is no room.
-template <class T>
-cudaError_t malloc_spare(T** p, size_t bytes) {
-  *p = nullptr;
-  if (bytes > spare_bytes()) return cudaSuccess;
-  const cudaError_t e = cudaMalloc(p, bytes);
-  if (e != cudaErrorMemoryAllocation) return e;
-  cudaGetLastError();
-  *p = nullptr;
-  return cudaSuccess;
 }
 
 // The anchor form's phase words for every trial of the lane, while they stay below

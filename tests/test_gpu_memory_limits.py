@@ -97,7 +97,7 @@ def shim(tmp_path_factory):
     return str(so)
 
 
-@pytest.mark.parametrize("case", ["stack_without_table", "trials_without_words"])
+@pytest.mark.parametrize("case", ["stack_without_table", "trials_without_words", "segments_one_by_one"])
 def test_short_of_memory(shim, case):
     r = subprocess.run([sys.executable, os.path.abspath(__file__), case], cwd=ROOT, text=True, capture_output=True,
                        timeout=300, env=dict(os.environ, LD_PRELOAD=shim, SHIM=shim))
@@ -183,6 +183,18 @@ def trials_without_words():
     words = ndm * (nfft // 2) * 4
     out, less = engine(x, peak - words // 2, *args, **kw)
     assert less <= peak - words and same(out, ref)
+
+
+def segments_one_by_one():
+    """A single-DM plan without room for the buffers of a group of segments: the same outputs
+    from one segment per launch."""
+    nfft = 1 << 20
+    x = samples(19 * nfft + 4321)
+    args = (0.4, nfft, 16, 128, 0.0371)
+    ref, peak = engine(x, NO_LIMIT, *args)
+    slices = 15 * 2 * 2 * (nfft // 2) * 8      # 15 further segments, two slots, two spectra
+    out, less = engine(x, peak - slices, *args)
+    assert less <= peak - slices and same(out, ref)
 
 
 if __name__ == "__main__":
