@@ -404,11 +404,12 @@ int build_trial(pond_t h, const pond_opts* o, Trial* t) {
   // single-DM plans take the chirp from the per-bin table unless the anchors are
   // asked for: F2f of three-pass plans (with the table rows prefetched into L2 it
   // overlaps the other segment stream better), and I1 of FP32 four-pass plans with columns
-  // of 512 points and more (the anchors cost it about 25 instructions per bin)
+  // of 512 points and more (the anchors cost it about 25 instructions per bin) where there is room
   const bool four = !h->multi && !ln.fused && !h->tc_terms && inv_cols_table(ln.g);
   if ((o->chirp == POND_CHIRP_TABLE || o->chirp == POND_CHIRP_AUTO) && (ln.fused || four)) {
-    CK(cudaMalloc(&t->ctab, (size_t)ln.g.L * sizeof(float2)));
-    CK(launch_chirp_c64(t->ctab, ln.g, ln.fused, du, half, o->f0_mhz, alpha, h->sgn, h->st));
+    const size_t bytes = (size_t)ln.g.L * sizeof(float2);
+    CK(four ? malloc_spare(&t->ctab, bytes) : cudaMalloc(&t->ctab, bytes));
+    if (t->ctab) CK(launch_chirp_c64(t->ctab, ln.g, ln.fused, du, half, o->f0_mhz, alpha, h->sgn, h->st));
   }
   return POND_OK;
 }

@@ -97,7 +97,8 @@ def shim(tmp_path_factory):
     return str(so)
 
 
-@pytest.mark.parametrize("case", ["stack_without_table", "trials_without_words", "segments_one_by_one"])
+@pytest.mark.parametrize("case", ["stack_without_table", "trials_without_words", "segments_one_by_one",
+                                  "four_pass_without_table"])
 def test_short_of_memory(shim, case):
     r = subprocess.run([sys.executable, os.path.abspath(__file__), case], cwd=ROOT, text=True, capture_output=True,
                        timeout=300, env=dict(os.environ, LD_PRELOAD=shim, SHIM=shim))
@@ -195,6 +196,18 @@ def segments_one_by_one():
     slices = 15 * 2 * 2 * (nfft // 2) * 8      # 15 further segments, two slots, two spectra
     out, less = engine(x, peak - slices, *args)
     assert less <= peak - slices and same(out, ref)
+
+
+def four_pass_without_table():
+    """A four-pass plan without room for its per-bin chirp table takes the anchors."""
+    from paper_1503_01405_gb300 import pond
+    nfft = 1 << 21
+    x = samples(3 * nfft + 99)
+    args, kw = (0.3, nfft, 1, 128, 0.0371), dict(timing=True)      # one segment per launch
+    ref, _ = engine(x, NO_LIMIT, *args, chirp=pond.POND_CHIRP_ANCHORS, **kw)
+    _, peak = engine(x, NO_LIMIT, *args, **kw)
+    out, less = engine(x, peak - nfft // 2 * 8, *args, **kw)
+    assert less <= peak - nfft // 2 * 8 and same(out, ref)
 
 
 if __name__ == "__main__":
