@@ -405,8 +405,9 @@ int pond_voltages(pond_t h, float* out_c, size_t cap, size_t* n_out, int64_t* fi
  *   point in (row, sample) order wins).  A row with sigma = 0 has none.
  *   Candidates go to HOST out[cap], sorted by (trial, index); *n_found gets
  *   their number.  Takes device scratch from a pool
- *   (up to 256 MiB of it stay for the next call): about 3 bytes per series sample, and
- *   8 + 1 more where more points than expected reach the threshold.
+ *   (up to 256 MiB of it stay for the next call): about 3 bytes per series sample (at
+ *   most 9 in rows under 9,000 samples) and 1.1 MB, or, where more points than expected
+ *   reach the threshold or that cannot be had, 8 + 1 instead.
  *   Work runs on cuda_stream and the call waits for it.
  *   Errors: POND_E_ARG, POND_E_OVERRUN (more candidates than cap; *n_found is
  *   the number found), POND_E_OOM, POND_E_CUDA.

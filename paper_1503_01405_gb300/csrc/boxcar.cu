@@ -734,7 +734,9 @@ __global__ void k_suppress(const double* __restrict__ S, const unsigned char* __
 }
 
 // Scratch of a call: stream-ordered allocations from a pool of the library's own per
-// device, which keeps up to SCRATCH_KEPT bytes between calls and gives the rest back.
+// device, which keeps up to SCRATCH_KEPT bytes between calls and gives the rest back.  What
+// it keeps the driver takes when another allocation of the process would fail (seen with
+// cudaMalloc beyond the free memory).
 constexpr unsigned long long SCRATCH_KEPT = 256ull << 20;
 cudaError_t scratch_pool(cudaMemPool_t* out) {
   static std::mutex mu;
@@ -802,29 +804,35 @@ int deliver(std::vector<pond_cand>& v, unsigned long long found, long long dcap,
   return POND_OK;
 }
 
-// Every point in FP64: for thresholds that most points pass, and lists that overflow.
-int run_dense(const float* d_series, int ndm, long long n, long long stride, double thr, const double* mu,
+// Every point in FP64: for thresholds that most points pass, and lists that overflow.  The
+// caller's scratch is given back first (its rows' mu and sigma are kept), so a
+// call never holds more than the larger of the two forms.
+int run_dense(const float* d_series, int ndm, long long n, long long stride, double thr, Scratch* sc, const double* mu,
               const double* sig, pond_cand* host_out, size_t cap, size_t* n_found, cudaStream_t st) {
   const long long dcap = std::max<long long>(1024, (long long)cap);
-  double* S = nullptr;
+  double *stats = nullptr, *S = nullptr;
   unsigned char* W = nullptr;
   pond_cand* dc = nullptr;
   unsigned long long* cnt = nullptr;
-  auto cleanup = [&]() {
-    cudaFree(S);
-    cudaFree(W);
-    cudaFree(dc);
-    cudaFree(cnt);
+  cudaError_t e = cudaSuccess;
+  auto take = [&](auto** p, size_t count) {
+    if (e == cudaSuccess) e = cudaMalloc(p, count * sizeof(**p));
   };
-  cudaError_t e = cudaMalloc(&S, (size_t)ndm * n * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&W, (size_t)ndm * n);
-  if (e == cudaSuccess) e = cudaMalloc(&dc, dcap * sizeof(pond_cand));
-  if (e == cudaSuccess) e = cudaMalloc(&cnt, sizeof(unsigned long long));
+  take(&stats, 2 * (size_t)ndm);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(stats, mu, ndm * sizeof(double), cudaMemcpyDeviceToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(stats + ndm, sig, ndm * sizeof(double), cudaMemcpyDeviceToDevice, st);
+  cudaFreeAsync(sc->p, st);
+  sc->p = nullptr;
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  take(&S, (size_t)ndm * n);
+  take(&W, (size_t)ndm * n);
+  take(&dc, (size_t)dcap);
+  take(&cnt, 1);
   if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), st);
   unsigned long long found = 0;
   if (e == cudaSuccess) {
     const dim3 grid((unsigned)((n + BOX_THREADS - 1) / BOX_THREADS), (unsigned)ndm);
-    k_boxcar<<<grid, BOX_THREADS, 0, st>>>(d_series, n, stride, mu, sig, S, W);
+    k_boxcar<<<grid, BOX_THREADS, 0, st>>>(d_series, n, stride, stats, stats + ndm, S, W);
     const long long tot = (long long)ndm * n;
     k_suppress<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(S, W, ndm, n, thr, 2, dc, dcap, cnt);
     e = cudaGetLastError();
@@ -833,7 +841,11 @@ int run_dense(const float* d_series, int ndm, long long n, long long stride, dou
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   std::vector<pond_cand> v;
   const int rc = e == cudaSuccess ? deliver(v, found, dcap, dc, host_out, cap, n_found, st) : boxcar_fail(e);
-  cleanup();
+  cudaFree(stats);
+  cudaFree(S);
+  cudaFree(W);
+  cudaFree(dc);
+  cudaFree(cnt);
   return rc;
 }
 
@@ -844,10 +856,10 @@ int run_boxcar(const float* d_series, int ndm, long long n, long long stride, do
   // At a threshold of 1 and more under half of a noise row's points reach the exact
   // evaluation; the list holds a sixteenth of all points, and a block where more reach it
   // takes the dense form.  (Points are listed with 32-bit sample indices.)
-  const bool sparse = thr >= 1.0 && n < (1ll << 31);
+  bool sparse = thr >= 1.0 && n < (1ll << 31);
   const long long dcap = std::max<long long>(1024, (long long)cap), tot = (long long)ndm * n;
   const long long chunks = (n + SCREEN_T - 1) / SCREEN_T, jobs = chunks * ndm;
-  const unsigned ccap = (unsigned)std::min<long long>(n, n / 8 + 8192), dlist = (unsigned)std::min<long long>(n, n / 4 + 16384);
+  unsigned ccap = (unsigned)std::min<long long>(n, n / 8 + 8192), dlist = (unsigned)std::min<long long>(n, n / 4 + 16384);
   const unsigned hotcap = (unsigned)std::min<long long>(1ll << 30, std::max<long long>(1 << 16, tot / 16));
   constexpr size_t FIRST = 512;   // candidates copied with the counters
   struct Head {
@@ -855,11 +867,17 @@ int run_boxcar(const float* d_series, int ndm, long long n, long long stride, do
     pond_cand first[FIRST];
   };
   Scratch sc;
-  const size_t o_mu = sc.cut(ndm * sizeof(double)), o_sig = sc.cut(ndm * sizeof(double));
-  const size_t o_br = sc.cut(ndm * sizeof(Bracket)), o_scr = sc.cut(ndm * sizeof(Screen));
-  const size_t o_C = sc.cut((size_t)ndm * ccap * sizeof(float)), o_D = sc.cut((size_t)ndm * dlist * sizeof(float));
-  size_t o_head = 0, o_bits = 0, o_base = 0, o_hot = 0, o_S = 0, o_W = 0;
-  if (sparse) {
+  size_t o_mu = 0, o_sig = 0, o_br = 0, o_scr = 0, o_C = 0, o_D = 0, o_head = 0, o_bits = 0, o_base = 0, o_hot = 0, o_S = 0,
+         o_W = 0;
+  auto lay_out = [&]() {
+    sc.bytes = 0;
+    o_mu = sc.cut(ndm * sizeof(double));
+    o_sig = sc.cut(ndm * sizeof(double));
+    o_br = sc.cut(ndm * sizeof(Bracket));
+    o_scr = sc.cut(ndm * sizeof(Screen));
+    o_C = sc.cut((size_t)ndm * ccap * sizeof(float));
+    o_D = sc.cut((size_t)ndm * dlist * sizeof(float));
+    if (!sparse) return;
     // counters, then the candidates
     o_head = sc.cut(offsetof(Head, first) + (size_t)std::max<long long>(dcap, FIRST) * sizeof(pond_cand));
     o_bits = sc.cut((size_t)jobs * SCREEN_W * sizeof(unsigned));
@@ -867,10 +885,20 @@ int run_boxcar(const float* d_series, int ndm, long long n, long long stride, do
     o_hot = sc.cut((size_t)hotcap * sizeof(uint2));
     o_S = sc.cut((size_t)hotcap * sizeof(double));
     o_W = sc.cut(hotcap);
-  }
+  };
   cudaMemPool_t pool = nullptr;
   cudaError_t e = scratch_pool(&pool);
-  if (e == cudaSuccess) e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&sc.p), sc.bytes, pool, st);
+  if (e != cudaSuccess) return boxcar_fail(e);
+  lay_out();
+  e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&sc.p), sc.bytes, pool, st);
+  if (e == cudaErrorMemoryAllocation) {
+    // no room for the lists: every row by radix selects, every point in FP64
+    cudaGetLastError();
+    sparse = false;
+    ccap = dlist = 0;
+    lay_out();
+    e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&sc.p), sc.bytes, pool, st);
+  }
   if (e != cudaSuccess) return boxcar_fail(e);
   double *mu = sc.at<double>(o_mu), *sig = sc.at<double>(o_sig);
   Bracket* br = sc.at<Bracket>(o_br);
@@ -915,9 +943,9 @@ int run_boxcar(const float* d_series, int ndm, long long n, long long stride, do
     }
   }
   if (e == cudaSuccess && dense)
-    rc = run_dense(d_series, ndm, n, stride, thr, mu, sig, host_out, cap, n_found, st);
+    rc = run_dense(d_series, ndm, n, stride, thr, &sc, mu, sig, host_out, cap, n_found, st);
   if (e != cudaSuccess) rc = boxcar_fail(e);
-  cudaFreeAsync(sc.p, st);
+  if (sc.p) cudaFreeAsync(sc.p, st);
   return rc;
 }
 

@@ -98,7 +98,8 @@ def shim(tmp_path_factory):
 
 
 @pytest.mark.parametrize("case", ["stack_without_table", "trials_without_words", "segments_one_by_one",
-                                  "four_pass_without_table"])
+                                  "four_pass_without_table",
+                                  "boxcar_without_lists"])
 def test_short_of_memory(shim, case):
     r = subprocess.run([sys.executable, os.path.abspath(__file__), case], cwd=ROOT, text=True, capture_output=True,
                        timeout=300, env=dict(os.environ, LD_PRELOAD=shim, SHIM=shim))
@@ -208,6 +209,26 @@ def four_pass_without_table():
     _, peak = engine(x, NO_LIMIT, *args, **kw)
     out, less = engine(x, peak - nfft // 2 * 8, *args, **kw)
     assert less <= peak - nfft // 2 * 8 and same(out, ref)
+
+
+def boxcar_without_lists():
+    """The detector never needs more than the 9 bytes per series sample of its dense form and
+    its candidate array: where too many points reach the threshold for the lists
+    (0.9: not screened at all, 1.0: they overflow), and where the lists of short rows do not fit."""
+    import torch
+
+    from paper_1503_01405_gb300 import pond
+    cap = 1 << 17
+    for ndm, n, thr in ((48, 20_000, 0.9), (48, 20_000, 1.0), (1500, 700, 6.0)):
+        g = torch.Generator(device="cuda")
+        g.manual_seed(n)
+        x = torch.randn((ndm, n), generator=g, device="cuda") * 3 + 10
+        x[ndm // 2, n // 2:n // 2 + 8] += 9.0
+        torch.cuda.synchronize()
+        ref = pond.boxcar(x.data_ptr(), ndm, n, n, thr, cap)
+        with Budget(9 * ndm * n + cap * ctypes.sizeof(pond.pond_cand) + ndm * 256 + 4096):
+            got = pond.boxcar(x.data_ptr(), ndm, n, n, thr, cap)
+        assert ref and got == ref, (ndm, n, thr, len(ref), len(got))
 
 
 if __name__ == "__main__":
