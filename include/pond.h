@@ -280,7 +280,9 @@ int pond_push(pond_t h, const int8_t* x, size_t n);
  *   stream, which then waits for the legacy default stream), in stream order,
  *   and reads d_x directly for segments that lie inside it.  d_x must stay
  *   valid and unmodified until the work enqueued on cuda_stream has finished;
- *   the library itself does not touch d_x after that work completes.
+ *   the library itself does not touch d_x after that work completes.  Where the
+ *   undrained series would outgrow the device ring, the call waits for the
+ *   complete samples and keeps them on the host for pond_timeseries.
  *   Errors: as pond_push.
  */
 int pond_push_device(pond_t h, const int8_t* d_x, size_t n, void* cuda_stream);
@@ -419,7 +421,9 @@ int pond_boxcar(const float* d_series, int32_t ndm, int64_t n, int64_t stride, d
  * pond_candidates: pond_boxcar over the handle's completed series samples that
  *   have not been drained yet (all trials of a batched plan), with index = the
  *   series sample index j and dm = the trial's DM.  Call it before
- *   pond_timeseries drains the samples.  Sec. 5 names automatic detection of
+ *   pond_timeseries drains the samples (after one push whose series is longer than the device
+ *   ring of 2^22 samples, 2^19 per trial of a batched plan, the device holds only its
+ *   end: POND_E_OVERRUN until they are drained).  Sec. 5 names automatic detection of
  *   transients as the paper's plan; the detector is this library's.  Besides
  *   the handle and the output array it takes the S/N threshold (the boxcar's
  *   detection level, 6 in the learned form), so callers choose it per call.

@@ -67,6 +67,7 @@ constexpr double K_DM = 1.0 / 2.41e-4;          // s MHz^2 (Eq. 1 constant)
 constexpr long long STAGE_BYTES = 128ll << 20;  // host-push staging chunk
 constexpr int NSTAGE = 2;                        // staging buffers: copies run up to one piece ahead
 constexpr long long FIRST_STAGE_BYTES = 32ll << 20;  // first piece of a stream's host push
+constexpr long long OPEN_END = 1ll << 62;   // g_end of segments that are not the stream's last
 constexpr long long TS_RING_SINGLE = 1ll << 22; // time-series samples held on the device (one trial)
 constexpr long long TS_RING_MULTI = 1ll << 19;  // ... per trial of a batched plan
 constexpr int MAX_TRIALS = 4096;
@@ -222,6 +223,8 @@ struct pond_s {
   long long outputs = 0;
   // time series: [ts_drained, ts_complete) complete on the device; ts_hi = one past the last touched
   long long ts_first = -1, ts_drained = 0, ts_hi = 0, ts_complete = 0;
+  long long ts_pushed = 0;                  // ts_complete when the current ingest began
+  bool ts_split = false;                    // one ingest filled the ring: the device holds only its later samples
   std::vector<std::vector<float>> ts_host;  // per trial
   std::vector<int32_t> ts_host_cnt;
   void* ts_pin = nullptr;                   // pinned staging of one ring row (ring * 4 B)
@@ -649,11 +652,12 @@ int drain_ts(pond_t h, long long n, DstRow dst, int32_t* cnt) {
   return POND_OK;
 }
 
-int spill_ts(pond_t h) {
-  if (h->ts_first < 0 || h->ts_complete <= h->ts_drained) return POND_OK;
+// Move the complete samples before `upto` to the host.
+int spill_ts(pond_t h, long long upto) {
+  if (h->ts_first < 0 || upto <= h->ts_drained) return POND_OK;
   RC(join_streams(h));
   CK(cudaStreamSynchronize(h->st));
-  const long long n = h->ts_complete - h->ts_drained;
+  const long long n = upto - h->ts_drained;
   const int ntr = (int)h->trials.size();
   if (h->ts_host[0].empty()) h->ts_host_first = h->ts_drained;
   const size_t off = h->ts_host[0].size();
@@ -723,7 +727,15 @@ int run_segments(pond_t h, int li, const SegSrc& src, long long s, int nseg, lon
     h->ts_drained = j_lo;
     h->ts_complete = j_lo;
   }
-  if (j_hi - h->ts_drained >= h->ring) RC(spill_ts(h));
+  if (j_hi - h->ts_drained >= h->ring) {
+    RC(spill_ts(h, h->ts_pushed));
+    if (j_hi - h->ts_drained >= h->ring) {   // one ingest alone fills the ring
+      h->ts_split = true;
+      RC(spill_ts(h, h->ts_complete));
+    }
+    if (j_hi - h->ts_drained >= h->ring)
+      return fail(POND_E_OVERRUN, "%lld undrained series samples exceed the device ring", j_hi - h->ts_drained + 1);
+  }
   float2* vout = nullptr;
   if (h->want_voltages) {
     if (h->v_base < 0) h->v_base = g0;
@@ -849,7 +861,8 @@ int run_segments(pond_t h, int li, const SegSrc& src, long long s, int nseg, lon
 }
 
 // Run the lane's next n segments (their input in the carry and the avail bytes at d) in
-// groups of at most ln.group; a group's series samples stay well inside the device ring.
+// groups of at most ln.group and a quarter of the series ring; the samples that every lane has
+// passed count as complete after each group, so that a long push can drain them.
 int run_lane(pond_t h, int li, const int8_t* d, long long avail, long long n, long long g_end) {
   Lane& ln = h->lanes[li];
   const Geom& g = ln.g;
@@ -868,6 +881,7 @@ int run_lane(pond_t h, int li, const int8_t* d, long long avail, long long n, lo
     RC(run_segments(h, li, src, ln.seg_start / g.S, k, g_end));
     ln.seg_start += k * g.S;
     n -= k;
+    if (g_end == OPEN_END) update_complete(h);
   }
   return POND_OK;
 }
@@ -877,11 +891,19 @@ int run_lane(pond_t h, int li, const int8_t* d, long long avail, long long n, lo
 int ingest_device(pond_t h, const int8_t* d, long long n) {
   const long long end = h->total_in + n;
   const long long ch = h->ch;                // bytes per sample at d and in the carry
+  h->ts_pushed = h->ts_complete;
   RC(fork_streams(h));
-  for (size_t li = 0; li < h->lanes.size(); ++li) {
-    Lane& ln = h->lanes[li];
-    const Geom& g = ln.g;
-    if (ln.seg_start + g.N <= end) RC(run_lane(h, (int)li, d, n * ch, (end - g.N - ln.seg_start) / g.S + 1, 1ll << 62));
+  // several lanes take a long push in stretches of a quarter of the series ring, so that none
+  // runs further ahead of the others than the ring holds
+  const double most = h->ring / 4 * ((double)h->dec_num / (double)h->dec_den) * 2.0 * h->nchan;
+  const long long step = h->lanes.size() > 1 && most < (double)n ? std::max(1ll, (long long)most) : n;
+  for (long long lim = std::min(end, h->total_in + step);; lim = std::min(end, lim + step)) {
+    for (size_t li = 0; li < h->lanes.size(); ++li) {
+      Lane& ln = h->lanes[li];
+      const Geom& g = ln.g;
+      if (ln.seg_start + g.N <= lim) RC(run_lane(h, (int)li, d, n * ch, (lim - g.N - ln.seg_start) / g.S + 1, OPEN_END));
+    }
+    if (lim == end) break;
   }
   // Each lane's carry is double-buffered: the buffer rewritten below was last
   // read by the previous ingest's segments, so st waits for that ingest's
@@ -1611,7 +1633,13 @@ int plan_impl(pond_t* out, const pond_opts* o) {
     }
   // outputs
   const int ntr = (int)dms.size();
+  // at least one segment's samples, or, of several lanes, a quarter of the ring, the longest
+  // segment and its overlap (see ingest_device)
   h->ring = multi ? TS_RING_MULTI : TS_RING_SINGLE;
+  for (const Lane& ln : h->lanes) {
+    const bool lone = h->lanes.size() == 1;
+    h->ring = std::max(h->ring, (long long)std::ceil((double)(lone ? ln.g.S_c : 3 * ln.g.M) * (double)h->dec_den / (double)h->dec_num) + 16);
+  }
   CKD(cudaMalloc(&h->ts, (size_t)ntr * h->ring * sizeof(float)));
   CKD(cudaMalloc(&h->ts_cnt, (size_t)ntr * h->ring * sizeof(int)));
   CKD(cudaMemsetAsync(h->ts, 0, (size_t)ntr * h->ring * sizeof(float), h->st));
@@ -1768,6 +1796,7 @@ int pond_flush(pond_t h) {
   CK(cudaSetDevice(h->device));
   const long long total_c = h->total_in / (2ll * h->nchan);
   const long long g_end = total_c - h->n_fut_max;
+  h->ts_pushed = h->ts_complete;
   RC(fork_streams(h));
   for (size_t li = 0; li < h->lanes.size(); ++li) {
     Lane& ln = h->lanes[li];
@@ -1816,7 +1845,8 @@ int pond_reset(pond_t h) {
   h->outputs = 0;
   h->launches = 0;
   h->ts_first = -1;
-  h->ts_drained = h->ts_hi = h->ts_complete = 0;
+  h->ts_drained = h->ts_hi = h->ts_complete = h->ts_pushed = 0;
+  h->ts_split = false;
   for (auto& v : h->ts_host) v.clear();
   h->ts_host_cnt.clear();
   h->ts_host_first = 0;
@@ -1871,7 +1901,8 @@ int pond_timeseries(pond_t h, float* out, int32_t* counts, size_t cap, size_t* n
     *n_out = (size_t)n;
     return POND_OK;
   }
-  RC(spill_ts(h));
+  RC(spill_ts(h, h->ts_complete));
+  h->ts_split = false;
   const size_t n = std::min(cap, h->ts_host[0].size());
   if (n) {
     for (size_t d = 0; d < h->trials.size(); ++d) {
@@ -1953,7 +1984,8 @@ static int candidates_impl(pond_t h, pond_cnn_t net, double threshold, pond_cand
   CK(cudaStreamSynchronize(h->st));
   const long long j0 = h->ts_drained, n = h->ts_complete - h->ts_drained;
   if (n <= 0) return POND_OK;
-  if (n > h->ring) return fail(POND_E_OVERRUN, "more undrained series samples than the device ring holds");
+  if (n > h->ring || h->ts_split)
+    return fail(POND_E_OVERRUN, "more undrained series samples than the device ring holds");
   const int ntr = (int)h->trials.size();
   float* blk = nullptr;
   CK(cudaMalloc(&blk, (size_t)ntr * n * sizeof(float)));
