@@ -98,3 +98,21 @@ def test_training_on_unaligned_patches(batch):
     loss2, grad2 = net.gradient(x.clone(), y)
     net.close()
     assert loss == loss2 and np.array_equal(grad, grad2)
+
+
+def test_pushes_of_a_running_stream_are_not_cut():
+    """A 100 MiB push behind another one reaches the device in one piece: one launch, the
+    copy, more than the same pushes from the device."""
+    import torch
+    p = pcd.make_plan(326.5, 16.0, 32e6, 26.8, 1 << 24, 64, 128, 0.03)
+    sizes = [20 << 20, 100 << 20]
+    h = torch.empty(max(sizes), dtype=torch.int8, pin_memory=True).zero_()
+    d = h.cuda()
+    launches = []
+    for src in (d, h.numpy()):
+        with pond.Engine(p.f0, p.bw, p.fs, p.dm, p.nfft, p.nchan, p.nbins, p.period) as e:
+            for n in sizes:
+                e.push_tensor(src[:n]) if src is d else e.push(src[:n])
+            e.sync()
+            launches.append(e.stats()["kernel_launches"])
+    assert launches[1] == launches[0] + len(sizes)
