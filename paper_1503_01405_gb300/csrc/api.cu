@@ -869,7 +869,10 @@ int run_lane(pond_t h, int li, const int8_t* d, long long avail, long long n, lo
   const long long per = (g.S_c * h->dec_den) / h->dec_num + 2;   // series samples per segment
   const long long most = std::max(1ll, std::min<long long>(ln.group, h->ring / (4 * per)));
   while (n > 0) {
-    const int k = (int)std::min(n, most);
+    // Two segments that each fill the chip (1.7 waves of CTAs and more) run faster on the two
+    // streams than in one launch: pushes of 28 MiB at nfft 2^24 288 us against 314, of 16 MiB at
+    // 2^23 157 against 174; at 2^22 the pair wins (33 MiB: 312 against 328).
+    const int k = n == 2 && most > 2 && g.L >= 1 << 22 ? 1 : (int)std::min(n, most);
     SegSrc src;
     src.carry_end = ln.carry[ln.carry_cur] + (h->total_in - ln.carry_pos) * h->ch;
     src.d = d;
