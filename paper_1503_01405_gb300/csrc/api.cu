@@ -149,7 +149,7 @@ struct Lane {
   float* partm[NSLOT] = {};                 // [kt][G][M] column-pass group partials
   int* cntm[NSLOT] = {};                    // [kt][FUSED_J] column-pass tickets
   unsigned* atab = nullptr;                 // table form: Q0.32 phase of one DM step per bin (row layout)
-  unsigned* words = nullptr;                // anchor form: [trial][L] phase words, or null
+  unsigned* words = nullptr;                // anchor and per-trial forms: [trial][L] phase words, or null
   unsigned* d_nmul = nullptr;               // per lane trial: its DM in DM steps
   const ChirpAnchor** d_anc = nullptr;      // per lane trial: its anchor table
   int* d_clog = nullptr;
@@ -699,6 +699,9 @@ void update_complete(pond_t h) {
   h->ts_complete = std::max(h->ts_complete, (gn * h->dec_den) / h->dec_num);
 }
 
+// The phase words of the lane's q-th trial (null: from its anchors).
+const unsigned* trial_words(const Lane& ln, size_t q) { return ln.words ? ln.words + q * ln.g.L : nullptr; }
+
 // The column pass of a three-pass lane: FP32 or tensor-core form.
 cudaError_t launch_ic(pond_t h, const Lane& ln, const float2* in, float* P, float* part, int* cnt, float2* vout,
                       long long vstride, long long vofs, const MSpan& span, cudaStream_t st, int nu = 1) {
@@ -833,7 +836,7 @@ int run_segments(pond_t h, int li, const SegSrc& src, long long s, int nseg, lon
         const Trial& t = h->trials[d];
         if (ln.mode == POND_TRIALS_PER_TRIAL) {
           // the trial's chirp and the first inverse factor as Ir loads the shared spectrum's rows
-          CK(launch_inv_rows_chirp(g, bufB, bufA, ln.tw2L, t.anc, t.clog, cs));
+          CK(launch_inv_rows_chirp(g, bufB, bufA, ln.tw2L, trial_words(ln, q), t.anc, t.clog, cs));
           if (q == 0) RC(record(h, 1 + ST_IR, cs));
           CK(launch_ic(h, ln, bufA, P, ln.part[slot], ln.cnt[slot], nullptr, 0, 0, span, cs));
           if (q == 0) RC(record(h, 1 + ST_IC, cs));
@@ -1069,7 +1072,7 @@ int measure_lane(pond_t h, const pond_opts* o, long long nfft, double* t_fwd, do
   for (int it = 0; it <= reps && ce == cudaSuccess; ++it) {
     if (it == 1) ce = cudaEventRecord(e[2], h->st);
     if (ln.fused_multi) {   // the per-trial passes the plan will run
-      if (ce == cudaSuccess) ce = launch_inv_rows_chirp(g, ln.bufB[0], ln.bufA[0], ln.tw2L, anc, clog, h->st);
+      if (ce == cudaSuccess) ce = launch_inv_rows_chirp(g, ln.bufB[0], ln.bufA[0], ln.tw2L, nullptr, anc, clog, h->st);
       if (ce == cudaSuccess)
         ce = launch_ic(h, ln, ln.bufA[0], ln.P[0], ln.part[0], ln.cnt[0], nullptr, 0, 0, span, h->st);
     } else {
@@ -1265,7 +1268,7 @@ int time_trials(pond_t h, Lane* ln, int mode, int kt, int split, double* us) {
     } else if (mode == POND_TRIALS_PER_TRIAL) {
       for (int q = 0; q < nq && ce == cudaSuccess; ++q) {
         const Trial& t = h->trials[ln->trials[q]];
-        ce = launch_inv_rows_chirp(g, ln->bufB[0], ln->bufA[0], ln->tw2L, t.anc, t.clog, h->st);
+        ce = launch_inv_rows_chirp(g, ln->bufB[0], ln->bufA[0], ln->tw2L, trial_words(*ln, q), t.anc, t.clog, h->st);
         if (ce == cudaSuccess)
           ce = launch_ic(h, *ln, ln->bufA[0], ln->P[0], ln->part[0], ln->cnt[0], nullptr, 0, 0, span, h->st);
         if (ce == cudaSuccess)
@@ -1361,16 +1364,17 @@ int apply_tune(pond_t h, Lane* ln, const TrialTune& t) {
   ln->cand_split = t.csplit;
   ln->cand_us = t.cus;
   if (t.mode == POND_TRIALS_FOUR_PASS) RC(use_split(h, ln, t.split));
-  if (t.mode != POND_TRIALS_MULTI_ANCHOR) {
+  const bool words = t.mode == POND_TRIALS_MULTI_ANCHOR || t.mode == POND_TRIALS_PER_TRIAL;
+  if (!words) {
     cudaFree(ln->words);
     ln->words = nullptr;
   }
   if (t.mode == POND_TRIALS_PER_TRIAL || t.mode == POND_TRIALS_FOUR_PASS) {
     free_multi(ln);
-    return POND_OK;
+    return words && !ln->words ? make_words(h, ln) : POND_OK;
   }
   if (t.kt != ln->kt || !ln->bufT[0]) RC(alloc_multi(ln, t.kt));
-  return t.mode == POND_TRIALS_MULTI_ANCHOR && !ln->words ? make_words(h, ln) : POND_OK;
+  return words && !ln->words ? make_words(h, ln) : POND_OK;
 }
 
 // Choose how the lane runs its trials (after its trials' anchors exist and the
@@ -1423,7 +1427,7 @@ int setup_trials(pond_t h, const pond_opts* o, Lane* ln) {
   const int kt_req = o->trials_per_launch ? std::min(o->trials_per_launch, ntr) : 0;
   if (!tune) {
     // the requested form (the table form only where the DMs allow it), else the table form where possible
-    if (!multi_ok) return POND_OK;
+    if (!multi_ok) return ln->mode == POND_TRIALS_PER_TRIAL ? make_words(h, ln) : POND_OK;
     ln->mode = (req == POND_TRIALS_MULTI_ANCHOR) ? POND_TRIALS_MULTI_ANCHOR : best_multi;
     RC(alloc_multi(ln, kt_req ? kt_req : std::min(32, ntr)));
     return ln->mode == POND_TRIALS_MULTI_ANCHOR ? make_words(h, ln) : POND_OK;
@@ -1452,10 +1456,8 @@ int setup_trials(pond_t h, const pond_opts* o, Lane* ln) {
     auto it = g_trial_tune.find(key);
     if (it != g_trial_tune.end()) return apply_tune(h, ln, it->second);
   }
-  if (!kts.empty()) {
-    RC(alloc_multi(ln, *std::max_element(kts.begin(), kts.end())));
-    RC(make_words(h, ln));
-  }
+  if (!kts.empty()) RC(alloc_multi(ln, *std::max_element(kts.begin(), kts.end())));
+  if (ln->fused_multi) RC(make_words(h, ln));
   CK(cudaMemsetAsync(ln->bufB[0], 0, (size_t)g.L * sizeof(float2), h->st));
   TrialTune t;
   size_t best = 0;

@@ -885,8 +885,13 @@ static cudaError_t launch_inv_rows_anchor(const Geom& g, const float2* in, float
   return cudaGetLastError();
 }
 
-cudaError_t launch_inv_rows_chirp(const Geom& g, const float2* in, float2* out, Tw2 tw2L,
+cudaError_t launch_inv_rows_chirp(const Geom& g, const float2* in, float2* out, Tw2 tw2L, const unsigned* words,
                                   const ChirpAnchor* anc, int clog, cudaStream_t st) {
+  if (words) {
+    MultiChirp mc{};
+    mc.words = words;
+    return launch_inv_rows_chirp_multi(g, in, out, 1, tw2L, mc, false, st);
+  }
   return launch_inv_rows_anchor(g, in, out, 1, tw2L, MultiChirp{}, anc, clog, st);
 }
 

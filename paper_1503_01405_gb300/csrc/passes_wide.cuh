@@ -311,7 +311,9 @@ size_t table_smem_bytes(const RowTile& rt) {
 // per plan.  A CTA keeps its rows resident and runs tpc trials of the launch on
 // them (blockIdx.x: trials x tpc ..), so a trial reads 4 bytes per bin and
 // writes 8.  21 trials of 2^19 bins: 53 us per launch with
-// the anchors evaluated per bin and trial, 36 here.
+// the anchors evaluated per bin and trial, 36 here.  Also one trial per launch, where the
+// anchors' evaluation adds to each tile's serial path (2^17 bins, a trial with its column
+// pass and decimation: 18 us against 26).
 template <int R1>
 __global__ void __launch_bounds__(WIDE_NT, 3)
     k_inv_rows_words(const float2* __restrict__ in, float2* __restrict__ out, long long out_tstride, RowTile rt,
@@ -355,7 +357,9 @@ __global__ void __launch_bounds__(WIDE_NT, 3)
 
 // Anchor form: one CTA per (trial, row tile), the chirp evaluated from the trial's anchors
 // as the tile is loaded (lanes over consecutive columns: their anchors lie side by side).
-// For lanes whose word tables would be too large, and for one trial per launch.
+// For lanes whose word tables would be too large, and for the length tuner's trial (2^23 bins, one
+// trial with its column pass and decimation: 94 us, with the words 82; the whole tile loaded
+// first and an anchor per value: 116).
 // blockIdx.x is the trial and runs fastest, so the CTAs that share rows are
 // adjacent in launch order and all but the first find them in L2.  With mc.anc null
 // the launch's one trial takes its anchors from anc1, clog1.
@@ -370,9 +374,6 @@ __global__ void __launch_bounds__(WIDE_NT, 3)
   const int r0 = blockIdx.y * NLR, t = blockIdx.x;
   const float2* src = in + ((size_t)r0 << LOGR1);
   {
-    float2 v[64];   // the tile: 64 loads in flight per thread
-#pragma unroll
-    for (int u = 0; u < 64; ++u) v[u] = __ldg(src + threadIdx.x + u * WIDE_NT);
     if (t == 0 && threadIdx.x == 0) {
       // the first trial's CTA of a row tile warms L2 with the rows of a later tile
       const unsigned rn = blockIdx.y + max(1u, (unsigned)WIDE_PF / gridDim.x);
@@ -380,12 +381,30 @@ __global__ void __launch_bounds__(WIDE_NT, 3)
     }
     const ChirpAnchor* anc = mc.anc ? mc.anc[t] : anc1;
     const int clog = mc.anc ? __ldg(mc.clog + t) : clog1;
+    // 16 values at a time, all rows of CB columns: their anchors fit the registers beside them
+    constexpr int CB = 16 / NLR, COLS = R1 / WIDE_NT;
+    const bool shared = (1 << clog) >= NLR;   // the tile's rows of a column have one anchor
+#pragma unroll 1
+    for (int c0 = 0; c0 < COLS; c0 += CB) {
+      float2 v[CB][NLR];
 #pragma unroll
-    for (int u = 0; u < 64; ++u) {
-      const int i = (int)threadIdx.x + u * WIDE_NT, slot = i >> LOGR1, k1 = i & (R1 - 1);
-      const unsigned k = (unsigned)(r0 + slot) + ((unsigned)k1 << rt.logR2);
-      const ChirpAnchor a = anc[k >> clog];
-      rows[slot * rt.rstr + k1 + (k1 >> 6)] = cmul(v[u], chirp_from(a, clog, k));
+      for (int q = 0; q < CB; ++q)
+#pragma unroll
+        for (int slot = 0; slot < NLR; ++slot) v[q][slot] = __ldg(src + slot * R1 + threadIdx.x + (c0 + q) * WIDE_NT);
+      ChirpAnchor a[CB];
+#pragma unroll
+      for (int q = 0; q < CB; ++q)
+        a[q] = anc[((unsigned)r0 + ((threadIdx.x + (unsigned)(c0 + q) * WIDE_NT) << rt.logR2)) >> clog];
+#pragma unroll
+      for (int q = 0; q < CB; ++q) {
+        const int k1 = (int)threadIdx.x + (c0 + q) * WIDE_NT;
+#pragma unroll
+        for (int slot = 0; slot < NLR; ++slot) {
+          const unsigned k = (unsigned)(r0 + slot) + ((unsigned)k1 << rt.logR2);
+          if (!shared && slot > 0) a[q] = anc[k >> clog];
+          rows[slot * rt.rstr + k1 + (k1 >> 6)] = cmul(v[q][slot], chirp_from(a[q], clog, k));
+        }
+      }
     }
   }
   make_twk<R1>(twk, tw2L, NLR, [&](int slot) { return r0 + slot; });

@@ -167,7 +167,8 @@ cudaError_t launch_fwd_rows_inv(const Geom& g, const float2* in, float2* out, Tw
                                 cudaStream_t st, int nseg = 1);
 cudaError_t launch_chirp_c64(float2* tab, const Geom& g, bool runs, double du, double half, double f0, double alpha, int sgn,
                              cudaStream_t st);
-cudaError_t launch_inv_rows_chirp(const Geom& g, const float2* in, float2* out, Tw2 tw2L,
+// words: the trial's launch_chirp_words, or null (from its anchors)
+cudaError_t launch_inv_rows_chirp(const Geom& g, const float2* in, float2* out, Tw2 tw2L, const unsigned* words,
                                   const ChirpAnchor* anc, int clog, cudaStream_t st);
 // nu > 1: one launch over nu trials or segments, the u-th reading in + u L and writing
 // P + u M, part + u G M, cnt + u FUSED_J (G = fused_groups); wtw: launch_wide_tw of R2

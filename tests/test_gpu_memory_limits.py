@@ -173,18 +173,18 @@ def same(a, b):
 
 
 def trials_without_words():
-    """The anchor form over several trials per launch without its per-trial phase words
-    (blocks of three and of two trials): the same series."""
+    """The anchor form over several trials per launch (blocks of three and of two) and the
+    per-trial form without the trials' phase words: the same series."""
     from paper_1503_01405_gb300 import pond
     nfft, ndm = 1 << 20, 8
     x = samples(5 * nfft + 1234)
     args = (0.0, nfft, 16, 1, 1.0)
-    kw = dict(t_dec=32e-6, dms=[0.31 + 0.0137 * d ** 1.3 for d in range(ndm)],
-              trial_mode=pond.POND_TRIALS_MULTI_ANCHOR, trials_per_launch=3)
-    ref, peak = engine(x, NO_LIMIT, *args, **kw)
     words = ndm * (nfft // 2) * 4
-    out, less = engine(x, peak - words // 2, *args, **kw)
-    assert less <= peak - words and same(out, ref)
+    for mode in (pond.POND_TRIALS_MULTI_ANCHOR, pond.POND_TRIALS_PER_TRIAL):
+        kw = dict(t_dec=32e-6, dms=[0.31 + 0.0137 * d ** 1.3 for d in range(ndm)], trial_mode=mode, trials_per_launch=3)
+        ref, peak = engine(x, NO_LIMIT, *args, **kw)
+        out, less = engine(x, peak - words // 2, *args, **kw)
+        assert less <= peak - words and same(out, ref), mode
 
 
 def segments_one_by_one():
