@@ -984,13 +984,13 @@ cudaError_t set_kernel_attributes() {
   // L1 and shared memory: an SM changes it only when idle, and the CTAs of the next
   // kernel crowd on the SMs that could (after a carry copy at the default division
   // a segment's fold took 31.8 us instead of 8.1, four 64-bit-bound CTAs to an SM).  Not
-  // the copy from host memory: its loads in flight need the L1 (end to end 1057 -> 1230 us).
+  // the copy from host memory: its loads in flight need the L1 (end to end 1057 -> 1230 us), nor
+  // the per-trial forms' decimation (24 trials at nfft 2^20: 2,132 us without, 2,230 with).
   auto shared_first = [&](auto* f) {
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   };
   shared_first(k_copy_bytes);
-  shared_first(k_decimate_short);
   shared_first(k_decimate_short_multi);
 #define SET_F(R)                                                                                               \
   {                                                                                                            \
