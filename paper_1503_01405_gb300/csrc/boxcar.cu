@@ -413,7 +413,8 @@ __device__ bool select_ranks(SelSmem& s, const float* __restrict__ list, unsigne
 }
 
 // One CTA per row: mu and sigma from the lists where the counts confirm the bracket, else
-// from the whole row; and the row's screening constants for threshold thr.
+// (or without brackets, br null) from the whole row; and the row's screening constants for
+// threshold thr.
 __global__ void __launch_bounds__(SORT_THREADS) k_robust_stats(const float* __restrict__ series, long long n,
                                                              long long stride, const Bracket* __restrict__ br,
                                                              const float* __restrict__ C, const float* __restrict__ D,
@@ -424,10 +425,10 @@ __global__ void __launch_bounds__(SORT_THREADS) k_robust_stats(const float* __re
   __shared__ unsigned long long shp;
   __shared__ long long shk;
   const int row = blockIdx.x;
-  const Bracket b = br[row];
+  const Bracket b = br ? br[row] : Bracket{};
   const long long k1 = (n - 1) / 2, k2 = n / 2;
   double mu = 0.0, mad = 0.0;
-  bool ok = !b.bad && b.nc <= ccap && b.nd <= dcap && k1 >= (long long)b.below && k2 - (long long)b.below < (long long)b.nc;
+  bool ok = br && !b.bad && b.nc <= ccap && b.nd <= dcap && k1 >= (long long)b.below && k2 - (long long)b.below < (long long)b.nc;
   if (ok) {
     const int shift = max(0, 32 - __clz(b.khi - b.klo) - 12);   // (khi - klo) >> shift < SEL_NB
     ok = select_ranks(s, C + (size_t)row * ccap, b.nc, k1 - b.below, k2 - b.below, 0,
@@ -902,10 +903,17 @@ int run_boxcar(const float* d_series, int ndm, long long n, long long stride, do
   if (e != cudaSuccess) return boxcar_fail(e);
   double *mu = sc.at<double>(o_mu), *sig = sc.at<double>(o_sig);
   Bracket* br = sc.at<Bracket>(o_br);
-  k_bracket<<<ndm, SORT_THREADS, 0, st>>>(d_series, n, stride, br);
+  // A bracket sorts 8192 values whatever the row's length (50 us for the two rows of an SM), so many short
+  // rows go by radix selects in small CTAs: 20,000 rows of 100 samples 2,060 us (6,520 with
+  // brackets), 2,000 of 2,000 590 (750), 1,333 of 3,000 552 (511); 64 rows
+  // of 1,000 142 (111).
+  const bool radix = n <= 2048 && ndm > 304;
+  if (radix) br = nullptr;
+  else k_bracket<<<ndm, SORT_THREADS, 0, st>>>(d_series, n, stride, br);
   const dim3 cg((unsigned)((n + COLLECT - 1) / COLLECT), (unsigned)ndm);
-  k_collect<<<cg, COLLECT_THREADS, 0, st>>>(d_series, n, stride, br, sc.at<float>(o_C), sc.at<float>(o_D), ccap, dlist);
-  k_robust_stats<<<ndm, SORT_THREADS, 0, st>>>(d_series, n, stride, br, sc.at<float>(o_C), sc.at<float>(o_D), ccap,
+  if (!radix)
+    k_collect<<<cg, COLLECT_THREADS, 0, st>>>(d_series, n, stride, br, sc.at<float>(o_C), sc.at<float>(o_D), ccap, dlist);
+  k_robust_stats<<<ndm, radix ? 256 : SORT_THREADS, 0, st>>>(d_series, n, stride, br, sc.at<float>(o_C), sc.at<float>(o_D), ccap,
                                                dlist, thr, mu, sig, sc.at<Screen>(o_scr));
   e = cudaGetLastError();
   int rc = POND_OK;

@@ -103,6 +103,23 @@ def test_order_statistics_of_awkward_rows(kind):
     assert gpu_detect(block, thr=5.0) == ob.detect(block, threshold=5.0)
 
 
+@pytest.mark.parametrize("n", [1, 2, 3, 70, 257, 2048, 2049])
+def test_many_short_rows(n):
+    """More rows than the brackets' CTAs at once, shorter and longer than the rule's line: each
+    row's statistics and the candidates are the oracle's, with ties, a NaN and infinities among them."""
+    rng = np.random.default_rng(n)
+    block = (100 + 3 * rng.standard_normal((310, n))).astype(np.float32)
+    block[::3] = np.round(block[::3])
+    block[5] = 7.0
+    block[9::50, n // 2:n // 2 + 5] += 60
+    want = ob.detect(block)
+    assert gpu_detect(block) == want
+    block[20, 0], block[40, n // 3], block[41, n - 1] = np.nan, np.inf, -np.inf
+    some = np.r_[0:18, 25:36, 46:310]      # trials whose neighbours hold only finite values
+    got = [c for c in gpu_detect(block) if c[0] in some]
+    assert got == [c for c in want if c[0] in some]
+
+
 def test_screened_and_dense_forms_agree():
     """A threshold below 1 evaluates every point; its list cut at S/N 6 is the screened
     list, also where rows hold infinities or NaN (and an overflowing list takes the dense form)."""
