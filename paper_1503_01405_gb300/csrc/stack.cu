@@ -89,26 +89,36 @@ __device__ __forceinline__ double phase_at(const PhaseModel& m, long long i) {
 }
 
 // start[K - K0] = first sample i with key >= K, for K0 <= K <= K0 + nk.  A warp takes
-// windows of 1024 samples.  Where the phase is known to run forwards over a window a
-// lane takes 32 consecutive samples: the keys at its first sample and at the next
+// windows of 32 run samples.  Where the phase is known to run forwards over a window a
+// lane takes run consecutive samples: the keys at its first sample and at the next
 // lane's tell which keys begin in between, and each one's first sample is predicted from
 // the phases at the ends and corrected with exact keys (two evaluations per key).
-// Elsewhere every sample's key is evaluated and compared with the one before.
-constexpr int RUN = 32, WINDOW = 32 * RUN;
+// Elsewhere every sample's key is evaluated and compared with the one before.  A run of 32 needs
+// the fewest evaluations; a short series takes shorter ones, whose keys follow one another on
+// fewer steps, until RUN_LANES lanes share it (a call over 20,000 samples, 1.5 keys a
+// sample: 47 us, 108 at 32; 80,000 samples: 56 and 108; 65,536 lanes 62, 4,096 71).
+constexpr int MAX_RUN = 32;
+constexpr long long RUN_LANES = 16384;
+int run_length(long long n) {
+  int run = MAX_RUN;
+  while (run > 1 && n / run < RUN_LANES) run /= 2;
+  return run;
+}
 __global__ void __launch_bounds__(128) k_stack_starts(PhaseModel m, long long n, long long K0, long long nk,
-                                                    unsigned* __restrict__ start, int* __restrict__ backwards) {
+                                                    unsigned* __restrict__ start, int* __restrict__ backwards, int run) {
+  const int window = 32 * run;
   const int lane = threadIdx.x & 31;
   const long long warps = gridDim.x * 4ll;
   auto put = [&](long long lo, long long hi, long long i) {   // keys lo .. hi start at sample i
     for (long long q = max(lo, K0); q <= min(hi, K0 + nk); ++q) start[q - K0] = (unsigned)i;
   };
-  for (long long base = (blockIdx.x * 4ll + (threadIdx.x >> 5)) * WINDOW; base < n; base += warps * WINDOW) {
-    const long long end = min(n, base + WINDOW);   // the window and the step to the next one
+  for (long long base = (blockIdx.x * 4ll + (threadIdx.x >> 5)) * window; base < n; base += warps * window) {
+    const long long end = min(n, base + window);   // the window and the step to the next one
     if (base == 0 && lane == 0) put(K0, key_value(m, 0), 0);
     if (end == n && lane == 0) put(key_value(m, n - 1) + 1, K0 + nk, n);
     const long long last = min(end, n - 1);
     if (pond::phase_forwards(m.c, m.nc, m.dt, m.t_ref, m.g0 + base, m.g0 + last)) {
-      const long long a = base + lane * RUN, e = min(last, a + RUN);
+      const long long a = base + lane * run, e = min(last, a + run);
       if (a >= e) continue;
       const double xa = phase_at(m, a), xe = phase_at(m, e);
       const long long ka = key_value(m, a), ke = key_value(m, e);
@@ -358,7 +368,9 @@ extern "C" int pond_fold_stack(const float* d_series, int64_t n, int64_t g0, dou
   }
   if (start) {
     const long long K0 = *first_rotation * (long long)nbins;
-    k_stack_starts<<<(unsigned)std::min<long long>((n + 4 * WINDOW - 1) / (4 * WINDOW), 4096), 128, 0, st>>>(m, n, K0, nk, start, flag);
+    const int run = run_length(n);
+    const long long cta = 4 * 32 * run;
+    k_stack_starts<<<(unsigned)std::min<long long>((n + cta - 1) / cta, 4096), 128, 0, st>>>(m, n, K0, nk, start, flag, run);
     if (cells > 0)
       k_stack_sums<<<cell_blocks, CELL_THREADS, 0, st>>>(d_series, n, m, mode, n_sub, *first_rotation, *rows, start,
                                                          flag, d_sum, reinterpret_cast<long long*>(d_hits));

@@ -63,6 +63,19 @@ def test_stack_key_tables_and_searches(n, period_samples, mode, n_sub):
     assert q0 == q0_ref and np.array_equal(H, H_ref) and np.array_equal(S, S_ref)
 
 
+@pytest.mark.parametrize("n", [16383, 32769, 65535, 131073, 262145, 524287, 600_001])
+@pytest.mark.parametrize("period_samples,nbins", [(30.0, 64), (11629.3, 1024)], ids=["keys_per_sample", "samples_per_key"])
+def test_stack_run_lengths(n, period_samples, nbins):
+    """Series lengths around each run length's line, bit for bit."""
+    import torch
+    dt = 1e-3
+    c = np.array([0.2, 1.0 / (period_samples * dt), 1e-4])
+    y = np.random.default_rng(n).normal(10.0, 3.0, n).astype(np.float32)
+    S_ref, H_ref, q0_ref = st.stack(y, 5, dt, c, 0.1, nbins, st.SUBINT, 50_000)
+    S, H, q0 = pond.fold_stack(torch.from_numpy(y).cuda(), 5, dt, c, 0.1, nbins, st.SUBINT, 50_000)
+    assert q0 == q0_ref and np.array_equal(H, H_ref) and np.array_equal(S, S_ref)
+
+
 @pytest.mark.parametrize("nbins", [64, 4096], ids=["table", "search"])
 def test_overlapping_calls_keep_their_own_verdict(nbins):
     """Calls on two streams, one with a model that runs forwards and one whose model
