@@ -437,7 +437,7 @@ size_t fb_smem_bytes() {
 // ---------------------------------------------------------------------------
 
 struct pond_incoh_s {
-  int device = 0;
+  int device = 0, sms = 0;
   pond_incoh_opts o{};
   int nch = 0, logR = 0, lognint = 0, form = 0;
   double ts = 0.0, inc = 0.0;
@@ -502,28 +502,40 @@ cudaError_t fb_attr() {
     attr(pond::k_fb_power_w<R, pond::FB_AID1>, pond::fbw_smem_bytes<R>());
     attr(pond::k_fb_power_w<R, pond::FB_AID2>, pond::fbw_smem_bytes<R>());
     attr(pond::k_fb_power_w<R, pond::FB_CID>, pond::fbw_smem_bytes<R>());
-  } else {
+  }
+  if constexpr (R != 512) {
     attr(pond::k_fb_power<R, false>, (int)pond::fb_smem_bytes<R>());
     attr(pond::k_fb_power<R, true>, (int)pond::fb_smem_bytes<R>());
   }
   return e;
 }
 
-// Lines of 512 samples and more take 64 values per thread; shorter ones have no 64-point stage to fill.
+// Lines of 512 samples and more take 64 values per thread (shorter ones have no 64-point stage
+// to fill), but those of 1024 and more only in launches of more CTAs than SMs: alone on
+// an SM, the 512 threads of the radix-16 form run through a CTA's spectra sooner (40 M pairs in
+// 2048 channels, cross-power of 64 spectra, 153 CTAs: 150 us against 191; 12 M pairs, 16
+// spectra, 184 CTAs: 78 against 53).  tw: launch_wide_tw's table, then launch_stage_tw's.
 template <int R>
-cudaError_t fb_launch(const FbArgs& a, const float2* tw, cudaStream_t st) {
+cudaError_t fb_launch(const FbArgs& a, const float2* tw, int sms, cudaStream_t st) {
   const unsigned blocks = (unsigned)((a.n_spec + a.s_cta - 1) / a.s_cta);
+  const float2* stw = tw + pond::wide_tw_entries(R, true);
+  bool wide = false;
   if constexpr (R >= 512) {
-    constexpr int bytes = pond::fbw_smem_bytes<R>();
-    if (a.form == pond::FB_AID1) pond::k_fb_power_w<R, pond::FB_AID1><<<blocks, pond::WIDE_NT, bytes, st>>>(a, tw);
-    else if (a.form == pond::FB_AID2) pond::k_fb_power_w<R, pond::FB_AID2><<<blocks, pond::WIDE_NT, bytes, st>>>(a, tw);
-    else pond::k_fb_power_w<R, pond::FB_CID><<<blocks, pond::WIDE_NT, bytes, st>>>(a, tw);
-  } else {
+    wide = R == 512 || blocks > (unsigned)sms;
+    if (wide) {
+      constexpr int bytes = pond::fbw_smem_bytes<R>();
+      if (a.form == pond::FB_AID1) pond::k_fb_power_w<R, pond::FB_AID1><<<blocks, pond::WIDE_NT, bytes, st>>>(a, tw);
+      else if (a.form == pond::FB_AID2) pond::k_fb_power_w<R, pond::FB_AID2><<<blocks, pond::WIDE_NT, bytes, st>>>(a, tw);
+      else pond::k_fb_power_w<R, pond::FB_CID><<<blocks, pond::WIDE_NT, bytes, st>>>(a, tw);
+    }
+  }
+  if constexpr (R != 512) {
     const long long per_pass = (long long)(a.form == pond::FB_CID ? 1 : 2) * (pond::TILE / R);
-    if (a.s_cta <= per_pass)
-      pond::k_fb_power<R, true><<<blocks, pond::NT, pond::fb_smem_bytes<R>(), st>>>(a, tw);
+    if (wide) {
+    } else if (a.s_cta <= per_pass)
+      pond::k_fb_power<R, true><<<blocks, pond::NT, pond::fb_smem_bytes<R>(), st>>>(a, stw);
     else
-      pond::k_fb_power<R, false><<<blocks, pond::NT, pond::fb_smem_bytes<R>(), st>>>(a, tw);
+      pond::k_fb_power<R, false><<<blocks, pond::NT, pond::fb_smem_bytes<R>(), st>>>(a, stw);
   }
   return cudaGetLastError();
 }
@@ -551,10 +563,10 @@ cudaError_t ips_dispatch(int logL, bool attr, const float* c, long long J, const
   }
 }
 
-cudaError_t fb_dispatch(int logR, bool attr, const FbArgs& a, const float2* tw, cudaStream_t st) {
+cudaError_t fb_dispatch(int logR, bool attr, const FbArgs& a, const float2* tw, int sms, cudaStream_t st) {
   switch (logR) {
 #define FB_CASE(L) \
-  case L: return attr ? fb_attr<1 << L>() : fb_launch<1 << L>(a, tw, st);
+  case L: return attr ? fb_attr<1 << L>() : fb_launch<1 << L>(a, tw, sms, st);
     FB_CASE(7) FB_CASE(8) FB_CASE(9) FB_CASE(10) FB_CASE(11) FB_CASE(12)
 #undef FB_CASE
     default: return cudaErrorInvalidValue;
@@ -644,7 +656,8 @@ extern "C" int pond_incoh_create(pond_incoh_t* out, const pond_incoh_opts* o) {
     return bail(err(POND_E_CUDA, "pond_incoh_create: no CUDA device %d", o->device));
   cudaError_t e = cudaSetDevice(o->device);
   if (e == cudaSuccess) e = pond::set_kernel_attributes();
-  if (e == cudaSuccess) e = fb_dispatch(h->logR, true, FbArgs{}, nullptr, nullptr);
+  if (e == cudaSuccess) e = fb_dispatch(h->logR, true, FbArgs{}, nullptr, 0, nullptr);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, o->device);
   if (e == cudaSuccess && o->ips_len) {
     const int logL = ilog2(o->ips_len);
     e = ips_dispatch(logL, true, nullptr, 0, nullptr, nullptr, nullptr);
@@ -655,9 +668,9 @@ extern "C" int pond_incoh_create(pond_incoh_t* out, const pond_incoh_opts* o) {
     if (e == cudaSuccess) e = cudaMemset(h->ips, 0, (o->ips_len / 2 + 1) * sizeof(double));
   }
   if (e == cudaSuccess) e = cudaMalloc(&h->d_delay, o->nchan * sizeof(int));
-  const int wide = pond::wide_tw_entries(1 << h->logR, true);   // 0: radix-16 stages
+  const int wide = pond::wide_tw_entries(1 << h->logR, true);   // 0 below 512 samples
   if (e == cudaSuccess)
-    e = cudaMalloc(&h->stw, std::max(1, wide ? wide : pond::stage_tw_entries(1 << h->logR)) * sizeof(float2));
+    e = cudaMalloc(&h->stw, std::max(1, wide + pond::stage_tw_entries(1 << h->logR)) * sizeof(float2));
   if (e == cudaSuccess) e = cudaMalloc(&h->psum, (size_t)pond::MAX_FOLD_PARTS * o->nbins * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&h->phits, (size_t)pond::MAX_FOLD_PARTS * o->nbins * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&h->prof_sum, o->nbins * sizeof(double));
@@ -667,8 +680,8 @@ extern "C" int pond_incoh_create(pond_incoh_t* out, const pond_incoh_opts* o) {
   if (e == cudaSuccess)
     e = cudaMemcpy(h->d_delay, h->delay.data(), o->nchan * sizeof(int), cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
-    e = wide ? pond::launch_wide_tw(h->stw, 1 << h->logR, true, nullptr)
-             : pond::launch_stage_tw(h->stw, 1 << h->logR, nullptr);
+    e = pond::launch_wide_tw(h->stw, 1 << h->logR, true, nullptr);
+  if (e == cudaSuccess) e = pond::launch_stage_tw(h->stw + wide, 1 << h->logR, nullptr);
   if (e == cudaSuccess) e = cudaMemset(h->prof_sum, 0, o->nbins * sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(h->prof_hits, 0, o->nbins * sizeof(long long));
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -722,7 +735,7 @@ extern "C" int pond_incoh_run(pond_incoh_t h, const int8_t* d_x, size_t nbytes, 
     a.lognint = h->lognint;
     a.form = h->form;
     a.F = h->F;
-    ICK(fb_dispatch(h->logR, false, a, h->stw, st));
+    ICK(fb_dispatch(h->logR, false, a, h->stw, h->sms, st));
     ++launches;
   }
   ICK(cudaEventRecord(h->ev[1], st));

@@ -55,6 +55,28 @@ def _compare(e, p, raw):
     return F, D, s, h
 
 
+LINES = [(ch, mode) for ch, mode in ((1, inc.AID), (2, inc.AID), (2, inc.CID))]
+
+
+@pytest.mark.parametrize("form", LINES, ids=["AID1", "AID2", "CID2"])
+@pytest.mark.parametrize("nchan", [256, 512, 1024, 2048])
+def test_filterbank_of_few_and_many_blocks(nchan, form):
+    """Both forms of the filterbank: launches of fewer and of more CTAs than SMs (a CTA takes
+    4096 / nchan lines of one spectrum, or of two for AID), with a ragged last CTA."""
+    import torch
+    ch, mode = form
+    per = (1 if mode == inc.CID else 2) * 4096 // nchan
+    p = inc.make_plan(326.5, 16.0, 32e6, 1.0, nchan, 1, mode, ch, 64, 0.02)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    with _engine(p) as e:
+        for blocks in (3, 2 * sms):
+            spectra = blocks * per - per // 2 - 1
+            x = np.random.default_rng(blocks + nchan).integers(-60, 61, ch * (spectra * 2 * nchan + 5)).astype(np.int8)
+            e.run_tensor(torch.from_numpy(x).cuda())
+            F, r = e.filterbank(), inc.run(p, x)
+            assert F.shape == r.F.T.shape and F.shape[0] == spectra and rel(F, r.F.T) <= TOL
+
+
 CASES = [  # nchan, nint, mode, channels, bw, dm, input samples
     (1024, 1, inc.AID, 1, 16.0, 10.0, (1 << 21) + 333),
     (256, 4, inc.AID, 2, 16.0, 5.0, (1 << 21) + 7),
