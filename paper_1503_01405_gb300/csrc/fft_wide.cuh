@@ -17,9 +17,13 @@
 // memory the line is RB rows of RA values with one value of padding per row,
 // so stage 1 writes rows and stage 2 reads columns without bank conflicts.
 // Stage 2's twiddles are factored: j = NB a + b gives w^{NB a t} w^{b t}, the
-// first applied before the inner DFTs over a, the second after them, so a
-// thread keeps NA + NB - 2 (10 for RB = 32, 14 for 64) values in registers
-// instead of reading RB - 1 from a table for every butterfly.
+// first applied before the inner DFTs over a, the second after them.  There the RB-point DFT
+// has a factor of its own, exp(-+2 pi i b ka / RB) for output ka; WideTw reads the
+// product of the two, rounded once, from a table (a value passes three products instead
+// of four: an FP32 line of 2048 points is off by 1.05e-7 relative to 64 bits, by
+// 1.13e-7 with two products, by 1.05e-7 with three radix-16 stages).  The column pass
+// after F2f multiplies twice (WideTwPair): it keeps NA + NB - 2 (10 for RB = 32) values in
+// registers for its butterflies and has none to spare.
 #pragma once
 #include "fft_block.cuh"
 
@@ -60,9 +64,9 @@ template <> struct WideSplit<32> { static constexpr int NA = 4, NB = 8; };
 template <> struct WideSplit<16> { static constexpr int NA = 4, NB = 4; };
 template <> struct WideSplit<8> { static constexpr int NA = 2, NB = 4; };
 
-// N-point DFT of v, natural order in and out.  before(v, j) may scale input
-// j = NB a + b ahead of the inner DFT over a; between(v, b) scales everything of
-// one b after it.
+// N-point DFT of v, natural order in and out.  before(v, a) may scale input
+// NB a + b ahead of the inner DFT over a; between(v, b, ka) scales its output ka
+// after it, by the DFT's own factor exp(-+2 pi i b ka / N) among others.
 template <int N, bool INV, class Before, class Between>
 __device__ __forceinline__ void wide_dft(float2* v, Before before, Between between) {
   constexpr int NA = WideSplit<N>::NA, NB = WideSplit<N>::NB;
@@ -73,7 +77,7 @@ __device__ __forceinline__ void wide_dft(float2* v, Before before, Between betwe
     for (int a = 0; a < NA; ++a) x[a] = before(v[NB * a + b], a);
     Dft<NA, INV>::run(x);
 #pragma unroll
-    for (int ka = 0; ka < NA; ++ka) v[NB * ka + b] = tw64<INV>(between(x[ka], b), b * ka * (64 / N));
+    for (int ka = 0; ka < NA; ++ka) v[NB * ka + b] = between(x[ka], b, ka);
   }
 #pragma unroll
   for (int ka = 0; ka < NA; ++ka) Dft<NB, INV>::run(v + NB * ka);
@@ -89,28 +93,53 @@ __device__ __forceinline__ void wide_dft(float2* v, Before before, Between betwe
 
 template <int N, bool INV>
 __device__ __forceinline__ void wide_dft(float2* v) {
-  wide_dft<N, INV>(v, [](float2 x, int) { return x; }, [](float2 x, int) { return x; });
+  wide_dft<N, INV>(v, [](float2 x, int) { return x; },
+                   [](float2 x, int b, int ka) { return tw64<INV>(x, b * ka * (64 / N)); });
 }
 
-// Stage 2's twiddles of butterfly t: w^{NB a t} (a = 1 .. NA-1) and w^{b t}
-// (b = 1 .. NB-1), w = exp(-2 pi i / (RA RB)).  In memory (FP64-built): row r
-// of RA entries per exponent factor, the b rows first.
+// Stage 2's twiddles of butterfly t, w = exp(-2 pi i / (RA RB)): w^{NB a t} (a = 1 .. NA-1)
+// and w^{b (t + RA ka)} (b = 1 .. NB-1), which is w^{b t} times the RB-point DFT's own factor.
+// In memory (FP64-built): a row of RA entries per (b, ka), then one per a.
 template <int RA, int RB> struct WideTw {
   static constexpr int NA = WideSplit<RB>::NA, NB = WideSplit<RB>::NB;
-  static constexpr int ROWS = NA + NB - 2;
+  static constexpr int ROWS = NB * NA - 1;
   static constexpr int SIZE = ROWS * RA;
-  float2 wa[NA - 1], wb[NB - 1];
+  float2 wa[NA - 1];
+  const float2* wb;
   __device__ __forceinline__ void load(const float2* __restrict__ tw, int t) {
+    wb = tw + t;
 #pragma unroll
-    for (int b = 1; b < NB; ++b) wb[b - 1] = __ldg(tw + (b - 1) * RA + t);
-#pragma unroll
-    for (int a = 1; a < NA; ++a) wa[a - 1] = __ldg(tw + (NB - 2 + a) * RA + t);
+    for (int a = 1; a < NA; ++a) wa[a - 1] = __ldg(tw + ((NB - 1) * NA + a - 1) * RA + t);
   }
   // the twiddled RB-point DFT
   template <bool INV> __device__ __forceinline__ void dft(float2* v) const {
     wide_dft<RB, INV>(
         v, [&](float2 x, int a) { return a == 0 ? x : cmul(x, INV ? cconj(wa[a - 1]) : wa[a - 1]); },
-        [&](float2 x, int b) { return b == 0 ? x : cmul(x, INV ? cconj(wb[b - 1]) : wb[b - 1]); });
+        [&](float2 x, int b, int ka) {
+          if (b == 0) return x;
+          const float2 w = __ldg(wb + ((b - 1) * NA + ka) * RA);
+          return cmul(x, INV ? cconj(w) : w);
+        });
+  }
+};
+
+// The same with w^{b t} alone, in registers, and the DFT's own factor multiplied after it; from
+// the ka = 0 rows of the same table.
+template <int RA, int RB> struct WideTwPair {
+  static constexpr int NA = WideSplit<RB>::NA, NB = WideSplit<RB>::NB;
+  float2 wa[NA - 1], wb[NB - 1];
+  __device__ __forceinline__ void load(const float2* __restrict__ tw, int t) {
+#pragma unroll
+    for (int b = 1; b < NB; ++b) wb[b - 1] = __ldg(tw + (b - 1) * NA * RA + t);
+#pragma unroll
+    for (int a = 1; a < NA; ++a) wa[a - 1] = __ldg(tw + ((NB - 1) * NA + a - 1) * RA + t);
+  }
+  template <bool INV> __device__ __forceinline__ void dft(float2* v) const {
+    wide_dft<RB, INV>(
+        v, [&](float2 x, int a) { return a == 0 ? x : cmul(x, INV ? cconj(wa[a - 1]) : wa[a - 1]); },
+        [&](float2 x, int b, int ka) {
+          return tw64<INV>(b == 0 ? x : cmul(x, INV ? cconj(wb[b - 1]) : wb[b - 1]), b * ka * (64 / RB));
+        });
   }
 };
 

@@ -40,13 +40,13 @@ __global__ void k_make_stage_tw(float2* out, int R) {
 }
 
 // Stage 2's twiddles of the (ra, rb) line FFT (fft_wide.cuh), rb = na nb: row
-// b - 1 (b = 1 .. nb-1) holds w^{b t}, row nb - 2 + a (a = 1 .. na-1) w^{nb a t},
-// t < ra, w = exp(-2 pi i / (ra rb)).
+// (b - 1) na + ka (b = 1 .. nb-1, ka < na) holds w^{b (t + ra ka)}, row (nb - 1) na + a - 1
+// (a = 1 .. na-1) w^{nb a t}, t < ra, w = exp(-2 pi i / (ra rb)).
 __global__ void k_make_wide_tw(float2* out, int ra, int rb, int na, int nb) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (na + nb - 2) * ra) return;
+  if (i >= (nb * na - 1) * ra) return;
   const int row = i / ra, t = i % ra;
-  const int e = row < nb - 1 ? (row + 1) * t : nb * (row - nb + 2) * t;
+  const int e = row < (nb - 1) * na ? (row / na + 1) * (t + ra * (row % na)) : nb * (row - (nb - 1) * na + 1) * t;
   double s, c;
   sincospi(-2.0 * (double)e / (double)(ra * rb), &s, &c);
   out[i] = make_float2((float)c, (float)s);

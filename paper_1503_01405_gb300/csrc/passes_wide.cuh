@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(WIDE_NT, 3) k_inv_cols_det_w(const float2* __r
   }
   // stage 2's thread: column t, half h (lane bit 4) of the lines
   const int t2 = (tid & 15) | ((tid >> 5) << 4), h = (tid >> 4) & 1;
-  WideTw<RA, RB> w2;
+  WideTwPair<RA, RB> w2;
   {
     // stage 1 straight from global memory: butterfly t of line ci (sub-channels
     // fastest, so consecutive lanes read consecutive elements) reads rows t + RB j
@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(WIDE_NT, MODE == ROW_SPECTRUM && R1 > 1024 ? 3
     const float2* un = uni + slot * 16;
     wide_dft<64, false>(
         v, [&](float2 x, int a) { return a == 0 ? x : cmul(x, un[8 + a]); },
-        [&](float2 x, int b) { return cmul(x, b == 0 ? wt : cmul(wt, un[b])); });
+        [&](float2 x, int b, int ka) { return tw64<false>(cmul(x, b == 0 ? wt : cmul(wt, un[b])), b * ka); });
     float2* dst = sm + slot * rt.rstr + 65 * t;
 #pragma unroll
     for (int j = 0; j < 64; ++j) dst[j] = v[j];
@@ -720,7 +720,7 @@ __global__ void __launch_bounds__(WIDE_NT, 2)
     for (int b = 0; b < 8; ++b) wb[b] = tw3(st3, m2 * (unsigned)(t + RB * b));
     wide_dft<RA, true>(
         v, [&](float2 x, int a) { return a == 0 ? x : cmul(x, wa[a - 1]); },
-        [&](float2 x, int b) { return cmul(x, wb[b]); });
+        [&](float2 x, int b, int ka) { return tw64<true>(cmul(x, wb[b]), b * ka); });
     float2* dst = sm + line * WSTR + (RA + 1) * t;
 #pragma unroll
     for (int j = 0; j < RA; ++j) dst[j] = v[j];
