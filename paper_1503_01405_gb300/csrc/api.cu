@@ -2014,8 +2014,8 @@ static int candidates_impl(pond_t h, pond_cnn_t net, double threshold, pond_cand
     return fail(POND_E_CUDA, "gather series: %s", cudaGetErrorString(e));
   }
   int rc = run_boxcar(blk, ntr, n, n, threshold, out, cap, n_found, h->st);
-  const size_t m = std::min(*n_found, cap);
-  if (net && m > 0 && (rc == POND_OK || rc == POND_E_OVERRUN)) {
+  const size_t m = rc == POND_OK ? *n_found : 0;   // after an overrun out holds no candidates
+  if (net && m > 0) {
     const int maxb = cnn_max_batch(net);
     std::vector<int32_t> corners(2 * m);
     for (size_t i = 0; i < m; ++i) {

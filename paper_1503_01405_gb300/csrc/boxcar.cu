@@ -795,11 +795,11 @@ int deliver(std::vector<pond_cand>& v, unsigned long long found, long long dcap,
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return set_error(POND_E_CUDA, cudaGetErrorString(e));
   }
+  *n_found = (size_t)found;
   if (found > (unsigned long long)dcap) return set_error(POND_E_OVERRUN, "boxcar: more candidates than capacity");
   std::sort(v.begin(), v.end(), [](const pond_cand& x, const pond_cand& y) {
     return x.trial != y.trial ? x.trial < y.trial : x.index < y.index;
   });
-  *n_found = v.size();
   if (v.size() > cap) return set_error(POND_E_OVERRUN, "boxcar: more candidates than capacity");
   std::copy(v.begin(), v.end(), out);
   return POND_OK;

@@ -120,6 +120,34 @@ def test_many_short_rows(n):
     assert got == [c for c in want if c[0] in some]
 
 
+@pytest.mark.parametrize("cap", [3, 1500], ids=["within_scratch", "beyond_scratch"])
+def test_more_candidates_than_room(cap):
+    """An overrun reports the number found and touches nothing of the caller's array, from the
+    detector and from a plan's series."""
+    import ctypes
+
+    import torch
+    rng = np.random.default_rng(2)
+    block = (100 + 3 * rng.standard_normal((1 if cap == 3 else 120, 20000))).astype(np.float32)
+    block[:, 100::300 if cap == 3 else 130] += 80
+    found = len(gpu_detect(block))
+    assert found > cap
+    d = torch.from_numpy(block).cuda()
+    out = (pond.pond_cand * cap)()
+    ctypes.memset(out, 0x7f, ctypes.sizeof(out))
+    before, nf = bytes(out), ctypes.c_size_t()
+    rc = pond.lib().pond_boxcar(d.data_ptr(), *block.shape, block.shape[1], 6.0, out, cap, ctypes.byref(nf), None)
+    assert rc == pond.POND_E_OVERRUN and nf.value == found and bytes(out) == before
+    x = torch.randint(-60, 61, (1 << 22,), dtype=torch.int8)
+    x[::65536] = 127
+    with pond.Engine(326.5, 16.0, 32e6, 0.0, 1 << 14, 4, 1, 1.0, t_dec=1e-6, dms=[0.0, 0.001]) as e:
+        e.push(x.numpy())
+        e.flush()
+        rc = pond.lib().pond_candidates(e._h, 3.0, out, 2, ctypes.byref(nf))
+        assert rc == pond.POND_E_OVERRUN and nf.value > 2 and bytes(out) == before
+        assert nf.value == len(e.candidates(3.0))
+
+
 def test_screened_and_dense_forms_agree():
     """A threshold below 1 evaluates every point; its list cut at S/N 6 is the screened
     list, also where rows hold infinities or NaN (and an overflowing list takes the dense form)."""
