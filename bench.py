@@ -41,12 +41,14 @@ sys.path.insert(0, ROOT)
 METRIC = "Msamples/s dedisperse+detect+fold (×real-time) and % HBM roofline vs plain FP32"
 UNIT = "Msamples/s"
 F0, BW, FS = 326.5, 16.0, 32e6
-# kernel behind each stage name of pond_stats
-KERNEL_OF_STAGE = {"fwd_cols_unpack": "k_fwd_cols", "fwd_rows_split": "k_fwd_rows",
-                   "fwd_rows_chirp_inv": "k_fwd_rows_inv", "inv_rows_chirp": "k_inv_rows_chirp",
+# kernel behind each stage name of pond_stats, at the full-rate plans' sizes.  The line keeps the
+# label k_fwd_rows_inv for the fused row pass, which k_fwd_rows_w runs
+KERNEL_OF_STAGE = {"fwd_cols_unpack": "k_fwd_cols", "fwd_rows_split": "k_fwd_rows_w",
+                   "fwd_rows_chirp_inv": "k_fwd_rows_inv", "inv_rows_chirp": "k_inv_rows_table",
                    "inv_cols_chirp": "k_inv_cols",
-                   "inv_rows_detect": "k_inv_rows", "inv_cols_detect": "k_inv_cols_det",
+                   "inv_rows_detect": "k_inv_rows", "inv_cols_detect": "k_inv_cols_det_w",
                    "fold": "k_fold_dec", "decimate": "k_decimate"}
+RUN_AS = {"k_fwd_rows_inv": "k_fwd_rows_w"}
 PLAN = dict(dm=26.8, nfft=1 << 24, nchan=64, nbins=1024, period=0.7145, t_dec=61.44e-6)
 REALTIME_MSPS = FS / 1e6
 
@@ -294,9 +296,11 @@ def pass_sources_hash(root: str | None = None) -> str:
     """Hash of the pass sources (the kernels the traffic counters describe)."""
     import hashlib
     h = hashlib.sha256()
-    for f in ("passes.cuh", "fft_block.cuh", "tc_dft.cuh"):
-        with open(os.path.join(root or ROOT, "paper_1503_01405_gb300", "csrc", f), "rb") as fh:
-            h.update(fh.read())
+    for f in ("passes.cuh", "fft_block.cuh", "tc_dft.cuh", "passes_wide.cuh", "fft_wide.cuh"):
+        path = os.path.join(root or ROOT, "paper_1503_01405_gb300", "csrc", f)
+        if os.path.exists(path):
+            with open(path, "rb") as fh:
+                h.update(fh.read())
     return h.hexdigest()[:16]
 
 
@@ -599,7 +603,7 @@ def run_incoherent(args, rank, ws, dist):
     value = ws * n * args.steps / (ms / 1e3) / 1e6
     info = eng.info()   # the last timed run: CUDA events around each stage on its stream
     peaks = measured_peaks()
-    stages = {"filterbank": (info["ms_filterbank"], info["algo_bytes_filterbank"], "k_fb_power"),
+    stages = {"filterbank": (info["ms_filterbank"], info["algo_bytes_filterbank"], "k_fb_power_w"),
               "dedisperse": (info["ms_dedisperse"], info["algo_bytes_dedisperse"], "k_incoh_sum")}
     dom = max(stages, key=lambda k: stages[k][0])
     t_ms, nbytes, kname = stages[dom]
@@ -951,7 +955,7 @@ def roofline(stages: dict, t_steps: int, ms_step: float, n: int, ch: int, st: di
             "peak_src": "nominal FP32 (152 SMs x 128 lanes x 2 flop x 2.07 GHz)",
             "peak_measured": fp32["tflops"], "frac_of_measured": achieved / fp32["tflops"],
             # the committed counters are of the single-channel launches
-            "traffic": traffic_from_profiles(kname) if ch == 1 else None,
+            "traffic": traffic_from_profiles(RUN_AS.get(kname, kname)) if ch == 1 else None,
             "kernel": kname, "algo_flops_per_launch": d["algo_flops"], "launch_us": avg_s * 1e6,
             "algo_hbm_gbs": seg_bytes / avg_s / 1e9, "algo_hbm_frac": seg_bytes / avg_s / 1e9 / peaks["hbm_gbs"],
             "pass_bytes_gbs": d["pass_bytes"] / avg_s / 1e9,

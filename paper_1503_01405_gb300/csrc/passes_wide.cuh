@@ -261,8 +261,8 @@ __device__ __forceinline__ void make_twk(float2* twk, const Tw2& tw2L, int nl, R
 // barrier after the tile's load.  Bound by the issue slots (chirp and DFT, 34
 // instructions per value) next to the 64 MiB that each trial writes (4.8 TB/s).
 // Full-rate batched plan: 19.9 us per trial with the runs split over four lanes
-// and exchanged through shared memory (78 % of that pipe), 13.5 here; the 8 s
-// chunk of 128 trials 126 -> 103 ms.
+// and exchanged through shared memory (78 % of that pipe), 13.5 here (16 in a launch of 16 trials
+// that starts with a cold L2); the 8 s chunk of 128 trials 126 -> 103 ms on the device.
 constexpr int TAB_GROUPS = 3;   // 384 threads of 168 registers: one CTA per SM
 
 template <int R1>
@@ -462,9 +462,10 @@ enum RowMode { ROW_SPECTRUM = 0, ROW_ANCHORS = 1, ROW_TABLE = 2 };
 // three for rows of 2048 and 4096 points (33.3 us against 36.9 per 2^23 bins); shorter rows
 // belong to segments of at most 128 tiles, which do not fill the SMs once, and take
 // the registers instead (2^20 bins beside another trial's passes: 8.0 us against 12.2).
-// Bound by instruction issue (43 %) and memory latency in turn.  Full rate, launches of
-// four 2^24-point segments: 56.0 -> 45 us per segment; 24.8 M warp
-// instructions per segment against 31.0 M with radix-16 stages.  blockIdx.x is
+// Bound by instruction issue (40 % in launches of four segments, 31 % in one's) and memory
+// latency in turn.  Full rate, launches of four 2^24-point segments: 56 -> 47 us per
+// segment; 22.6 M warp instructions per segment against 31.0 M with radix-16 stages.  A launch of one
+// segment has 3.4 waves and takes 71 us where 512 threads per tile took 69.  blockIdx.x is
 // the segment and runs fastest, so the segments of a launch share the chirp table's
 // rows in L2 (launches of four: 215 -> 188 us).
 template <int R1, int MODE>
