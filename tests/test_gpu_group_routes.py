@@ -7,6 +7,7 @@ import pytest
 
 from oracle import pcd
 from paper_1503_01405_gb300 import pond, synth
+from test_gpu_parity import CONFIGS, THREE_PASS, _stream, check, run_engine
 
 pytestmark = pytest.mark.gpu
 
@@ -34,6 +35,15 @@ def cut(x, sizes):
         n = sizes.pop(0) if sizes else len(x) - a
         yield x[a:a + n]
         a += n
+
+
+@pytest.mark.parametrize("cfg", CONFIGS + THREE_PASS, ids=lambda c: f"N{c[0]}_c{c[1]}_dm{c[2]}_bw{c[3]}")
+def test_grouped_plans_match_oracle(cfg):
+    """The parity suite's plans without voltages, which launch groups of segments."""
+    nfft, nchan, dm, bw, nbins, period = cfg
+    p = pcd.make_plan(326.5, bw, 32e6, dm, nfft, nchan, nbins, period)
+    x = _stream(p, seed=nfft + nchan, extra=17)
+    check(run_engine(x, p, want_voltages=False, device_push=True), pcd.run(p, x), voltages=False)
 
 
 @pytest.mark.parametrize("ch", [1, 2], ids=["one_channel", "pairs"])
